@@ -47,6 +47,26 @@ def test_random_grids_match_oracle_bit_for_bit(ccm):
         ccm.ccm_context_destroy(ctx)
 
 
+@pytest.mark.parametrize("r", [2, 31, 64, 65, 255, 256, 257, 300])
+def test_group_sizes_around_the_sorts(ccm, r):
+    """Sizes at the edges of the in-register and block-wide sorts, with zeros of
+    both signs (equal), infinities (left out), a constant group and a group
+    without a value."""
+    rng = np.random.default_rng(r)
+    rho = rng.normal(0.0, 0.3, size=(4, 9, r))
+    rho[0] = np.round(rho[0], 1) * np.where(rng.random((9, r)) < 0.5, 1.0, -1.0)
+    rho[1, 3:6] = 0.5
+    rho[2, 4] = np.nan
+    rho[3, :, ::5] = np.where(rng.random((9, (r + 4) // 5)) < 0.5, np.inf, -np.inf)
+    L = np.array([70, 10, 60, 20, 50, 30, 40, 90, 80])
+    ctx = ccm.ccm_context_create(0)
+    try:
+        got = as_rows(ccm.ccm_convergence(ctx, rho, L))
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    assert same(got, oracle.convergence(rho, L))
+
+
 def test_sweep_rho_on_device(ccm):
     torch = pytest.importorskip("torch")
     base = I.sweep_problem()

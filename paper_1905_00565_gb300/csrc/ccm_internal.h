@@ -62,18 +62,37 @@ struct ObsJob {
 // (zero past the tile's end), then mean(x) and sum of (x_q - mean(x))^2.
 constexpr int kObsStride = 264;        // doubles per record (64-byte multiple)
 
-// One work item of the fused kernels: query tiles [tile, tile + chunk) of a
-// unit (chunk = kBruteChunk for the brute-force kernel, kTableChunk for the
-// table kernel; the last item of a unit may hold fewer tiles).
+// One work item of the fused kernels: query tiles of a unit, from `tile` on.  A
+// brute-force item holds up to `count` tiles (brute_chunk), a table item up to
+// kTableChunk; the last item of a unit may hold fewer.
 // A table item may cover `count` consecutive realizations of one cell (units
 // unit .. unit + count - 1): one walk of each query's table row serves all of
-// them.  Brute-force items have count 1.
+// them.
 struct WorkItem {
   int32_t unit;
   int32_t tile;
   int32_t count;
 };
-constexpr int kBruteChunk = 8;         // query tiles per brute-force work item (one staging)
+constexpr int kBruteChunk = 8;         // query tiles per brute-force work item, at most
+// Points of a staged library tile in the brute-force kernel: kTileBytes of
+// packed coordinate pairs (padded to even E) and indices, whole warps of them.
+constexpr int kTileBytes = 20 * 1024;
+constexpr int brute_tile_points(int E) {
+  return (kTileBytes / ((E + (E & 1)) * 8 + 8)) * 2 / 64 * 64;
+}
+// Query tiles per brute-force item, for libraries of L points in a launch of
+// `tiles` tiles.  An item is the unit of balance, and a launch of few
+// realizations has too few of eight tiles for the 152 SMs x 3 CTA slots (50
+// realizations of N = 10^4, L = 1500: 250 items of 8 tiles 620 us, 2000 items
+// 440 us).  A library that fits one staged tile is staged once per item (3-8 %
+// of a tile's time), so there one item per slot is enough: with eight, 2400
+// tiles of N = 1000 and L <= 200 took 1.5 % longer.  Longer libraries are
+// staged for every tile anyway and are split to eight items per slot.
+constexpr int64_t kBruteSlots = 3 * 152;
+inline int32_t brute_chunk(int64_t tiles, int64_t L, int E) {
+  const int64_t c = tiles / (L <= brute_tile_points(E) ? kBruteSlots : 8 * kBruteSlots);
+  return c < 1 ? 1 : c > kBruteChunk ? kBruteChunk : (int32_t)c;
+}
 constexpr int kTableGroup = 4;         // realizations per grouped table item, at most
 constexpr int kTableGroupMaxNm = 32768;  // grouping needs a byte membership map (bit b: realization b)
 

@@ -10,7 +10,7 @@
 //
 // Design (GB300, FP32 on the CUDA cores; E <= 10 is not a dense contraction):
 //  * persistent CTAs pull work items, sorted by cost, from an atomic counter;
-//    a brute-force item is up to eight query tiles of one realization, so a
+//    a brute-force item is one to eight query tiles of one realization, so a
 //    library that fits one shared-memory tile is staged once for all of them;
 //  * each thread owns one query; library points sit in shared memory in
 //    pairs, packed {a_e, b_e} per coordinate, so one sub.f32x2 + fma.f32x2
@@ -83,7 +83,8 @@ struct TileShape {
   static constexpr int EP = E + (E & 1);                        // coordinates padded to even
   static constexpr int D = E < 3 ? E : 3;                       // coordinates a chunk box bounds
   // library points per tile: a point pair takes EP*8 bytes of coordinates + 8 of indices
-  static constexpr int LT = ((kCoordBytes - kBoxBytes) / (EP * 8 + 8)) * 2 / 64 * 64;
+  static constexpr int LT = brute_tile_points(E);
+  static_assert(kTileBytes == kCoordBytes - kBoxBytes, "the tile fills its region");
   static_assert(LT >= 64 && LT % 32 == 0, "tile must hold whole warps of chunks");
   static_assert((LT / kChunk) * 2 * D * 4 <= kBoxBytes, "chunk boxes must fit");
 };
@@ -567,8 +568,8 @@ __device__ __forceinline__ void sort_column(u64* col, int n) {
   }
 }
 
-// Brute-force search of one work item: query tiles [tile0, tile0 +
-// kBruteChunk) of a unit.  When the whole library fits one shared-memory tile
+// Brute-force search of one work item: query tiles [tile0, tile0 + n_chunk)
+// of a unit.  When the whole library fits one shared-memory tile
 // it is staged once for all of them; each warp starts its scan at the library
 // run nearest its own 32 queries (the library is in query order) and wraps
 // around.  Larger libraries are staged tile by tile for every query tile.
@@ -588,7 +589,7 @@ __device__ __forceinline__ void sort_column(u64* col, int n) {
 // exactly the list the sorted insertion of every candidate would give.
 template <int E, int V, bool kStats>
 __device__ void process_item(const KnnParams& p, const UnitDesc& u, int unit, int tile0,
-                             unsigned char* smem, RingMeta* meta, int& ring_n) {
+                             int n_chunk, unsigned char* smem, RingMeta* meta, int& ring_n) {
   constexpr int K = E + 1;  // the window keeps m itself out, so E+1 slots suffice
   constexpr int EP = TileShape<E>::EP;
   constexpr int LT = TileShape<E>::LT;
@@ -628,7 +629,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int unit, in
   static_assert(kInit <= kChunk, "the initial points lie in the first chunk");
   u64* col = s_buf + tid;  // this thread's candidate column
 
-  const int tile1 = min(u.n_tiles, tile0 + kBruteChunk);
+  const int tile1 = min(u.n_tiles, tile0 + n_chunk);
   if (single) {
     __syncthreads();  // the previous item's readers of the tile are done
     stage_library<E>(sj, lib, off, tau, 0, L, s_coord, s_lidx, s_box);
@@ -1207,9 +1208,9 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
       continue;
     }
     if (p.variant[E] == 1)
-      process_item<E, 1, kStats>(p, u, w.unit, w.tile, smem, s_meta, ring_n);
+      process_item<E, 1, kStats>(p, u, w.unit, w.tile, w.count, smem, s_meta, ring_n);
     else
-      process_item<E, 0, kStats>(p, u, w.unit, w.tile, smem, s_meta, ring_n);
+      process_item<E, 0, kStats>(p, u, w.unit, w.tile, w.count, smem, s_meta, ring_n);
   }
   if (ring_n > 0)
     flush_ring(p, reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);

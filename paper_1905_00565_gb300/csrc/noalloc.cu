@@ -78,6 +78,7 @@ struct CellArgs {
   int64_t n;
   uint64_t seed;
   int32_t j, i, E, tau, L, r, n_m, n_tiles;
+  int32_t chunk;  // query tiles per work item
 };
 
 // Writes the descriptors and work items of the cell into the scratch and
@@ -86,13 +87,13 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, 
   UnitDesc* units = reinterpret_cast<UnitDesc*>(scratch + lay.units);
   WorkItem* items = reinterpret_cast<WorkItem*>(scratch + lay.items);
   uint32_t* done = reinterpret_cast<uint32_t*>(scratch + lay.done);
-  const int64_t per_unit = (c.n_tiles + kBruteChunk - 1) / kBruteChunk;  // items per realization
+  const int64_t per_unit = (c.n_tiles + c.chunk - 1) / c.chunk;  // items per realization
   const int64_t n_items = (int64_t)c.r * per_unit;
   for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < n_items;
        w += (int64_t)gridDim.x * blockDim.x) {
     items[w].unit = (int32_t)(w / per_unit);
-    items[w].tile = (int32_t)((w % per_unit) * kBruteChunk);
-    items[w].count = 1;
+    items[w].tile = (int32_t)((w % per_unit) * c.chunk);
+    items[w].count = c.chunk;
   }
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < c.r;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -221,6 +222,7 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   c.r = r;
   c.n_m = (int32_t)n_m;
   c.n_tiles = (int32_t)n_tiles;
+  c.chunk = brute_chunk(r * n_tiles, L, E);
   noalloc_setup_kernel<<<(unsigned)((r * n_tiles + 255) / 256), 256, 0, s>>>(scratch, lay, c);
   e = launch_order(d_series, reinterpret_cast<const OrderJob*>(scratch + lay.orderjob), 1,
                    (int)n_m, reinterpret_cast<int32_t*>(scratch + lay.order), nullptr, s);
@@ -242,7 +244,7 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   kp.units = reinterpret_cast<const UnitDesc*>(scratch + lay.units);
   kp.targets = reinterpret_cast<const TargetDesc*>(scratch + lay.target);
   kp.items = reinterpret_cast<const WorkItem*>(scratch + lay.items);
-  kp.n_items = (int64_t)r * ((n_tiles + kBruteChunk - 1) / kBruteChunk);
+  kp.n_items = (int64_t)r * ((n_tiles + c.chunk - 1) / c.chunk);
   kp.lib = reinterpret_cast<const int32_t*>(scratch + lay.lib);
   kp.order = reinterpret_cast<const int32_t*>(scratch + lay.order);
   kp.partials = reinterpret_cast<double*>(scratch + lay.part);

@@ -388,14 +388,26 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           ul->tables.push_back(tj);
         }
   }
+  // Query tiles per brute-force item, from the tiles of each E's launch.
+  std::map<int32_t, int64_t> brute_tiles;
+  for (int32_t j : lib_vars)
+    for (int32_t E : pc.E)
+      for (int32_t tau : pc.tau) {
+        const int64_t n_m = pc.n - (int64_t)(E - 1) * tau;
+        const bool tab = table_of.count(std::make_tuple(j, E, tau)) != 0;
+        for (int64_t L : pc.L)
+          if (!tab || (double)L < table_min_L(E, n_m, tt))
+            brute_tiles[E] += (n_m + tileq - 1) / tileq * pc.r;
+      }
   for (int32_t j : lib_vars) {
     const std::vector<int64_t>& tp = pairs_of[j];
     for (int64_t e = 0; e < nE; ++e)
       for (int64_t t = 0; t < nT; ++t)
-        for (int64_t l = 0; l < nL; ++l)
+        for (int64_t l = 0; l < nL; ++l) {
+          const int32_t E = pc.E[(size_t)e], tau = pc.tau[(size_t)t];
+          const int64_t L = pc.L[(size_t)l];
+          const int32_t chunk = brute_chunk(brute_tiles[E], L, E);
           for (int32_t k = 0; k < pc.r; ++k) {
-            const int32_t E = pc.E[(size_t)e], tau = pc.tau[(size_t)t];
-            const int64_t L = pc.L[(size_t)l];
             UnitDesc u;
             std::memset(&u, 0, sizeof(u));
             u.series_off = series_off;
@@ -456,11 +468,11 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
                     (double)nq * 12.0 * (E + 2) * (double)u.n_m / (double)L * (1.0 + 0.1 * count) +
                     (double)u.n_targets * nq * 64.0 * count;
               } else {
-                // one item per kBruteChunk tiles: one library staging (when it
+                // one item per `chunk` tiles: one library staging (when it
                 // fits a shared-memory tile), then per tile the search and the
                 // per-target epilogue
-                if (q % kBruteChunk == 0) {
-                  ul->items.push_back(WorkItem{uidx, q, 1});
+                if (q % chunk == 0) {
+                  ul->items.push_back(WorkItem{uidx, q, chunk});
                   ul->item_cost.push_back(64.0 * E * (double)L);
                 }
                 ul->item_cost.back() += (double)L * (double)nq * (2.0 * E + 1.0) +
@@ -483,6 +495,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             ul->flops += 3.0 * E * (double)u.n_m * (double)L;
             ul->units.push_back(u);
           }
+        }
   }
 }
 

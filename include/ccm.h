@@ -25,10 +25,12 @@
  *       optionally raised to a floor f (ccm_problem.weight_floor),
  *       w_i = u_i / sum u, Xhat(m) = sum_i w_i s_i[t_i];
  *     - the skill rho = Pearson(s_i[t_m], Xhat(m)) over m (Sect. 2.1),
- *       accumulated in FP64; NaN when either variance is zero.
+ *       accumulated in FP64 precision; NaN when either variance is zero.
  *
  * Precision: distances, selection, weights and predictions in FP32;
- * rho moments in FP64.
+ * rho moments in FP64 and, for the predictions' sums over a tile of 256
+ * queries, in unevaluated pairs of FP32 numbers (48 bits, the target scaled by
+ * a power of two).
  *
  * Output layout: rho[pair][E][tau][L][k], FP64, C order, where the axes index
  * the arrays of ccm_problem in the order given.
@@ -161,7 +163,7 @@ ccm_status ccm_plan_destroy(ccm_plan_t* plan);
 
 ccm_status ccm_plan_get_info(const ccm_plan_t* plan, ccm_plan_info* info);
 
-/* Run the whole sweep: query order, observed-value tile moments (the target's
+/* Run the whole sweep: query order, observed-value tile records (the target's
  * mean and centred values per query tile of each (pair, E, tau), shared by
  * every L and realization), distance indexing tables (unless
  * CCM_NO_TABLE or none pays off), library sampler, one persistent fused
@@ -195,8 +197,9 @@ ccm_status ccm_run_ex(ccm_plan_t* plan, const float* series, double* rho,
 ccm_status ccm_plan_kernel_times(const ccm_plan_t* plan, double* sampler_ms, double* knn_ms);
 
 /* The same events per stage: stage_ms[0] query order + observed-value tile
- * moments + distance indexing tables, [1] library sampler, [2] brute-force fused kernel, [3] table-scan
- * fused kernel (0 when the stage launched nothing). */
+ * records + distance indexing tables, [1] library sampler, [2] brute-force
+ * fused kernel, [3] table-scan fused kernel and the merge of the tiles' moments
+ * into rho. */
 ccm_status ccm_plan_stage_times(const ccm_plan_t* plan, double* stage_ms /* [4] */);
 
 /* Work counts of the neighbour search in the plan's last completed run
@@ -266,8 +269,8 @@ ccm_status ccm_job_times(ccm_context* ctx, uint64_t ticket, double* submit_s, do
  * d_series: device [n_series][n] FP32 (not checked for non-finite values);
  * d_rho: device [r] FP64, written in stream order.  All scratch lives in one
  * fixed 16 MiB device array held by every GPU that loads the library until
- * exit; a cell needing more (about r*L*4 + r*ceil(N_m/256)*56 + r*160 +
- * N_m*4 + ceil(N_m/256)*2112 bytes) returns CCM_ETOOLARGE with a message and runs nothing.  Nothing is
+ * exit; a cell needing more (about r*L*4 + r*ceil(N_m/256)*44 + r*176 +
+ * N_m*4 + ceil(N_m/256)*2080 bytes) returns CCM_ETOOLARGE with a message and runs nothing.  Nothing is
  * allocated.  The first call on a device (with that device current) finds
  * the array's address and sets kernel attributes; make it before any stream
  * capture.  Every call reuses the same array: calls that overlap on the GPU

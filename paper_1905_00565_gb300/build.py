@@ -1,6 +1,6 @@
 """Build ``libccm_gb300.so`` in-tree with nvcc for sm_103a.
 
-Each CUDA translation unit is compiled in parallel (one ``-gencode`` for
+Each CUDA translation unit (the search kernels: one per E) is compiled in parallel (one ``-gencode`` for
 sm_103a, ``-lineinfo``, IEEE FP32: no fast-math, so ``sqrtf``, division and
 ``expf`` keep their documented accuracy) and linked with the static CUDA
 runtime into one shared library exporting the C ABI of include/ccm.h.
@@ -19,8 +19,12 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libccm_gb300.so")
-SOURCES = ["runtime.cu", "sampler.cu", "knn_fused.cu", "plain.cu", "noalloc.cu", "order.cu",
-           "table.cu", "convergence.cu"]
+# (source, E): the search kernels are compiled once per embedding dimension, in parallel
+SOURCES = [("knn_fused.cu", e) for e in range(10, 0, -1)] + [
+    (name, 0) for name in ("table.cu", "runtime.cu", "sampler.cu", "knn_dispatch.cu", "plain.cu",
+                           "noalloc.cu", "order.cu", "convergence.cu")]
+HEADERS = [os.path.join(CSRC, "ccm_internal.h"), os.path.join(CSRC, "moments.cuh"),
+           os.path.join(INCLUDE, "ccm.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -29,13 +33,13 @@ def _nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
-def _compile(src: str, verbose: bool) -> str:
-    obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
-    deps = [os.path.join(CSRC, src), os.path.join(CSRC, "ccm_internal.h"),
-            os.path.join(INCLUDE, "ccm.h")]
+def _compile(src: str, E: int, verbose: bool) -> str:
+    obj = os.path.join(BUILD, os.path.splitext(src)[0] + (f"_e{E}" if E else "") + ".o")
+    deps = [os.path.join(CSRC, src), *HEADERS]
     if os.path.exists(obj) and os.path.getmtime(obj) >= max(os.path.getmtime(d) for d in deps):
         return obj
     cmd = [_nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
+           *([f"-DCCM_E={E}"] if E else []),
            *os.environ.get("CCM_EXTRA_NVCC_FLAGS", "").split(),
            "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, src), "-o", obj + ".tmp"]
     if verbose:
@@ -56,7 +60,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         for f in os.listdir(BUILD):
             os.remove(os.path.join(BUILD, f))
     with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(lambda s: _compile(s, verbose), SOURCES))
+        objs = list(ex.map(lambda s: _compile(*s, verbose), SOURCES))
     if force or not os.path.exists(LIB) or os.path.getmtime(LIB) < max(os.path.getmtime(o) for o in objs):
         tmp = LIB + f".tmp{os.getpid()}"
         cmd = [_nvcc(), *ARCH, "-shared", "-Xcompiler", "-fPIC", "-cudart", "static", *objs,

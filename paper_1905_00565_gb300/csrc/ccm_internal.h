@@ -17,10 +17,11 @@ struct UnitDesc {
   int64_t series_off;   // element offset of the job's series block [V][n]
   int64_t n;            // series length of the job
   int64_t lib_off;      // offset of this unit's library in the library buffer
-  int64_t part_off;     // first partial-moment slot: target t, tile q at part_off + t*n_tiles + q
+  int64_t part_off;     // first partial-sum slot: target t, tile q at part_off + t*n_tiles + q
   int64_t order_off;    // first entry of this unit's query order (per variable, E, tau)
   int64_t tgt_off;      // first TargetDesc of this unit
   int64_t table_off;    // distance indexing table of (j, E, tau), when table_R > 0
+  int64_t st_off;       // the job's series by time, [n][st_stride] (n_targets >= kLaneTargets)
   uint64_t seed;        // library sampler seed of the job
   int32_t j;            // library variable
   int32_t E, tau;
@@ -32,7 +33,13 @@ struct UnitDesc {
   int32_t theiler;      // exclusion window W >= 0: candidates l of query m need |l - m| > W
   float wfloor;         // simplex weight floor f >= 0: u_i = max(u_i, f)
   int32_t table_tv;     // 1: the table also holds this unit's (single) target's values
+  int32_t st_stride;
+  int32_t pad;
 };
+// Units with at least this many targets form their predictions with one lane
+// per target (coalesced reads of the time-major series); fewer, one thread per
+// query and target after target.
+constexpr int kLaneTargets = 12;
 
 // One target of a unit: the pair (j, i) and where its outputs go.
 struct TargetDesc {
@@ -40,27 +47,46 @@ struct TargetDesc {
   int64_t q_off;        // first query of this pair-realization in the debug predictions
   int64_t nbr_off;      // first entry in the debug neighbour lists
   int64_t lib_dbg_off;  // first entry in the debug libraries
-  int64_t obs_tile;     // observed-moment record of query tile 0 of (j, i, E, tau)
+  int64_t obs_tile;     // observed-value record of query tile 0 of (j, i, E, tau)
   int32_t i;            // target variable
-  int32_t pad;
+  int32_t unit;         // the unit it belongs to
 };
 
-// Observed-moment job: one per (job, library variable j, target i, E, tau).
+// Observed-value job: one per (job, library variable j, target i, E, tau).
 // The observed values of a query tile (the target at the tile's manifold
 // points) do not depend on L or the realization, so their tile mean, centred
 // values and centred sum of squares are computed once per run and read by the
-// epilogue of every realization of that (j, i, E, tau).
+// epilogue of every realization of that (j, i, E, tau).  All values are scaled
+// by the target series' power of two (moments.cuh).
 struct ObsJob {
   int64_t series_off;   // element offset of the job's series block
   int64_t n;            // series length
   int64_t order_off;    // query order of (j, E, tau)
-  int64_t obs_tile;     // first tile record; the jobs' records are consecutive
+  int64_t obs_tile;     // first tile's ObsStat; the jobs' records are consecutive
+  int64_t a_off;        // centred values: element of query 0 of tile 0
+  int32_t a_step;       // 0: a tile's 256 values in obs_slot order; T > 0: query q of tile t at
+                        // a_off + (256t + q)*T (the T targets of a query side by side)
+  int32_t scale;        // index of the target series' scale
   int32_t i, E, tau, n_m, n_tiles;
   int32_t pad;
 };
-// One tile record: x_q - mean(x) for the tile's 256 queries in query order
-// (zero past the tile's end), then mean(x) and sum of (x_q - mean(x))^2.
-constexpr int kObsStride = 264;        // doubles per record (64-byte multiple)
+// One tile of an observed target: mean(x), sum of (x_q - mean(x))^2 and the
+// scale.  Beside it 256 float2 {h, l}, h + l = x_q - mean(x) to 48 bits (zero
+// past the tile's end).
+struct ObsStat {
+  double mx, sxx;
+  float scale;
+  float pad[3];
+};
+// Per-series preparation (one CTA of the order launch): the power of two that
+// brings the series' largest magnitude into [1, 2), and, for jobs with units
+// of kLaneTargets targets, the series' column of the time-major copy.
+struct SeriesJob {
+  int64_t off, n;       // the series
+  int64_t st_off;       // element of (t = 0, this variable) in the time-major copy; -1: none
+  int32_t st_stride;
+  int32_t scale;        // where the scale goes
+};
 
 // One work item of the fused kernels: query tiles of a unit, from `tile` on.  A
 // brute-force item holds up to `count` tiles (brute_chunk), a table item up to
@@ -145,15 +171,16 @@ struct KnnParams {
                             // layout; table_pairs: float2 {distance, target value} per entry
   int32_t table_pairs;    // 1: the tables store (distance, target value) pairs (TableJob::tv_i)
   int32_t table_u16;      // 1: uint16 entries (every manifold below 65536 points), 0: int32
-  double* partials;       // 6 doubles per query tile
-  const double* obs;      // observed-moment tile records (TargetDesc::obs_tile)
-  uint32_t* unit_done;    // per-unit tile counters (reset by the unit's last tile)
+  float4* partials;       // two float4 per (target, query tile): its sums (moments.cuh)
+  const float2* obs;      // centred observations, 256 per record (TargetDesc::obs_tile)
+  const ObsStat* obs_stat;  // one per record
+  const float* st;        // time-major series of jobs with units of kLaneTargets targets
   uint32_t* item_counter; // dynamic scheduling counter (zeroed before each launch)
-  double* rho;            // output (device), indexed by UnitDesc::out_idx
   int32_t* dbg_nbr;       // optional [sum N_m][E+1]
   float* dbg_xhat;        // optional [sum N_m]
   int32_t* err;
   unsigned long long* stats;  // optional search counters [kStatCount] (kStat*), nullptr: none
+  int32_t lane_scratch;   // table kernel: where the lane-per-target scratch starts in shared memory
   int32_t persistent;     // 1: CTAs pull items from item_counter; 0: item = blockIdx.x
   int32_t merge_at[kMaxE + 1];  // per E: merge pending candidates once a lane holds this many
   int32_t variant[kMaxE + 1];   // per E: kernel variant (0 narrow, 1 wide); same results
@@ -225,8 +252,10 @@ cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t c
 
 // Query order (order.cu).
 cudaError_t order_prepare();
+// The same launch prepares the target series (SeriesJob).
 cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jobs, int max_nm,
-                         int32_t* order, unsigned long long* scratch, cudaStream_t s);
+                         int32_t* order, unsigned long long* scratch, const SeriesJob* series_jobs,
+                         int64_t n_series_jobs, float* scales, float* st, cudaStream_t s);
 
 // Distance indexing table (table.cu).
 cudaError_t table_prepare();
@@ -235,21 +264,41 @@ cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_
                                int max_nm, int max_R, const int32_t* order, void* table,
                                float* table_dist, int table_pairs, int table_u16, cudaStream_t s);
 
-// Fused kernel (knn_fused.cu).
+// Search kernels of one E (knn_fused.cu, compiled once per E; each kernel keeps
+// its registers for that E's lists).
+template <int E>
+struct KnnKernels {
+  static cudaError_t prepare();
+  static cudaError_t occupancy(int* ctas);
+  static cudaError_t launch(const KnnParams& p, bool lanes, int grid, cudaStream_t s);
+  static cudaError_t prepare_table();
+  static cudaError_t occupancy_table(int max_nm, bool lanes, int* ctas);
+  static cudaError_t launch_table(const KnnParams& p, int max_nm, bool lanes, int grid,
+                                  cudaStream_t s);
+};
+
+// Their dispatch, and what surrounds the search (knn_dispatch.cu).
 int knn_block_threads();
 int knn_queries_per_thread();
 cudaError_t knn_prepare();
 cudaError_t knn_occupancy(int E, int* ctas_per_sm);
-cudaError_t launch_knn(const KnnParams& p, int E, int grid, cudaStream_t s);
-// Observed-moment records of every ObsJob (after the query order): one warp
+// lane_targets: the launch's units have kLaneTargets targets or more (a kernel
+// of their own).
+cudaError_t launch_knn(const KnnParams& p, int E, bool lane_targets, int grid, cudaStream_t s);
+// Observed-value records of every ObsJob (after the query order): one warp
 // per tile, n_tiles tiles in all.
 cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* jobs,
-                       int64_t n_jobs, int64_t n_tiles, double* obs, cudaStream_t s);
+                       int64_t n_jobs, int64_t n_tiles, const float* scales, float2* obs,
+                       ObsStat* obs_stat, cudaStream_t s);
+// rho of every target from its tiles' sums (after the search kernels).
+cudaError_t launch_rho(const UnitDesc* units, const TargetDesc* targets, int64_t n_targets,
+                       const float4* partials, const ObsStat* obs_stat, double* rho,
+                       cudaStream_t s);
 // Table path: same work items, neighbours read from the distance indexing table.
-size_t knn_table_smem(int max_nm);
 cudaError_t knn_table_prepare();
-cudaError_t knn_table_occupancy(int max_nm, int* ctas_per_sm);
-cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, int grid, cudaStream_t s);
+cudaError_t knn_table_occupancy(int max_nm, bool lane_targets, int* ctas_per_sm);
+cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lane_targets, int grid,
+                             cudaStream_t s);
 
 // Sets the thread-local message returned by ccm_last_error() (runtime.cu).
 void set_last_error(const char* msg);

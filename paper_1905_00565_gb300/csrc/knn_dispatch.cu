@@ -1,0 +1,202 @@
+// Observed-value records, rho and the dispatch of the search kernels by E.
+#include "ccm_internal.h"
+#include "moments.cuh"
+
+namespace ccm {
+namespace {
+
+constexpr int kThreads = 256;
+constexpr unsigned kFull = 0xffffffffu;
+
+// Butterfly sum over the warp: every lane ends with the same bits (each
+// level adds the same two values in either order).
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(kFull, v, o));
+  return v;
+}
+
+constexpr int kPer = kQT / 32;  // queries per lane
+
+// Observed-value records (see ObsJob), one warp per tile: x_q is the target
+// at the tile's manifold points (Sect. 2.1: the value the cross map
+// predicts).  Two passes in FP64, then split into float pairs.
+__global__ void __launch_bounds__(kThreads) obs_kernel(const float* series, const int32_t* order,
+                                                      const ObsJob* jobs, int64_t n_jobs,
+                                                      int64_t n_tiles, const float* scales,
+                                                      float2* obs, ObsStat* obs_stat) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n_tiles;
+       g += n_warps) {
+    int64_t lo = 0, hi = n_jobs - 1;  // the job holding tile g: last obs_tile <= g
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) >> 1;
+      if (jobs[mid].obs_tile <= g) lo = mid;
+      else hi = mid - 1;
+    }
+    const ObsJob jb = jobs[lo];
+    const int tile = (int)(g - jb.obs_tile);
+    const int nq = min(kQT, jb.n_m - tile * kQT);
+    const float* si = series + jb.series_off + (int64_t)jb.i * jb.n;
+    const int32_t* ord = order + jb.order_off + (int64_t)tile * kQT;
+    const int off = (jb.E - 1) * jb.tau;
+    const float scale = scales[jb.scale];
+    double x[kPer];
+    double sv = 0.0;
+#pragma unroll
+    for (int c = 0; c < kPer; ++c) {
+      const int q = lane + 32 * c;
+      x[c] = (q < nq) ? (double)__fmul_rn(si[ord[q] + off], scale) : 0.0;
+      sv = __dadd_rn(sv, x[c]);
+    }
+    const double mx = __ddiv_rn(warp_sum(sv), (double)nq);
+    double sxx = 0.0;
+#pragma unroll
+    for (int c = 0; c < kPer; ++c) {
+      const int q = lane + 32 * c;
+      const double a = (q < nq) ? __dsub_rn(x[c], mx) : 0.0;
+      sxx = __fma_rn(a, a, sxx);
+      const float h = __double2float_rn(a);
+      const float2 v = make_float2(h, __double2float_rn(__dsub_rn(a, (double)h)));
+      if (jb.a_step == 0) obs[jb.a_off + (int64_t)tile * kQT + obs_slot(q)] = v;
+      else obs[jb.a_off + ((int64_t)tile * kQT + q) * jb.a_step] = v;
+    }
+    sxx = warp_sum(sxx);
+    if (lane == 0) {
+      ObsStat& o = obs_stat[g];
+      o.mx = mx;
+      o.sxx = sxx;
+      o.scale = scale;
+    }
+  }
+}
+
+// rho of one target: the tile moments merged.  With the grand means MX =
+// sum(n_t mx_t)/N, the centred sums are exactly
+//   Sxx = sum_t [Sxx_t + n_t (mx_t - MX)^2]   (likewise Syy, Sxy),
+// a sum of non-negative terms (no cancellation).  kRhoLanes lanes per target
+// take every kRhoLanes-th tile and are added in a fixed order, so rho does not
+// depend on which CTA ran which tile, or when.  A launch of its own: FP64
+// instructions cost the same for one lane as for 32, and merging inside the
+// search kernels kept whole warps on it (and a fence and a counter per tile).
+constexpr int kRhoLanes = 4;
+__device__ __forceinline__ double rho_sum(double v) {
+#pragma unroll
+  for (int o = 1; o < kRhoLanes; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(kFull, v, o));
+  return v;
+}
+__global__ void __launch_bounds__(kThreads) rho_kernel(const UnitDesc* units,
+                                                      const TargetDesc* targets,
+                                                      int64_t n_targets, const float4* partials,
+                                                      const ObsStat* obs_stat, double* rho) {
+  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kRhoLanes;
+  const int sub = threadIdx.x & (kRhoLanes - 1);
+  const TargetDesc tg = targets[g < n_targets ? g : n_targets - 1];  // whole warps shuffle
+  const UnitDesc& u = units[tg.unit];
+  const int n_tiles = u.n_tiles, n_m = u.n_m;
+  const int64_t t = (g < n_targets ? g : n_targets - 1) - u.tgt_off;
+  const float4* base = partials + 2 * (u.part_off + t * n_tiles);
+  const ObsStat* stat = obs_stat + tg.obs_tile;
+  auto count = [&](int q) { return (double)min(kQT, n_m - q * kQT); };
+  // mean(y) - c and Syy, Sxy of tile q
+  auto tile = [&](int q, double n, double& my, double& syy, double& sxy) {
+    const float4 a = __ldg(base + 2 * q), b = __ldg(base + 2 * q + 1);
+    const double b1 = __dadd_rn((double)a.y, (double)a.z);
+    const double b2 = __dadd_rn((double)a.w, (double)b.x);
+    const double d = (n == (double)kQT) ? __dmul_rn(b1, 1.0 / kQT) : __ddiv_rn(b1, n);
+    my = __dadd_rn((double)a.x, d);
+    syy = fmax(__fma_rn(-b1, d, b2), 0.0);
+    sxy = __dadd_rn((double)b.y, (double)b.z);
+  };
+  double SX = 0.0, SY = 0.0, my, syy, sxy;
+  for (int q = sub; q < n_tiles; q += kRhoLanes) {
+    const double n = count(q);
+    tile(q, n, my, syy, sxy);
+    SX = __fma_rn(n, stat[q].mx, SX);
+    SY = __fma_rn(n, my, SY);
+  }
+  const double inv = (double)n_m;
+  const double MX = __ddiv_rn(rho_sum(SX), inv), MY = __ddiv_rn(rho_sum(SY), inv);
+  double SXX = 0.0, SYY = 0.0, SXY = 0.0;
+  for (int q = sub; q < n_tiles; q += kRhoLanes) {
+    const double n = count(q);
+    tile(q, n, my, syy, sxy);
+    const double dx = __dsub_rn(stat[q].mx, MX), dy = __dsub_rn(my, MY);
+    const double wx = __dmul_rn(n, dx);
+    SXX = __fma_rn(wx, dx, __dadd_rn(SXX, stat[q].sxx));
+    SYY = __fma_rn(__dmul_rn(n, dy), dy, __dadd_rn(SYY, syy));
+    SXY = __fma_rn(wx, dy, __dadd_rn(SXY, sxy));
+  }
+  SXX = rho_sum(SXX);
+  SYY = rho_sum(SYY);
+  SXY = rho_sum(SXY);
+  if (sub == 0 && g < n_targets)
+    rho[tg.out_idx] = (SXX > 0.0 && SYY > 0.0) ? __ddiv_rn(SXY, __dsqrt_rn(__dmul_rn(SXX, SYY)))
+                                               : nan("");
+}
+
+}  // namespace
+
+int knn_block_threads() { return kThreads; }
+int knn_queries_per_thread() { return 1; }
+
+#define CCM_FOR_E(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10)
+#define CCM_CASE_PREPARE(EV)                                             \
+  if (const cudaError_t e = KnnKernels<EV>::prepare(); e != cudaSuccess) return e;
+#define CCM_CASE_PREPARE_TABLE(EV)                                       \
+  if (const cudaError_t e = KnnKernels<EV>::prepare_table(); e != cudaSuccess) return e;
+#define CCM_CASE_OCCUPANCY(EV) \
+  case EV: return KnnKernels<EV>::occupancy(ctas);
+#define CCM_CASE_LAUNCH(EV) \
+  case EV: return KnnKernels<EV>::launch(p, lanes, grid, s);
+#define CCM_CASE_LAUNCH_TABLE(EV) \
+  case EV: return KnnKernels<EV>::launch_table(p, max_nm, lanes, grid, s);
+
+cudaError_t knn_prepare() {
+  CCM_FOR_E(CCM_CASE_PREPARE)
+  return cudaSuccess;
+}
+cudaError_t knn_table_prepare() {
+  CCM_FOR_E(CCM_CASE_PREPARE_TABLE)
+  return cudaSuccess;
+}
+cudaError_t knn_occupancy(int E, int* ctas) {
+  switch (E) { CCM_FOR_E(CCM_CASE_OCCUPANCY) }
+  return cudaErrorInvalidValue;
+}
+cudaError_t launch_knn(const KnnParams& p, int E, bool lanes, int grid, cudaStream_t s) {
+  switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH) }
+  return cudaErrorInvalidValue;
+}
+cudaError_t knn_table_occupancy(int max_nm, bool lanes, int* ctas) {
+  return KnnKernels<kMaxE>::occupancy_table(max_nm, lanes, ctas);
+}
+cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lanes, int grid,
+                             cudaStream_t s) {
+  switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH_TABLE) }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* jobs,
+                       int64_t n_jobs, int64_t n_tiles, const float* scales, float2* obs,
+                       ObsStat* obs_stat, cudaStream_t s) {
+  if (n_jobs <= 0 || n_tiles <= 0) return cudaSuccess;
+  const int64_t want = (n_tiles + kThreads / 32 - 1) / (kThreads / 32);  // a warp per tile
+  const int64_t blocks = want < 65536 ? want : 65536;
+  obs_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(series, order, jobs, n_jobs, n_tiles, scales,
+                                                   obs, obs_stat);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rho(const UnitDesc* units, const TargetDesc* targets, int64_t n_targets,
+                       const float4* partials, const ObsStat* obs_stat, double* rho,
+                       cudaStream_t s) {
+  if (n_targets <= 0) return cudaSuccess;
+  const int64_t blocks = (n_targets * kRhoLanes + kThreads - 1) / kThreads;
+  rho_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(units, targets, n_targets, partials, obs_stat,
+                                                   rho);
+  return cudaGetLastError();
+}
+
+}  // namespace ccm

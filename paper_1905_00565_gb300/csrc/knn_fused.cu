@@ -30,12 +30,13 @@
 //    runs full and sorted at the end, so the E+1 nearest come out in
 //    (distance, index) order however the library was visited;
 //  * the epilogue forms u_i = exp(-d_i/d_1) (optionally floored), the
-//    prediction, and the FP64 moments of each (tile, target): predictions go
-//    to a shared-memory ring whose eight slots are reduced by eight warps at
-//    once (the FP64 pipe is the scarce unit); the observed values' half is
+//    prediction, and the moments of each (tile, target) in paired FP32
+//    (moments.cuh): predictions go to a shared-memory ring whose eight slots
+//    are reduced by eight warps at once; a unit of many targets sums them with
+//    a lane per target instead (lane_targets); the observed values' half is
 //    done once per (j, i, E, tau) by obs_kernel, not once per realization;
-//    the last (tile, target) of a realization to finish merges the tiles'
-//    moments in a fixed order, so rho does not depend on the schedule.
+//    rho_kernel merges the tiles' moments in a fixed order, so rho does not
+//    depend on the schedule.
 #include <float.h>
 #include <limits.h>
 #include <math.h>
@@ -43,6 +44,7 @@
 #include <initializer_list>
 
 #include "ccm_internal.h"
+#include "moments.cuh"
 
 namespace ccm {
 namespace {
@@ -50,17 +52,21 @@ namespace {
 using u64 = unsigned long long;
 
 constexpr int kThreads = 256;             // threads per CTA = queries per tile
-constexpr int kQT = kThreads;             // queries per tile (one per thread)
-static_assert((kQT & (kQT - 1)) == 0, "tile moments rely on a power-of-two tile");
+static_assert(kQT == kThreads, "one query per thread");
 constexpr int kBuf = 20;                  // candidate keys per query (a column of the buffer)
 constexpr int kCoordBytes = 24 * 1024;    // shared memory for one library tile + chunk boxes
 constexpr int kBoxBytes = 4 * 1024;       // chunk bounding boxes, at the end of that region
 constexpr int kChunk = 16;                // library points per bounding box
 constexpr int kBufBytes = kBuf * kThreads * 8;
-// Predictions staged for their FP64 moments: kRing (tile, target) vectors of
-// kQT floats, reduced together, one warp each, when the ring is full.
+// Predictions staged for their moments: kRing (tile, target) vectors, reduced
+// together, one warp each, when the ring is full.
 constexpr int kRing = kThreads / 32;
-constexpr int kRingBytes = kRing * kThreads * 4;
+constexpr int kRingBytes = kRing * kVecStride * 4;
+// Scratch of the lane-per-target epilogue: 1 / sum of weights per query, then
+// two buffers of the eight warps' sums (six floats a lane).
+constexpr int kLaneScratch = kThreads * 4 + 2 * (kThreads / 32) * 6 * 32 * 4;
+static_assert(kBuf * kThreads * 8 >= (kMaxE + 1) * kThreads * 8 + kLaneScratch,
+              "the lane-per-target epilogue's scratch fits the candidate buffer");
 constexpr int kSmemBytes = kCoordBytes + kBufBytes + kRingBytes;
 constexpr unsigned kFull = 0xffffffffu;
 // Kernel variants picked per E by the autotuner (results are identical):
@@ -193,193 +199,104 @@ __device__ __forceinline__ void insert_prefix(u64 (&ku)[K], u64 x, int n) {
   ku[0] = below[0] ? x : ku[0];
 }
 
-// Butterfly sum over the warp: every lane ends with the same bits (each
-// level adds the same two values in either order).
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(kFull, v, o));
-  return v;
-}
-
-// Two-pass FP64 moments of one tile's (observed x, predicted y) pairs, by one
-// warp: each lane sums a fixed strided subset, then the butterfly.  The
-// predictions are staged in shared memory (ys[0..nq)); the observed half comes
-// from the tile's record (obs_kernel: x_q - mean(x), mean(x), Sxx), computed
-// there with the same lane order and butterfly.  Writes (n, mean_x, mean_y,
-// Sxx, Syy, Sxy) about the tile means.
-constexpr int kPer = kQT / 32;  // queries per lane
-
-// Mean of the nq lane-strided values v(c) = value lane + 32c (the sum in lane
-// order, then the butterfly); a full tile divides by 256 = 2^8, and
-// multiplying by 2^-8 gives the same bits and spares the FP64 pipe a division.
-template <class V>
-__device__ __forceinline__ double tile_mean(V v, int nq) {
-  const int lane = threadIdx.x & 31;
-  double sv = 0.0;
-#pragma unroll
-  for (int c = 0; c < kPer; ++c)
-    if (lane + 32 * c < nq) sv = __dadd_rn(sv, v(c));
-  sv = warp_sum(sv);
-  return (nq == kQT) ? __dmul_rn(sv, 1.0 / kQT) : __ddiv_rn(sv, (double)nq);
-}
-
-__device__ __forceinline__ void tile_moments(const float* ys, const double* rec, int nq,
-                                             double* part) {
-  const int lane = threadIdx.x & 31;
-  double y[kPer];
-#pragma unroll
-  for (int c = 0; c < kPer; ++c) y[c] = (double)ys[lane + 32 * c];
-  const double my = tile_mean([&](int c) { return y[c]; }, nq);
-  double syy = 0.0, sxy = 0.0;
-#pragma unroll
-  for (int c = 0; c < kPer; ++c) {
-    const int q = lane + 32 * c;
-    if (q < nq) {
-      const double b = __dsub_rn(y[c], my);
-      syy = __fma_rn(b, b, syy);
-      sxy = __fma_rn(__ldg(rec + q), b, sxy);
-    }
-  }
-  syy = warp_sum(syy);
-  sxy = warp_sum(sxy);
-  if (lane == 0) {
-    part[0] = (double)nq;
-    part[1] = __ldg(rec + kQT);
-    part[2] = my;
-    part[3] = __ldg(rec + kQT + 1);
-    part[4] = syy;
-    part[5] = sxy;
-  }
-}
-
-// Observed-moment records (see ObsJob), one warp per tile: x_q is the target
-// at the tile's manifold points (Sect. 2.1: the value the cross map
-// predicts).  The same lane order and butterfly as tile_moments.
-__global__ void __launch_bounds__(kThreads) obs_kernel(const float* series, const int32_t* order,
-                                                      const ObsJob* jobs, int64_t n_jobs,
-                                                      int64_t n_tiles, double* obs) {
-  const int lane = threadIdx.x & 31;
-  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n_tiles;
-       g += n_warps) {
-    int64_t lo = 0, hi = n_jobs - 1;  // the job holding tile g: last obs_tile <= g
-    while (lo < hi) {
-      const int64_t mid = (lo + hi + 1) >> 1;
-      if (jobs[mid].obs_tile <= g) lo = mid;
-      else hi = mid - 1;
-    }
-    const ObsJob jb = jobs[lo];
-    const int tile = (int)(g - jb.obs_tile);
-    const int nq = min(kQT, jb.n_m - tile * kQT);
-    const float* si = series + jb.series_off + (int64_t)jb.i * jb.n;
-    const int32_t* ord = order + jb.order_off + (int64_t)tile * kQT;
-    const int off = (jb.E - 1) * jb.tau;
-    double x[kPer];
-#pragma unroll
-    for (int c = 0; c < kPer; ++c) {
-      const int q = lane + 32 * c;
-      x[c] = (q < nq) ? (double)si[ord[q] + off] : 0.0;
-    }
-    const double mx = tile_mean([&](int c) { return x[c]; }, nq);
-    double* rec = obs + g * kObsStride;
-    double sxx = 0.0;
-#pragma unroll
-    for (int c = 0; c < kPer; ++c) {
-      const int q = lane + 32 * c;
-      double a = 0.0;
-      if (q < nq) {
-        a = __dsub_rn(x[c], mx);
-        sxx = __fma_rn(a, a, sxx);
-      }
-      rec[q] = a;
-    }
-    sxx = warp_sum(sxx);
-    if (lane == 0) {
-      rec[kQT] = mx;
-      rec[kQT + 1] = sxx;
-    }
-  }
-}
-
-// Merge the tile moments of one (realization, target) into rho, by one warp.
-// With the grand means MX = sum(n_t mx_t)/N, the centred sums are exactly
-//   Sxx = sum_t [Sxx_t + n_t (mx_t - MX)^2]   (likewise Syy, Sxy),
-// a sum of non-negative terms (no cancellation), taken in a fixed lane and
-// butterfly order: rho does not depend on which CTA ran which tile, or when.
-__device__ __forceinline__ double merge_moments(const double* base, int n_tiles) {
-  const int lane = threadIdx.x & 31;
-  double N = 0.0, SX = 0.0, SY = 0.0;
-  for (int q = lane; q < n_tiles; q += 32) {
-    const double* pt = base + 6 * q;
-    const double nq = __ldcg(pt + 0);
-    N = __dadd_rn(N, nq);
-    SX = __fma_rn(nq, __ldcg(pt + 1), SX);
-    SY = __fma_rn(nq, __ldcg(pt + 2), SY);
-  }
-  N = warp_sum(N);
-  SX = warp_sum(SX);
-  SY = warp_sum(SY);
-  const double MX = __ddiv_rn(SX, N), MY = __ddiv_rn(SY, N);
-  double SXX = 0.0, SYY = 0.0, SXY = 0.0;
-  for (int q = lane; q < n_tiles; q += 32) {
-    const double* pt = base + 6 * q;
-    const double nq = __ldcg(pt + 0);
-    const double dx = __dsub_rn(__ldcg(pt + 1), MX), dy = __dsub_rn(__ldcg(pt + 2), MY);
-    const double wx = __dmul_rn(nq, dx);
-    SXX = __fma_rn(wx, dx, __dadd_rn(SXX, __ldcg(pt + 3)));
-    SYY = __fma_rn(__dmul_rn(nq, dy), dy, __dadd_rn(SYY, __ldcg(pt + 4)));
-    SXY = __fma_rn(wx, dy, __dadd_rn(SXY, __ldcg(pt + 5)));
-  }
-  SXX = warp_sum(SXX);
-  SYY = warp_sum(SYY);
-  SXY = warp_sum(SXY);
-  return (SXX > 0.0 && SYY > 0.0) ? __ddiv_rn(SXY, __dsqrt_rn(__dmul_rn(SXX, SYY))) : nan("");
-}
-
-// Called by a reducer warp after its lane 0 wrote the moments of one (tile,
-// target) of a realization: the fence orders them before the completion
-// count, and the last of the realization's n_tiles * n_targets to arrive
-// merges every target's moments.  Out of line: inlined its registers would
-// crowd the search.
-__device__ __noinline__ void complete_tile(const KnnParams& p, int unit) {
-  const int lane = threadIdx.x & 31;
-  unsigned prev = 0u;
-  if (lane == 0) {
-    __threadfence();
-    prev = atomicAdd(&p.unit_done[unit], 1u);
-  }
-  prev = __shfl_sync(kFull, prev, 0);
-  const UnitDesc& u = p.units[unit];
-  const int n_tiles = u.n_tiles, n_targets = u.n_targets;
-  if (prev != (unsigned)(n_tiles * n_targets - 1)) return;
-  __threadfence();
-  for (int t = 0; t < n_targets; ++t) {
-    const double r = merge_moments(p.partials + 6 * (u.part_off + (int64_t)t * n_tiles), n_tiles);
-    if (lane == 0) p.rho[p.targets[u.tgt_off + t].out_idx] = r;
-  }
-  if (lane == 0) p.unit_done[unit] = 0u;  // ready for the next run
-}
-
-// A staged (tile, target) prediction vector awaiting its FP64 moments.
+// A staged (tile, target) prediction vector awaiting its moments.
 struct RingMeta {
-  const double* rec;  // the tile's observed-value record
-  double* part;       // where its six moments go
-  int32_t unit;       // its realization
+  const float2* a;    // the tile's centred observations
+  float4* part;       // where its sums go
   int32_t nq;         // valid queries of the tile
 };
 
-// The staged vectors' moments: warps 0..n-1 take one each, in parallel (so the
-// FP64 pipes of all four SM sub-partitions share the work), and count it
-// towards its realization's completion.  Between two block barriers: the
-// slots are complete on entry and free again on exit.
-__device__ __forceinline__ void flush_ring(const KnnParams& p, const float* ring,
-                                           const RingMeta* meta, int n) {
+// The staged vectors' sums: warps 0..n-1 take one each, in parallel.  Between
+// two block barriers: the slots are complete on entry and free again on exit.
+__device__ __forceinline__ void flush_ring(const float* ring, const RingMeta* meta, int n) {
   __syncthreads();
   const int warp = threadIdx.x >> 5;
   if (warp < n) {
     const RingMeta mt = meta[warp];
-    tile_moments(ring + warp * kQT, mt.rec, mt.nq, mt.part);
-    complete_tile(p, mt.unit);
+    tile_sums_warp(ring + warp * kVecStride, mt.a, mt.nq, mt.part);
+  }
+  __syncthreads();
+}
+
+// The epilogue of a unit with many targets (>= kLaneTargets): a lane per
+// target.  The weights and neighbours of the tile's queries lie in shared
+// memory (keep[s][query], {weight, neighbour}); warp w takes queries 32w ..
+// 32w+31 and 32 targets at a time, so a neighbour's values of 32 targets are
+// one coalesced read of the time-major series and every lane sums its own
+// target's moments in registers, group of eight after group of eight; the
+// warps' sums meet in shared memory.  One thread per query and target after
+// target instead gathered 4 bytes a lane from as many lines and spent five
+// FP64 operations a prediction.  64 variables, N = 5000, r = 25, all pairs:
+// brute force and table scan 222 -> 62 ms a run.
+// Block-wide; the caller's next use of keep and scratch is behind the closing
+// barrier.
+template <int E>
+__device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc& u, int tile, int nq,
+                                          const u64* keep, const float* rus, float* sums) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int T = u.n_targets, n_tiles = u.n_tiles, stride = u.st_stride;
+  const float* st = p.st + u.st_off + (int64_t)(E - 1) * u.tau * stride;
+  const TargetDesc* tgs = p.targets + u.tgt_off;
+  const float2* obs = p.obs + tgs[0].obs_tile * kQT + (int64_t)tile * kQT * T;
+  const int q0 = warp * 32, q1 = min(nq, q0 + 32);
+  const int32_t* order = p.order + u.order_off + (int64_t)tile * kQT;
+  for (int tc = 0, turn = 0; tc < T; tc += 32, ++turn) {
+    const int t = min(tc + lane, T - 1);  // lanes past the last target repeat it
+    const TargetDesc& tg = tgs[t];
+    const float* col = st + tg.i;
+    const float scale = p.obs_stat[tg.obs_tile + tile].scale;
+    auto predict = [&](int q) {
+      float acc = 0.f;
+#pragma unroll
+      for (int s = 0; s <= E; ++s) {
+        const u64 k = keep[s * kThreads + q];
+        acc = __fmaf_rn(key_dist(k), __ldg(col + (int64_t)key_index(k) * stride), acc);
+      }
+      return __fmul_rn(acc, rus[q]);
+    };
+    const float c = __fmul_rn(predict(0), scale);
+    const float2* a = obs + t;
+    TileSums part[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      part[g] = zero_sums();
+      const int qa = q0 + kMomentGroup * g;
+      if (qa + kMomentGroup <= q1 && p.dbg_xhat == nullptr) {
+#pragma unroll 4
+        for (int i = 0; i < kMomentGroup; ++i)
+          add_query(part[g], __fmul_rn(predict(qa + i), scale), __ldg(a + (int64_t)(qa + i) * T), c);
+      } else {
+        for (int q = qa; q < min(qa + kMomentGroup, q1); ++q) {
+          const float y = predict(q);
+          if (p.dbg_xhat && tc + lane < T) p.dbg_xhat[tg.q_off + order[q]] = y;
+          add_query(part[g], __fmul_rn(y, scale), __ldg(a + (int64_t)q * T), c);
+        }
+      }
+      if (g == 1) part[0] = merge_sums(part[0], part[1]);
+    }
+    part[0] = merge_sums(part[0], merge_sums(part[2], part[3]));
+    // [turn & 1][value][warp][lane]
+    float* mine = sums + (turn & 1) * (kThreads / 32) * 6 * 32 + warp * 32 + lane;
+    const float v[6] = {part[0].b1.h, part[0].b1.l, part[0].b2.h,
+                        part[0].b2.l, part[0].ab.h, part[0].ab.l};
+#pragma unroll
+    for (int x = 0; x < 6; ++x) mine[x * kThreads] = v[x];
+    __syncthreads();
+    if (warp == (turn & 7) && tc + lane < T) {
+      const float* all = sums + (turn & 1) * (kThreads / 32) * 6 * 32 + lane;
+      auto load = [&](int w) {
+        const float* f = all + w * 32;
+        TileSums m;
+        m.b1 = Pair32{f[0], f[kThreads]};
+        m.b2 = Pair32{f[2 * kThreads], f[3 * kThreads]};
+        m.ab = Pair32{f[4 * kThreads], f[5 * kThreads]};
+        return m;
+      };
+      const TileSums lo = merge_sums(merge_sums(load(0), load(1)), merge_sums(load(2), load(3)));
+      const TileSums hi = merge_sums(merge_sums(load(4), load(5)), merge_sums(load(6), load(7)));
+      store_sums(p.partials + 2 * (u.part_off + (int64_t)t * n_tiles + tile), c,
+                 merge_sums(lo, hi));
+    }
   }
   __syncthreads();
 }
@@ -390,20 +307,20 @@ __device__ __forceinline__ void flush_ring(const KnnParams& p, const float* ring
 // (itself excluded).  Simplex weights and the
 // prediction of every target; each target's prediction vector goes to the
 // next ring slot (ring_n, the same in every thread), and a full ring is
-// reduced (flush_ring).  The CTA flushes what is left when it runs out of
+// reduced (flush_ring); units of many targets (kLanes: a kernel of their own, so
+// that neither epilogue costs the other registers) take lane_targets instead.  The CTA flushes what is left when it runs out of
 // work.  rho does not depend on which warp reduced which vector, or when.
 // `keep` (brute-force path: the thread's own column of the candidate buffer,
 // which only this thread uses and which is free once its search is done)
 // holds the weights and neighbours in shared memory, so that a reduction
 // between two targets finds no live registers to spill; other warps may still
-// be searching, so nothing else of the buffer is touched.  kKeep false: they
-// stay in registers.  nb_values (table path, one target, no checking copy of
+// be searching, so nothing else of the buffer is touched before a barrier.
+// kKeep false: they stay in registers (keep: the lane-per-target scratch).  nb_values (table path, one target, no checking copy of
 // the neighbours): nb holds the bits of the target's values at the E+1
 // neighbours, read from the table instead of gathered.
 static_assert(kMaxE + 1 <= kBuf, "the epilogue keeps E+1 entries in a candidate column");
-template <int E, bool kKeep, bool kDist = false>
-__device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& u, int unit,
-                                            int tile, int m, bool valid, const float (&dd)[E + 1],
+template <int E, bool kLanes, bool kKeep, bool kDist = false>
+__device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& u, int tile, int m, bool valid, const float (&dd)[E + 1],
                                             const int (&nb)[E + 1], float* ring, RingMeta* meta,
                                             int& ring_n, u64* keep, bool nb_values = false) {
   const int tid = threadIdx.x;
@@ -437,6 +354,23 @@ __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& 
     nbc[s] = kDist ? nb[s] : min(max(nb[s], 0), n_m - 1);
     if (kKeep) keep[s * kThreads + tid] = ((u64)__float_as_uint(w[s]) << 32) | (uint32_t)nbc[s];
   }
+  if constexpr (kLanes) {
+    if (!kKeep) {
+#pragma unroll
+      for (int s = 0; s <= E; ++s)
+        keep[s * kThreads + tid] = ((u64)__float_as_uint(w[s]) << 32) | (uint32_t)nbc[s];
+    }
+    if (p.dbg_nbr && valid)
+      for (int t = 0; t < u.n_targets; ++t)
+        for (int s = 0; s <= E; ++s)
+          p.dbg_nbr[p.targets[u.tgt_off + t].nbr_off + (int64_t)m * (E + 1) + s] =
+              key_index(keep[s * kThreads + tid]);
+    float* rus = reinterpret_cast<float*>(keep + (E + 1) * kThreads);
+    if (kKeep) __syncthreads();  // other warps' columns reach beyond E+1 keys while they search
+    rus[tid] = rcp_hw(usum);
+    __syncthreads();
+    lane_targets<E>(p, u, tile, nq, keep, rus, rus + kThreads);
+  } else {
   auto weight = [&](int s) {
     return kKeep ? __uint_as_float((uint32_t)(keep[s * kThreads + tid] >> 32)) : w[s];
   };
@@ -460,20 +394,21 @@ __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& 
         for (int s = 0; s <= E; ++s) p.dbg_nbr[tg.nbr_off + (int64_t)m * (E + 1) + s] = nbr(s);
       }
     }
-    ring[ring_n * kQT + tid] = valid ? xhat : 0.f;
+    const int64_t rec = tg.obs_tile + tile;
+    ring[ring_n * kVecStride + vec_slot(tid)] = __fmul_rn(xhat, p.obs_stat[rec].scale);
     if (tid == 0)
-      meta[ring_n] = RingMeta{p.obs + (tg.obs_tile + tile) * kObsStride,
-                              p.partials + 6 * (u.part_off + (int64_t)t * u.n_tiles + tile), unit,
-                              nq};
+      meta[ring_n] = RingMeta{p.obs + rec * kQT,
+                              p.partials + 2 * (u.part_off + (int64_t)t * u.n_tiles + tile), nq};
     // a full ring is reduced before the next target's vector, or at the end
     if (++ring_n == kRing && t + 1 < u.n_targets) {
-      flush_ring(p, ring, meta, kRing);
+      flush_ring(ring, meta, kRing);
       ring_n = 0;
     }
   }
   if (ring_n == kRing) {  // the weights and neighbours are dead here
-    flush_ring(p, ring, meta, kRing);
+    flush_ring(ring, meta, kRing);
     ring_n = 0;
+  }
   }
 }
 
@@ -587,9 +522,9 @@ __device__ __forceinline__ void sort_column(u64* col, int n) {
 // to the K smallest keys.  At the end the column is compacted and sorted: its
 // first K keys are the E+1 nearest neighbours in (distance, index) order,
 // exactly the list the sorted insertion of every candidate would give.
-template <int E, int V, bool kStats>
-__device__ void process_item(const KnnParams& p, const UnitDesc& u, int unit, int tile0,
-                             int n_chunk, unsigned char* smem, RingMeta* meta, int& ring_n) {
+template <int E, int V, bool kLanes, bool kStats>
+__device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, int n_chunk,
+                             unsigned char* smem, RingMeta* meta, int& ring_n) {
   constexpr int K = E + 1;  // the window keeps m itself out, so E+1 slots suffice
   constexpr int EP = TileShape<E>::EP;
   constexpr int LT = TileShape<E>::LT;
@@ -612,7 +547,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int unit, in
   }
   u64* s_buf = reinterpret_cast<u64*>(smem + buf_off);
   const int cap = (int)((kCoordBytes + kBufBytes - buf_off) / (kThreads * 8));  // >= kBuf
-  float* s_ring = reinterpret_cast<float*>(smem + kCoordBytes + kBufBytes);      // [kRing][kQT]
+  float* s_ring = reinterpret_cast<float*>(smem + kCoordBytes + kBufBytes);      // [kRing][kVecStride]
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int off = (E - 1) * tau;
@@ -880,7 +815,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int unit, in
       nb[s] = key_index(k);
     }
     if (kPrefetch && tile + 1 < tile1) load_query(tile + 1);
-    finish_tile<E, true>(p, u, unit, tile, m, valid, dd, nb, s_ring, meta, ring_n, s_buf);
+    finish_tile<E, kLanes, true>(p, u, tile, m, valid, dd, nb, s_ring, meta, ring_n, s_buf);
     // the next tile's search starts behind a barrier (this also keeps the
     // search's registers free of spills)
     __syncthreads();
@@ -994,7 +929,7 @@ __device__ __forceinline__ void table_walk(const KnnParams& p, int64_t at, int n
   }
 }
 
-template <int E, bool kStats>
+template <int E, bool kLanes, bool kStats>
 __device__ void process_table_item(const KnnParams& p, int unit0, int count, int tile0,
                                    unsigned char* smem, RingMeta* meta, int& ring_n) {
   // `count` consecutive realizations of one cell (the same manifold, table, L
@@ -1009,6 +944,7 @@ __device__ void process_table_item(const KnnParams& p, int unit0, int count, int
   float* s_ring = reinterpret_cast<float*>(smem);
   uint16_t* s_rec = reinterpret_cast<uint16_t*>(smem + kRingBytes);  // [count][K][kThreads]
   unsigned char* map = smem + kRingBytes + kRecBytes;
+  u64* s_keep = reinterpret_cast<u64*>(smem + p.lane_scratch);
   const bool bytes = n_m <= kByteMapMax;
   const int words = bytes ? (n_m + 3) >> 2 : (n_m + 31) >> 5;  // 32-bit words of the map
   uint32_t* mw = reinterpret_cast<uint32_t*>(map);
@@ -1061,8 +997,7 @@ __device__ void process_table_item(const KnnParams& p, int unit0, int count, int
       }
     }
     for (int b = 0; b < count; ++b) {
-      const int unit = unit0 + b;
-      const UnitDesc u = (b == 0) ? u0 : p.units[unit];
+      const UnitDesc u = (b == 0) ? u0 : p.units[unit0 + b];
       const bool full = ((counts >> (8 * b)) & 0xffu) >= (uint32_t)K;
       if (kStats) {
         const unsigned fb = __popc(__ballot_sync(kFull, valid && !full));
@@ -1149,8 +1084,7 @@ __device__ void process_table_item(const KnnParams& p, int unit0, int count, int
         }
         tv = false;  // gathered as for brute force
       }
-      finish_tile<E, false, true>(p, u, unit, tile, m, valid, dd, nb, s_ring, meta, ring_n, nullptr,
-                                  tv);
+      finish_tile<E, kLanes, false, true>(p, u, tile, m, valid, dd, nb, s_ring, meta, ring_n, s_keep, tv);
     }
   }
 }
@@ -1161,7 +1095,7 @@ __device__ void process_table_item(const KnnParams& p, int unit0, int count, int
 // three).  Three (80 registers) for longer manifolds (bitmap, one realization
 // an item, tables beyond L2), which want the registers (the N = 10^5 series'
 // scan: 110 ms, 120 ms with four).
-template <int E, bool kStats, int kMinCtas>
+template <int E, bool kLanes, bool kStats, int kMinCtas>
 __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -1177,17 +1111,17 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams
     if ((int64_t)it >= p.n_items) break;
     const WorkItem w = p.items[it];
     const UnitDesc u = p.units[w.unit];
-    if (u.E != E || w.count < 1 || w.count > kTableGroup ||
+    if (u.E != E || (u.n_targets >= kLaneTargets) != kLanes || w.count < 1 || w.count > kTableGroup ||
         (w.count > 1 && u.n_m > kByteMapMax)) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrBadUnit);
       continue;
     }
-    process_table_item<E, kStats>(p, w.unit, w.count, w.tile, smem, s_meta, ring_n);
+    process_table_item<E, kLanes, kStats>(p, w.unit, w.count, w.tile, smem, s_meta, ring_n);
   }
-  if (ring_n > 0) flush_ring(p, reinterpret_cast<const float*>(smem), s_meta, ring_n);
+  if (ring_n > 0) flush_ring(reinterpret_cast<const float*>(smem), s_meta, ring_n);
 }
 
-template <int E, bool kStats>
+template <int E, bool kLanes, bool kStats>
 __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -1203,119 +1137,99 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
     if ((int64_t)it >= p.n_items) break;
     const WorkItem w = p.items[it];
     const UnitDesc u = p.units[w.unit];
-    if (u.E != E) {
+    if (u.E != E || (u.n_targets >= kLaneTargets) != kLanes) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrBadUnit);
       continue;
     }
     if (p.variant[E] == 1)
-      process_item<E, 1, kStats>(p, u, w.unit, w.tile, w.count, smem, s_meta, ring_n);
+      process_item<E, 1, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, ring_n);
     else
-      process_item<E, 0, kStats>(p, u, w.unit, w.tile, w.count, smem, s_meta, ring_n);
+      process_item<E, 0, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, ring_n);
   }
   if (ring_n > 0)
-    flush_ring(p, reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);
+    flush_ring(reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);
+}
+
+// Ring, records and map: every manifold of the launch fits (bytes up to
+// kByteMapMax points, bits above).
+size_t table_base_smem(int max_nm) {
+  const size_t bits = (size_t)((max_nm + 31) / 32) * 4;
+  const size_t map = (max_nm <= kByteMapMax) ? (size_t)(max_nm + 3) / 4 * 4
+                                             : (bits > (size_t)kByteMapMax ? bits : kByteMapMax);
+  return ((size_t)kRingBytes + (size_t)kRecBytes + map + 15) / 16 * 16;
+}
+size_t table_smem(int max_nm, bool lane_targets) {
+  return table_base_smem(max_nm) +
+         (lane_targets ? (size_t)(kMaxE + 1) * kThreads * 8 + kLaneScratch : 0);
 }
 
 }  // namespace
 
-int knn_block_threads() { return kThreads; }
-
-size_t knn_table_smem(int max_nm) {
-  // every manifold of the launch fits: bytes up to kByteMapMax points, bits above
-  const size_t bits = (size_t)((max_nm + 31) / 32) * 4;
-  const size_t map = (max_nm <= kByteMapMax) ? (size_t)(max_nm + 3) / 4 * 4
-                                             : (bits > (size_t)kByteMapMax ? bits : kByteMapMax);
-  return (size_t)kRingBytes + (size_t)kRecBytes + map + 16;
+// The kernels of one E, in a translation unit of their own (CCM_E).
+template <int E>
+cudaError_t KnnKernels<E>::launch(const KnnParams& p, bool lanes, int grid, cudaStream_t s) {
+  const auto fn = lanes ? (p.stats ? knn_fused_kernel<E, true, true> : knn_fused_kernel<E, true, false>)
+                        : (p.stats ? knn_fused_kernel<E, false, true> : knn_fused_kernel<E, false, false>);
+  fn<<<grid, kThreads, kSmemBytes, s>>>(p);
+  return cudaGetLastError();
 }
 
-#define CCM_FOR_E(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10)
-
-cudaError_t knn_table_prepare() {
-  // the largest bitmap any plan may need (manifolds up to kTableMaxNm points);
-  // set once, so that plans of different sizes never lower it for each other
-#define CCM_TPREP(EV)                                                             \
-  for (const auto fn : {knn_table_kernel<EV, false, 4>, knn_table_kernel<EV, true, 4>,  \
-                        knn_table_kernel<EV, false, 3>}) {                          \
-    const cudaError_t e = cudaFuncSetAttribute(                                   \
-        fn, cudaFuncAttributeMaxDynamicSharedMemorySize,                          \
-        (int)knn_table_smem(kTableMaxNm));                                        \
-    if (e != cudaSuccess) return e;                                               \
+template <int E>
+cudaError_t KnnKernels<E>::prepare() {
+  for (const auto fn : {knn_fused_kernel<E, false, false>, knn_fused_kernel<E, false, true>,
+                        knn_fused_kernel<E, true, false>, knn_fused_kernel<E, true, true>}) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) return e;
   }
-  CCM_FOR_E(CCM_TPREP)
-#undef CCM_TPREP
   return cudaSuccess;
+}
+
+template <int E>
+cudaError_t KnnKernels<E>::occupancy(int* ctas) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, knn_fused_kernel<E, false, false>,
+                                                       kThreads, kSmemBytes);
 }
 
 // Launches whose manifolds exceed the byte map use the three-CTA kernels
 // (the counting variant always the four-CTA ones).
-cudaError_t knn_table_occupancy(int max_nm, int* ctas) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      ctas, max_nm > kByteMapMax ? knn_table_kernel<kMaxE, false, 3> : knn_table_kernel<kMaxE, false, 4>,
-      kThreads, knn_table_smem(max_nm));
+template <int E>
+static auto table_kernel(int max_nm, bool lanes, bool stats) {
+  if (lanes) return stats ? knn_table_kernel<E, true, true, 2> : knn_table_kernel<E, true, false, 2>;
+  if (stats) return knn_table_kernel<E, false, true, 4>;
+  return max_nm > kByteMapMax ? knn_table_kernel<E, false, false, 3>
+                              : knn_table_kernel<E, false, false, 4>;
 }
 
-cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, int grid, cudaStream_t s) {
-#define CCM_TLAUNCH(EV)                                                           \
-  if (E == EV) {                                                                  \
-    if (p.stats)                                                                  \
-      knn_table_kernel<EV, true, 4><<<grid, kThreads, knn_table_smem(max_nm), s>>>(p); \
-    else if (max_nm > kByteMapMax)                                                \
-      knn_table_kernel<EV, false, 3><<<grid, kThreads, knn_table_smem(max_nm), s>>>(p); \
-    else                                                                          \
-      knn_table_kernel<EV, false, 4><<<grid, kThreads, knn_table_smem(max_nm), s>>>(p); \
-    return cudaGetLastError();                                                    \
-  }
-  CCM_FOR_E(CCM_TLAUNCH)
-#undef CCM_TLAUNCH
-  return cudaErrorInvalidValue;
-}
-int knn_queries_per_thread() { return 1; }
-
-cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* jobs,
-                       int64_t n_jobs, int64_t n_tiles, double* obs, cudaStream_t s) {
-  if (n_jobs <= 0 || n_tiles <= 0) return cudaSuccess;
-  const int64_t want = (n_tiles + kThreads / 32 - 1) / (kThreads / 32);  // a warp per tile
-  const int64_t blocks = want < 65536 ? want : 65536;
-  obs_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(series, order, jobs, n_jobs, n_tiles, obs);
+template <int E>
+cudaError_t KnnKernels<E>::launch_table(const KnnParams& params, int max_nm, bool lanes, int grid,
+                                        cudaStream_t s) {
+  KnnParams p = params;
+  p.lane_scratch = (int32_t)table_base_smem(max_nm);
+  table_kernel<E>(max_nm, lanes, p.stats != nullptr)<<<grid, kThreads, table_smem(max_nm, lanes), s>>>(p);
   return cudaGetLastError();
 }
 
-// One kernel per E (each keeps all its registers for that E's lists).
-
-cudaError_t launch_knn(const KnnParams& p, int E, int grid, cudaStream_t s) {
-#define CCM_LAUNCH(EV)                                                          \
-  if (E == EV) {                                                                \
-    if (p.stats)                                                                \
-      knn_fused_kernel<EV, true><<<grid, kThreads, kSmemBytes, s>>>(p);         \
-    else                                                                        \
-      knn_fused_kernel<EV, false><<<grid, kThreads, kSmemBytes, s>>>(p);        \
-    return cudaGetLastError();                                                  \
+template <int E>
+cudaError_t KnnKernels<E>::prepare_table() {
+  // the largest bitmap any plan may need (manifolds up to kTableMaxNm points);
+  // set once, so that plans of different sizes never lower it for each other
+  for (const auto fn : {knn_table_kernel<E, false, false, 4>, knn_table_kernel<E, false, true, 4>,
+                        knn_table_kernel<E, false, false, 3>, knn_table_kernel<E, true, false, 2>,
+                        knn_table_kernel<E, true, true, 2>}) {
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)table_smem(kTableMaxNm, true));
+    if (e != cudaSuccess) return e;
   }
-  CCM_FOR_E(CCM_LAUNCH)
-#undef CCM_LAUNCH
-  return cudaErrorInvalidValue;
-}
-
-cudaError_t knn_prepare() {
-#define CCM_PREP(EV)                                                            \
-  for (const auto fn : {knn_fused_kernel<EV, false>, knn_fused_kernel<EV, true>}) { \
-    const cudaError_t e = cudaFuncSetAttribute(                                 \
-        fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);           \
-    if (e != cudaSuccess) return e;                                             \
-  }
-  CCM_FOR_E(CCM_PREP)
-#undef CCM_PREP
   return cudaSuccess;
 }
 
-cudaError_t knn_occupancy(int E, int* ctas) {
-#define CCM_OCC(EV)                                                             \
-  if (E == EV)                                                                  \
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, knn_fused_kernel<EV, false>,   \
-                                                         kThreads, kSmemBytes);
-  CCM_FOR_E(CCM_OCC)
-#undef CCM_OCC
-  return cudaErrorInvalidValue;
+template <int E>
+cudaError_t KnnKernels<E>::occupancy_table(int max_nm, bool lanes, int* ctas) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, table_kernel<E>(max_nm, lanes, false),
+                                                       kThreads, table_smem(max_nm, lanes));
 }
+
+template struct KnnKernels<CCM_E>;
 
 }  // namespace ccm

@@ -1,0 +1,127 @@
+// Skill moments of one query tile in paired FP32 (shared by the search
+// kernels; not part of the public ABI).
+//
+// A tile of kQT queries of one (realization, target) contributes its count, the
+// means and centred sums of observed x and predicted y.  x's half is computed
+// in FP64 once per (pair, E, tau) (obs_kernel); y's half once per realization,
+// which in FP64 is what the epilogue used to wait for: GB300's FP64 pipe takes
+// two lanes per SM per clock, five operations a prediction.  Here every
+// quantity is an unevaluated sum h + l of two FP32 numbers, built from
+// error-free additions and products, so a sum carries about 48 bits; the
+// predictions themselves are FP32 values (24 bits).
+//
+// Values are scaled by a power of two that brings the target series' largest
+// magnitude into [1, 2) (exact; rho does not change), so that no product
+// leaves FP32's range.  With c the tile's first prediction and b = y - c
+// (exact as h + l), the sums are B1 = sum b, B2 = sum b^2 and AB = sum a b,
+// a = x - mean(x) (exact to 48 bits).  y constant over a tile gives exactly
+// zero.  From them mean(y) = c + B1/n, Syy = B2 - B1^2/n, Sxy = AB (sum a = 0).
+//
+// Order of the sums, the same in every kernel: eight consecutive queries one
+// after the other, then a binary tree over the tile's 32 such groups.
+#pragma once
+
+#include "ccm_internal.h"
+
+namespace ccm {
+
+constexpr int kQT = 256;                  // queries per tile
+constexpr int kMomentGroup = 8;           // queries summed one after the other
+constexpr int kVecStride = kQT + 8;       // floats of a staged prediction vector
+constexpr unsigned kAllLanes = 0xffffffffu;
+
+// Where query q of a tile lies in a staged prediction vector: one pad word per
+// 32 queries, so that lanes walking different groups hit different banks.
+__device__ __forceinline__ int vec_slot(int q) { return q + (q >> 5); }
+// Where query q of a tile lies in a record of centred observations: lanes
+// walking the tile's eight runs of 32 queries read consecutive elements.
+__device__ __forceinline__ int obs_slot(int q) { return ((q & 31) << 3) | (q >> 5); }
+
+struct Pair32 {
+  float h, l;
+};
+
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+  return s;
+}
+__device__ __forceinline__ void accumulate(Pair32& acc, float h, float l) {
+  float e;
+  acc.h = two_sum(acc.h, h, e);
+  acc.l = __fadd_rn(acc.l, __fadd_rn(e, l));
+}
+// Symmetric in its arguments (both add to the same bits).
+__device__ __forceinline__ Pair32 merge_pairs(const Pair32& a, const Pair32& b) {
+  Pair32 r;
+  float e;
+  r.h = two_sum(a.h, b.h, e);
+  r.l = __fadd_rn(__fadd_rn(a.l, b.l), e);
+  return r;
+}
+
+struct TileSums {
+  Pair32 b1, b2, ab;
+};
+__device__ __forceinline__ TileSums zero_sums() {
+  TileSums z;
+  z.b1 = z.b2 = z.ab = Pair32{0.f, 0.f};
+  return z;
+}
+
+// One query: y its scaled prediction, a its centred observation {h, l}.
+__device__ __forceinline__ void add_query(TileSums& m, float y, float2 a, float c) {
+  const float b = __fsub_rn(y, c);  // b + e = y - c exactly
+  const float v = __fsub_rn(b, y);
+  const float e = __fsub_rn(__fsub_rn(y, __fsub_rn(b, v)), __fadd_rn(c, v));
+  accumulate(m.b1, b, e);
+  float p = __fmul_rn(b, b);
+  float pe = __fmaf_rn(__fadd_rn(b, b), e, __fmaf_rn(b, b, -p));
+  accumulate(m.b2, p, pe);
+  p = __fmul_rn(a.x, b);
+  pe = __fmaf_rn(a.x, e, __fmaf_rn(a.y, b, __fmaf_rn(a.x, b, -p)));
+  accumulate(m.ab, p, pe);
+}
+__device__ __forceinline__ TileSums merge_sums(const TileSums& a, const TileSums& b) {
+  TileSums r;
+  r.b1 = merge_pairs(a.b1, b.b1);
+  r.b2 = merge_pairs(a.b2, b.b2);
+  r.ab = merge_pairs(a.ab, b.ab);
+  return r;
+}
+__device__ __forceinline__ TileSums merge_across(const TileSums& a, int mask) {
+  TileSums o;
+  o.b1.h = __shfl_xor_sync(kAllLanes, a.b1.h, mask);
+  o.b1.l = __shfl_xor_sync(kAllLanes, a.b1.l, mask);
+  o.b2.h = __shfl_xor_sync(kAllLanes, a.b2.h, mask);
+  o.b2.l = __shfl_xor_sync(kAllLanes, a.b2.l, mask);
+  o.ab.h = __shfl_xor_sync(kAllLanes, a.ab.h, mask);
+  o.ab.l = __shfl_xor_sync(kAllLanes, a.ab.l, mask);
+  return merge_sums(a, o);
+}
+__device__ __forceinline__ void store_sums(float4* part, float c, const TileSums& m) {
+  part[0] = make_float4(c, m.b1.h, m.b1.l, m.b2.h);
+  part[1] = make_float4(m.b2.l, m.ab.h, m.ab.l, 0.f);
+}
+
+// Moments of one staged vector by one warp: lane g sums queries 8g .. 8g+7,
+// then the tree.  ys: the scaled predictions (vec_slot order, queries past nq
+// ignored), a: the tile's record (obs_slot order, zero past nq).
+__device__ __forceinline__ void tile_sums_warp(const float* ys, const float2* a, int nq,
+                                               float4* part) {
+  const int lane = threadIdx.x & 31;
+  const float c = ys[0];
+  TileSums m = zero_sums();
+#pragma unroll
+  for (int i = 0; i < kMomentGroup; ++i) {
+    const int q = kMomentGroup * lane + i;
+    const float y = ys[vec_slot(q)];
+    add_query(m, q < nq ? y : c, __ldg(a + obs_slot(q)), c);
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) m = merge_across(m, o);
+  if (lane == 0) store_sums(part, c, m);
+}
+
+}  // namespace ccm

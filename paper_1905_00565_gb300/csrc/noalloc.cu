@@ -38,7 +38,8 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 namespace {
 
 struct NoallocLayout {
-  size_t units, items, lib, part, done, err, counter, order, orderjob, target, obs, obsjob, total;
+  size_t units, items, lib, part, err, counter, order, orderjob, target, obs, obs_stat, obsjob,
+      seriesjob, scale, total;
 };
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
@@ -53,9 +54,7 @@ NoallocLayout noalloc_layout(int64_t r, int64_t L, int64_t n_tiles, int64_t n_m)
   a.lib = o;
   o = up256(o + sizeof(int32_t) * (size_t)(r * L));
   a.part = o;
-  o = up256(o + 6 * sizeof(double) * (size_t)(r * n_tiles));
-  a.done = o;
-  o = up256(o + sizeof(uint32_t) * (size_t)r);
+  o = up256(o + 2 * sizeof(float4) * (size_t)(r * n_tiles));
   a.err = o;
   o = up256(o + sizeof(int32_t));
   a.counter = o;
@@ -67,9 +66,15 @@ NoallocLayout noalloc_layout(int64_t r, int64_t L, int64_t n_tiles, int64_t n_m)
   a.target = o;
   o = up256(o + sizeof(TargetDesc) * (size_t)r);
   a.obs = o;
-  o = up256(o + sizeof(double) * kObsStride * (size_t)n_tiles);
+  o = up256(o + sizeof(float2) * (size_t)knn_block_threads() * (size_t)n_tiles);
+  a.obs_stat = o;
+  o = up256(o + sizeof(ObsStat) * (size_t)n_tiles);
   a.obsjob = o;
   o = up256(o + sizeof(ObsJob));
+  a.seriesjob = o;
+  o = up256(o + sizeof(SeriesJob));
+  a.scale = o;
+  o = up256(o + sizeof(float));
   a.total = o;
   return a;
 }
@@ -86,7 +91,6 @@ struct CellArgs {
 __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, CellArgs c) {
   UnitDesc* units = reinterpret_cast<UnitDesc*>(scratch + lay.units);
   WorkItem* items = reinterpret_cast<WorkItem*>(scratch + lay.items);
-  uint32_t* done = reinterpret_cast<uint32_t*>(scratch + lay.done);
   const int64_t per_unit = (c.n_tiles + c.chunk - 1) / c.chunk;  // items per realization
   const int64_t n_items = (int64_t)c.r * per_unit;
   for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < n_items;
@@ -118,6 +122,9 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, 
     u.theiler = 0;
     u.wfloor = 0.f;
     u.table_tv = 0;
+    u.st_off = 0;
+    u.st_stride = 0;
+    u.pad = 0;
     TargetDesc tg;
     tg.out_idx = k;
     tg.q_off = k * (int64_t)c.n_m;
@@ -125,10 +132,9 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, 
     tg.lib_dbg_off = k * (int64_t)c.L;
     tg.obs_tile = 0;
     tg.i = c.i;
-    tg.pad = 0;
+    tg.unit = (int32_t)k;
     reinterpret_cast<TargetDesc*>(scratch + lay.target)[k] = tg;
     units[k] = u;
-    done[k] = 0u;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     OrderJob oj;
@@ -151,8 +157,18 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, 
     ob.tau = c.tau;
     ob.n_m = c.n_m;
     ob.n_tiles = c.n_tiles;
+    ob.a_off = 0;
+    ob.a_step = 0;
+    ob.scale = 0;
     ob.pad = 0;
     *reinterpret_cast<ObsJob*>(scratch + lay.obsjob) = ob;
+    SeriesJob sj;
+    sj.off = (int64_t)c.i * c.n;
+    sj.n = c.n;
+    sj.st_off = -1;
+    sj.st_stride = 0;
+    sj.scale = 0;
+    *reinterpret_cast<SeriesJob*>(scratch + lay.seriesjob) = sj;
     *reinterpret_cast<int32_t*>(scratch + lay.err) = 0;
     *reinterpret_cast<uint32_t*>(scratch + lay.counter) = 0u;
   }
@@ -225,11 +241,15 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   c.chunk = brute_chunk(r * n_tiles, L, E);
   noalloc_setup_kernel<<<(unsigned)((r * n_tiles + 255) / 256), 256, 0, s>>>(scratch, lay, c);
   e = launch_order(d_series, reinterpret_cast<const OrderJob*>(scratch + lay.orderjob), 1,
-                   (int)n_m, reinterpret_cast<int32_t*>(scratch + lay.order), nullptr, s);
+                   (int)n_m, reinterpret_cast<int32_t*>(scratch + lay.order), nullptr,
+                   reinterpret_cast<const SeriesJob*>(scratch + lay.seriesjob), 1,
+                   reinterpret_cast<float*>(scratch + lay.scale), nullptr, s);
   if (e == cudaSuccess)
     e = launch_obs(d_series, reinterpret_cast<const int32_t*>(scratch + lay.order),
                    reinterpret_cast<const ObsJob*>(scratch + lay.obsjob), 1, n_tiles,
-                   reinterpret_cast<double*>(scratch + lay.obs), s);
+                   reinterpret_cast<const float*>(scratch + lay.scale),
+                   reinterpret_cast<float2*>(scratch + lay.obs),
+                   reinterpret_cast<ObsStat*>(scratch + lay.obs_stat), s);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));
   SamplerParams sp{};
   sp.units = reinterpret_cast<const UnitDesc*>(scratch + lay.units);
@@ -247,18 +267,19 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   kp.n_items = (int64_t)r * ((n_tiles + c.chunk - 1) / c.chunk);
   kp.lib = reinterpret_cast<const int32_t*>(scratch + lay.lib);
   kp.order = reinterpret_cast<const int32_t*>(scratch + lay.order);
-  kp.partials = reinterpret_cast<double*>(scratch + lay.part);
-  kp.obs = reinterpret_cast<const double*>(scratch + lay.obs);
-  kp.unit_done = reinterpret_cast<uint32_t*>(scratch + lay.done);
+  kp.partials = reinterpret_cast<float4*>(scratch + lay.part);
+  kp.obs = reinterpret_cast<const float2*>(scratch + lay.obs);
+  kp.obs_stat = reinterpret_cast<const ObsStat*>(scratch + lay.obs_stat);
   kp.item_counter = reinterpret_cast<uint32_t*>(scratch + lay.counter);
-  kp.rho = d_rho;
   kp.err = reinterpret_cast<int32_t*>(scratch + lay.err);
   kp.persistent = 0;
   for (int q = 0; q <= kMaxE; ++q) {
     kp.merge_at[q] = kDefaultMergeAt;
     kp.variant[q] = kDefaultVariant;
   }
-  e = launch_knn(kp, E, (int)kp.n_items, s);
+  e = launch_knn(kp, E, false, (int)kp.n_items, s);
+  if (e == cudaSuccess)
+    e = launch_rho(kp.units, kp.targets, r, kp.partials, kp.obs_stat, d_rho, s);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));
   if (!cuda_stream) {
     int32_t err = 0;

@@ -115,10 +115,33 @@ __device__ void bitonic_sort(unsigned long long* k, int n2) {
   }
 }
 
+// Preparation of one target series (SeriesJob), by one CTA: the power of two
+// 2^-e, e the exponent of the series' largest magnitude (clamped so that it is
+// a normal number; 1 for an all-zero or non-finite series), and its column of
+// the time-major copy.
+__device__ void prepare_series(const float* series, const SeriesJob& jb, float* scales, float* st) {
+  const float* s = series + jb.off;
+  float lo, hi;
+  series_range(s, jb.n, &lo, &hi);
+  if (threadIdx.x == 0) {
+    const float top = fmaxf(fabsf(lo), fabsf(hi));
+    const int e = (int)((__float_as_uint(top) >> 23) & 0xffu) - 127;  // -127: zero or subnormal
+    scales[jb.scale] = (top == 0.f || e == 128)
+                           ? 1.f
+                           : __uint_as_float((uint32_t)(127 - max(-126, min(e, 126))) << 23);
+  }
+  if (jb.st_off >= 0)
+    for (int64_t t = threadIdx.x; t < jb.n; t += blockDim.x) st[jb.st_off + t * jb.st_stride] = s[t];
+}
+
 __global__ void __launch_bounds__(kOrderThreads)
-order_kernel(const float* series, const OrderJob* jobs, int32_t* order,
-             unsigned long long* scratch) {
+order_kernel(const float* series, const OrderJob* jobs, int64_t n_jobs, int32_t* order,
+             unsigned long long* scratch, const SeriesJob* series_jobs, float* scales, float* st) {
   extern __shared__ unsigned long long s_key[];
+  if (blockIdx.x >= n_jobs) {
+    prepare_series(series, series_jobs[blockIdx.x - n_jobs], scales, st);
+    return;
+  }
   const OrderJob jb = jobs[blockIdx.x];
   const float* s = series + jb.series_off + (int64_t)jb.j * jb.n;
   const int n_m = jb.n_m, E = jb.E, tau = jb.tau, off = (E - 1) * tau;
@@ -191,12 +214,14 @@ cudaError_t order_prepare() {
 }
 
 cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jobs, int max_nm,
-                         int32_t* order, unsigned long long* scratch, cudaStream_t s) {
-  if (n_jobs <= 0) return cudaSuccess;
+                         int32_t* order, unsigned long long* scratch, const SeriesJob* series_jobs,
+                         int64_t n_series_jobs, float* scales, float* st, cudaStream_t s) {
+  if (n_jobs + n_series_jobs <= 0) return cudaSuccess;
   int n2 = 1;
   while (n2 < max_nm && n2 < kOrderMaxSort) n2 <<= 1;
   const size_t smem = (size_t)n2 * sizeof(unsigned long long);
-  order_kernel<<<(unsigned)n_jobs, kOrderThreads, smem, s>>>(series, jobs, order, scratch);
+  order_kernel<<<(unsigned)(n_jobs + n_series_jobs), kOrderThreads, smem, s>>>(
+      series, jobs, n_jobs, order, scratch, series_jobs, scales, st);
   return cudaGetLastError();
 }
 

@@ -142,18 +142,27 @@ bool all_finite(const float* x, size_t count) {
 }
 
 // ------------------------------------------------------------- unit lists ---
+// The work items of one search launch: one E, and units of few or of many
+// targets (a kernel each).
+struct ItemGroup {
+  int32_t E;
+  bool lanes;
+  int64_t first, count;
+};
+
 struct UnitList {
   std::vector<UnitDesc> units;        // library realizations
   std::vector<TargetDesc> targets;    // their targets (one per output rho)
   std::vector<WorkItem> items;        // brute-force items, grouped by E (see sort_items)
   std::vector<double> item_cost;
-  int64_t e_first[kMaxE + 1] = {};    // items of E: e_count[E] from index e_first[E]
-  int64_t e_count[kMaxE + 1] = {};
-  int64_t te_first[kMaxE + 1] = {};   // the same for the table items
-  int64_t te_count[kMaxE + 1] = {};
+  std::vector<ItemGroup> groups;      // brute-force launches, in stream order
+  std::vector<ItemGroup> groups_table;  // the same for the table items
   std::vector<OrderJob> orders;       // one per (job, library variable, E, tau)
   std::vector<ObsJob> obs_jobs;       // one per (job, library variable, target, E, tau)
-  int64_t obs_total = 0;              // observed-moment tile records
+  int64_t obs_total = 0;              // observed-value tile records
+  std::vector<SeriesJob> series_jobs; // one per (job, target variable)
+  int64_t st_total = 0;               // elements of the time-major series copies
+  bool lane_targets = false;          // some unit has kLaneTargets targets
   std::vector<TableJob> tables;       // distance indexing tables to build
   std::vector<WorkItem> items_table;  // work items of units that read a table
   std::vector<double> item_cost_table;
@@ -181,6 +190,20 @@ struct UnitList {
   int64_t search_queries = 0;         // N_m summed over the units
   int64_t table_queries = 0;          // N_m summed over the units that read a table
   bool table_tv = false;              // some table stores its target's values (TableJob::tv_i)
+  bool lanes(const WorkItem& w) const {
+    return units[(size_t)w.unit].n_targets >= kLaneTargets;
+  }
+  // The launches of a sorted item list.
+  std::vector<ItemGroup> group_items(const std::vector<WorkItem>& list) const {
+    std::vector<ItemGroup> g;
+    for (size_t q = 0; q < list.size(); ++q) {
+      const int32_t E = units[(size_t)list[q].unit].E;
+      if (g.empty() || g.back().E != E || g.back().lanes != lanes(list[q]))
+        g.push_back(ItemGroup{E, lanes(list[q]), (int64_t)q, 0});
+      ++g.back().count;
+    }
+    return g;
+  }
   int table_u16() const { return max_nm < 65536 ? 1 : 0; }
   size_t table_elem() const { return table_u16() ? 2 : 4; }
   int64_t n_rho = 0, q_total = 0, nbr_total = 0, lib_dbg_total = 0;  // per output realization
@@ -302,30 +325,57 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         }
         ul->orders.push_back(oj);
       }
-  // Observed-moment records per (j, i, E, tau), shared by every L and k.
-  std::map<std::tuple<int32_t, int32_t, int32_t, int32_t>, int64_t> obs_of;
+  // Target series: their scales and, when some library variable has many
+  // targets, the time-major copy of the whole series block.
+  bool lanes = false;
+  for (int32_t j : lib_vars) lanes |= pairs_of[j].size() >= (size_t)kLaneTargets;
+  ul->lane_targets |= lanes;
+  const int64_t st_off = ul->st_total;
+  const int32_t st_stride = (pc.V + 31) / 32 * 32;
+  if (lanes) ul->st_total += pc.n * st_stride;
+  std::vector<int32_t> scale_of((size_t)pc.V, -1);
+  for (int64_t p = 0; p < nP; ++p) {
+    const int32_t i = pc.pairs[2 * p + 1];
+    if (scale_of[(size_t)i] >= 0) continue;
+    SeriesJob sj;
+    std::memset(&sj, 0, sizeof(sj));
+    sj.off = series_off + (int64_t)i * pc.n;
+    sj.n = pc.n;
+    sj.st_off = lanes ? st_off + i : -1;
+    sj.st_stride = st_stride;
+    sj.scale = scale_of[(size_t)i] = (int32_t)ul->series_jobs.size();
+    ul->series_jobs.push_back(sj);
+  }
+  // Observed-value records per (j, E, tau) and target, shared by every L and k:
+  // the targets of one (j, E, tau) lie side by side.
+  std::map<std::tuple<int32_t, int32_t, int32_t>, int64_t> obs_of;  // first target's first record
   for (int32_t j : lib_vars)
-    for (int64_t p : pairs_of[j])
-      for (int32_t E : pc.E)
-        for (int32_t tau : pc.tau) {
-          const int32_t i = pc.pairs[2 * p + 1];
-          const auto key = std::make_tuple(j, i, E, tau);
-          if (obs_of.count(key)) continue;
+    for (int32_t E : pc.E)
+      for (int32_t tau : pc.tau) {
+        const auto key = std::make_tuple(j, E, tau);
+        if (!obs_of.emplace(key, ul->obs_total).second) continue;
+        const int64_t base = ul->obs_total;
+        const std::vector<int64_t>& tp = pairs_of[j];
+        for (size_t t = 0; t < tp.size(); ++t) {
           ObsJob ob;
           std::memset(&ob, 0, sizeof(ob));
           ob.series_off = series_off;
           ob.n = pc.n;
-          ob.order_off = combo[std::make_tuple(j, E, tau)];
+          ob.order_off = combo[key];
           ob.obs_tile = ul->obs_total;
-          ob.i = i;
+          ob.i = pc.pairs[2 * tp[t] + 1];
+          ob.scale = scale_of[(size_t)ob.i];
           ob.E = E;
           ob.tau = tau;
           ob.n_m = (int32_t)(pc.n - (int64_t)(E - 1) * tau);
           ob.n_tiles = (ob.n_m + tileq - 1) / tileq;
-          obs_of[key] = ob.obs_tile;
+          const bool side = tp.size() >= (size_t)kLaneTargets;
+          ob.a_step = side ? (int32_t)tp.size() : 0;
+          ob.a_off = side ? base * tileq + (int64_t)t : ob.obs_tile * tileq;
           ul->obs_total += ob.n_tiles;
           ul->obs_jobs.push_back(ob);
         }
+      }
   // Distance indexing tables (unless CCM_NO_TABLE): per (j, E, tau),
   // realizations with L >= table_min_L read their neighbours from a table of
   // the R nearest points of every query (R from table_row_length at the
@@ -425,8 +475,11 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             u.wfloor = pc.weight_floor;
             u.lib_off = ul->lib_total;
             u.part_off = ul->part_total;
+            u.st_off = st_off;
+            u.st_stride = st_stride;
             u.order_off = combo[std::make_tuple(j, E, tau)];
             u.tgt_off = (int64_t)ul->targets.size();
+            int64_t obs_tile = obs_of[std::make_tuple(j, E, tau)];
             for (int64_t p : tp) {
               const int64_t o = (((p * nE + e) * nT + t) * nL + l) * pc.r + k;  // rho order
               TargetDesc tg;
@@ -436,7 +489,9 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
               tg.nbr_off = nbr_off[(size_t)o];
               tg.lib_dbg_off = lib_off[(size_t)o];
               tg.i = pc.pairs[2 * p + 1];
-              tg.obs_tile = obs_of[std::make_tuple(j, tg.i, E, tau)];
+              tg.obs_tile = obs_tile;
+              tg.unit = (int32_t)ul->units.size();
+              obs_tile += u.n_tiles;
               ul->targets.push_back(tg);
             }
             const auto tab = table_of.find(std::make_tuple(j, E, tau));
@@ -515,6 +570,8 @@ void sort_items(UnitList* ul) {
       const int32_t ea = ul->units[(size_t)ul->items[(size_t)a].unit].E;
       const int32_t eb = ul->units[(size_t)ul->items[(size_t)b].unit].E;
       if (ea != eb) return ea > eb;
+      const bool la = ul->lanes(ul->items[(size_t)a]), lb = ul->lanes(ul->items[(size_t)b]);
+      if (la != lb) return la;
       return ul->item_cost[(size_t)a] > ul->item_cost[(size_t)b];
     });
     std::vector<WorkItem> sorted(order.size());
@@ -525,13 +582,7 @@ void sort_items(UnitList* ul) {
     }
     ul->items.swap(sorted);
     ul->item_cost.swap(cost);
-    for (int E = 0; E <= kMaxE; ++E) ul->e_first[E] = ul->e_count[E] = 0;
-    for (const WorkItem& w : ul->items) ++ul->e_count[ul->units[(size_t)w.unit].E];
-    int64_t at = 0;  // groups are stored from E = 10 down to E = 1
-    for (int E = kMaxE; E >= 1; --E) {
-      ul->e_first[E] = at;
-      at += ul->e_count[E];
-    }
+    ul->groups = ul->group_items(ul->items);
   }
   // Table items: grouped by E (one launch per E), then by table (a table of
   // 5-30 MB stays in L2 while its realizations run), larger items first.
@@ -541,26 +592,27 @@ void sort_items(UnitList* ul) {
     const UnitDesc& ua = ul->units[(size_t)ul->items_table[(size_t)a].unit];
     const UnitDesc& ub = ul->units[(size_t)ul->items_table[(size_t)b].unit];
     if (ua.E != ub.E) return ua.E > ub.E;
+    const bool la = ua.n_targets >= kLaneTargets, lb = ub.n_targets >= kLaneTargets;
+    if (la != lb) return la;
     if (ua.table_off != ub.table_off) return ua.table_off < ub.table_off;
     return ul->item_cost_table[(size_t)a] > ul->item_cost_table[(size_t)b];
   });
   std::vector<WorkItem> sorted(order.size());
   for (size_t q = 0; q < order.size(); ++q) sorted[q] = ul->items_table[(size_t)order[q]];
   ul->items_table.swap(sorted);
-  for (int E = 0; E <= kMaxE; ++E) ul->te_first[E] = ul->te_count[E] = 0;
-  for (const WorkItem& w : ul->items_table) ++ul->te_count[ul->units[(size_t)w.unit].E];
-  int64_t at = 0;
-  for (int E = kMaxE; E >= 1; --E) {
-    ul->te_first[E] = at;
-    at += ul->te_count[E];
-  }
+  ul->groups_table = ul->group_items(ul->items_table);
 }
+
+// Search launches of one run, at most: per E, few or many targets, brute force
+// or table.
+constexpr int kMaxSearchLaunches = 4 * kMaxE;
 
 // Device arena layout for a unit list.
 struct Arena {
-  size_t series = 0, units = 0, items = 0, lib = 0, part = 0, done = 0, rho = 0, err = 0,
+  size_t series = 0, units = 0, items = 0, lib = 0, part = 0, rho = 0, err = 0,
          counter = 0, scratch = 0, order = 0, orders = 0, targets = 0, table = 0, tables = 0,
-         items_table = 0, order_scratch = 0, obs = 0, obs_jobs = 0, table_dist = 0, stats = 0,
+         items_table = 0, order_scratch = 0, obs = 0, obs_stat = 0, obs_jobs = 0, series_jobs = 0,
+         scales = 0, st = 0, table_dist = 0, stats = 0,
          total = 0;
 };
 
@@ -576,11 +628,10 @@ Arena layout(int64_t series_elems, const UnitList& ul, int64_t n_rho, int64_t sc
   a.units = take(sizeof(UnitDesc) * ul.units.size());
   a.items = take(sizeof(WorkItem) * ul.items.size());
   a.lib = take(sizeof(int32_t) * (size_t)ul.lib_total);
-  a.part = take(6 * sizeof(double) * (size_t)ul.part_total);
-  a.done = take(sizeof(uint32_t) * ul.units.size());
+  a.part = take(2 * sizeof(float4) * (size_t)ul.part_total);
   a.rho = take(sizeof(double) * (size_t)n_rho);
   a.err = take(sizeof(int32_t));
-  a.counter = take(2 * (kMaxE + 1) * sizeof(uint32_t));  // [E] brute force, [kMaxE+1+E] table
+  a.counter = take(kMaxSearchLaunches * sizeof(uint32_t));
   a.scratch = take(sizeof(float) * (size_t)scratch_floats);
   a.order = take(sizeof(int32_t) * (size_t)ul.order_total);
   a.order_scratch = take(sizeof(unsigned long long) * (size_t)ul.order_scratch_total);
@@ -590,8 +641,12 @@ Arena layout(int64_t series_elems, const UnitList& ul, int64_t n_rho, int64_t sc
   a.table_dist = take((ul.table_tv ? sizeof(float2) : sizeof(float)) * (size_t)ul.table_total);
   a.tables = take(sizeof(TableJob) * ul.tables.size());
   a.items_table = take(sizeof(WorkItem) * ul.items_table.size());
-  a.obs = take(sizeof(double) * kObsStride * (size_t)ul.obs_total);
+  a.obs = take(sizeof(float2) * (size_t)knn_block_threads() * (size_t)ul.obs_total);
+  a.obs_stat = take(sizeof(ObsStat) * (size_t)ul.obs_total);
   a.obs_jobs = take(sizeof(ObsJob) * ul.obs_jobs.size());
+  a.series_jobs = take(sizeof(SeriesJob) * ul.series_jobs.size());
+  a.scales = take(sizeof(float) * ul.series_jobs.size());
+  a.st = take(sizeof(float) * (size_t)ul.st_total);
   a.stats = take(sizeof(unsigned long long) * kStatCount);
   a.total = o;
   return a;
@@ -756,11 +811,11 @@ KnnParams knn_params(char* base, const Arena& ar, const UnitList& ul, int persis
   kp.table_dist = reinterpret_cast<const float*>(base + ar.table_dist);
   kp.table_pairs = ul.table_tv ? 1 : 0;
   kp.table_u16 = ul.table_u16();
-  kp.partials = reinterpret_cast<double*>(base + ar.part);
-  kp.obs = reinterpret_cast<const double*>(base + ar.obs);
-  kp.unit_done = reinterpret_cast<uint32_t*>(base + ar.done);
+  kp.partials = reinterpret_cast<float4*>(base + ar.part);
+  kp.obs = reinterpret_cast<const float2*>(base + ar.obs);
+  kp.obs_stat = reinterpret_cast<const ObsStat*>(base + ar.obs_stat);
+  kp.st = reinterpret_cast<const float*>(base + ar.st);
   kp.item_counter = reinterpret_cast<uint32_t*>(base + ar.counter);
-  kp.rho = reinterpret_cast<double*>(base + ar.rho);
   kp.err = reinterpret_cast<int32_t*>(base + ar.err);
   kp.persistent = persistent;
   for (int e = 0; e <= kMaxE; ++e) {
@@ -770,12 +825,23 @@ KnnParams knn_params(char* base, const Arena& ar, const UnitList& ul, int persis
   return kp;
 }
 
-cudaError_t enqueue_obs(char* base, const Arena& ar, const UnitList& ul, cudaStream_t s) {
+// Query order and target series, then the observed-value records.
+cudaError_t enqueue_order(char* base, const Arena& ar, const UnitList& ul, cudaStream_t s) {
+  float* scales = reinterpret_cast<float*>(base + ar.scales);
+  const cudaError_t e =
+      launch_order(reinterpret_cast<const float*>(base + ar.series),
+                   reinterpret_cast<const OrderJob*>(base + ar.orders), (int64_t)ul.orders.size(),
+                   ul.max_nm, reinterpret_cast<int32_t*>(base + ar.order),
+                   reinterpret_cast<unsigned long long*>(base + ar.order_scratch),
+                   reinterpret_cast<const SeriesJob*>(base + ar.series_jobs),
+                   (int64_t)ul.series_jobs.size(), scales, reinterpret_cast<float*>(base + ar.st), s);
+  if (e != cudaSuccess) return e;
   return launch_obs(reinterpret_cast<const float*>(base + ar.series),
                     reinterpret_cast<const int32_t*>(base + ar.order),
                     reinterpret_cast<const ObsJob*>(base + ar.obs_jobs),
-                    (int64_t)ul.obs_jobs.size(), ul.obs_total,
-                    reinterpret_cast<double*>(base + ar.obs), s);
+                    (int64_t)ul.obs_jobs.size(), ul.obs_total, scales,
+                    reinterpret_cast<float2*>(base + ar.obs),
+                    reinterpret_cast<ObsStat*>(base + ar.obs_stat), s);
 }
 
 // Enqueue sampler + fused kernel for a whole unit list on stream s.
@@ -794,16 +860,10 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
                      : cudaEventRecord(e, s);
   };
   CCM_CUDA(cudaMemsetAsync(base + ar.err, 0, sizeof(int32_t), s));
-  CCM_CUDA(cudaMemsetAsync(base + ar.counter, 0, 2 * (kMaxE + 1) * sizeof(uint32_t), s));
-  CCM_CUDA(cudaMemsetAsync(base + ar.done, 0, sizeof(uint32_t) * ul.units.size(), s));
+  CCM_CUDA(cudaMemsetAsync(base + ar.counter, 0, kMaxSearchLaunches * sizeof(uint32_t), s));
   if (stats) CCM_CUDA(cudaMemsetAsync(base + ar.stats, 0, sizeof(unsigned long long) * kStatCount, s));
   if (ev) CCM_CUDA(record(ev[0]));
-  CCM_CUDA(launch_order(reinterpret_cast<const float*>(base + ar.series),
-                        reinterpret_cast<const OrderJob*>(base + ar.orders),
-                        (int64_t)ul.orders.size(), ul.max_nm,
-                        reinterpret_cast<int32_t*>(base + ar.order),
-                        reinterpret_cast<unsigned long long*>(base + ar.order_scratch), s));
-  CCM_CUDA(enqueue_obs(base, ar, ul, s));
+  CCM_CUDA(enqueue_order(base, ar, ul, s));
   for (size_t g0 = 0; g0 < ul.tables.size();) {  // one launch per (sort size, E)
     const int rc = UnitList::table_rcap(ul.tables[g0].R), te = ul.tables[g0].E;
     size_t g1 = g0;
@@ -835,25 +895,26 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   // One launch per E (a kernel specialised for one E keeps its registers for
   // that E); each drains its own queue, larger items first, so the launches
   // follow each other with short tails.
-  for (int E = kMaxE; E >= 1; --E) {
-    if (ul.e_count[E] == 0) continue;
+  uint32_t* counter = reinterpret_cast<uint32_t*>(base + ar.counter);  // one per launch
+  for (const ItemGroup& ig : ul.groups) {
     KnnParams ke = kp;
-    ke.items = kp.items + ul.e_first[E];
-    ke.n_items = ul.e_count[E];
-    ke.item_counter = reinterpret_cast<uint32_t*>(base + ar.counter) + E;
-    const int g = persistent ? grid : (int)std::min<int64_t>(ul.e_count[E], 0x7fffffff);
-    CCM_CUDA(launch_knn(ke, E, g, s));
+    ke.items = kp.items + ig.first;
+    ke.n_items = ig.count;
+    ke.item_counter = counter++;
+    const int g = persistent ? grid : (int)std::min<int64_t>(ig.count, 0x7fffffff);
+    CCM_CUDA(launch_knn(ke, ig.E, ig.lanes, g, s));
   }
   if (ev) CCM_CUDA(record(ev[3]));
-  for (int E = kMaxE; E >= 1; --E) {
-    if (ul.te_count[E] == 0) continue;
+  for (const ItemGroup& ig : ul.groups_table) {
     KnnParams kt = kp;
-    kt.items = reinterpret_cast<const WorkItem*>(base + ar.items_table) + ul.te_first[E];
-    kt.n_items = ul.te_count[E];
-    kt.item_counter = reinterpret_cast<uint32_t*>(base + ar.counter) + (kMaxE + 1) + E;
-    const int g = persistent ? grid_table : (int)std::min<int64_t>(ul.te_count[E], 0x7fffffff);
-    CCM_CUDA(launch_knn_table(kt, E, ul.max_nm, g, s));
+    kt.items = reinterpret_cast<const WorkItem*>(base + ar.items_table) + ig.first;
+    kt.n_items = ig.count;
+    kt.item_counter = counter++;
+    const int g = persistent ? grid_table : (int)std::min<int64_t>(ig.count, 0x7fffffff);
+    CCM_CUDA(launch_knn_table(kt, ig.E, ul.max_nm, ig.lanes, g, s));
   }
+  CCM_CUDA(launch_rho(kp.units, kp.targets, (int64_t)ul.targets.size(), kp.partials, kp.obs_stat,
+                      reinterpret_cast<double*>(base + ar.rho), s));
   if (ev) CCM_CUDA(record(ev[4]));
   return CCM_OK;
 }
@@ -936,12 +997,7 @@ ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
   const Arena& ar = pl->ar;
   const UnitList& ul = pl->ul;
   // libraries and query orders for the timing launches
-  CCM_CUDA(launch_order(reinterpret_cast<const float*>(base + ar.series),
-                        reinterpret_cast<const OrderJob*>(base + ar.orders),
-                        (int64_t)ul.orders.size(), ul.max_nm,
-                        reinterpret_cast<int32_t*>(base + ar.order),
-                        reinterpret_cast<unsigned long long*>(base + ar.order_scratch), s));
-  CCM_CUDA(enqueue_obs(base, ar, ul, s));
+  CCM_CUDA(enqueue_order(base, ar, ul, s));
   SamplerParams sp = sampler_params(base, ar);
   CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, s));
   const int want = 6 * ctx->sm_count;
@@ -953,9 +1009,12 @@ ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
   ccm_status st = CCM_OK;
   for (int E = ul.emin; E <= ul.emax && st == CCM_OK; ++E) {
     if (pl->tuning.known[E]) continue;
+    // (units of many targets only where a plan has no others of this E)
+    bool lanes = true;
+    for (const ItemGroup& ig : ul.groups) lanes &= ig.E != E || ig.lanes;
     std::vector<WorkItem> all;
     for (const WorkItem& w : ul.items)
-      if (ul.units[(size_t)w.unit].E == E) all.push_back(w);
+      if (ul.units[(size_t)w.unit].E == E && ul.lanes(w) == lanes) all.push_back(w);
     if ((int)all.size() < want) continue;
     std::vector<WorkItem> sample;  // evenly spaced over the cost-sorted list
     for (int q = 0; q < want; ++q) sample.push_back(all[(size_t)q * all.size() / (size_t)want]);
@@ -975,7 +1034,7 @@ ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
         float ms = 0.f;
         for (int rep = 0; rep < 2 && ce == cudaSuccess; ++rep) {  // warm-up, then timed
           ce = cudaEventRecord(e0, s);
-          if (ce == cudaSuccess) ce = launch_knn(kp, E, (int)sample.size(), s);
+          if (ce == cudaSuccess) ce = launch_knn(kp, E, lanes, (int)sample.size(), s);
           if (ce == cudaSuccess) ce = cudaEventRecord(e1, s);
           if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
           if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
@@ -1087,7 +1146,8 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
     e = cudaMemcpy(pl->d_arena + pl->ar.items_table, pl->ul.items_table.data(),
                    sizeof(WorkItem) * pl->ul.items_table.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
-    e = cudaMemset(pl->d_arena + pl->ar.done, 0, sizeof(uint32_t) * pl->ul.units.size());
+    e = cudaMemcpy(pl->d_arena + pl->ar.series_jobs, pl->ul.series_jobs.data(),
+                   sizeof(SeriesJob) * pl->ul.series_jobs.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(pl->d_arena);
     if (pl->stream) cudaStreamDestroy(pl->stream);
@@ -1097,7 +1157,7 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
   pl->grid = persistent_grid(ctx, pl->ul.emin, pl->ul.emax);
   {
     int per_sm = 1;
-    if (knn_table_occupancy(pl->ul.max_nm, &per_sm) != cudaSuccess || per_sm < 1) per_sm = 1;
+    if (knn_table_occupancy(pl->ul.max_nm, pl->ul.lane_targets, &per_sm) != cudaSuccess || per_sm < 1) per_sm = 1;
     pl->grid_table = ctx->sm_count * per_sm;
   }
   {
@@ -1120,10 +1180,9 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
   in.table_bytes = (pl->ul.table_elem() + sizeof(float) * (pl->ul.table_tv ? 2 : 1)) *
                    (size_t)pl->ul.table_total;
   // launches of one ccm_run: order, tables, sampler, one brute-force and one
-  // table-scan kernel per E present
-  in.launches_per_run = 3 + pl->ul.table_groups();  // order, observed moments, sampler, tables
-  for (int E = 1; E <= kMaxE; ++E)
-    in.launches_per_run += (pl->ul.e_count[E] > 0 ? 1 : 0) + (pl->ul.te_count[E] > 0 ? 1 : 0);
+  // table-scan kernel per E present, rho
+  in.launches_per_run = 4 + pl->ul.table_groups();  // order, observed values, sampler, rho, tables
+  in.launches_per_run += (int64_t)(pl->ul.groups.size() + pl->ul.groups_table.size());
   *out = pl.release();
   return CCM_OK;
 }
@@ -1291,11 +1350,7 @@ ccm_status ccm_run_plain(ccm_plan_t* plan, const float* series, double* rho, voi
   const SamplerParams sp = sampler_params(base, ar);
   const UnitDesc* d_units = reinterpret_cast<const UnitDesc*>(base + ar.units);
   const TargetDesc* d_targets = reinterpret_cast<const TargetDesc*>(base + ar.targets);
-  CCM_CUDA(launch_order(reinterpret_cast<const float*>(base + ar.series),
-                        reinterpret_cast<const OrderJob*>(base + ar.orders),
-                        (int64_t)plan->ul.orders.size(), plan->ul.max_nm,
-                        reinterpret_cast<int32_t*>(base + ar.order),
-                        reinterpret_cast<unsigned long long*>(base + ar.order_scratch), s));
+  CCM_CUDA(enqueue_order(base, ar, plan->ul, s));
   for (size_t q = 0; q < plan->ul.units.size(); ++q) {
     const UnitDesc& u = plan->ul.units[q];
     CCM_CUDA(launch_sampler(sp, (int64_t)q, 1, u.n_m, s));
@@ -1436,20 +1491,21 @@ ccm_status launch_batch(ccm_context* ctx, Batch* b, bool inject) {
   // Descriptors go through pinned staging: a copy from pageable memory would
   // wait for earlier work on this (reused) stream.
   // (units, work items, order jobs, targets, table jobs, table work items,
-  // observed-moment jobs)
-  constexpr int kMeta = 7;
+  // observed-value jobs, series jobs)
+  constexpr int kMeta = 8;
   const void* src[kMeta] = {b->ul.units.data(),   b->ul.items.data(),  b->ul.orders.data(),
                             b->ul.targets.data(), b->ul.tables.data(), b->ul.items_table.data(),
-                            b->ul.obs_jobs.data()};
+                            b->ul.obs_jobs.data(),  b->ul.series_jobs.data()};
   const size_t len[kMeta] = {sizeof(UnitDesc) * b->ul.units.size(),
                              sizeof(WorkItem) * b->ul.items.size(),
                              sizeof(OrderJob) * b->ul.orders.size(),
                              sizeof(TargetDesc) * b->ul.targets.size(),
                              sizeof(TableJob) * b->ul.tables.size(),
                              sizeof(WorkItem) * b->ul.items_table.size(),
-                             sizeof(ObsJob) * b->ul.obs_jobs.size()};
+                             sizeof(ObsJob) * b->ul.obs_jobs.size(),
+                             sizeof(SeriesJob) * b->ul.series_jobs.size()};
   const size_t dst[kMeta] = {b->ar.units,  b->ar.items,       b->ar.orders,  b->ar.targets,
-                             b->ar.tables, b->ar.items_table, b->ar.obs_jobs};
+                             b->ar.tables, b->ar.items_table, b->ar.obs_jobs, b->ar.series_jobs};
   b->meta_bytes = 0;
   for (int q = 0; q < kMeta; ++q) b->meta_bytes += len[q];
   b->h_meta = pinned_get(ctx, b->meta_bytes);
@@ -1461,7 +1517,6 @@ ccm_status launch_batch(ccm_context* ctx, Batch* b, bool inject) {
     CCM_CUDA(cudaMemcpyAsync(base + dst[q], hm, len[q], cudaMemcpyHostToDevice, b->stream));
     hm += len[q];
   }
-  CCM_CUDA(cudaMemsetAsync(base + b->ar.done, 0, sizeof(uint32_t) * b->ul.units.size(), b->stream));
   Tuning tn;
   {
     std::lock_guard<std::mutex> g(ctx->mu);

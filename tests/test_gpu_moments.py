@@ -1,0 +1,111 @@
+"""Skill moments on the GPU: the epilogues of few and of many targets per library
+variable, and the paired-FP32 sums against the plain comparator's FP64 ones
+(needs a GB300)."""
+
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1905_00565_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+# Both sides sum the same FP32 predictions, the comparator in FP64.  A paired sum
+# carries 48 bits over 256 terms and its shift by the first prediction costs at
+# most (range / std)^2 <= 1e3 here: 256 * 2^-48 * 1e3 = 1e-9 in the worst case of
+# all roundings one way, 16 * 2^-48 * 1e3 = 6e-11 for independent ones.
+MOMENT_TOL = 1e-10
+
+
+@pytest.fixture(scope="module")
+def ccm():
+    from paper_1905_00565_gb300 import ccm as c
+    return c
+
+
+def run(ccm, ctx, p, flags=0, plain=False):
+    plan = ccm.plan_problem(ctx, p, flags)
+    try:
+        rho = np.zeros(ccm.rho_shape(p))
+        (ccm.ccm_run_plain if plain else ccm.ccm_run)(plan, p.series, rho)
+    finally:
+        ccm.ccm_plan_destroy(plan)
+    return rho
+
+
+def many_series(n, V, seed):
+    rng = np.random.default_rng(seed)
+    base = I.logistic_pair(n).astype(np.float64)
+    mix = rng.random((V, 2))
+    out = mix @ base + 0.05 * rng.standard_normal((V, n))
+    out[0] = base[0]
+    return np.ascontiguousarray(out.astype(np.float32))
+
+
+@pytest.mark.parametrize("targets,n", [(11, 1000), (12, 1000), (31, 513), (32, 770), (33, 1287),
+                                       (70, 300)])
+def test_many_targets_equal_one_by_one(ccm, targets, n):
+    """A library variable with many targets gives every target the bits of a plan
+    of that pair alone, from brute force and from tables."""
+    s = many_series(n, targets + 1, targets)
+    kw = dict(E=np.array([1, 3, 10], np.int32), tau=np.array([2], np.int32),
+              L=np.array([40, 260], np.int64), r=5, seed=11)
+    pairs = np.array([[0, i] for i in range(1, targets + 1)], np.int32)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        for flags in (0, ccm.CCM_NO_TABLE):
+            both = run(ccm, ctx, I.Problem(series=s, pairs=pairs, **kw), flags)
+            for t in (0, targets // 2, targets - 1):
+                one = run(ccm, ctx, I.Problem(series=s, pairs=pairs[t:t + 1], **kw), flags)
+                np.testing.assert_array_equal(both[t], one[0])
+    finally:
+        ccm.ccm_context_destroy(ctx)
+
+
+def test_repeated_pairs(ccm):
+    s = many_series(700, 9, 3)
+    pairs = np.array([[0, 1 + i % 8] for i in range(20)] + [[2, 0], [2, 0]], np.int32)
+    p = I.Problem(series=s, pairs=pairs, E=np.array([2], np.int32), tau=np.array([1], np.int32),
+                  L=np.array([50, 300], np.int64), r=3, seed=5)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        rho = run(ccm, ctx, p)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    np.testing.assert_array_equal(rho[:8], rho[8:16])
+    np.testing.assert_array_equal(rho[:4], rho[16:20])
+    np.testing.assert_array_equal(rho[20], rho[21])
+    assert np.all(np.isfinite(rho))
+
+
+@pytest.mark.parametrize("targets", [1, 14])
+def test_scaled_shifted_and_sparse_targets(ccm, targets):
+    """Targets of extreme scale, far from zero, constant, and mostly zero: the same
+    skill as the plain comparator's, and a value exactly where it has one."""
+    n = 1100
+    s = many_series(n, targets + 1, 7)
+    rows = [s[0]]
+    rng = np.random.default_rng(2)
+    made = [s[1] * np.float32(1e30), s[1] * np.float32(1e-30), s[1] + np.float32(300),
+            s[1] * np.float32(1e-41), np.full(n, 0.1, np.float32),
+            np.where(rng.random(n) < 0.002, s[1], 0).astype(np.float32)]
+    ctx = ccm.ccm_context_create(0)
+    try:
+        for odd in made:
+            series = np.ascontiguousarray(np.stack(rows + [odd] + list(s[2:])))
+            p = I.Problem(series=series,
+                          pairs=np.array([[0, i] for i in range(1, targets + 1)], np.int32),
+                          E=np.array([2, 4], np.int32), tau=np.array([1], np.int32),
+                          L=np.array([20, 120, 700], np.int64), r=4, seed=9)
+            got, want = run(ccm, ctx, p), run(ccm, ctx, p, plain=True)
+            assert np.array_equal(np.isnan(got[1:]), np.isnan(want[1:]))
+            nan = np.isnan(got[0]) != np.isnan(want[0])
+            if not np.any(np.diff(odd)):          # constant: no skill
+                assert np.all(np.isnan(got[0]))
+            else:
+                assert not np.any(nan)
+            fine = np.isfinite(got) & np.isfinite(want)
+            np.testing.assert_allclose(got[fine], want[fine], rtol=0, atol=MOMENT_TOL)
+    finally:
+        ccm.ccm_context_destroy(ctx)

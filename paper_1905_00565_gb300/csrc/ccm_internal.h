@@ -16,7 +16,11 @@ constexpr int kMaxE = 10;
 struct UnitDesc {
   int64_t series_off;   // element offset of the job's series block [V][n]
   int64_t n;            // series length of the job
-  int64_t lib_off;      // offset of this unit's library in the library buffer
+  int64_t lib_off;      // offset of this unit's library in the library buffer (units that read a
+                        // table share one slot there: only the plain comparator lists them)
+  int64_t bits_off;     // table_R > 0: this unit's membership bits, by position of the query order
+                        // (consecutive units of one cell lie back to back)
+  int64_t words_off;    // table_R > 0 and one target: its scan group's membership words
   int64_t part_off;     // first partial-sum slot: target t, tile q at part_off + t*n_tiles + q
   int64_t order_off;    // first entry of this unit's query order (per variable, E, tau)
   int64_t tgt_off;      // first TargetDesc of this unit
@@ -29,12 +33,10 @@ struct UnitDesc {
   int32_t n_m;          // manifold points = queries
   int32_t n_tiles;      // query tiles of the fused kernel
   int32_t n_targets;    // targets cross-mapped from this library (>= 1)
-  int32_t table_R;      // > 0: neighbours read from the table (R entries per query)
+  int32_t table_R;      // > 0: neighbours read from the table (its row length, a multiple of 64)
   int32_t theiler;      // exclusion window W >= 0: candidates l of query m need |l - m| > W
   float wfloor;         // simplex weight floor f >= 0: u_i = max(u_i, f)
-  int32_t table_tv;     // 1: the table also holds this unit's (single) target's values
   int32_t st_stride;
-  int32_t pad;
 };
 // Units with at least this many targets form their predictions with one lane
 // per target (coalesced reads of the time-major series); fewer, one thread per
@@ -88,12 +90,12 @@ struct SeriesJob {
   int32_t scale;        // where the scale goes
 };
 
-// One work item of the fused kernels: query tiles of a unit, from `tile` on.  A
-// brute-force item holds up to `count` tiles (brute_chunk), a table item up to
-// kTableChunk; the last item of a unit may hold fewer.
-// A table item may cover `count` consecutive realizations of one cell (units
-// unit .. unit + count - 1): one walk of each query's table row serves all of
-// them.
+// One work item of the search kernels: query tiles of a unit, from `tile` on;
+// the last item of a unit may hold fewer than its count says.
+//   brute force: up to `count` tiles (brute_chunk)
+//   table scan of units with one target (knn_scan.cu): (count >> 8) tiles of
+//     count & 255 consecutive units, realizations of one (j, E, tau)
+//   table walk of units with several targets: up to kTableChunk tiles
 struct WorkItem {
   int32_t unit;
   int32_t tile;
@@ -119,8 +121,17 @@ inline int32_t brute_chunk(int64_t tiles, int64_t L, int E) {
   const int64_t c = tiles / (L <= brute_tile_points(E) ? kBruteSlots : 8 * kBruteSlots);
   return c < 1 ? 1 : c > kBruteChunk ? kBruteChunk : (int32_t)c;
 }
-constexpr int kTableGroup = 4;         // realizations per grouped table item, at most
-constexpr int kTableGroupMaxNm = 32768;  // grouping needs a byte membership map (bit b: realization b)
+constexpr int kScanGroup = 32;         // realizations per scan item: one lane each
+constexpr int kScanChunk = 8;          // query tiles per scan item, at most
+constexpr size_t kScanSmemMax = 112 * 1024;  // shared memory of a scan CTA: two fit an SM
+// Membership words of a scan group: one per position of the query order, and
+// zeros up to a whole number of 32 beyond the last (table rows are padded with
+// position n_m).
+__host__ __device__ constexpr int member_words(int n_m) { return (n_m + 32) / 32 * 32; }
+// One scan group: `count` consecutive units from `unit` on.
+struct MemberGroup {
+  int32_t unit, count;
+};
 
 // Query order job: one per (job, library variable, E, tau).
 struct OrderJob {
@@ -139,9 +150,12 @@ struct TableJob {
   int64_t series_off;   // element offset of the job's series block
   int64_t n;            // series length
   int64_t order_off;    // query order of this combination
-  int64_t table_off;    // first entry: table[table_off + r * n_m + pos]
-  int32_t j, E, tau, n_m, R;
+  int64_t table_off;    // first entry: rank r of query position pos at table_off + pos*stride + r
+  int32_t j, E, tau, n_m;
+  int32_t R;            // entries per row; padded with position n_m to
+  int32_t stride;       // a multiple of 64
   int32_t tv_i;         // >= 0: also store target variable tv_i's value at every entry's point
+  int32_t pad;
 };
 constexpr int kTableMaxR = 2048;       // entries per query row, at most
 constexpr int kTableChunk = 8;         // query tiles per table work item (one bitmap each)
@@ -153,6 +167,8 @@ struct SamplerParams {
   const TargetDesc* targets;  // for the debug copies (lib_dbg_off per target)
   const int32_t* order;   // query orders (per variable, E, tau); libraries follow them
   int32_t* lib;           // library buffer (sum of L), each library in query order
+  uint32_t* bits;         // membership bits of the units that read a table (no list is written)
+  int32_t list_all;       // 1: list those too (at lib_off)
   int32_t* dbg_lib;       // optional: libraries in ascending m, once per target, in rho order
   int32_t* err;           // error flag (set, never cleared, by the kernels)
 };
@@ -166,10 +182,13 @@ struct KnnParams {
   int64_t n_items;
   const int32_t* lib;
   const int32_t* order;   // query order (manifold index per position)
+  const uint32_t* bits;   // membership bits of the units that read a table
+  const uint32_t* words;  // membership words of the scan groups
   const void* table;      // distance indexing tables (units with table_R > 0)
   const float* table_dist;  // every table entry's distance sqrt_hw(FP32 squared distance), same
                             // layout; table_pairs: float2 {distance, target value} per entry
   int32_t table_pairs;    // 1: the tables store (distance, target value) pairs (TableJob::tv_i)
+  int32_t window;         // 1: some unit has an exclusion window
   int32_t table_u16;      // 1: uint16 entries (every manifold below 65536 points), 0: int32
   float4* partials;       // two float4 per (target, query tile): its sums (moments.cuh)
   const float2* obs;      // centred observations, 256 per record (TargetDesc::obs_tile)
@@ -245,24 +264,28 @@ constexpr int32_t kErrSampler = 2;
 
 // Sampler (sampler.cu).
 constexpr int kSamplerThreads = 256;
-constexpr int kSamplerSmemKeys = 40960;   // keys kept in shared memory up to this N_m
+constexpr int kSamplerBitsMax = 1 << 20;  // membership bits in shared memory up to this N_m
 cudaError_t sampler_prepare();
 cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t count,
                            int max_nm, cudaStream_t s);
+// Membership words of the scan groups from their units' bits.
+cudaError_t launch_member_words(const UnitDesc* units, const MemberGroup* groups, int64_t n_groups,
+                                int max_nm, const uint32_t* bits, uint32_t* words, cudaStream_t s);
 
 // Query order (order.cu).
 cudaError_t order_prepare();
+// inverse (optional): the position of every manifold index, same offsets.
 // The same launch prepares the target series (SeriesJob).
 cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jobs, int max_nm,
-                         int32_t* order, unsigned long long* scratch, const SeriesJob* series_jobs,
-                         int64_t n_series_jobs, float* scales, float* st, cudaStream_t s);
+                         int32_t* order, int32_t* inverse, unsigned long long* scratch,
+                         const SeriesJob* series_jobs, int64_t n_series_jobs, float* scales, float* st, cudaStream_t s);
 
 // Distance indexing table (table.cu).
 cudaError_t table_prepare();
 // One launch builds the tables of jobs[0..n_jobs), all of embedding dimension E.
 cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_t n_jobs, int E,
-                               int max_nm, int max_R, const int32_t* order, void* table,
-                               float* table_dist, int table_pairs, int table_u16, cudaStream_t s);
+                               int max_nm, int max_R, const int32_t* order,
+                               const int32_t* inverse, void* table, float* table_dist, int table_pairs, int table_u16, cudaStream_t s);
 
 // Search kernels of one E (knn_fused.cu, compiled once per E; each kernel keeps
 // its registers for that E's lists).
@@ -275,6 +298,8 @@ struct KnnKernels {
   static cudaError_t occupancy_table(int max_nm, bool lanes, int* ctas);
   static cudaError_t launch_table(const KnnParams& p, int max_nm, bool lanes, int grid,
                                   cudaStream_t s);
+  static cudaError_t prepare_scan();
+  static cudaError_t launch_scan(const KnnParams& p, int max_nm, int grid, cudaStream_t s);
 };
 
 // Their dispatch, and what surrounds the search (knn_dispatch.cu).
@@ -299,6 +324,9 @@ cudaError_t knn_table_prepare();
 cudaError_t knn_table_occupancy(int max_nm, bool lane_targets, int* ctas_per_sm);
 cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lane_targets, int grid,
                              cudaStream_t s);
+// Units with one target: grouped realizations (two CTAs per SM).
+cudaError_t knn_scan_prepare();
+cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, cudaStream_t s);
 
 // Sets the thread-local message returned by ccm_last_error() (runtime.cu).
 void set_last_error(const char* msg);

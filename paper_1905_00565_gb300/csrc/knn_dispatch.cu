@@ -146,6 +146,10 @@ int knn_queries_per_thread() { return 1; }
   if (const cudaError_t e = KnnKernels<EV>::prepare(); e != cudaSuccess) return e;
 #define CCM_CASE_PREPARE_TABLE(EV)                                       \
   if (const cudaError_t e = KnnKernels<EV>::prepare_table(); e != cudaSuccess) return e;
+#define CCM_CASE_PREPARE_SCAN(EV)                                        \
+  if (const cudaError_t e = KnnKernels<EV>::prepare_scan(); e != cudaSuccess) return e;
+#define CCM_CASE_LAUNCH_SCAN(EV) \
+  case EV: return KnnKernels<EV>::launch_scan(p, max_nm, grid, s);
 #define CCM_CASE_OCCUPANCY(EV) \
   case EV: return KnnKernels<EV>::occupancy(ctas);
 #define CCM_CASE_LAUNCH(EV) \
@@ -160,6 +164,14 @@ cudaError_t knn_prepare() {
 cudaError_t knn_table_prepare() {
   CCM_FOR_E(CCM_CASE_PREPARE_TABLE)
   return cudaSuccess;
+}
+cudaError_t knn_scan_prepare() {
+  CCM_FOR_E(CCM_CASE_PREPARE_SCAN)
+  return cudaSuccess;
+}
+cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, cudaStream_t s) {
+  switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH_SCAN) }
+  return cudaErrorInvalidValue;
 }
 cudaError_t knn_occupancy(int E, int* ctas) {
   switch (E) { CCM_FOR_E(CCM_CASE_OCCUPANCY) }

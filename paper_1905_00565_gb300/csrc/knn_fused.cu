@@ -315,14 +315,12 @@ __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc&
 // holds the weights and neighbours in shared memory, so that a reduction
 // between two targets finds no live registers to spill; other warps may still
 // be searching, so nothing else of the buffer is touched before a barrier.
-// kKeep false: they stay in registers (keep: the lane-per-target scratch).  nb_values (table path, one target, no checking copy of
-// the neighbours): nb holds the bits of the target's values at the E+1
-// neighbours, read from the table instead of gathered.
+// kKeep false: they stay in registers (keep: the lane-per-target scratch).
 static_assert(kMaxE + 1 <= kBuf, "the epilogue keeps E+1 entries in a candidate column");
 template <int E, bool kLanes, bool kKeep, bool kDist = false>
 __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& u, int tile, int m, bool valid, const float (&dd)[E + 1],
                                             const int (&nb)[E + 1], float* ring, RingMeta* meta,
-                                            int& ring_n, u64* keep, bool nb_values = false) {
+                                            int& ring_n, u64* keep) {
   const int tid = threadIdx.x;
   const int n_m = u.n_m;
   const int off = (E - 1) * u.tau;
@@ -379,13 +377,8 @@ __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& 
     const TargetDesc tg = p.targets[u.tgt_off + t];
     const float* si = p.series + u.series_off + (int64_t)tg.i * u.n;
     float acc = 0.f;
-    if (nb_values) {  // nb holds the table's copy of the target at the neighbours
 #pragma unroll
-      for (int s = 0; s <= E; ++s) acc = __fmaf_rn(weight(s), __int_as_float(nbr(s)), acc);
-    } else {
-#pragma unroll
-      for (int s = 0; s <= E; ++s) acc = __fmaf_rn(weight(s), si[nbr(s) + off], acc);
-    }
+    for (int s = 0; s <= E; ++s) acc = __fmaf_rn(weight(s), si[nbr(s) + off], acc);
     const float xhat = __fmul_rn(acc, rcp_hw(usum));  // usum >= exp(-1)
     if (valid) {
       if (p.dbg_xhat) p.dbg_xhat[tg.q_off + m] = xhat;
@@ -823,12 +816,14 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
 }
 
 // --------------------------------------------------------------------------
-// Table path: the library's members are marked in a shared-memory bitmap and
-// each query walks its row of the distance indexing table (sorted by (FP32
-// squared distance, index) over the whole manifold, the query itself left
-// out) until it has met E+1 library members outside the exclusion window.  Those are, in order, the E+1 nearest
-// library neighbours -- the same list the brute-force scan produces.  A query
-// whose R table entries hold fewer members falls back to scanning the library.
+// Table path of units with several targets (units with one: knn_scan.cu): the
+// unit's membership bits (by position of the query order) are copied to shared
+// memory and each query walks its row of the distance indexing table (sorted
+// by (FP32 squared distance, index) over the whole manifold, the query itself
+// left out) until it has met E+1 library members outside the exclusion window.
+// Those are, in order, the E+1 nearest library neighbours -- the same list the
+// brute-force scan produces.  A query whose row holds fewer members scans the
+// library.
 template <int E>
 __device__ __forceinline__ float d2_point(const float* sj, int off, int tau, const float (&q)[E],
                                           int x) {
@@ -843,227 +838,143 @@ __device__ __forceinline__ float d2_point(const float* sj, int off, int tau, con
 }
 
 // Shared memory of the table kernel: the epilogue's ring of predictions, the
-// walk's records (below), then the library membership map: one byte per
-// manifold point when the manifold has at most kByteMapMax points (bit b: the
-// point is in realization b's library), else one bit (one realization).
+// walk's records (below), then the membership bits.
 //
 // A record is one step of the walk (eight consecutive ranks of the row) that
-// held members of a realization: (step << 8) | flags, flag c marking rank
-// 8*step + c.  A realization stops recording once it has E+1 members, so it
-// keeps at most E+1 records: [kTableGroup][kMaxE+1][kThreads] 16-bit words.
-constexpr int kRecBytes = kTableGroup * (kMaxE + 1) * kThreads * 2;
-constexpr int kByteMapMax = 32768;
+// held members: (step << 8) | flags, flag c marking rank 8*step + c.  A query
+// keeps at most E+1 records: [kMaxE+1][kThreads] 16-bit words.
+constexpr int kRecBytes = (kMaxE + 1) * kThreads * 2;
 static_assert(kTableMaxR / 8 <= 256, "a record's step index has eight bits");
-static_assert(kTableGroupMaxNm <= kByteMapMax, "grouped table items need the byte map");
-static_assert(kTableGroup <= 4, "one byte of member flags per realization in 32 bits");
 
-// One query's walk along its table row (see process_table_item): `at` is the
-// element of its rank group 0, `rec` its column of the records, and act,
-// counts and nrec the per-realization bytes described there.  The map is a
-// byte map (kBytes) or a bitmap, fixed per work item, so each kind gets its
-// own loop.
-template <int K, bool kBytes, bool kStats>
-__device__ __forceinline__ void table_walk(const KnnParams& p, int64_t at, int n_m, int groups, int m,
-                                           int W, const unsigned char* map, uint16_t* rec,
-                                           uint32_t& act, uint32_t& counts, uint32_t& nrec,
-                                           uint32_t& st_entries) {
-  const uint32_t table_limit = (uint32_t)(0x80 - K) * 0x01010101u;
-  for (int g = 0; __any_sync(kFull, act != 0u && g < groups); g += 2) {
-    const bool w0 = act != 0u && g < groups, w1 = act != 0u && g + 1 < groups;
-    if (kStats) st_entries += (w0 ? 4u : 0u) + (w1 ? 4u : 0u);
-    int x[8];  // ranks 4g .. 4g+7 of this query's row (index 0 when not loaded)
-    if (p.table_u16) {
-      const uint16_t* t16 = static_cast<const uint16_t*>(p.table) + at;
-      const uint2 v0 = w0 ? __ldg(reinterpret_cast<const uint2*>(t16 + (int64_t)g * 4 * n_m))
-                          : make_uint2(0u, 0u);
-      const uint2 v1 = w1 ? __ldg(reinterpret_cast<const uint2*>(t16 + (int64_t)(g + 1) * 4 * n_m))
-                          : make_uint2(0u, 0u);
-      x[0] = v0.x & 0xffffu; x[1] = v0.x >> 16; x[2] = v0.y & 0xffffu; x[3] = v0.y >> 16;
-      x[4] = v1.x & 0xffffu; x[5] = v1.x >> 16; x[6] = v1.y & 0xffffu; x[7] = v1.y >> 16;
+// One query's walk along its table row (`row`: its entries): records the steps
+// with members until it has K of them; returns the members met.
+template <int K, typename Index, bool kStats>
+__device__ __forceinline__ int table_walk(const Index* row, const int32_t* order, int steps, int m,
+                                          int W, const uint32_t* bits, uint16_t* rec, bool active,
+                                          uint32_t& st_entries) {
+  int got = 0, nrec = 0;
+  for (int g = 0; __any_sync(kFull, active && got < K && g < steps); ++g) {
+    if (!(active && got < K && g < steps)) continue;
+    if (kStats) st_entries += 8u;
+    int x[8];  // ranks 8g .. 8g+7
+    if (sizeof(Index) == 2) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + g);
+      x[0] = v.x & 0xffffu; x[1] = v.x >> 16; x[2] = v.y & 0xffffu; x[3] = v.y >> 16;
+      x[4] = v.z & 0xffffu; x[5] = v.z >> 16; x[6] = v.w & 0xffffu; x[7] = v.w >> 16;
     } else {
-      const int32_t* t32 = static_cast<const int32_t*>(p.table) + at;
-      const int4 v0 = w0 ? __ldg(reinterpret_cast<const int4*>(t32 + (int64_t)g * 4 * n_m))
-                         : make_int4(0, 0, 0, 0);
-      const int4 v1 = w1 ? __ldg(reinterpret_cast<const int4*>(t32 + (int64_t)(g + 1) * 4 * n_m))
-                         : make_int4(0, 0, 0, 0);
+      const int4 v0 = __ldg(reinterpret_cast<const int4*>(row) + 2 * g);
+      const int4 v1 = __ldg(reinterpret_cast<const int4*>(row) + 2 * g + 1);
       x[0] = v0.x; x[1] = v0.y; x[2] = v0.z; x[3] = v0.w;
       x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
     }
-    // member flags: the map byte's bit b moved to bit c of byte b (the
-    // multiply spreads bits 0..3 to bits 0, 8, 16, 24)
     uint32_t flags = 0u;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const uint32_t mb = kBytes ? (uint32_t)map[x[c]]
-                                 : ((reinterpret_cast<const uint32_t*>(map)[x[c] >> 5] >> (x[c] & 31)) & 1u);
-      flags |= (kBytes ? ((mb * 0x00204081u) & 0x01010101u) : mb) << c;  // a bitmap: one realization
-    }
-    flags &= act & ((w0 ? 0x0f0f0f0fu : 0u) | (w1 ? 0xf0f0f0f0u : 0u));
-    if (W > 0) {
-      // points inside the exclusion window |x - m| <= W are no neighbours
+    for (int c = 0; c < 8; ++c) flags |= ((bits[x[c] >> 5] >> (x[c] & 31)) & 1u) << c;
+    if (W > 0 && flags != 0u) {
+      // points inside the exclusion window |l - m| <= W are no neighbours
       // (the row never holds m itself, so W = 0 excludes nothing)
-      uint32_t win = 0u;
 #pragma unroll
       for (int c = 0; c < 8; ++c)
-        win |= (((unsigned)x[c] - (unsigned)m + (unsigned)W <= 2u * (unsigned)W) ? 1u : 0u) << c;
-      flags &= ~(win * 0x01010101u);
+        if ((flags >> c) & 1u) {
+          const int l = order[x[c]];
+          if ((unsigned)l - (unsigned)m + (unsigned)W <= 2u * (unsigned)W) flags &= ~(1u << c);
+        }
     }
     if (flags != 0u) {
-      // one record per realization with members in this step
-#pragma unroll
-      for (int b = 0; b < kTableGroup; ++b) {
-        const uint32_t fb = (flags >> (8 * b)) & 0xffu;
-        if (fb != 0u) {
-          const uint32_t i = (nrec >> (8 * b)) & 0xffu;  // < K: the realization was short
-          rec[(b * K + (int)i) * kThreads] = (uint16_t)(((uint32_t)(g >> 1) << 8) | fb);
-          nrec += 1u << (8 * b);
-        }
-      }
-      // per-byte population counts, then the realizations now complete
-      uint32_t v = flags - ((flags >> 1) & 0x55555555u);
-      v = (v & 0x33333333u) + ((v >> 2) & 0x33333333u);
-      counts += (v + (v >> 4)) & 0x0f0f0f0fu;  // each byte stays below K + 8
-      const uint32_t done = ((counts + table_limit) & 0x80808080u) >> 7;  // counts_b >= K
-      act &= ~(done * 0xffu);
+      rec[nrec * kThreads] = (uint16_t)(((uint32_t)g << 8) | flags);
+      ++nrec;
+      got += __popc(flags);
     }
   }
+  return got;
 }
 
 template <int E, bool kLanes, bool kStats>
-__device__ void process_table_item(const KnnParams& p, int unit0, int count, int tile0,
+__device__ void process_table_item(const KnnParams& p, const UnitDesc& u, int tile0,
                                    unsigned char* smem, RingMeta* meta, int& ring_n) {
-  // `count` consecutive realizations of one cell (the same manifold, table, L
-  // and target; count > 1 only with a byte map): one walk of each query's row
-  // finds the E+1 nearest members of every one of them.
   constexpr int K = E + 1;
   const int tid = threadIdx.x;
-  const UnitDesc u0 = p.units[unit0];
-  const int n_m = u0.n_m, L = u0.L, tau = u0.tau, R = u0.table_R, W = u0.theiler;
+  const int n_m = u.n_m, tau = u.tau, stride = u.table_R, W = u.theiler;
   const int off = (E - 1) * tau;
-  const float* sj = p.series + u0.series_off + (int64_t)u0.j * u0.n;
+  const float* sj = p.series + u.series_off + (int64_t)u.j * u.n;
+  const int32_t* order = p.order + u.order_off;
   float* s_ring = reinterpret_cast<float*>(smem);
-  uint16_t* s_rec = reinterpret_cast<uint16_t*>(smem + kRingBytes);  // [count][K][kThreads]
-  unsigned char* map = smem + kRingBytes + kRecBytes;
+  uint16_t* s_rec = reinterpret_cast<uint16_t*>(smem + kRingBytes);  // [K][kThreads]
+  uint32_t* s_bits = reinterpret_cast<uint32_t*>(smem + kRingBytes + kRecBytes);
   u64* s_keep = reinterpret_cast<u64*>(smem + p.lane_scratch);
-  const bool bytes = n_m <= kByteMapMax;
-  const int words = bytes ? (n_m + 3) >> 2 : (n_m + 31) >> 5;  // 32-bit words of the map
-  uint32_t* mw = reinterpret_cast<uint32_t*>(map);
-  // Library membership, once for the item's tiles: byte x holds bit b when
-  // point x is in realization b's library (a bitmap of one realization for
-  // manifolds above kByteMapMax points).
-  __syncthreads();  // the previous item's readers of the map are done
-  for (int w = tid; w < words; w += kThreads) mw[w] = 0u;
-  __syncthreads();
-  for (int b = 0; b < count; ++b) {
-    const int32_t* lib = p.lib + p.units[unit0 + b].lib_off;
-    for (int a = tid; a < L; a += kThreads) {
-      const int l = lib[a];
-      if (!bytes) atomicOr(&mw[l >> 5], 1u << (l & 31));
-      else if (count == 1) map[l] = 1;
-      else atomicOr(&mw[l >> 2], (1u << b) << (8 * (l & 3)));
-    }
-  }
+  const int words = (n_m + 31) >> 5;
+  __syncthreads();  // the previous item's readers of the bits are done
+  for (int w = tid; w < (n_m + 32) >> 5; w += kThreads)  // one beyond the last position at least
+    s_bits[w] = w < words ? p.bits[u.bits_off + w] : 0u;
   __syncthreads();
 
-  const int tile1 = min(u0.n_tiles, tile0 + kTableChunk);
-  const int groups = R >> 2;  // groups of four ranks
-  const uint32_t all = (count >= 4) ? 0xffffffffu : (1u << (8 * count)) - 1u;
+  const int tile1 = min(u.n_tiles, tile0 + kTableChunk);
   for (int tile = tile0; tile < tile1; ++tile) {
     const int pos = tile * kQT + tid;
     const bool valid = pos < n_m;
-    const int m = p.order[u0.order_off + (valid ? pos : n_m - 1)];
-
-    // Walk the row (every manifold point but m, in (distance, index) order),
-    // eight ranks a step; for each realization the first E+1 members outside
-    // the window are its neighbours, in order.  Everything below works on four bytes at once,
-    // byte b for realization b: `flags` the step's members (bit c: rank
-    // 8*step + c), `counts` the members found so far, `act` 0xff while a
-    // realization still lacks some, `nrec` its records.
-    uint32_t act = valid ? all : 0u, counts = 0u, nrec = 0u;
-    const int64_t col = (int64_t)(valid ? pos : 0) * 4;
+    const int m = order[valid ? pos : n_m - 1];
+    const int64_t row = u.table_off + (int64_t)(valid ? pos : 0) * stride;
     uint32_t st_entries = 0;
-    if (bytes)
-      table_walk<K, true, kStats>(p, u0.table_off + col, n_m, groups, m, W, map, s_rec + tid, act,
-                                  counts, nrec, st_entries);
-    else
-      table_walk<K, false, kStats>(p, u0.table_off + col, n_m, groups, m, W, map, s_rec + tid, act,
-                                   counts, nrec, st_entries);
+    uint16_t* rec = s_rec + tid;
+    const int got =
+        p.table_u16 ? table_walk<K, uint16_t, kStats>(static_cast<const uint16_t*>(p.table) + row,
+                                                      order, stride >> 3, m, W, s_bits, rec, valid,
+                                                      st_entries)
+                    : table_walk<K, int32_t, kStats>(static_cast<const int32_t*>(p.table) + row,
+                                                     order, stride >> 3, m, W, s_bits, rec, valid,
+                                                     st_entries);
+    const bool full = got >= K;
     if (kStats) {
       const uint32_t ent = __reduce_add_sync(kFull, st_entries);
       const unsigned vq = __popc(__ballot_sync(kFull, valid));
+      const unsigned fb = __popc(__ballot_sync(kFull, valid && !full));
       if ((tid & 31) == 0) {
         atomicAdd(&p.stats[kStatTableEntries], (unsigned long long)ent);
-        atomicAdd(&p.stats[kStatTableQueries], (unsigned long long)vq * count);
+        atomicAdd(&p.stats[kStatTableQueries], (unsigned long long)vq);
+        if (fb) atomicAdd(&p.stats[kStatTableFallbacks], (unsigned long long)fb);
       }
     }
-    for (int b = 0; b < count; ++b) {
-      const UnitDesc u = (b == 0) ? u0 : p.units[unit0 + b];
-      const bool full = ((counts >> (8 * b)) & 0xffu) >= (uint32_t)K;
-      if (kStats) {
-        const unsigned fb = __popc(__ballot_sync(kFull, valid && !full));
-        if ((tid & 31) == 0 && fb) atomicAdd(&p.stats[kStatTableFallbacks], (unsigned long long)fb);
+    int nb[E + 1];
+    float dd[E + 1];
+    if (full) {
+      // the first E+1 flagged ranks; their points and distances are read from
+      // the table (the stored distances are the bits the epilogue would
+      // compute: the build used the same rounding sequence and square root)
+      int ri = 0;
+      uint32_t cur = rec[0];
+#pragma unroll
+      for (int s2 = 0; s2 <= E; ++s2) {
+        if ((cur & 0xffu) == 0u) cur = rec[(++ri) * kThreads];
+        const int c = __ffs(cur & 0xffu) - 1;
+        cur &= ~(1u << c);
+        const int64_t at = row + 8 * (int)(cur >> 8) + c;
+        dd[s2] = p.table_pairs ? __ldg(reinterpret_cast<const float2*>(p.table_dist) + at).x
+                               : __ldg(p.table_dist + at);
+        nb[s2] = order[p.table_u16 ? (int)__ldg(static_cast<const uint16_t*>(p.table) + at)
+                                   : __ldg(static_cast<const int32_t*>(p.table) + at)];
       }
-      int nb[E + 1];
-      float dd[E + 1];
-      // target values from the table (not when the neighbours are checked)
-      bool tv = u.table_tv != 0 && p.table_pairs && p.dbg_nbr == nullptr;
-      if (full || !valid) {
-        // the first E+1 flagged ranks of the realization's records; their
-        // indices and distances are read from the table (the stored distances
-        // are the bits the epilogue would compute: the build used the same
-        // rounding sequence and the same square root)
-        const int nr = (int)((nrec >> (8 * b)) & 0xffu);
-        const uint16_t* rec = s_rec + b * K * kThreads + tid;
-        int ri = 0;
-        uint32_t cur = valid ? rec[0] : 0u;
+    } else if (!valid) {
 #pragma unroll
-        for (int s2 = 0; s2 <= E; ++s2) {
-          while ((cur & 0xffu) == 0u && ri + 1 < nr) cur = rec[(++ri) * kThreads];
-          const uint32_t fl = cur & 0xffu;
-          const int c = fl ? __ffs(fl) - 1 : 0;  // fl > 0 whenever the walk was full
-          cur &= ~(1u << c);
-          nb[s2] = 8 * (int)(cur >> 8) + c;  // the rank, for now
-        }
-        // the distances (not squared) and, when the table holds them, the
-        // target's values at the neighbours (one 8-byte load each), else the
-        // neighbours' indices (for the gather)
-        auto at = [&](int rank) {
-          return u0.table_off + (int64_t)(rank >> 2) * 4 * n_m + col + (rank & 3);
-        };
-        const float2* dv2 = reinterpret_cast<const float2*>(p.table_dist);
-        if (tv) {
+      for (int s2 = 0; s2 <= E; ++s2) {
+        dd[s2] = 0.f;
+        nb[s2] = 0;
+      }
+    } else {
+      // Rare: fewer than E+1 members in the row; scan the library, keeping the
+      // E+1 smallest (distance, index) keys.
+      float q[E];
 #pragma unroll
-          for (int s2 = 0; s2 <= E; ++s2) {
-            const float2 dv = valid ? __ldg(dv2 + at(nb[s2])) : make_float2(0.f, 0.f);
-            dd[s2] = dv.x;
-            nb[s2] = __float_as_int(dv.y);
-          }
-        } else {
+      for (int e = 0; e < E; ++e) q[e] = sj[m + off - e * tau];
+      float kd[E + 1];
+      int kl[E + 1];
 #pragma unroll
-          for (int s2 = 0; s2 <= E; ++s2) {
-            const int64_t a2 = at(nb[s2]);
-            dd[s2] = !valid ? 0.f : p.table_pairs ? __ldg(dv2 + a2).x : __ldg(p.table_dist + a2);
-            nb[s2] = !valid ? 0
-                            : (p.table_u16 ? (int)__ldg(static_cast<const uint16_t*>(p.table) + a2)
-                                           : __ldg(static_cast<const int32_t*>(p.table) + a2));
-          }
-        }
-      } else {
-        // Rare: fewer than E+1 members among the R nearest points; scan the
-        // library, keeping the E+1 smallest (distance, index) keys.
-        const int32_t* lib = p.lib + u.lib_off;
-        float q[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) q[e] = sj[m + off - e * tau];
-        float kd[E + 1];
-        int kl[E + 1];
-#pragma unroll
-        for (int s2 = 0; s2 <= E; ++s2) {
-          kd[s2] = INFINITY;
-          kl[s2] = INT_MAX;
-        }
-        for (int a = 0; a < L; ++a) {
-          const int l = lib[a];
+      for (int s2 = 0; s2 <= E; ++s2) {
+        kd[s2] = INFINITY;
+        kl[s2] = INT_MAX;
+      }
+      for (int w = 0; w < words; ++w) {
+        for (uint32_t left = s_bits[w]; left != 0u; left &= left - 1u) {
+          const int l = order[32 * w + __ffs(left) - 1];
           if (abs(l - m) <= W) continue;
           const float d = d2_point<E>(sj, off, tau, q, l);
           if (key_less(d, l, kd[E], kl[E])) {
@@ -1077,24 +988,19 @@ __device__ void process_table_item(const KnnParams& p, int unit0, int count, int
             kl[s2] = l;
           }
         }
-#pragma unroll
-        for (int s2 = 0; s2 <= E; ++s2) {
-          nb[s2] = min(max(kl[s2], 0), n_m - 1);  // in bounds however few points qualified
-          dd[s2] = sqrt_hw(kd[s2]);
-        }
-        tv = false;  // gathered as for brute force
       }
-      finish_tile<E, kLanes, false, true>(p, u, tile, m, valid, dd, nb, s_ring, meta, ring_n, s_keep, tv);
+#pragma unroll
+      for (int s2 = 0; s2 <= E; ++s2) {
+        nb[s2] = min(max(kl[s2], 0), n_m - 1);  // in bounds however few points qualified
+        dd[s2] = sqrt_hw(kd[s2]);
+      }
     }
+    finish_tile<E, kLanes, false, true>(p, u, tile, m, valid, dd, nb, s_ring, meta, ring_n, s_keep);
   }
 }
 
-// kMinCtas CTAs per SM.  Four (64 registers a thread) for manifolds with a
-// byte map: the walk waits on L2, and more resident warps hide more of it
-// than the few spilled registers cost (the sweep's scan: 151 ms, 165 ms with
-// three).  Three (80 registers) for longer manifolds (bitmap, one realization
-// an item, tables beyond L2), which want the registers (the N = 10^5 series'
-// scan: 110 ms, 120 ms with four).
+// kMinCtas CTAs per SM: two (128 registers) with a lane per target, whose
+// epilogue is the work; four (64 registers) else, where the walk waits on L2.
 template <int E, bool kLanes, bool kStats, int kMinCtas>
 __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1111,12 +1017,11 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams
     if ((int64_t)it >= p.n_items) break;
     const WorkItem w = p.items[it];
     const UnitDesc u = p.units[w.unit];
-    if (u.E != E || (u.n_targets >= kLaneTargets) != kLanes || w.count < 1 || w.count > kTableGroup ||
-        (w.count > 1 && u.n_m > kByteMapMax)) {
+    if (u.E != E || (u.n_targets >= kLaneTargets) != kLanes) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrBadUnit);
       continue;
     }
-    process_table_item<E, kLanes, kStats>(p, w.unit, w.count, w.tile, smem, s_meta, ring_n);
+    process_table_item<E, kLanes, kStats>(p, u, w.tile, smem, s_meta, ring_n);
   }
   if (ring_n > 0) flush_ring(reinterpret_cast<const float*>(smem), s_meta, ring_n);
 }
@@ -1150,13 +1055,10 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
     flush_ring(reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);
 }
 
-// Ring, records and map: every manifold of the launch fits (bytes up to
-// kByteMapMax points, bits above).
+// Ring, records and bits: every manifold of the launch fits.
 size_t table_base_smem(int max_nm) {
-  const size_t bits = (size_t)((max_nm + 31) / 32) * 4;
-  const size_t map = (max_nm <= kByteMapMax) ? (size_t)(max_nm + 3) / 4 * 4
-                                             : (bits > (size_t)kByteMapMax ? bits : kByteMapMax);
-  return ((size_t)kRingBytes + (size_t)kRecBytes + map + 15) / 16 * 16;
+  const size_t bits = (size_t)((max_nm + 32) / 32) * 4;
+  return ((size_t)kRingBytes + (size_t)kRecBytes + bits + 15) / 16 * 16;
 }
 size_t table_smem(int max_nm, bool lane_targets) {
   return table_base_smem(max_nm) +
@@ -1191,14 +1093,10 @@ cudaError_t KnnKernels<E>::occupancy(int* ctas) {
                                                        kThreads, kSmemBytes);
 }
 
-// Launches whose manifolds exceed the byte map use the three-CTA kernels
-// (the counting variant always the four-CTA ones).
 template <int E>
-static auto table_kernel(int max_nm, bool lanes, bool stats) {
+static auto table_kernel(bool lanes, bool stats) {
   if (lanes) return stats ? knn_table_kernel<E, true, true, 2> : knn_table_kernel<E, true, false, 2>;
-  if (stats) return knn_table_kernel<E, false, true, 4>;
-  return max_nm > kByteMapMax ? knn_table_kernel<E, false, false, 3>
-                              : knn_table_kernel<E, false, false, 4>;
+  return stats ? knn_table_kernel<E, false, true, 4> : knn_table_kernel<E, false, false, 4>;
 }
 
 template <int E>
@@ -1206,7 +1104,7 @@ cudaError_t KnnKernels<E>::launch_table(const KnnParams& params, int max_nm, boo
                                         cudaStream_t s) {
   KnnParams p = params;
   p.lane_scratch = (int32_t)table_base_smem(max_nm);
-  table_kernel<E>(max_nm, lanes, p.stats != nullptr)<<<grid, kThreads, table_smem(max_nm, lanes), s>>>(p);
+  table_kernel<E>(lanes, p.stats != nullptr)<<<grid, kThreads, table_smem(max_nm, lanes), s>>>(p);
   return cudaGetLastError();
 }
 
@@ -1215,8 +1113,7 @@ cudaError_t KnnKernels<E>::prepare_table() {
   // the largest bitmap any plan may need (manifolds up to kTableMaxNm points);
   // set once, so that plans of different sizes never lower it for each other
   for (const auto fn : {knn_table_kernel<E, false, false, 4>, knn_table_kernel<E, false, true, 4>,
-                        knn_table_kernel<E, false, false, 3>, knn_table_kernel<E, true, false, 2>,
-                        knn_table_kernel<E, true, true, 2>}) {
+                        knn_table_kernel<E, true, false, 2>, knn_table_kernel<E, true, true, 2>}) {
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)table_smem(kTableMaxNm, true));
     if (e != cudaSuccess) return e;
@@ -1226,7 +1123,7 @@ cudaError_t KnnKernels<E>::prepare_table() {
 
 template <int E>
 cudaError_t KnnKernels<E>::occupancy_table(int max_nm, bool lanes, int* ctas) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, table_kernel<E>(max_nm, lanes, false),
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, table_kernel<E>(lanes, false),
                                                        kThreads, table_smem(max_nm, lanes));
 }
 

@@ -121,10 +121,10 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, 
     u.table_R = 0;
     u.theiler = 0;
     u.wfloor = 0.f;
-    u.table_tv = 0;
     u.st_off = 0;
     u.st_stride = 0;
-    u.pad = 0;
+    u.bits_off = 0;
+    u.words_off = 0;
     TargetDesc tg;
     tg.out_idx = k;
     tg.q_off = k * (int64_t)c.n_m;
@@ -241,7 +241,7 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   c.chunk = brute_chunk(r * n_tiles, L, E);
   noalloc_setup_kernel<<<(unsigned)((r * n_tiles + 255) / 256), 256, 0, s>>>(scratch, lay, c);
   e = launch_order(d_series, reinterpret_cast<const OrderJob*>(scratch + lay.orderjob), 1,
-                   (int)n_m, reinterpret_cast<int32_t*>(scratch + lay.order), nullptr,
+                   (int)n_m, reinterpret_cast<int32_t*>(scratch + lay.order), nullptr, nullptr,
                    reinterpret_cast<const SeriesJob*>(scratch + lay.seriesjob), 1,
                    reinterpret_cast<float*>(scratch + lay.scale), nullptr, s);
   if (e == cudaSuccess)

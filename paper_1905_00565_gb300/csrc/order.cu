@@ -136,7 +136,7 @@ __device__ void prepare_series(const float* series, const SeriesJob& jb, float* 
 
 __global__ void __launch_bounds__(kOrderThreads)
 order_kernel(const float* series, const OrderJob* jobs, int64_t n_jobs, int32_t* order,
-             unsigned long long* scratch, const SeriesJob* series_jobs, float* scales, float* st) {
+             int32_t* inverse, unsigned long long* scratch, const SeriesJob* series_jobs, float* scales, float* st) {
   extern __shared__ unsigned long long s_key[];
   if (blockIdx.x >= n_jobs) {
     prepare_series(series, series_jobs[blockIdx.x - n_jobs], scales, st);
@@ -145,9 +145,13 @@ order_kernel(const float* series, const OrderJob* jobs, int64_t n_jobs, int32_t*
   const OrderJob jb = jobs[blockIdx.x];
   const float* s = series + jb.series_off + (int64_t)jb.j * jb.n;
   const int n_m = jb.n_m, E = jb.E, tau = jb.tau, off = (E - 1) * tau;
-  int32_t* out = order + jb.order_off;
+  // position q of the query order holds manifold point m
+  auto put = [&](int q, int m) {
+    order[jb.order_off + q] = m;
+    if (inverse) inverse[jb.order_off + m] = q;
+  };
   if (n_m > kOrderMaxSort && jb.scratch_off < 0) {  // no scratch: time order
-    for (int m = threadIdx.x; m < n_m; m += blockDim.x) out[m] = m;
+    for (int m = threadIdx.x; m < n_m; m += blockDim.x) put(m, m);
     return;
   }
   float lo, hi;
@@ -160,7 +164,7 @@ order_kernel(const float* series, const OrderJob* jobs, int64_t n_jobs, int32_t*
       s_key[q] = (q < n_m) ? morton_key(s, off, tau, E, lo, inv, q) : ~0ull;
     __syncthreads();
     bitonic_sort(s_key, n2);
-    for (int q = threadIdx.x; q < n_m; q += blockDim.x) out[q] = (int32_t)(s_key[q] & 0xffffffffu);
+    for (int q = threadIdx.x; q < n_m; q += blockDim.x) put(q, (int32_t)(s_key[q] & 0xffffffffu));
     return;
   }
   // Long manifold: sorted runs of kOrderMaxSort keys, then pairwise merges.
@@ -203,7 +207,7 @@ order_kernel(const float* series, const OrderJob* jobs, int64_t n_jobs, int32_t*
     }
     __syncthreads();
   }
-  for (int q = threadIdx.x; q < n_m; q += blockDim.x) out[q] = (int32_t)(buf[src][q] & 0xffffffffu);
+  for (int q = threadIdx.x; q < n_m; q += blockDim.x) put(q, (int32_t)(buf[src][q] & 0xffffffffu));
 }
 
 }  // namespace
@@ -214,14 +218,15 @@ cudaError_t order_prepare() {
 }
 
 cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jobs, int max_nm,
-                         int32_t* order, unsigned long long* scratch, const SeriesJob* series_jobs,
-                         int64_t n_series_jobs, float* scales, float* st, cudaStream_t s) {
+                         int32_t* order, int32_t* inverse, unsigned long long* scratch,
+                         const SeriesJob* series_jobs, int64_t n_series_jobs, float* scales,
+                         float* st, cudaStream_t s) {
   if (n_jobs + n_series_jobs <= 0) return cudaSuccess;
   int n2 = 1;
   while (n2 < max_nm && n2 < kOrderMaxSort) n2 <<= 1;
   const size_t smem = (size_t)n2 * sizeof(unsigned long long);
   order_kernel<<<(unsigned)(n_jobs + n_series_jobs), kOrderThreads, smem, s>>>(
-      series, jobs, n_jobs, order, scratch, series_jobs, scales, st);
+      series, jobs, n_jobs, order, inverse, scratch, series_jobs, scales, st);
   return cudaGetLastError();
 }
 

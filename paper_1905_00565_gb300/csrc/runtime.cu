@@ -142,11 +142,12 @@ bool all_finite(const float* x, size_t count) {
 }
 
 // ------------------------------------------------------------- unit lists ---
-// The work items of one search launch: one E, and units of few or of many
-// targets (a kernel each).
+// The work items of one search launch: one E, and units of one, few or many
+// targets (a kernel each; brute force: one and few share theirs).
+enum class Targets : int32_t { kOne, kFew, kMany };
 struct ItemGroup {
   int32_t E;
-  bool lanes;
+  Targets targets;
   int64_t first, count;
 };
 
@@ -162,9 +163,13 @@ struct UnitList {
   int64_t obs_total = 0;              // observed-value tile records
   std::vector<SeriesJob> series_jobs; // one per (job, target variable)
   int64_t st_total = 0;               // elements of the time-major series copies
+  bool window = false;                // some unit has an exclusion window
   bool lane_targets = false;          // some unit has kLaneTargets targets
   std::vector<TableJob> tables;       // distance indexing tables to build
   std::vector<WorkItem> items_table;  // work items of units that read a table
+  std::vector<MemberGroup> member_groups;  // scan groups (units of one target)
+  int64_t bits_total = 0, words_total = 0;  // their membership bits and words
+  int64_t lib_scratch = 0;            // longest library of the units that read a table
   std::vector<double> item_cost_table;
   int64_t lib_total = 0, part_total = 0, order_total = 0, table_total = 0;
   int64_t order_scratch_total = 0;    // 64-bit keys for sorting manifolds above kOrderMaxSort
@@ -190,16 +195,18 @@ struct UnitList {
   int64_t search_queries = 0;         // N_m summed over the units
   int64_t table_queries = 0;          // N_m summed over the units that read a table
   bool table_tv = false;              // some table stores its target's values (TableJob::tv_i)
-  bool lanes(const WorkItem& w) const {
-    return units[(size_t)w.unit].n_targets >= kLaneTargets;
+  Targets targets_of(const WorkItem& w) const {
+    const UnitDesc& u = units[(size_t)w.unit];
+    if (u.n_targets >= kLaneTargets) return Targets::kMany;
+    return u.table_R > 0 && u.n_targets == 1 ? Targets::kOne : Targets::kFew;
   }
   // The launches of a sorted item list.
   std::vector<ItemGroup> group_items(const std::vector<WorkItem>& list) const {
     std::vector<ItemGroup> g;
     for (size_t q = 0; q < list.size(); ++q) {
       const int32_t E = units[(size_t)list[q].unit].E;
-      if (g.empty() || g.back().E != E || g.back().lanes != lanes(list[q]))
-        g.push_back(ItemGroup{E, lanes(list[q]), (int64_t)q, 0});
+      if (g.empty() || g.back().E != E || g.back().targets != targets_of(list[q]))
+        g.push_back(ItemGroup{E, targets_of(list[q]), (int64_t)q, 0});
       ++g.back().count;
     }
     return g;
@@ -330,6 +337,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
   bool lanes = false;
   for (int32_t j : lib_vars) lanes |= pairs_of[j].size() >= (size_t)kLaneTargets;
   ul->lane_targets |= lanes;
+  ul->window |= pc.theiler > 0;
   const int64_t st_off = ul->st_total;
   const int32_t st_stride = (pc.V + 31) / 32 * 32;
   if (lanes) ul->st_total += pc.n * st_stride;
@@ -406,18 +414,14 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             }
           if (lmin < 0 || lsum < 8.0 * (double)n_m) continue;
           int64_t R = table_row_length(E, n_m, lmin, pc.theiler, safety);
-          // whole groups of four ranks (the table's layout), from the n_m - 1
-          // points other than the query
-          R = std::min<int64_t>(std::min<int64_t>((R + 31) / 32 * 32, kTableMaxR),
-                                (n_m - 1) / 4 * 4);
-          // indices (2 or 4 bytes), distances, and (a variable with one target,
-          // a manifold below 65536 points) the target's values: the scan then
-          // reads them beside the distances instead of gathering them through
-          // the indices (on longer manifolds the extra array's cold lines cost
-          // more than the gather: 120 -> 129 ms on the N = 10^5 series)
-          const bool tv = pairs_of[j].size() == 1 && n_m < 65536;
+          // from the n_m - 1 points other than the query; rows are padded to 64
+          R = std::min<int64_t>(std::min<int64_t>((R + 31) / 32 * 32, kTableMaxR), n_m - 1);
+          const int64_t stride = (R + 63) / 64 * 64;
+          // positions (2 or 4 bytes), distances, and for a variable with one
+          // target the target's values
+          const bool tv = pairs_of[j].size() == 1;
           const double bytes =
-              (double)n_m * (double)R * ((n_m < 65536 ? 2.0 : 4.0) + 4.0 + (tv ? 4.0 : 0.0));
+              (double)n_m * (double)stride * ((n_m < 65536 ? 2.0 : 4.0) + 4.0 + (tv ? 4.0 : 0.0));
           if (table_bytes + bytes > table_cap_bytes) continue;
           table_bytes += bytes;
           TableJob tj;
@@ -431,30 +435,37 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           tj.tau = tau;
           tj.n_m = (int32_t)n_m;
           tj.R = (int32_t)R;
+          tj.stride = (int32_t)stride;
           tj.tv_i = tv ? pc.pairs[2 * pairs_of[j][0] + 1] : -1;
           if (tv) ul->table_tv = true;
-          table_of[std::make_tuple(j, E, tau)] = std::make_pair(tj.table_off, tj.R);
-          ul->table_total += n_m * R;
+          table_of[std::make_tuple(j, E, tau)] = std::make_pair(tj.table_off, tj.stride);
+          ul->table_total += n_m * stride;
           ul->tables.push_back(tj);
         }
   }
-  // Query tiles per brute-force item, from the tiles of each E's launch.
-  std::map<int32_t, int64_t> brute_tiles;
+  // Query tiles per brute-force and scan item, from the tiles of each E's launch.
+  std::map<int32_t, int64_t> brute_tiles, scan_tiles;
   for (int32_t j : lib_vars)
     for (int32_t E : pc.E)
       for (int32_t tau : pc.tau) {
         const int64_t n_m = pc.n - (int64_t)(E - 1) * tau;
         const bool tab = table_of.count(std::make_tuple(j, E, tau)) != 0;
-        for (int64_t L : pc.L)
+        int64_t tabled = 0;
+        for (int64_t L : pc.L) {
           if (!tab || (double)L < table_min_L(E, n_m, tt))
             brute_tiles[E] += (n_m + tileq - 1) / tileq * pc.r;
+          else
+            tabled += pc.r;
+        }
+        scan_tiles[E] += (n_m + tileq - 1) / tileq * ((tabled + kScanGroup - 1) / kScanGroup);
       }
   for (int32_t j : lib_vars) {
     const std::vector<int64_t>& tp = pairs_of[j];
     for (int64_t e = 0; e < nE; ++e)
-      for (int64_t t = 0; t < nT; ++t)
+      for (int64_t t = 0; t < nT; ++t) {
+        const int32_t E = pc.E[(size_t)e], tau = pc.tau[(size_t)t];
+        const size_t first_unit = ul->units.size();
         for (int64_t l = 0; l < nL; ++l) {
-          const int32_t E = pc.E[(size_t)e], tau = pc.tau[(size_t)t];
           const int64_t L = pc.L[(size_t)l];
           const int32_t chunk = brute_chunk(brute_tiles[E], L, E);
           for (int32_t k = 0; k < pc.r; ++k) {
@@ -498,30 +509,25 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             if (tab != table_of.end() && (double)L >= table_min_L(E, u.n_m, tt)) {
               u.table_off = tab->second.first;
               u.table_R = tab->second.second;
-              u.table_tv = (tp.size() == 1 && u.n_m < 65536) ? 1 : 0;  // as the table's job
+              u.bits_off = ul->bits_total;
+              ul->bits_total += (u.n_m + 31) / 32;
+              ul->lib_scratch = std::max(ul->lib_scratch, L);
             }
             const int32_t uidx = (int32_t)ul->units.size();
-            // Table realizations of one cell with a single target and a byte
-            // membership map are grouped kTableGroup at a time (consecutive k):
-            // the item of the group's first realization covers all of them.
-            const bool groupable = u.table_R > 0 && u.n_targets == 1 && u.n_m <= kTableGroupMaxNm;
-            const int32_t count =
-                groupable ? std::min<int32_t>(kTableGroup, pc.r - (k / kTableGroup) * kTableGroup) : 1;
-            const bool owns_items = !groupable || k % kTableGroup == 0;
+            // units of one target that read a table get their items below, in groups
+            const bool owns_items = !(u.table_R > 0 && u.n_targets == 1);
             for (int32_t q = 0; q < u.n_tiles && owns_items; ++q) {
               const int64_t nq = std::min<int64_t>(tileq, u.n_m - (int64_t)q * tileq);
               if (u.table_R > 0) {
-                // one item per kTableChunk tiles: one membership map, then per
-                // tile one walk of each row (longer for a group: it ends when
-                // every realization has its E+1) and one epilogue per
-                // realization and target
+                // one item per kTableChunk tiles: one copy of the membership
+                // bits, then per tile one walk of each row and the epilogue
                 if (q % kTableChunk == 0) {
-                  ul->items_table.push_back(WorkItem{uidx, q, count});
-                  ul->item_cost_table.push_back((double)L * count);
+                  ul->items_table.push_back(WorkItem{uidx, q, kTableChunk});
+                  ul->item_cost_table.push_back((double)u.n_m);
                 }
                 ul->item_cost_table.back() +=
-                    (double)nq * 12.0 * (E + 2) * (double)u.n_m / (double)L * (1.0 + 0.1 * count) +
-                    (double)u.n_targets * nq * 64.0 * count;
+                    (double)nq * 12.0 * (E + 2) * (double)u.n_m / (double)L +
+                    (double)u.n_targets * nq * 64.0;
               } else {
                 // one item per `chunk` tiles: one library staging (when it
                 // fits a shared-memory tile), then per tile the search and the
@@ -541,7 +547,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
               ul->table_queries += u.n_m;
             }
             ul->search_queries += u.n_m;
-            ul->lib_total += L;
+            if (u.table_R == 0) ul->lib_total += L;
             ul->part_total += (int64_t)u.n_tiles * u.n_targets;
             ul->emin = std::min(ul->emin, E);
             ul->emax = std::max(ul->emax, E);
@@ -551,10 +557,40 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             ul->units.push_back(u);
           }
         }
+        if (tp.size() != 1) continue;
+        // Scan groups: consecutive units of this (j, E, tau) that read the table,
+        // whatever their L (the lanes of a partly filled group would idle; the
+        // walk of a mixed one is as long as its smallest L's).
+        int64_t slots = scan_tiles[E] / (4 * 2 * 152);
+        const int32_t chunk = (int32_t)std::min<int64_t>(std::max<int64_t>(slots, 1), kScanChunk);
+        for (size_t a = first_unit; a < ul->units.size();) {
+          if (ul->units[a].table_R == 0) {
+            ++a;
+            continue;
+          }
+          size_t b = a;
+          int32_t lmin = ul->units[a].L;
+          for (; b < ul->units.size() && b - a < (size_t)kScanGroup && ul->units[b].table_R > 0; ++b) {
+            ul->units[b].words_off = ul->words_total;
+            lmin = std::min(lmin, ul->units[b].L);
+          }
+          const UnitDesc& u = ul->units[a];
+          ul->words_total += member_words(u.n_m);
+          ul->member_groups.push_back(MemberGroup{(int32_t)a, (int32_t)(b - a)});
+          for (int32_t q = 0; q < u.n_tiles; q += chunk) {
+            ul->items_table.push_back(WorkItem{(int32_t)a, q, (int32_t)(b - a) | chunk << 8});
+            ul->item_cost_table.push_back(std::min(chunk, u.n_tiles - q) *
+                                          (64.0 + (E + 4.0) * u.n_m / lmin));
+          }
+          a = b;
+        }
+      }
   }
 }
 
 void sort_items(UnitList* ul) {
+  for (UnitDesc& u : ul->units)
+    if (u.table_R > 0) u.lib_off = ul->lib_total;  // one slot behind the lists
   std::stable_sort(ul->tables.begin(), ul->tables.end(), [](const TableJob& a, const TableJob& b) {
     const int ra = UnitList::table_rcap(a.R), rb = UnitList::table_rcap(b.R);
     if (ra != rb) return ra < rb;
@@ -570,8 +606,9 @@ void sort_items(UnitList* ul) {
       const int32_t ea = ul->units[(size_t)ul->items[(size_t)a].unit].E;
       const int32_t eb = ul->units[(size_t)ul->items[(size_t)b].unit].E;
       if (ea != eb) return ea > eb;
-      const bool la = ul->lanes(ul->items[(size_t)a]), lb = ul->lanes(ul->items[(size_t)b]);
-      if (la != lb) return la;
+      const Targets ta = ul->targets_of(ul->items[(size_t)a]);
+      const Targets tb = ul->targets_of(ul->items[(size_t)b]);
+      if (ta != tb) return ta > tb;
       return ul->item_cost[(size_t)a] > ul->item_cost[(size_t)b];
     });
     std::vector<WorkItem> sorted(order.size());
@@ -584,17 +621,20 @@ void sort_items(UnitList* ul) {
     ul->item_cost.swap(cost);
     ul->groups = ul->group_items(ul->items);
   }
-  // Table items: grouped by E (one launch per E), then by table (a table of
-  // 5-30 MB stays in L2 while its realizations run), larger items first.
+  // Table items: grouped by E (one launch per E and kind), then by table and,
+  // for the scan, by query tiles, so that all realizations that walk a row do
+  // so while it is in L2; larger items first.
   std::vector<int64_t> order(ul->items_table.size());
   for (size_t q = 0; q < order.size(); ++q) order[q] = (int64_t)q;
   std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) {
     const UnitDesc& ua = ul->units[(size_t)ul->items_table[(size_t)a].unit];
     const UnitDesc& ub = ul->units[(size_t)ul->items_table[(size_t)b].unit];
     if (ua.E != ub.E) return ua.E > ub.E;
-    const bool la = ua.n_targets >= kLaneTargets, lb = ub.n_targets >= kLaneTargets;
-    if (la != lb) return la;
+    const WorkItem &wa = ul->items_table[(size_t)a], &wb = ul->items_table[(size_t)b];
+    const Targets ta = ul->targets_of(wa), tb = ul->targets_of(wb);
+    if (ta != tb) return ta > tb;
     if (ua.table_off != ub.table_off) return ua.table_off < ub.table_off;
+    if (ta == Targets::kOne && wa.tile != wb.tile) return wa.tile < wb.tile;
     return ul->item_cost_table[(size_t)a] > ul->item_cost_table[(size_t)b];
   });
   std::vector<WorkItem> sorted(order.size());
@@ -603,16 +643,17 @@ void sort_items(UnitList* ul) {
   ul->groups_table = ul->group_items(ul->items_table);
 }
 
-// Search launches of one run, at most: per E, few or many targets, brute force
-// or table.
-constexpr int kMaxSearchLaunches = 4 * kMaxE;
+// Search launches of one run, at most: per E, brute force of few or many
+// targets, tables of one, few or many.
+constexpr int kMaxSearchLaunches = 5 * kMaxE;
 
 // Device arena layout for a unit list.
 struct Arena {
   size_t series = 0, units = 0, items = 0, lib = 0, part = 0, rho = 0, err = 0,
          counter = 0, scratch = 0, order = 0, orders = 0, targets = 0, table = 0, tables = 0,
          items_table = 0, order_scratch = 0, obs = 0, obs_stat = 0, obs_jobs = 0, series_jobs = 0,
-         scales = 0, st = 0, table_dist = 0, stats = 0,
+         scales = 0, st = 0, table_dist = 0, stats = 0, inverse = 0, bits = 0, words = 0,
+         member_groups = 0,
          total = 0;
 };
 
@@ -627,13 +668,17 @@ Arena layout(int64_t series_elems, const UnitList& ul, int64_t n_rho, int64_t sc
   a.series = take(sizeof(float) * (size_t)series_elems);
   a.units = take(sizeof(UnitDesc) * ul.units.size());
   a.items = take(sizeof(WorkItem) * ul.items.size());
-  a.lib = take(sizeof(int32_t) * (size_t)ul.lib_total);
+  a.lib = take(sizeof(int32_t) * (size_t)(ul.lib_total + ul.lib_scratch));
+  a.bits = take(sizeof(uint32_t) * (size_t)ul.bits_total);
+  a.words = take(sizeof(uint32_t) * (size_t)ul.words_total);
+  a.member_groups = take(sizeof(MemberGroup) * ul.member_groups.size());
   a.part = take(2 * sizeof(float4) * (size_t)ul.part_total);
   a.rho = take(sizeof(double) * (size_t)n_rho);
   a.err = take(sizeof(int32_t));
   a.counter = take(kMaxSearchLaunches * sizeof(uint32_t));
   a.scratch = take(sizeof(float) * (size_t)scratch_floats);
   a.order = take(sizeof(int32_t) * (size_t)ul.order_total);
+  a.inverse = take(ul.tables.empty() ? 0 : sizeof(int32_t) * (size_t)ul.order_total);
   a.order_scratch = take(sizeof(unsigned long long) * (size_t)ul.order_scratch_total);
   a.orders = take(sizeof(OrderJob) * ul.orders.size());
   a.targets = take(sizeof(TargetDesc) * ul.targets.size());
@@ -778,7 +823,7 @@ struct ccm_plan_s {
   cudaStream_t stream = nullptr;
   cudaGraphExec_t graph = nullptr;
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // stage boundaries
-  int grid = 0, grid_table = 0;
+  int grid = 0, grid_table = 0, grid_scan = 0;
   Tuning tuning = default_tuning();
   bool tuned = false;
   std::mutex run_mu;
@@ -793,6 +838,7 @@ SamplerParams sampler_params(char* base, const Arena& ar) {
   sp.targets = reinterpret_cast<const TargetDesc*>(base + ar.targets);
   sp.order = reinterpret_cast<const int32_t*>(base + ar.order);
   sp.lib = reinterpret_cast<int32_t*>(base + ar.lib);
+  sp.bits = reinterpret_cast<uint32_t*>(base + ar.bits);
   sp.err = reinterpret_cast<int32_t*>(base + ar.err);
   return sp;
 }
@@ -807,6 +853,9 @@ KnnParams knn_params(char* base, const Arena& ar, const UnitList& ul, int persis
   kp.n_items = (int64_t)ul.items.size();
   kp.lib = reinterpret_cast<const int32_t*>(base + ar.lib);
   kp.order = reinterpret_cast<const int32_t*>(base + ar.order);
+  kp.bits = reinterpret_cast<const uint32_t*>(base + ar.bits);
+  kp.words = reinterpret_cast<const uint32_t*>(base + ar.words);
+  kp.window = ul.window ? 1 : 0;
   kp.table = base + ar.table;
   kp.table_dist = reinterpret_cast<const float*>(base + ar.table_dist);
   kp.table_pairs = ul.table_tv ? 1 : 0;
@@ -832,6 +881,7 @@ cudaError_t enqueue_order(char* base, const Arena& ar, const UnitList& ul, cudaS
       launch_order(reinterpret_cast<const float*>(base + ar.series),
                    reinterpret_cast<const OrderJob*>(base + ar.orders), (int64_t)ul.orders.size(),
                    ul.max_nm, reinterpret_cast<int32_t*>(base + ar.order),
+                   ul.tables.empty() ? nullptr : reinterpret_cast<int32_t*>(base + ar.inverse),
                    reinterpret_cast<unsigned long long*>(base + ar.order_scratch),
                    reinterpret_cast<const SeriesJob*>(base + ar.series_jobs),
                    (int64_t)ul.series_jobs.size(), scales, reinterpret_cast<float*>(base + ar.st), s);
@@ -849,7 +899,7 @@ cudaError_t enqueue_order(char* base, const Arena& ar, const UnitList& ul, cudaS
 // ev[2] after the sampler, ev[3] after the brute-force launch, ev[4] after the
 // table-scan launch.
 ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const Tuning& tn,
-                         int grid, int grid_table, int persistent, int32_t* dbg_lib,
+                         int grid, int grid_table, int grid_scan, int persistent, int32_t* dbg_lib,
                          int32_t* dbg_nbr, float* dbg_xhat, cudaStream_t s,
                          cudaEvent_t* ev = nullptr, bool capturing = false,
                          bool stats = false) {
@@ -878,6 +928,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
                                 reinterpret_cast<const TableJob*>(base + ar.tables) + g0,
                                 (int64_t)(g1 - g0), te, nm, rmax,
                                 reinterpret_cast<const int32_t*>(base + ar.order),
+                                reinterpret_cast<const int32_t*>(base + ar.inverse),
                                 base + ar.table, reinterpret_cast<float*>(base + ar.table_dist),
                                 ul.table_tv ? 1 : 0,
                                 ul.table_u16(), s));
@@ -887,6 +938,11 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   SamplerParams sp = sampler_params(base, ar);
   sp.dbg_lib = dbg_lib;
   CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, s));
+  if (!ul.member_groups.empty())
+    CCM_CUDA(launch_member_words(reinterpret_cast<const UnitDesc*>(base + ar.units),
+                                 reinterpret_cast<const MemberGroup*>(base + ar.member_groups),
+                                 (int64_t)ul.member_groups.size(), ul.max_nm, sp.bits,
+                                 reinterpret_cast<uint32_t*>(base + ar.words), s));
   if (ev) CCM_CUDA(record(ev[2]));
   KnnParams kp = knn_params(base, ar, ul, persistent, tn);
   kp.dbg_nbr = dbg_nbr;
@@ -902,7 +958,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     ke.n_items = ig.count;
     ke.item_counter = counter++;
     const int g = persistent ? grid : (int)std::min<int64_t>(ig.count, 0x7fffffff);
-    CCM_CUDA(launch_knn(ke, ig.E, ig.lanes, g, s));
+    CCM_CUDA(launch_knn(ke, ig.E, ig.targets == Targets::kMany, g, s));
   }
   if (ev) CCM_CUDA(record(ev[3]));
   for (const ItemGroup& ig : ul.groups_table) {
@@ -911,7 +967,10 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     kt.n_items = ig.count;
     kt.item_counter = counter++;
     const int g = persistent ? grid_table : (int)std::min<int64_t>(ig.count, 0x7fffffff);
-    CCM_CUDA(launch_knn_table(kt, ig.E, ul.max_nm, ig.lanes, g, s));
+    if (ig.targets == Targets::kOne)
+      CCM_CUDA(launch_knn_scan(kt, ig.E, ul.max_nm, persistent ? grid_scan : g, s));
+    else
+      CCM_CUDA(launch_knn_table(kt, ig.E, ul.max_nm, ig.targets == Targets::kMany, g, s));
   }
   CCM_CUDA(launch_rho(kp.units, kp.targets, (int64_t)ul.targets.size(), kp.partials, kp.obs_stat,
                       reinterpret_cast<double*>(base + ar.rho), s));
@@ -1010,11 +1069,12 @@ ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
   for (int E = ul.emin; E <= ul.emax && st == CCM_OK; ++E) {
     if (pl->tuning.known[E]) continue;
     // (units of many targets only where a plan has no others of this E)
-    bool lanes = true;
-    for (const ItemGroup& ig : ul.groups) lanes &= ig.E != E || ig.lanes;
+    Targets kind = Targets::kMany;
+    for (const ItemGroup& ig : ul.groups)
+      if (ig.E == E) kind = std::min(kind, ig.targets);
     std::vector<WorkItem> all;
     for (const WorkItem& w : ul.items)
-      if (ul.units[(size_t)w.unit].E == E && ul.lanes(w) == lanes) all.push_back(w);
+      if (ul.units[(size_t)w.unit].E == E && ul.targets_of(w) == kind) all.push_back(w);
     if ((int)all.size() < want) continue;
     std::vector<WorkItem> sample;  // evenly spaced over the cost-sorted list
     for (int q = 0; q < want; ++q) sample.push_back(all[(size_t)q * all.size() / (size_t)want]);
@@ -1034,7 +1094,7 @@ ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
         float ms = 0.f;
         for (int rep = 0; rep < 2 && ce == cudaSuccess; ++rep) {  // warm-up, then timed
           ce = cudaEventRecord(e0, s);
-          if (ce == cudaSuccess) ce = launch_knn(kp, E, lanes, (int)sample.size(), s);
+          if (ce == cudaSuccess) ce = launch_knn(kp, E, kind == Targets::kMany, (int)sample.size(), s);
           if (ce == cudaSuccess) ce = cudaEventRecord(e1, s);
           if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
           if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
@@ -1090,6 +1150,7 @@ ccm_status ccm_context_create(int device, size_t hbm_budget_bytes, ccm_context**
   CCM_CUDA(table_prepare());
   CCM_CUDA(convergence_prepare());
   CCM_CUDA(knn_table_prepare());
+  CCM_CUDA(knn_scan_prepare());
   size_t free_b = 0, total_b = 0;
   CCM_CUDA(cudaMemGetInfo(&free_b, &total_b));
   std::unique_ptr<ccm_context> ctx(new ccm_context());
@@ -1146,6 +1207,9 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
     e = cudaMemcpy(pl->d_arena + pl->ar.items_table, pl->ul.items_table.data(),
                    sizeof(WorkItem) * pl->ul.items_table.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
+    e = cudaMemcpy(pl->d_arena + pl->ar.member_groups, pl->ul.member_groups.data(),
+                   sizeof(MemberGroup) * pl->ul.member_groups.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
     e = cudaMemcpy(pl->d_arena + pl->ar.series_jobs, pl->ul.series_jobs.data(),
                    sizeof(SeriesJob) * pl->ul.series_jobs.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
@@ -1159,6 +1223,7 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
     int per_sm = 1;
     if (knn_table_occupancy(pl->ul.max_nm, pl->ul.lane_targets, &per_sm) != cudaSuccess || per_sm < 1) per_sm = 1;
     pl->grid_table = ctx->sm_count * per_sm;
+    pl->grid_scan = ctx->sm_count * 2;
   }
   {
     std::lock_guard<std::mutex> g(ctx->mu);
@@ -1182,6 +1247,7 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
   // launches of one ccm_run: order, tables, sampler, one brute-force and one
   // table-scan kernel per E present, rho
   in.launches_per_run = 4 + pl->ul.table_groups();  // order, observed values, sampler, rho, tables
+  in.launches_per_run += pl->ul.member_groups.empty() ? 0 : 1;  // membership words
   in.launches_per_run += (int64_t)(pl->ul.groups.size() + pl->ul.groups_table.size());
   *out = pl.release();
   return CCM_OK;
@@ -1243,7 +1309,7 @@ ccm_status ccm_run_ex(ccm_plan_t* plan, const float* series, double* rho, const 
                                  : reinterpret_cast<float*>(tmp + align_up(lb, 256) + align_up(nb, 256)))
                       : nullptr;
     ccm_status st =
-        enqueue_sweep(base, plan->ar, ul, plan->tuning, plan->grid, plan->grid_table, 1, d_lib,
+        enqueue_sweep(base, plan->ar, ul, plan->tuning, plan->grid, plan->grid_table, plan->grid_scan, 1, d_lib,
                       d_nbr, d_xh, s, plan->ev, false, (pc.flags & CCM_SEARCH_STATS) != 0);
     if (st != CCM_OK) return st;
     if (!out_dev) {
@@ -1267,7 +1333,7 @@ ccm_status ccm_run_ex(ccm_plan_t* plan, const float* series, double* rho, const 
       cudaGraph_t graph = nullptr;
       CCM_CUDA(cudaStreamBeginCapture(plan->stream, cudaStreamCaptureModeThreadLocal));
       ccm_status st = enqueue_sweep(base, plan->ar, plan->ul, plan->tuning, plan->grid,
-                                    plan->grid_table, 1, nullptr, nullptr, nullptr, plan->stream,
+                                    plan->grid_table, plan->grid_scan, 1, nullptr, nullptr, nullptr, plan->stream,
                                     plan->ev, true, (pc.flags & CCM_SEARCH_STATS) != 0);
       const cudaError_t ce = cudaStreamEndCapture(plan->stream, &graph);
       if (st != CCM_OK) {
@@ -1347,7 +1413,8 @@ ccm_status ccm_run_plain(ccm_plan_t* plan, const float* series, double* rho, voi
   CCM_CUDA(cudaMemcpyAsync(base + ar.series, series, sizeof(float) * (size_t)pc.V * (size_t)pc.n,
                            in_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   CCM_CUDA(cudaMemsetAsync(base + ar.err, 0, sizeof(int32_t), s));
-  const SamplerParams sp = sampler_params(base, ar);
+  SamplerParams sp = sampler_params(base, ar);
+  sp.list_all = 1;
   const UnitDesc* d_units = reinterpret_cast<const UnitDesc*>(base + ar.units);
   const TargetDesc* d_targets = reinterpret_cast<const TargetDesc*>(base + ar.targets);
   CCM_CUDA(enqueue_order(base, ar, plan->ul, s));
@@ -1491,11 +1558,12 @@ ccm_status launch_batch(ccm_context* ctx, Batch* b, bool inject) {
   // Descriptors go through pinned staging: a copy from pageable memory would
   // wait for earlier work on this (reused) stream.
   // (units, work items, order jobs, targets, table jobs, table work items,
-  // observed-value jobs, series jobs)
-  constexpr int kMeta = 8;
+  // observed-value jobs, series jobs, scan groups)
+  constexpr int kMeta = 9;
   const void* src[kMeta] = {b->ul.units.data(),   b->ul.items.data(),  b->ul.orders.data(),
                             b->ul.targets.data(), b->ul.tables.data(), b->ul.items_table.data(),
-                            b->ul.obs_jobs.data(),  b->ul.series_jobs.data()};
+                            b->ul.obs_jobs.data(),  b->ul.series_jobs.data(),
+                            b->ul.member_groups.data()};
   const size_t len[kMeta] = {sizeof(UnitDesc) * b->ul.units.size(),
                              sizeof(WorkItem) * b->ul.items.size(),
                              sizeof(OrderJob) * b->ul.orders.size(),
@@ -1503,9 +1571,11 @@ ccm_status launch_batch(ccm_context* ctx, Batch* b, bool inject) {
                              sizeof(TableJob) * b->ul.tables.size(),
                              sizeof(WorkItem) * b->ul.items_table.size(),
                              sizeof(ObsJob) * b->ul.obs_jobs.size(),
-                             sizeof(SeriesJob) * b->ul.series_jobs.size()};
+                             sizeof(SeriesJob) * b->ul.series_jobs.size(),
+                             sizeof(MemberGroup) * b->ul.member_groups.size()};
   const size_t dst[kMeta] = {b->ar.units,  b->ar.items,       b->ar.orders,  b->ar.targets,
-                             b->ar.tables, b->ar.items_table, b->ar.obs_jobs, b->ar.series_jobs};
+                             b->ar.tables, b->ar.items_table, b->ar.obs_jobs, b->ar.series_jobs,
+                             b->ar.member_groups};
   b->meta_bytes = 0;
   for (int q = 0; q < kMeta; ++q) b->meta_bytes += len[q];
   b->h_meta = pinned_get(ctx, b->meta_bytes);
@@ -1523,7 +1593,7 @@ ccm_status launch_batch(ccm_context* ctx, Batch* b, bool inject) {
     tn = ctx->tuning;
   }
   ccm_status st =
-      enqueue_sweep(base, b->ar, b->ul, tn, 0, 0, 0, nullptr, nullptr, nullptr, b->stream);
+      enqueue_sweep(base, b->ar, b->ul, tn, 0, 0, 0, 0, nullptr, nullptr, nullptr, b->stream);
   if (st != CCM_OK) return st;
   int64_t ro = 0;
   for (auto& j : b->jobs) {

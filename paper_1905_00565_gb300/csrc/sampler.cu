@@ -10,14 +10,27 @@
 // points with the smallest keys, written in ascending m.  Keys are distinct,
 // so the selection is a pure function of the counter.
 //
-// One CTA per unit.  The high halves h(m) are computed once into shared memory
-// (or recomputed per pass when N_m is too large), an 8-bit radix select over
-// four passes (bins scanned by one warp) finds the L-th smallest key (h*, and
-// how many of the h == h* points, smallest m first, are taken; when some ties
-// are left out, one warp finds the last tie taken).  A warp-by-warp stable
-// compaction over the unit's query order writes the library in query order,
-// the order the neighbour search visits it in (spatially coherent runs); the
-// checking copy is compacted in ascending m.
+// One CTA per unit.  The L-th smallest of N_m uniform keys lies within a few
+// standard deviations of L/N_m, so one pass over the keys decides almost every
+// point: below a window of +-5 standard deviations it is a member, above it is
+// not, and the few hundred inside are listed in shared memory, where a
+// histogram and a rank count find the last member.  The keys are never stored
+// (one bit per point is).  When the window misses (about one unit in 10^6), an
+// 8-bit radix select over four passes recomputes the keys.
+//
+// Bound: issue (the 64-bit multiplies of Philox are half of the instructions)
+// and the latency between its barriers.  Sweep of 4*10^5 libraries of N_m =
+// 10^4: 17.9 ms with the scan's membership words (keys stored and four radix
+// passes over them: 20.0 ms); 10^4 libraries of N_m = 10^5: 3.9 ms (keys
+// recomputed in every pass: 26.4 ms).
+//
+// Output: realizations that read a distance indexing table get one bit per
+// position of the query order; the others their library as a list in query
+// order, the order the neighbour search visits it in (spatially coherent
+// runs).  The checking copy is compacted in ascending m.
+#include <algorithm>
+
+#include "bits.cuh"
 #include "ccm_internal.h"
 
 namespace ccm {
@@ -36,8 +49,9 @@ __device__ __forceinline__ void philox_block(uint64_t c0, uint64_t c1, uint64_t 
       k0 += W0;
       k1 += W1;
     }
-    const uint64_t hi0 = __umul64hi(M0, c0), lo0 = M0 * c0;
-    const uint64_t hi1 = __umul64hi(M1, c2), lo1 = M1 * c2;
+    const unsigned __int128 p0 = (unsigned __int128)M0 * c0, p1 = (unsigned __int128)M1 * c2;
+    const uint64_t hi0 = (uint64_t)(p0 >> 64), lo0 = (uint64_t)p0;
+    const uint64_t hi1 = (uint64_t)(p1 >> 64), lo1 = (uint64_t)p1;
     const uint64_t n0 = hi1 ^ c1 ^ k0, n2 = hi0 ^ c3 ^ k1;
     c0 = n0;
     c1 = lo1;
@@ -61,13 +75,6 @@ __device__ __forceinline__ uint32_t block_half(const uint64_t (&w)[4], int i) {
   const int q = i >> 1;
   const uint64_t x = (q == 0) ? w[0] : (q == 1) ? w[1] : (q == 2) ? w[2] : w[3];
   return (i & 1) ? (uint32_t)x : (uint32_t)(x >> 32);
-}
-
-// The high half of point m's key (one block per call).
-__device__ __forceinline__ uint32_t key_hi(const UnitDesc& u, int m) {
-  uint64_t w[4];
-  key_block(u, m >> 3, w);
-  return block_half(w, m & 7);
 }
 
 // Stable compaction of the members among positions [0, n) by the whole block,
@@ -112,66 +119,42 @@ __device__ uint32_t block_compact(int n, Item item, Member is_member, int32_t* o
   return total;
 }
 
-template <bool kInSmem>
-__global__ void __launch_bounds__(kSamplerThreads)
-sampler_kernel(SamplerParams p, int64_t first_unit) {
-  extern __shared__ __align__(16) uint32_t s_keys[];
-  __shared__ uint32_t s_hist[256];
-  __shared__ uint32_t s_warp[32];
-  __shared__ uint32_t s_prefix, s_rank, s_neq;
-  __shared__ int s_mtie;
-
-  const int64_t uidx = first_unit + blockIdx.x;
-  const UnitDesc u = p.units[uidx];
-  const int n_m = u.n_m, L = u.L;
+// The L-th smallest key of a unit whose window missed: an 8-bit radix select
+// of its high half h* over four passes of recomputed keys, then the last of the
+// points with that half that are taken (smallest m first).  Block-wide.
+struct SelectScratch {
+  uint32_t hist[256];
+  uint32_t prefix, rank;
+};
+__device__ __noinline__ unsigned long long select_by_radix(const UnitDesc& u, SelectScratch& sc) {
+  const int n_m = u.n_m, n_blocks = (n_m + 7) >> 3;
   const int lane = threadIdx.x & 31;
-  if (L < 1 || L > n_m) {
-    if (threadIdx.x == 0) atomicOr(p.err, kErrSampler);
-    return;
-  }
-  const int n_blocks = (n_m + 7) >> 3;
-  if (kInSmem) {  // the key array is padded to whole blocks of eight
-    for (int b = threadIdx.x; b < n_blocks; b += blockDim.x) {
-      uint64_t w[4];
-      key_block(u, b, w);
-      uint4* dst = reinterpret_cast<uint4*>(s_keys + 8 * b);
-      dst[0] = make_uint4(block_half(w, 0), block_half(w, 1), block_half(w, 2), block_half(w, 3));
-      dst[1] = make_uint4(block_half(w, 4), block_half(w, 5), block_half(w, 6), block_half(w, 7));
-    }
-  }
   if (threadIdx.x == 0) {
-    s_prefix = 0u;
-    s_rank = (uint32_t)L;  // 1-based rank still to find within the current prefix
+    sc.prefix = 0u;
+    sc.rank = (uint32_t)u.L;  // 1-based rank still to find within the current prefix
   }
   uint32_t mask = 0u;
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) s_hist[b] = 0u;
     __syncthreads();
-    const uint32_t prefix = s_prefix;
-    if (kInSmem) {
-      for (int m = threadIdx.x; m < n_m; m += blockDim.x) {
-        const uint32_t h = s_keys[m];
-        if ((h & mask) == prefix) atomicAdd(&s_hist[(h >> shift) & 255u], 1u);
-      }
-    } else {  // recomputed, a block of eight keys per call
-      for (int b = threadIdx.x; b < n_blocks; b += blockDim.x) {
-        uint64_t w[4];
-        key_block(u, b, w);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const uint32_t h = block_half(w, i);
-          if (8 * b + i < n_m && (h & mask) == prefix) atomicAdd(&s_hist[(h >> shift) & 255u], 1u);
-        }
+    for (int b = threadIdx.x; b < 256; b += blockDim.x) sc.hist[b] = 0u;
+    __syncthreads();
+    const uint32_t prefix = sc.prefix;
+    for (int b = threadIdx.x; b < n_blocks; b += blockDim.x) {
+      uint64_t w[4];
+      key_block(u, b, w);
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t h = block_half(w, i);
+        if (8 * b + i < n_m && (h & mask) == prefix) atomicAdd(&sc.hist[(h >> shift) & 255u], 1u);
       }
     }
     __syncthreads();
     if (threadIdx.x < 32) {
-      // the bin holding rank s_rank: lane l sums bins 8l..8l+7, then a warp scan
-      const uint32_t rank = s_rank;
+      // the bin holding the rank: lane l sums bins 8l..8l+7, then a warp scan
+      const uint32_t rank = sc.rank;
       uint32_t mine = 0u;
 #pragma unroll
-      for (int b = 0; b < 8; ++b) mine += s_hist[lane * 8 + b];
+      for (int b = 0; b < 8; ++b) mine += sc.hist[lane * 8 + b];
       uint32_t incl = mine;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -184,53 +167,224 @@ sampler_kernel(SamplerParams p, int64_t first_unit) {
         uint32_t cum = incl - mine;
         int b = lane * 8;
         for (; b < lane * 8 + 7; ++b) {
-          if (cum + s_hist[b] >= rank) break;
-          cum += s_hist[b];
+          if (cum + sc.hist[b] >= rank) break;
+          cum += sc.hist[b];
         }
-        s_prefix = prefix | ((uint32_t)b << shift);
-        s_rank = rank - cum;
-        s_neq = s_hist[b];  // after the last pass: the keys equal to h*
+        sc.prefix = prefix | ((uint32_t)b << shift);
+        sc.rank = rank - cum;
       }
     }
     mask |= 255u << shift;
-    __syncthreads();
-  }
-  const uint32_t hstar = s_prefix;   // high half of the L-th smallest key
-  const uint32_t take_ties = s_rank; // points with h == h* to take, smallest m first
-
-  // Members: h < h*, or h == h* and m <= mtie (the last tie taken).  Almost
-  // always every tie is taken; otherwise warp 0 finds the take_ties-th tie.
-  if (threadIdx.x < 32) {
-    int mtie = 0x7fffffff;
-    if (take_ties < s_neq) {
-      uint32_t seen = 0u;
-      mtie = -1;
-      for (int m0 = 0; m0 < n_m && mtie < 0; m0 += 32) {
-        const int m = m0 + lane;
-        const bool tie = m < n_m && (kInSmem ? s_keys[m] : key_hi(u, m)) == hstar;
-        const unsigned bal = __ballot_sync(0xffffffffu, tie);
-        if (seen + __popc(bal) >= take_ties) {
-          unsigned b = bal;
-          for (uint32_t k = seen + 1; k < take_ties; ++k) b &= b - 1u;  // drop earlier ties
-          mtie = m0 + __ffs(b) - 1;
-        }
-        seen += __popc(bal);
-      }
-    }
-    if (lane == 0) s_mtie = mtie;
   }
   __syncthreads();
-  const int mtie = s_mtie;
+  const uint32_t hstar = sc.prefix;    // high half of the L-th smallest key
+  const uint32_t take_ties = sc.rank;  // points with h == h* to take, smallest m first
+  __syncthreads();
+  // warp 0 finds the last tie taken (no shared state but the prefix word)
+  if (threadIdx.x < 32) {
+    uint32_t seen = 0u;
+    int mtie = -1;
+    for (int b0 = 0; b0 < n_blocks && mtie < 0; b0 += 32) {
+      uint64_t w[4];
+      key_block(u, min(b0 + lane, n_blocks - 1), w);
+      uint32_t ties = 0u;
+      for (int i = 0; i < 8; ++i)
+        if (b0 + lane < n_blocks && 8 * (b0 + lane) + i < n_m && block_half(w, i) == hstar)
+          ties |= 1u << i;
+      uint32_t incl = __popc(ties);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const unsigned hit = __ballot_sync(0xffffffffu, seen + incl >= take_ties);
+      if (hit) {
+        const int owner = __ffs(hit) - 1;
+        uint32_t before = seen + incl - __popc(ties);
+        for (uint32_t k = before + 1; k < take_ties; ++k) ties &= ties - 1u;  // drop earlier ties
+        mtie = __shfl_sync(0xffffffffu, 8 * (b0 + lane) + __ffs(ties) - 1, owner);
+      }
+      seen += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) sc.prefix = (uint32_t)mtie;
+  }
+  __syncthreads();
+  return ((unsigned long long)hstar << 32) | sc.prefix;
+}
+
+constexpr int kWindow = 2048;  // keys listed around the L-th smallest
+constexpr int kBinKeys = 64;   // of them, keys of the bin that holds it
+
+__global__ void __launch_bounds__(kSamplerThreads)
+sampler_kernel(SamplerParams p, int64_t first_unit) {
+  extern __shared__ __align__(16) uint32_t s_bits[];  // bit m: point m is a member
+  __shared__ unsigned long long s_win[kWindow], s_bin_keys[kBinKeys], s_last;
+  __shared__ SelectScratch s_sel;
+  __shared__ uint32_t s_warp[32];
+  __shared__ uint32_t s_below, s_listed, s_rank, s_bin, s_in_bin, s_total;
+
+  const int64_t uidx = first_unit + blockIdx.x;
+  const UnitDesc u = p.units[uidx];
+  const int n_m = u.n_m, L = u.L;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (L < 1 || L > n_m) {
+    if (tid == 0) atomicOr(p.err, kErrSampler);
+    return;
+  }
+  const int n_blocks = (n_m + 7) >> 3, words = (n_m + 31) >> 5;
+  // a manifold too long for the bits keeps only the last member's key
+  const bool keep = n_m <= kSamplerBitsMax;
+  unsigned char* bytes = reinterpret_cast<unsigned char*>(s_bits);
+
+  // The window [lo, hi] of high halves: L/N_m of the range, +-5 standard
+  // deviations of the rank (and a few keys more).
+  const float pf = (float)L / (float)n_m;
+  const float half_keys = 5.f * sqrtf((float)L * fmaxf(1.f - pf, 0.f)) + 8.f;
+  const uint64_t centre = ((uint64_t)L << 32) / (uint32_t)n_m;
+  const uint64_t half = (uint64_t)(half_keys * (4294967296.f / (float)n_m));
+  const uint32_t lo = centre > half ? (uint32_t)min(centre - half, (uint64_t)0xffffffffu) : 0u;
+  const uint32_t hi = (uint32_t)min(centre + half, (uint64_t)0xffffffffu);
+  for (int b = tid; b < 256; b += kSamplerThreads) s_sel.hist[b] = 0u;
+  if (tid == 0) {
+    s_below = s_listed = s_in_bin = s_total = 0u;
+    s_rank = 0u;
+    s_bin = 0xffffffffu;
+    for (int b = n_blocks; b < 4 * words && keep; ++b) bytes[b] = 0;  // the last word's unused bytes
+  }
+  __syncthreads();
+  uint32_t below = 0u;
+  for (int b = tid; b < n_blocks; b += kSamplerThreads) {
+    uint64_t w[4];
+    key_block(u, b, w);
+    uint32_t byte = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t h = block_half(w, i);
+      if (h < lo) byte |= 1u << i;
+      if (h - lo <= hi - lo && 8 * b + i < n_m) {
+        const uint32_t at = atomicAdd(&s_listed, 1u);
+        if (at < (uint32_t)kWindow) s_win[at] = ((unsigned long long)h << 32) | (uint32_t)(8 * b + i);
+      }
+    }
+    if (8 * b + 8 > n_m) byte &= (1u << (n_m - 8 * b)) - 1u;
+    below += __popc(byte);
+    if (keep) bytes[b] = (unsigned char)byte;
+  }
+  below = __reduce_add_sync(0xffffffffu, below);
+  if (lane == 0 && below) atomicAdd(&s_below, below);
+  __syncthreads();
+  const uint32_t listed = s_listed, sum_below = s_below;
+  // members among the listed keys; 0 and all of them need no search
+  const uint32_t want = (uint32_t)L - sum_below;
+  bool found = (uint32_t)L >= sum_below && listed <= (uint32_t)kWindow && want <= listed;
+  if (found && want > 0u && want < listed) {
+    // bins of equal width over the window: the one holding the last member,
+    // then its rank among that bin's keys
+    const uint64_t scale = (256ull << 24) / ((uint64_t)(hi - lo) + 1u);
+    auto bin_of = [&](unsigned long long key) {
+      return min(255u, (uint32_t)(((uint32_t)(key >> 32) - lo) * scale >> 24));
+    };
+    for (uint32_t q = tid; q < listed; q += kSamplerThreads) atomicAdd(&s_sel.hist[bin_of(s_win[q])], 1u);
+    __syncthreads();
+    if (tid < 32) {
+      uint32_t mine = 0u;
+#pragma unroll
+      for (int b = 0; b < 8; ++b) mine += s_sel.hist[lane * 8 + b];
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const unsigned hit = __ballot_sync(0xffffffffu, incl >= want);
+      if (lane == __ffs(hit) - 1) {
+        uint32_t cum = incl - mine;
+        int b = lane * 8;
+        for (; b < lane * 8 + 7; ++b) {
+          if (cum + s_sel.hist[b] >= want) break;
+          cum += s_sel.hist[b];
+        }
+        s_bin = (uint32_t)b;
+        s_rank = want - cum;
+      }
+    }
+    __syncthreads();
+    for (uint32_t q = tid; q < listed; q += kSamplerThreads) {
+      const unsigned long long key = s_win[q];
+      if (bin_of(key) == s_bin) {
+        const uint32_t at = atomicAdd(&s_in_bin, 1u);
+        if (at < (uint32_t)kBinKeys) s_bin_keys[at] = key;
+      }
+    }
+    __syncthreads();
+    const uint32_t in_bin = s_in_bin;
+    found = in_bin <= (uint32_t)kBinKeys;
+    if (found && tid < (int)in_bin) {
+      const unsigned long long key = s_bin_keys[tid];
+      uint32_t less = 0u;
+      for (uint32_t q = 0; q < in_bin; ++q) less += s_bin_keys[q] < key ? 1u : 0u;
+      if (less + 1u == s_rank) s_last = key;
+    }
+    __syncthreads();
+  }
+  // the last member's key; the members are the points whose key is not above it
+  const unsigned long long last = !found            ? select_by_radix(u, s_sel)
+                                  : want == 0u      ? ((unsigned long long)lo << 32) - 1ull
+                                  : want == listed ? ((unsigned long long)hi << 32) | 0xffffffffull
+                                                    : s_last;
+  if (keep && found) {
+    for (uint32_t q = tid; q < listed; q += kSamplerThreads) {
+      const unsigned long long key = s_win[q];
+      if (key <= last) atomicOr(&s_bits[(uint32_t)key >> 5], 1u << ((uint32_t)key & 31u));
+    }
+  } else if (keep) {
+    for (int b = tid; b < n_blocks; b += kSamplerThreads) {
+      uint64_t w[4];
+      key_block(u, b, w);
+      uint32_t byte = 0u;
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long key = ((unsigned long long)block_half(w, i) << 32) | (uint32_t)(8 * b + i);
+        if (8 * b + i < n_m && key <= last) byte |= 1u << i;
+      }
+      bytes[b] = (unsigned char)byte;
+    }
+  }
+  __syncthreads();
   auto is_member = [&](int m) {
-    const uint32_t h = kInSmem ? s_keys[m] : key_hi(u, m);
-    return h < hstar || (h == hstar && m <= mtie);
+    if (keep) return ((s_bits[m >> 5] >> (m & 31)) & 1u) != 0u;
+    uint64_t w[4];
+    key_block(u, m >> 3, w);
+    return (((unsigned long long)block_half(w, m & 7) << 32) | (uint32_t)m) <= last;
   };
-  // The library in query order (the order the neighbour search visits it in).
   const int32_t* ord = p.order + u.order_off;
-  const uint32_t total = block_compact(n_m, [&](int q) { return ord[q]; }, is_member,
-                                       p.lib + u.lib_off, (uint32_t)L, s_warp);
+  uint32_t total = 0u;
+  if (u.table_R > 0 && !p.list_all) {
+    // one bit per position of the query order, eight words at a time per warp
+    uint32_t* out = p.bits + u.bits_off;
+    uint32_t count = 0u;
+    for (int w0 = warp * 8; w0 < words; w0 += kSamplerThreads / 32 * 8) {
+      uint32_t mine = 0u;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int pos = (w0 + i) * 32 + lane;
+        const bool mem = pos < n_m && is_member(ord[min(pos, n_m - 1)]);
+        const uint32_t word = __ballot_sync(0xffffffffu, mem);
+        if (lane == i) mine = word;
+      }
+      if (lane < 8 && w0 + lane < words) out[w0 + lane] = mine;
+      count += __popc(mine);
+    }
+    count = __reduce_add_sync(0xffffffffu, count);
+    if (lane == 0) atomicAdd(&s_total, count);
+    __syncthreads();
+    total = s_total;
+  } else {
+    // the library in query order (the order the neighbour search visits it in)
+    total = block_compact(n_m, [&](int q) { return ord[q]; }, is_member,
+                          p.lib + u.lib_off, (uint32_t)L, s_warp);
+  }
   if (total != (uint32_t)L) {  // not a permutation, or a lost tie: report, never guess
-    if (threadIdx.x == 0) atomicOr(p.err, kErrSampler);
+    if (tid == 0) atomicOr(p.err, kErrSampler);
     return;
   }
   if (p.dbg_lib) {  // checking copy in ascending m, once per target of this library
@@ -245,24 +399,50 @@ sampler_kernel(SamplerParams p, int64_t first_unit) {
 }  // namespace
 
 cudaError_t sampler_prepare() {
-  return cudaFuncSetAttribute(sampler_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(kSamplerSmemKeys * sizeof(uint32_t)));
+  return cudaFuncSetAttribute(sampler_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              kSamplerBitsMax / 8);
 }
 
 cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t count, int max_nm,
                            cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  if (max_nm <= kSamplerSmemKeys) {
-    const size_t smem = (size_t)((max_nm + 7) / 8 * 8) * sizeof(uint32_t);  // whole blocks
-    for (int64_t off = 0; off < count; off += 0x7fffffff) {
-      const unsigned grid = (unsigned)((count - off) < 0x7fffffff ? (count - off) : 0x7fffffff);
-      sampler_kernel<true><<<grid, kSamplerThreads, smem, s>>>(p, first_unit + off);
-    }
-  } else {
-    for (int64_t off = 0; off < count; off += 0x7fffffff) {
-      const unsigned grid = (unsigned)((count - off) < 0x7fffffff ? (count - off) : 0x7fffffff);
-      sampler_kernel<false><<<grid, kSamplerThreads, 0, s>>>(p, first_unit + off);
-    }
+  const size_t smem = (size_t)((std::min(max_nm, kSamplerBitsMax) + 31) / 32) * 4;
+  for (int64_t off = 0; off < count; off += 0x7fffffff) {
+    const unsigned grid = (unsigned)std::min<int64_t>(count - off, 0x7fffffff);
+    sampler_kernel<<<grid, kSamplerThreads, smem, s>>>(p, first_unit + off);
+  }
+  return cudaGetLastError();
+}
+
+// Membership words of the scan's realization groups: word pos of a group holds
+// bit r when position pos of the query order is in the library of its r-th
+// realization; the words past the last position are zero (the positions that
+// pad a table row).  A warp turns 32 positions of 32 realizations at a time:
+// lane r reads the realization's bits, the transpose leaves a word per position.
+__global__ void __launch_bounds__(256) member_words_kernel(const UnitDesc* units,
+                                                          const MemberGroup* groups,
+                                                          const uint32_t* bits, uint32_t* words) {
+  const MemberGroup g = groups[blockIdx.y];
+  const UnitDesc& u = units[g.unit];
+  const int n_m = u.n_m, per_unit = (n_m + 31) >> 5;
+  const int lane = threadIdx.x & 31;
+  const BitTranspose tr(lane);
+  const uint32_t* src = bits + u.bits_off + (int64_t)min(lane, g.count - 1) * per_unit;
+  uint32_t* dst = words + u.words_off;
+  const int blocks = member_words(n_m) >> 5;
+  // eight consecutive blocks a warp: the 32-byte sectors of `src` are used whole
+  const int b0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 8;
+  for (int b = b0; b < min(b0 + 8, blocks); ++b) {
+    const uint32_t w = (lane < g.count && b < per_unit) ? src[b] : 0u;
+    dst[b * 32 + lane] = tr(w);
+  }
+}
+
+cudaError_t launch_member_words(const UnitDesc* units, const MemberGroup* groups, int64_t n_groups,
+                                int max_nm, const uint32_t* bits, uint32_t* words, cudaStream_t s) {
+  const unsigned gx = (unsigned)((member_words(max_nm) / 32 + 63) / 64);
+  for (int64_t off = 0; off < n_groups; off += 65535) {
+    const dim3 grid(gx, (unsigned)std::min<int64_t>(n_groups - off, 65535));
+    member_words_kernel<<<grid, 256, 0, s>>>(units, groups + off, bits, words);
   }
   return cudaGetLastError();
 }

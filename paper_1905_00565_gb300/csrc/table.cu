@@ -13,15 +13,16 @@
 // the exclusion window) are exactly its E+1 nearest library neighbours:
 // restricting a total order to a subset keeps its order.
 //
-// Layout: ranks in groups of four, table[table_off + (r/4) * 4*n_m + pos*4 +
-// r%4], so that one 8-byte (16-bit entries) or 16-byte (32-bit) load gives a
-// query four consecutive ranks and the 32 consecutive query positions of a
-// warp read one group with one coalesced access; 16-bit entries when every
-// manifold of the plan has fewer than 65536 points, else 32-bit.  A float
-// array of the same layout holds each entry's distance (the square root the
-// simplex weights take of the FP32 squared distance, computed the same way),
-// so that the scan reads the E+1 distances it needs instead of recomputing
-// them from E scattered coordinates each.
+// Layout: row after row, table[table_off + pos*stride + r], an entry being the
+// point's position in the query order (16 bits when every manifold of the plan
+// has fewer than 65536 points, else 32; rows are padded to a multiple of 64
+// with position n_m, which no library holds).  A warp that walks a row reads 32
+// ranks with one access, and neighbouring points have neighbouring positions,
+// so lookups by position are coherent.  A float array of the same layout holds
+// each entry's distance (the square root the simplex weights take of the FP32
+// squared distance, computed the same way), or pairs of it and the single
+// target's value at the point, so that the scan reads what the prediction needs
+// from the row.
 //
 // Build: one warp per query position, one kernel per E (its registers follow
 // that E).  A histogram of the top 11 bits of the
@@ -148,7 +149,8 @@ __device__ __forceinline__ uint32_t d2_bits_staged(const float* stage, int off, 
 // series values, or null.
 template <int E>
 __device__ void build_row(const float* s, const TableJob& jb, int pos, bool row,
-                          const int32_t* order, void* table, float* table_dist, int pairs,
+                          const int32_t* order, const int32_t* inverse, void* table,
+                          float* table_dist, int pairs,
                           const float* tv_series, int u16,
                           uint32_t* hist, unsigned long long* keys, unsigned long long* bnd,
                           uint32_t* cnt, int region_keys, float* stage) {
@@ -373,27 +375,23 @@ __device__ void build_row(const float* s, const TableJob& jb, int pos, bool row,
   }
   }
   __syncwarp();
-  const int64_t base = jb.table_off + (int64_t)pos * 4;
+  const int64_t base = jb.table_off + (int64_t)pos * jb.stride;
   // each entry's distance (the epilogue's square root), beside it; with pairs,
   // together with the target's value at the entry's point (what the
   // prediction weighs; 0 in a table without a target)
   for (int r = lane; r < R; r += 32) {
-    const int64_t at = base + (int64_t)(r >> 2) * 4 * n_m + (r & 3);
     const float d = sqrt_hw(__uint_as_float((uint32_t)(keys[r] >> 32)));
     if (pairs)
-      reinterpret_cast<float2*>(table_dist)[at] =
+      reinterpret_cast<float2*>(table_dist)[base + r] =
           make_float2(d, jb.tv_i >= 0 ? tv_series[(int)(keys[r] & 0xffffffffu) + off] : 0.f);
     else
-      table_dist[at] = d;
+      table_dist[base + r] = d;
   }
-  if (u16) {
-    uint16_t* out = static_cast<uint16_t*>(table) + base;
-    for (int r = lane; r < R; r += 32)
-      out[(int64_t)(r >> 2) * 4 * n_m + (r & 3)] = (uint16_t)(keys[r] & 0xffffu);
-  } else {
-    int32_t* out = static_cast<int32_t*>(table) + base;
-    for (int r = lane; r < R; r += 32)
-      out[(int64_t)(r >> 2) * 4 * n_m + (r & 3)] = (int32_t)(keys[r] & 0xffffffffu);
+  const int32_t* inv = inverse + jb.order_off;
+  for (int r = lane; r < jb.stride; r += 32) {
+    const int at = r < R ? inv[(int)(keys[r] & 0xffffffffu)] : n_m;
+    if (u16) static_cast<uint16_t*>(table)[base + r] = (uint16_t)at;
+    else static_cast<int32_t*>(table)[base + r] = at;
   }
   __syncwarp();
 }
@@ -404,8 +402,8 @@ __device__ void build_row(const float* s, const TableJob& jb, int pos, bool row,
 // the N = 10^5 series' 203 vs 185 ms).
 template <int E, int kMinCtas>
 __global__ void __launch_bounds__(kTableWarps * 32, kMinCtas)
-table_build_kernel(const float* series, const TableJob* jobs, const int32_t* order, void* table,
-                   float* table_dist, int pairs, int u16, int rcap, int staged) {
+table_build_kernel(const float* series, const TableJob* jobs, const int32_t* order,
+                   const int32_t* inverse, void* table, float* table_dist, int pairs, int u16, int rcap, int staged) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ uint32_t s_cnt[kTableWarps][2];  // per warp: entries below b1, entries of b1
   const TableJob jb = jobs[blockIdx.y];
@@ -426,7 +424,7 @@ table_build_kernel(const float* series, const TableJob* jobs, const int32_t* ord
                      ? reinterpret_cast<float*>(smem + kTableWarps * table_warp_bytes(rcap))
                      : nullptr;
   const float* tv_series = series + jb.series_off + (int64_t)(jb.tv_i >= 0 ? jb.tv_i : 0) * jb.n;
-  build_row<E>(s, jb, pos, pos < jb.n_m, order, table, table_dist, pairs, tv_series, u16, hist,
+  build_row<E>(s, jb, pos, pos < jb.n_m, order, inverse, table, table_dist, pairs, tv_series, u16, hist,
                keys, bnd,
                s_cnt[warp], (int)(table_warp_bytes(rcap) / 8), stage);
 }
@@ -453,8 +451,8 @@ cudaError_t table_prepare() {
 }
 
 cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_t n_jobs, int E,
-                               int max_nm, int max_R, const int32_t* order, void* table,
-                               float* table_dist, int table_pairs, int table_u16, cudaStream_t s) {
+                               int max_nm, int max_R, const int32_t* order,
+                               const int32_t* inverse, void* table, float* table_dist, int table_pairs, int table_u16, cudaStream_t s) {
   if (n_jobs <= 0) return cudaSuccess;
   int rcap = 32;
   while (rcap < max_R) rcap <<= 1;
@@ -465,10 +463,10 @@ cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_
   if (E == EV) {                                                                         \
     if (max_nm >= kSampleMinNm)                                                          \
       table_build_kernel<EV, 3><<<grid, kTableWarps * 32, table_smem(rcap, staged), s>>>( \
-          series, jobs, order, table, table_dist, table_pairs, table_u16, rcap, staged);   \
+          series, jobs, order, inverse, table, table_dist, table_pairs, table_u16, rcap, staged);   \
     else                                                                                 \
       table_build_kernel<EV, 2><<<grid, kTableWarps * 32, table_smem(rcap, staged), s>>>( \
-          series, jobs, order, table, table_dist, table_pairs, table_u16, rcap, staged);   \
+          series, jobs, order, inverse, table, table_dist, table_pairs, table_u16, rcap, staged);   \
     return cudaGetLastError();                                                           \
   }
   CCM_FOR_E(CCM_TBLAUNCH)

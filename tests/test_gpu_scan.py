@@ -1,0 +1,86 @@
+"""The grouped table scan and the window sampler at their edges, against brute
+force bit for bit and the oracle (needs a GB300)."""
+
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1905_00565_gb300 import inputs as I
+from tests.ccm_check import check_units, run_detailed
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ccm():
+    from paper_1905_00565_gb300 import ccm as c
+    return c
+
+
+def rho_only(ccm, ctx, p, flags):
+    plan = ccm.plan_problem(ctx, p, flags)
+    try:
+        assert (ccm.ccm_plan_get_info(plan)["table_bytes"] > 0) == (flags == 0)
+        rho = np.zeros(ccm.rho_shape(p))
+        ccm.ccm_run(plan, p.series, rho)
+    finally:
+        ccm.ccm_plan_destroy(plan)
+    return rho
+
+
+# r: one lane, groups that end inside a cell, exactly at it, and that span cells;
+# n: ragged tiles, membership words in shared memory and (20000, 70000) in L2,
+# 16- and 32-bit positions; unsorted L
+@pytest.mark.parametrize("n,E,L,r,theiler", [
+    (700, [1, 10], [400, 690, 300], 33, 0), (2049, [3], [2000, 300, 1024], 31, 0),
+    (3000, [2, 9], [2900, 700], 64, 4), (5000, [4], [300, 4999 - 3], 21, 0),
+    (20000, [1, 5], [900, 15000], 40, 0), (70000, [3], [20000, 69000], 11, 2)])
+def test_scan_equals_brute_force(ccm, n, E, L, r, theiler):
+    s = I.add_noise(I.logistic_pair(n), 0.001, 3) if n % 2 else I.logistic_pair(n)
+    p = I.Problem(series=s, pairs=I.BOTH_DIRECTIONS.copy(), E=np.array(E, np.int32),
+                  tau=np.array([1], np.int32), L=np.array(L, np.int64), r=r, seed=21,
+                  theiler=theiler)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        np.testing.assert_array_equal(rho_only(ccm, ctx, p, 0),
+                                      rho_only(ccm, ctx, p, ccm.CCM_NO_TABLE))
+    finally:
+        ccm.ccm_context_destroy(ctx)
+
+
+def test_scan_checking_outputs(ccm):
+    """Neighbours, predictions and libraries of the general variant."""
+    p = I.Problem(series=I.logistic_pair(1500), pairs=I.BOTH_DIRECTIONS.copy(),
+                  E=np.array([1, 6], np.int32), tau=np.array([3], np.int32),
+                  L=np.array([500, 1400], np.int64), r=18, seed=2, weight_floor=0.01)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        rho, lib, nbr, xh = run_detailed(ccm, ctx, p)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    check_units(p, rho, lib, nbr, xh, which={0, 17, 18, 35, 70, 143})
+
+
+@pytest.mark.parametrize("n,L", [(300, [5, 150, 299, 300]), (9, [4, 9]), (4096, [4, 4095, 2048]),
+                                 (65536, [100, 65000])])
+def test_libraries_at_the_edges(ccm, n, L):
+    """The sampler's window at both ends of its range: the smallest and the full
+    library, short and long manifolds."""
+    rng = np.random.default_rng(n)
+    p = I.Problem(series=rng.random((2, n)).astype(np.float32),
+                  pairs=np.array([[0, 1]], np.int32), E=np.array([1], np.int32),
+                  tau=np.array([1], np.int32), L=np.array(L, np.int64), r=9, seed=77)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        for flags in (0, ccm.CCM_NO_TABLE):
+            _, lib, _, _ = run_detailed(ccm, ctx, p, flags)
+            at = 0
+            for Lv in L:
+                for k in range(p.r):
+                    want = oracle.library(n, Lv, 0, 1, 1, k, p.seed)
+                    np.testing.assert_array_equal(lib[at:at + Lv], want)
+                    at += Lv
+    finally:
+        ccm.ccm_context_destroy(ctx)

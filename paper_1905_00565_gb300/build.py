@@ -20,7 +20,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libccm_gb300.so")
 # (source, E): the search kernels are compiled once per embedding dimension, in parallel
-SOURCES = [(name, e) for e in range(10, 0, -1) for name in ("knn_fused.cu", "knn_scan.cu")] + [
+SOURCES = [(name, e) for e in range(10, 0, -1) for name in ("knn_fused.cu", "table_build.cu", "knn_scan.cu")] + [
     (name, 0) for name in ("table.cu", "runtime.cu", "sampler.cu", "knn_dispatch.cu", "plain.cu",
                            "noalloc.cu", "order.cu", "convergence.cu")]
 HEADERS = [os.path.join(CSRC, name) for name in ("ccm_internal.h", "moments.cuh", "bits.cuh")] + [

@@ -154,10 +154,22 @@ struct TableJob {
   int32_t j, E, tau, n_m;
   int32_t R;            // entries per row; padded with position n_m to
   int32_t stride;       // a multiple of 64
+  int64_t pts_off;      // the points in query order: [chunk of 32][E][32] floats
+  int64_t box_off;      // chunk boxes [2E][32 * superchunks], superchunk boxes [2E][superchunks]
+  int64_t sbox_off;
+  int64_t sample_off;   // every sample-th point, [E][n_m / sample]
+  int32_t sample;       // (sample_stride)
   int32_t tv_i;         // >= 0: also store target variable tv_i's value at every entry's point
-  int32_t pad;
 };
-constexpr int kTableMaxR = 2048;       // entries per query row, at most
+// The sample a row's threshold is read from: at least about 1000 points and
+// about 24 of them inside the row.
+inline int32_t sample_stride(int64_t n_m, int64_t R) {
+  int32_t s = 1;
+  while (2 * s * 1024 <= n_m && 2 * s * 24 <= R) s <<= 1;
+  return s;
+}
+constexpr int kTableMaxR = 4096;       // entries per query row, at most
+constexpr int kWalkMaxR = 2048;        // the same for variables with several targets (knn_fused.cu)
 constexpr int kTableChunk = 8;         // query tiles per table work item (one bitmap each)
 constexpr int kTableMaxNm = 1 << 20;   // longest manifold that gets a table (bitmap in smem)
 
@@ -261,6 +273,7 @@ __device__ __forceinline__ float simplex_u(float d2, float d1, float inv_d1, flo
 // Error flag values written by kernels.
 constexpr int32_t kErrBadUnit = 1;
 constexpr int32_t kErrSampler = 2;
+constexpr int32_t kErrTable = 4;
 
 // Sampler (sampler.cu).
 constexpr int kSamplerThreads = 256;
@@ -282,10 +295,25 @@ cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jo
 
 // Distance indexing table (table.cu).
 cudaError_t table_prepare();
-// One launch builds the tables of jobs[0..n_jobs), all of embedding dimension E.
-cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_t n_jobs, int E,
-                               int max_nm, int max_R, const int32_t* order,
-                               const int32_t* inverse, void* table, float* table_dist, int table_pairs, int table_u16, cudaStream_t s);
+// The jobs' points and boxes (all jobs of a run).
+cudaError_t launch_table_points(const float* series, const TableJob* jobs, int64_t n_jobs,
+                                int max_nm, const int32_t* order, float* points, cudaStream_t s);
+// One launch builds the tables of jobs[0..n_jobs), all of embedding dimension E
+// (n_rows rows together).
+cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_t n_jobs,
+                               int64_t n_rows, int E, int max_nm, int max_R, const float* points,
+                               const int32_t* order, const int32_t* inverse, void* table,
+                               float* table_dist, int table_pairs, int table_u16, int32_t* err,
+                               cudaStream_t s);
+// Its kernels (table_build.cu, compiled once per E).
+template <int E>
+struct TableKernels {
+  static cudaError_t prepare();
+  static cudaError_t launch(const float* series, const TableJob* jobs, int64_t n_jobs,
+                            int64_t n_rows, int max_nm, int max_R, const float* points,
+                            const int32_t* order, const int32_t* inverse, void* table,
+                            float* table_dist, int pairs, int u16, int32_t* err, cudaStream_t s);
+};
 
 // Search kernels of one E (knn_fused.cu, compiled once per E; each kernel keeps
 // its registers for that E's lists).

@@ -844,7 +844,7 @@ __device__ __forceinline__ float d2_point(const float* sj, int off, int tau, con
 // held members: (step << 8) | flags, flag c marking rank 8*step + c.  A query
 // keeps at most E+1 records: [kMaxE+1][kThreads] 16-bit words.
 constexpr int kRecBytes = (kMaxE + 1) * kThreads * 2;
-static_assert(kTableMaxR / 8 <= 256, "a record's step index has eight bits");
+static_assert(kWalkMaxR / 8 <= 256, "a record's step index has eight bits");
 
 // One query's walk along its table row (`row`: its entries): records the steps
 // with members until it has K of them; returns the members met.

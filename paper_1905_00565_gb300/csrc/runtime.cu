@@ -172,11 +172,11 @@ struct UnitList {
   int64_t lib_scratch = 0;            // longest library of the units that read a table
   std::vector<double> item_cost_table;
   int64_t lib_total = 0, part_total = 0, order_total = 0, table_total = 0;
+  int64_t points_total = 0;           // floats: the tables' points and boxes
   int64_t order_scratch_total = 0;    // 64-bit keys for sorting manifolds above kOrderMaxSort
-  // Table jobs are sorted by (sort size, E) (sort_items) and built one launch
-  // per sort size (the power of two at or above R) and E: a launch's shared
-  // memory per warp follows its own largest row, so short rows run more warps
-  // per SM, and its registers follow its E.
+  // Table jobs are sorted by (size class, E) (sort_items) and built one launch
+  // per size class (the power of two at or above R) and E: a launch's shared
+  // memory follows its own longest row and its registers its E.
   static int table_rcap(int R) {
     int rc = 32;
     while (rc < R) rc <<= 1;
@@ -245,11 +245,11 @@ TableTuning read_table_tuning() {
 // N = 10^5 series (E = 3..6) brute force at L = 1000 beats walks of
 // (E+1)*100 entries, so libraries below N_m/max_ratio (40) points stay with
 // brute force.  The last term keeps the row length (table_row_length) within
-// kTableMaxR.
-double table_min_L(int32_t E, int64_t n_m, const TableTuning& t) {
+// max_R.
+double table_min_L(int32_t E, int64_t n_m, int max_R, const TableTuning& t) {
   return std::max({t.floor, std::ceil(std::sqrt(t.crossover * (double)n_m / (double)(E + 1))),
                    std::ceil((double)n_m / t.max_ratio),
-                   std::ceil(t.safety * 2.8 * (E + 2) * (double)n_m / (double)kTableMaxR)});
+                   std::ceil(t.safety * 2.8 * (E + 2) * (double)n_m / (double)max_R)});
 }
 
 // Row length R of a table whose smallest L is lmin.  A query of a realization
@@ -396,6 +396,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
   // The safety factor trades table memory and build time against how often a
   // query falls back to scanning its library.
   const TableTuning tt = read_table_tuning();
+  auto max_R_of = [&](int32_t j) { return pairs_of[j].size() == 1 ? kTableMaxR : kWalkMaxR; };
   const double safety = tt.safety;
   double table_bytes = 0.0;
   if (!(pc.flags & CCM_NO_TABLE)) {
@@ -404,7 +405,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         for (int32_t tau : pc.tau) {
           const int64_t n_m = pc.n - (int64_t)(E - 1) * tau;
           if (n_m > kTableMaxNm) continue;
-          const double ls = table_min_L(E, n_m, tt);
+          const double ls = table_min_L(E, n_m, max_R_of(j), tt);
           int64_t lmin = -1;
           double lsum = 0.0;
           for (int64_t L : pc.L)
@@ -415,7 +416,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           if (lmin < 0 || lsum < 8.0 * (double)n_m) continue;
           int64_t R = table_row_length(E, n_m, lmin, pc.theiler, safety);
           // from the n_m - 1 points other than the query; rows are padded to 64
-          R = std::min<int64_t>(std::min<int64_t>((R + 31) / 32 * 32, kTableMaxR), n_m - 1);
+          R = std::min<int64_t>(std::min<int64_t>((R + 31) / 32 * 32, max_R_of(j)), n_m - 1);
           const int64_t stride = (R + 63) / 64 * 64;
           // positions (2 or 4 bytes), distances, and for a variable with one
           // target the target's values
@@ -436,6 +437,13 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           tj.n_m = (int32_t)n_m;
           tj.R = (int32_t)R;
           tj.stride = (int32_t)stride;
+          const int64_t chunks = (n_m + 31) / 32, supers = (chunks + 31) / 32;
+          tj.pts_off = ul->points_total;
+          tj.box_off = tj.pts_off + chunks * 32 * E;
+          tj.sbox_off = tj.box_off + 2 * E * supers * 32;
+          tj.sample = sample_stride(n_m, R);
+          tj.sample_off = tj.sbox_off + 2 * E * supers;
+          ul->points_total = (tj.sample_off + n_m / tj.sample * E + 63) / 64 * 64;
           tj.tv_i = tv ? pc.pairs[2 * pairs_of[j][0] + 1] : -1;
           if (tv) ul->table_tv = true;
           table_of[std::make_tuple(j, E, tau)] = std::make_pair(tj.table_off, tj.stride);
@@ -452,7 +460,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         const bool tab = table_of.count(std::make_tuple(j, E, tau)) != 0;
         int64_t tabled = 0;
         for (int64_t L : pc.L) {
-          if (!tab || (double)L < table_min_L(E, n_m, tt))
+          if (!tab || (double)L < table_min_L(E, n_m, max_R_of(j), tt))
             brute_tiles[E] += (n_m + tileq - 1) / tileq * pc.r;
           else
             tabled += pc.r;
@@ -506,7 +514,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
               ul->targets.push_back(tg);
             }
             const auto tab = table_of.find(std::make_tuple(j, E, tau));
-            if (tab != table_of.end() && (double)L >= table_min_L(E, u.n_m, tt)) {
+            if (tab != table_of.end() && (double)L >= table_min_L(E, u.n_m, max_R_of(j), tt)) {
               u.table_off = tab->second.first;
               u.table_R = tab->second.second;
               u.bits_off = ul->bits_total;
@@ -653,7 +661,7 @@ struct Arena {
          counter = 0, scratch = 0, order = 0, orders = 0, targets = 0, table = 0, tables = 0,
          items_table = 0, order_scratch = 0, obs = 0, obs_stat = 0, obs_jobs = 0, series_jobs = 0,
          scales = 0, st = 0, table_dist = 0, stats = 0, inverse = 0, bits = 0, words = 0,
-         member_groups = 0,
+         member_groups = 0, points = 0,
          total = 0;
 };
 
@@ -684,6 +692,7 @@ Arena layout(int64_t series_elems, const UnitList& ul, int64_t n_rho, int64_t sc
   a.targets = take(sizeof(TargetDesc) * ul.targets.size());
   a.table = take(ul.table_elem() * (size_t)ul.table_total);
   a.table_dist = take((ul.table_tv ? sizeof(float2) : sizeof(float)) * (size_t)ul.table_total);
+  a.points = take(sizeof(float) * (size_t)ul.points_total);
   a.tables = take(sizeof(TableJob) * ul.tables.size());
   a.items_table = take(sizeof(WorkItem) * ul.items_table.size());
   a.obs = take(sizeof(float2) * (size_t)knn_block_threads() * (size_t)ul.obs_total);
@@ -914,24 +923,33 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   if (stats) CCM_CUDA(cudaMemsetAsync(base + ar.stats, 0, sizeof(unsigned long long) * kStatCount, s));
   if (ev) CCM_CUDA(record(ev[0]));
   CCM_CUDA(enqueue_order(base, ar, ul, s));
-  for (size_t g0 = 0; g0 < ul.tables.size();) {  // one launch per (sort size, E)
+  if (!ul.tables.empty())
+    CCM_CUDA(launch_table_points(reinterpret_cast<const float*>(base + ar.series),
+                                 reinterpret_cast<const TableJob*>(base + ar.tables),
+                                 (int64_t)ul.tables.size(), ul.max_nm,
+                                 reinterpret_cast<const int32_t*>(base + ar.order),
+                                 reinterpret_cast<float*>(base + ar.points), s));
+  for (size_t g0 = 0; g0 < ul.tables.size();) {  // one launch per (size class, E)
     const int rc = UnitList::table_rcap(ul.tables[g0].R), te = ul.tables[g0].E;
     size_t g1 = g0;
     int nm = 0, rmax = 0;
+    int64_t rows = 0;
     for (; g1 < ul.tables.size() && UnitList::table_rcap(ul.tables[g1].R) == rc &&
-           ul.tables[g1].E == te;
+           ul.tables[g1].E == te && g1 - g0 < 65535;
          ++g1) {
       nm = std::max(nm, ul.tables[g1].n_m);
       rmax = std::max(rmax, ul.tables[g1].R);
+      rows += ul.tables[g1].n_m;
     }
     CCM_CUDA(launch_table_build(reinterpret_cast<const float*>(base + ar.series),
                                 reinterpret_cast<const TableJob*>(base + ar.tables) + g0,
-                                (int64_t)(g1 - g0), te, nm, rmax,
+                                (int64_t)(g1 - g0), rows, te, nm, rmax,
+                                reinterpret_cast<const float*>(base + ar.points),
                                 reinterpret_cast<const int32_t*>(base + ar.order),
                                 reinterpret_cast<const int32_t*>(base + ar.inverse),
                                 base + ar.table, reinterpret_cast<float*>(base + ar.table_dist),
-                                ul.table_tv ? 1 : 0,
-                                ul.table_u16(), s));
+                                ul.table_tv ? 1 : 0, ul.table_u16(),
+                                reinterpret_cast<int32_t*>(base + ar.err), s));
     g0 = g1;
   }
   if (ev) CCM_CUDA(record(ev[1]));
@@ -1248,6 +1266,7 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
   // table-scan kernel per E present, rho
   in.launches_per_run = 4 + pl->ul.table_groups();  // order, observed values, sampler, rho, tables
   in.launches_per_run += pl->ul.member_groups.empty() ? 0 : 1;  // membership words
+  in.launches_per_run += pl->ul.tables.empty() ? 0 : 1;         // the tables' points
   in.launches_per_run += (int64_t)(pl->ul.groups.size() + pl->ul.groups_table.size());
   *out = pl.release();
   return CCM_OK;

@@ -50,6 +50,36 @@ def test_scan_equals_brute_force(ccm, n, E, L, r, theiler):
         ccm.ccm_context_destroy(ctx)
 
 
+@pytest.mark.parametrize("kind", ["clusters", "ints", "few", "line", "zeros"])
+def test_rows_of_unusual_distances(ccm, kind):
+    """Table rows whose threshold is hard to find: tight clusters 60 octaves of
+    squared distance below the manifold's extent, many exact ties (also at
+    distance 0), and a one-dimensional manifold."""
+    rng = np.random.default_rng(5)
+    n = 2600
+    if kind == "clusters":      # period 4, near-exact copies of four states
+        s = np.tile([0.1, 0.5, 0.35, 0.9], (2, n // 4)) + 1e-6 * rng.random((2, n))
+        s[:, ::97] += 3e4
+    elif kind == "ints":
+        s = rng.integers(0, 3, (2, n))
+    elif kind == "few":
+        s = rng.integers(0, 40, (2, n)) * 0.25
+    elif kind == "line":
+        s = np.stack([np.arange(n), np.arange(n)[::-1]]) * 0.125 + 0.01 * rng.random((2, n))
+    else:
+        s = np.where(rng.random((2, n)) < 0.6, 0.0, rng.random((2, n)))
+    p = I.Problem(series=np.ascontiguousarray(s.astype(np.float32)),
+                  pairs=I.BOTH_DIRECTIONS.copy(), E=np.array([1, 2, 4], np.int32),
+                  tau=np.array([1], np.int32), L=np.array([600, 1900, 2590], np.int64), r=9,
+                  seed=6)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        np.testing.assert_array_equal(rho_only(ccm, ctx, p, 0),
+                                      rho_only(ccm, ctx, p, ccm.CCM_NO_TABLE))
+    finally:
+        ccm.ccm_context_destroy(ctx)
+
+
 def test_scan_checking_outputs(ccm):
     """Neighbours, predictions and libraries of the general variant."""
     p = I.Problem(series=I.logistic_pair(1500), pairs=I.BOTH_DIRECTIONS.copy(),

@@ -80,8 +80,10 @@ typedef enum {
                                       CCM_TABLE_CROSSOVER (default 20), CCM_TABLE_FLOOR
                                       (default 256) and CCM_TABLE_MAX_RATIO (default 40):
                                       tables for L >= max(floor, sqrt(c*N_m/(E+1)),
-                                      N_m/max_ratio); CCM_TABLE_SAFETY (default 1): factor
-                                      on the table row length */
+                                      N_m/max_ratio); library variables with one target go
+                                      lower by an estimate of both sides' time unless one
+                                      of the three is set; CCM_TABLE_SAFETY (default 1):
+                                      factor on the table row length */
 #define CCM_SEARCH_STATS     0x20u /* the neighbour-search kernels also count their work
                                       (ccm_plan_search_stats); a separately compiled
                                       counting variant, slower, same results */

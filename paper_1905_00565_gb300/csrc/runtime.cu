@@ -222,12 +222,15 @@ struct UnitList {
 // manifold-to-library ratio of table_min_L, and a factor s on the row length
 // (see below).  The environment variables CCM_TABLE_CROSSOVER, CCM_TABLE_FLOOR,
 // CCM_TABLE_MAX_RATIO and CCM_TABLE_SAFETY replace the defaults (read at each
-// ccm_plan; tuning and measurement only).
+// ccm_plan; tuning and measurement only); any of the first three leaves the
+// decision to table_min_L.
 struct TableTuning {
   double crossover, floor, max_ratio, safety;
+  bool fixed;  // some threshold was given: the general rule alone decides
 };
 TableTuning read_table_tuning() {
-  TableTuning r{20.0, 256.0, 40.0, 1.0};
+  TableTuning r{20.0, 256.0, 40.0, 1.0, false};
+  r.fixed = getenv("CCM_TABLE_CROSSOVER") || getenv("CCM_TABLE_FLOOR") || getenv("CCM_TABLE_MAX_RATIO");
   if (const char* e = getenv("CCM_TABLE_CROSSOVER")) r.crossover = std::max(0.0, atof(e));
   if (const char* e = getenv("CCM_TABLE_FLOOR")) r.floor = std::max(16.0, atof(e));
   if (const char* e = getenv("CCM_TABLE_MAX_RATIO")) r.max_ratio = std::max(1.0, atof(e));
@@ -245,7 +248,8 @@ TableTuning read_table_tuning() {
 // N = 10^5 series (E = 3..6) brute force at L = 1000 beats walks of
 // (E+1)*100 entries, so libraries below N_m/max_ratio (40) points stay with
 // brute force.  The last term keeps the row length (table_row_length) within
-// max_R.
+// max_R.  (Measured with a walk per query and realization, which variables with
+// several targets still take.)
 double table_min_L(int32_t E, int64_t n_m, int max_R, const TableTuning& t) {
   return std::max({t.floor, std::ceil(std::sqrt(t.crossover * (double)n_m / (double)(E + 1))),
                    std::ceil((double)n_m / t.max_ratio),
@@ -272,6 +276,66 @@ int64_t table_row_length(int32_t E, int64_t n_m, int64_t lmin, int32_t theiler, 
     if (tail <= eps) break;
   }
   return (int64_t)std::ceil(safety * lambda * (double)n_m / (double)lmin) + 2 * (int64_t)theiler;
+}
+
+// Entries per row and their row stride (rows are padded to 64) of a table for
+// libraries from lmin on: from the n_m - 1 points other than the query.
+int64_t table_row_entries(int32_t E, int64_t n_m, int64_t lmin, int32_t theiler, double safety,
+                          int max_R) {
+  const int64_t R = table_row_length(E, n_m, lmin, theiler, safety);
+  return std::min<int64_t>(std::min<int64_t>((R + 31) / 32 * 32, max_R), n_m - 1);
+}
+
+// Estimated picoseconds on one GB300: brute-force search of a query of one
+// realization; table scan of it (W = ranks walked until the slowest of 32
+// realizations has its E+1); table row of R entries.  Fitted to measurements
+// at N = 1000..40000, E in {1, 3, 6, 10}, L = 20..1000 (e.g. N = 10^4, E = 6:
+// brute force 140 / 265 / 472 ps at L = 100 / 400 / 1000, scan 87 / 42 / 26 ps,
+// rows 58 / 22 / 15 ns), within a third of them.
+double brute_ps(int32_t E, double L) {
+  return 20.0 + 7.0 * E + (0.5 + 0.044 * E * E) * std::pow(L, 0.75);
+}
+double scan_ps(int32_t E, double n_m, double L) {
+  const double W = (E + 1 + 2.3 * std::sqrt(E + 1.0)) * n_m / L;
+  const bool in_smem = n_m <= 13000;  // membership words in shared memory (knn_scan.cu)
+  return 12.0 + 1.5 * E + 0.055 * W + (in_smem ? 0.0 : 15.0 + 0.03 * W);
+}
+double row_ps(int32_t E, double n_m, double R) {
+  return 1e3 * (3.0 + 1.2 * E + 0.03 * R + 1.5e-4 * n_m);
+}
+
+// Smallest tabled L of a library variable with one target: that of the general
+// rule (`base`; -1: no table), or the smaller one of the grid at which the
+// brute-force searches it saves outweigh the scans and the longer rows by
+// the estimates above (a table that the general rule does not build also costs
+// about 10 us of launches).  Sweep of N = 10^4 (L = 100..9000, r = 250): every
+// L tabled 172 ms a run, the general rule's 240 ms; two variables of N = 10^5
+// (L from 1000): 106 against 120 ms.
+int64_t cheapest_table_L(const ProblemCopy& pc, int32_t E, int64_t n_m, int64_t base, int max_R,
+                         double safety) {
+  auto cost = [&](int64_t lmin) {
+    double c = 0.0;
+    if (lmin >= 0) {
+      c += row_ps(E, (double)n_m, (double)table_row_entries(E, n_m, lmin, pc.theiler, safety, max_R));
+      if (base < 0) c += 10e6 / (double)n_m;
+    }
+    for (int64_t L : pc.L)
+      c += pc.r * (lmin >= 0 && L >= lmin ? scan_ps(E, (double)n_m, (double)L) : brute_ps(E, (double)L));
+    return c;
+  };
+  int64_t best = base;
+  double least = cost(base);
+  for (int64_t L : pc.L) {
+    if (base >= 0 && L >= base) continue;
+    // rows this long would not fit: too many queries would miss
+    if (table_row_length(E, n_m, L, pc.theiler, safety) > max_R && n_m - 1 > max_R) continue;
+    const double c = cost(L);
+    if (c < least) {
+      least = c;
+      best = L;
+    }
+  }
+  return best;
 }
 
 // Append the units of one problem.  Offsets: series block, first rho index.
@@ -385,18 +449,22 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         }
       }
   // Distance indexing tables (unless CCM_NO_TABLE): per (j, E, tau),
-  // realizations with L >= table_min_L read their neighbours from a table of
-  // the R nearest points of every query (R from table_row_length at the
-  // smallest such L).  A table is built only when the
+  // realizations from a smallest L on read their neighbours from a table of
+  // the R nearest points of every query (R from table_row_length at that L).
+  // The general rule takes L >= table_min_L and builds a table only when the
   // realizations that use it would otherwise scan at least 8*N_m library
-  // points in total (its build costs about N_m^2 distance evaluations), and
-  // while the plan's tables stay within table_cap_bytes; the realizations of
-  // a (j, E, tau) without a table use brute force.
-  std::map<std::tuple<int32_t, int32_t, int32_t>, std::pair<int64_t, int32_t>> table_of;
+  // points in total; for variables with one target, whose scan serves 32
+  // realizations a walk, cheapest_table_L may go lower.  The plan's tables stay
+  // within table_cap_bytes; the realizations of a (j, E, tau) without a table
+  // use brute force.
+  struct TableOf {
+    int64_t off, lmin;
+    int32_t stride;
+  };
+  std::map<std::tuple<int32_t, int32_t, int32_t>, TableOf> table_of;
   // The safety factor trades table memory and build time against how often a
   // query falls back to scanning its library.
   const TableTuning tt = read_table_tuning();
-  auto max_R_of = [&](int32_t j) { return pairs_of[j].size() == 1 ? kTableMaxR : kWalkMaxR; };
   const double safety = tt.safety;
   double table_bytes = 0.0;
   if (!(pc.flags & CCM_NO_TABLE)) {
@@ -405,25 +473,32 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         for (int32_t tau : pc.tau) {
           const int64_t n_m = pc.n - (int64_t)(E - 1) * tau;
           if (n_m > kTableMaxNm) continue;
-          const double ls = table_min_L(E, n_m, max_R_of(j), tt);
-          int64_t lmin = -1;
+          const bool tv = pairs_of[j].size() == 1;  // the target's values stand in the rows
+          const int max_R = tv ? kTableMaxR : kWalkMaxR;
+          const double ls = table_min_L(E, n_m, kWalkMaxR, tt);
+          int64_t base = -1;
           double lsum = 0.0;
           for (int64_t L : pc.L)
             if ((double)L >= ls) {
-              lmin = (lmin < 0) ? L : std::min(lmin, L);
+              base = (base < 0) ? L : std::min(base, L);
               lsum += (double)L * pc.r;
             }
-          if (lmin < 0 || lsum < 8.0 * (double)n_m) continue;
-          int64_t R = table_row_length(E, n_m, lmin, pc.theiler, safety);
-          // from the n_m - 1 points other than the query; rows are padded to 64
-          R = std::min<int64_t>(std::min<int64_t>((R + 31) / 32 * 32, max_R_of(j)), n_m - 1);
-          const int64_t stride = (R + 63) / 64 * 64;
-          // positions (2 or 4 bytes), distances, and for a variable with one
-          // target the target's values
-          const bool tv = pairs_of[j].size() == 1;
-          const double bytes =
-              (double)n_m * (double)stride * ((n_m < 65536 ? 2.0 : 4.0) + 4.0 + (tv ? 4.0 : 0.0));
-          if (table_bytes + bytes > table_cap_bytes) continue;
+          if (lsum < 8.0 * (double)n_m) base = -1;
+          int64_t lmin = base;
+          if (tv && !tt.fixed) lmin = cheapest_table_L(pc, E, n_m, base, max_R, safety);
+          int64_t R = 0, stride = 0;
+          double bytes = 0.0;
+          auto size = [&]() {  // positions (2 or 4 bytes), distances, values
+            R = table_row_entries(E, n_m, lmin, pc.theiler, safety, max_R);
+            stride = (R + 63) / 64 * 64;
+            bytes = (double)n_m * (double)stride * ((n_m < 65536 ? 2.0 : 4.0) + 4.0 + (tv ? 4.0 : 0.0));
+          };
+          if (lmin >= 0) size();
+          if (lmin != base && table_bytes + bytes > table_cap_bytes) {
+            lmin = base;  // too long for the cap: the general rule's
+            if (lmin >= 0) size();
+          }
+          if (lmin < 0 || table_bytes + bytes > table_cap_bytes) continue;
           table_bytes += bytes;
           TableJob tj;
           std::memset(&tj, 0, sizeof(tj));
@@ -446,7 +521,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           ul->points_total = (tj.sample_off + n_m / tj.sample * E + 63) / 64 * 64;
           tj.tv_i = tv ? pc.pairs[2 * pairs_of[j][0] + 1] : -1;
           if (tv) ul->table_tv = true;
-          table_of[std::make_tuple(j, E, tau)] = std::make_pair(tj.table_off, tj.stride);
+          table_of[std::make_tuple(j, E, tau)] = TableOf{tj.table_off, lmin, tj.stride};
           ul->table_total += n_m * stride;
           ul->tables.push_back(tj);
         }
@@ -457,10 +532,10 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
     for (int32_t E : pc.E)
       for (int32_t tau : pc.tau) {
         const int64_t n_m = pc.n - (int64_t)(E - 1) * tau;
-        const bool tab = table_of.count(std::make_tuple(j, E, tau)) != 0;
+        const auto tab = table_of.find(std::make_tuple(j, E, tau));
         int64_t tabled = 0;
         for (int64_t L : pc.L) {
-          if (!tab || (double)L < table_min_L(E, n_m, max_R_of(j), tt))
+          if (tab == table_of.end() || L < tab->second.lmin)
             brute_tiles[E] += (n_m + tileq - 1) / tileq * pc.r;
           else
             tabled += pc.r;
@@ -514,9 +589,9 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
               ul->targets.push_back(tg);
             }
             const auto tab = table_of.find(std::make_tuple(j, E, tau));
-            if (tab != table_of.end() && (double)L >= table_min_L(E, u.n_m, max_R_of(j), tt)) {
-              u.table_off = tab->second.first;
-              u.table_R = tab->second.second;
+            if (tab != table_of.end() && L >= tab->second.lmin) {
+              u.table_off = tab->second.off;
+              u.table_R = tab->second.stride;
               u.bits_off = ul->bits_total;
               ul->bits_total += (u.n_m + 31) / 32;
               ul->lib_scratch = std::max(ul->lib_scratch, L);
@@ -1189,17 +1264,27 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
   pl->ctx = ctx;
   ccm_status st = copy_problem(prob, &pl->pc);
   if (st != CCM_OK) return st;
-  append_units(pl->pc, 0, 0, &pl->ul, table_cap(ctx));
-  sort_items(&pl->ul);
   const int64_t series_elems = (int64_t)pl->pc.V * pl->pc.n;
-  pl->ar = layout(series_elems, pl->ul, pl->ul.n_rho, pl->ul.max_nm);
   CCM_CUDA(cudaSetDevice(ctx->device));
-  st = reserve(ctx, pl->ar.total);
-  if (st != CCM_OK) return st;
-  cudaError_t e = cudaMalloc(&pl->d_arena, pl->ar.total);
-  if (e != cudaSuccess) {
+  // where the plan does not fit, once more with smaller tables, then with none
+  cudaError_t e = cudaSuccess;
+  for (double cap : {table_cap(ctx), 0.1 * table_cap(ctx), 0.0}) {
+    pl->ul = UnitList();
+    append_units(pl->pc, 0, 0, &pl->ul, cap);
+    sort_items(&pl->ul);
+    pl->ar = layout(series_elems, pl->ul, pl->ul.n_rho, pl->ul.max_nm);
+    const bool last = pl->ul.tables.empty();
+    st = reserve(ctx, pl->ar.total);
+    if (st != CCM_OK) {
+      if (last) return st;
+      continue;
+    }
+    e = cudaMalloc(&pl->d_arena, pl->ar.total);
+    if (e == cudaSuccess) break;
+    pl->d_arena = nullptr;
     release(ctx, pl->ar.total);
-    return fail(CCM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    if (last) return fail(CCM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    (void)cudaGetLastError();  // reported by the next attempt if it fails too
   }
   e = cudaStreamCreateWithFlags(&pl->stream, cudaStreamNonBlocking);
   for (int q = 0; q < 5 && e == cudaSuccess; ++q) e = cudaEventCreate(&pl->ev[q]);
@@ -1514,6 +1599,7 @@ struct Job {
   int64_t n_units = 0;
   size_t footprint = 0;
   double pairs = 0.0;  // query-library pairs: the job's cost
+  double table_cap = 0.0;  // bytes its tables may take
   enum State { kQueued, kRunning, kDone, kFailed, kCancelled } state = kQueued;
   ccm_status status = CCM_PENDING;
   std::string err;
@@ -1535,11 +1621,19 @@ struct Batch {
 
 namespace {
 
-size_t job_footprint(const ccm_context* ctx, const ProblemCopy& pc, double* pairs) {
-  UnitList ul;
-  append_units(pc, 0, 0, &ul, table_cap(ctx));
-  *pairs = ul.pairs;
-  return layout((int64_t)pc.V * pc.n, ul, ul.n_rho, 0).total;
+// Device footprint of a job; where it exceeds the budget, with smaller tables,
+// then with none.
+size_t job_footprint(const ccm_context* ctx, const ProblemCopy& pc, double* pairs, double* cap) {
+  size_t total = 0;
+  for (double c : {table_cap(ctx), 0.1 * table_cap(ctx), 0.0}) {
+    UnitList ul;
+    append_units(pc, 0, 0, &ul, c);
+    *pairs = ul.pairs;
+    *cap = c;
+    total = layout((int64_t)pc.V * pc.n, ul, ul.n_rho, 0).total;
+    if (total <= ctx->budget || ul.tables.empty()) break;
+  }
+  return total;
 }
 
 void CUDART_CB on_batch_done(void* arg) {
@@ -1558,7 +1652,7 @@ void CUDART_CB on_batch_done(void* arg) {
 ccm_status launch_batch(ccm_context* ctx, Batch* b, bool inject) {
   int64_t series_elems = 0, out = 0;
   for (auto& j : b->jobs) {
-    append_units(j->pc, series_elems, out, &b->ul, table_cap(ctx));
+    append_units(j->pc, series_elems, out, &b->ul, j->table_cap);
     series_elems += (int64_t)j->pc.V * j->pc.n;
     out += j->n_units;
   }
@@ -1780,7 +1874,7 @@ ccm_status ccm_submit(ccm_context* ctx, const ccm_problem* prob, const float* se
   const size_t elems = (size_t)j->pc.V * (size_t)j->pc.n;
   if (!all_finite(series, elems)) return fail(CCM_EINVAL, "series holds a non-finite value");
   j->n_units = j->pc.n_units();
-  j->footprint = job_footprint(ctx, j->pc, &j->pairs);
+  j->footprint = job_footprint(ctx, j->pc, &j->pairs, &j->table_cap);
   if (j->footprint > ctx->budget)
     return fail(CCM_ETOOLARGE, "job footprint " + std::to_string(j->footprint) +
                                    " B exceeds the context budget");

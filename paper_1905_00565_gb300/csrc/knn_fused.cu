@@ -53,10 +53,9 @@ using u64 = unsigned long long;
 
 constexpr int kThreads = 256;             // threads per CTA = queries per tile
 static_assert(kQT == kThreads, "one query per thread");
-constexpr int kBuf = 20;                  // candidate keys per query (a column of the buffer)
-constexpr int kCoordBytes = 24 * 1024;    // shared memory for one library tile + chunk boxes
-constexpr int kBoxBytes = 4 * 1024;       // chunk bounding boxes, at the end of that region
-constexpr int kChunk = 16;                // library points per bounding box
+constexpr int kBuf = 22;                  // candidate keys per query (a column of the buffer)
+constexpr int kCoordBytes = kTileBytes;   // shared memory for one library tile
+constexpr int kChunk = 16;                // a tile is padded to whole chunks of points
 constexpr int kBufBytes = kBuf * kThreads * 8;
 // Predictions staged for their moments: kRing (tile, target) vectors, reduced
 // together, one warp each, when the ring is full.
@@ -84,15 +83,15 @@ constexpr int kStepE = (V == 1 && E <= 6) ? 8 : 4;
 template <int E, int V>
 constexpr int kE1 = (V == 1 && E >= 3) ? (E <= 6 ? 2 : 3) : E;
 
+constexpr int kBoxDims = 6;  // coordinates of a warp's query box, at most
+
 template <int E>
 struct TileShape {
   static constexpr int EP = E + (E & 1);                        // coordinates padded to even
-  static constexpr int D = E < 3 ? E : 3;                       // coordinates a chunk box bounds
+  static constexpr int D = E < 6 ? E : 6;                       // coordinates the pruning bounds
   // library points per tile: a point pair takes EP*8 bytes of coordinates + 8 of indices
   static constexpr int LT = brute_tile_points(E);
-  static_assert(kTileBytes == kCoordBytes - kBoxBytes, "the tile fills its region");
   static_assert(LT >= 64 && LT % 32 == 0, "tile must hold whole warps of chunks");
-  static_assert((LT / kChunk) * 2 * D * 4 <= kBoxBytes, "chunk boxes must fit");
 };
 
 __device__ __forceinline__ u64 pack2(float a, float b) {
@@ -406,60 +405,23 @@ __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& 
 }
 
 // Stage library points [t0, t0 + nt) of a unit's library (query order) into
-// shared memory: coordinates in packed pairs, indices, and the bounding box
-// of every kChunk consecutive points over the first D coordinates.  The tile
-// is padded to whole chunks with sentinel points (NaN coordinates, index
-// INT_MAX) that are never selected.  Block-wide; the caller brackets it with
-// barriers.  Sentinel coordinates are NaN: every distance to a sentinel is
-// NaN, which compares false against any threshold.
+// shared memory: coordinates in packed pairs, and indices.  The tile is padded
+// to whole chunks with sentinel points (NaN coordinates, index INT_MAX): every
+// distance to one is NaN, which compares false against any threshold.
+// Block-wide; the caller brackets it with barriers.
 template <int E>
 __device__ __noinline__ void stage_library(const float* sj, const int32_t* lib, int off, int tau,
-                                              int t0, int nt, u64* s_coord, int32_t* s_lidx,
-                                              float* s_box) {
+                                              int t0, int nt, u64* s_coord, int32_t* s_lidx) {
   constexpr int EP = TileShape<E>::EP;
-  constexpr int D = TileShape<E>::D;
-  const int tid = threadIdx.x;
   const int ntp = (nt + kChunk - 1) / kChunk * kChunk;
-  for (int a = tid; a < (ntp + 31) / 32 * 32; a += kThreads) {  // whole warps: the box shuffles
-    const int pp = a >> 1, half = a & 1;
-    float c0[D];
-    if (a < nt) {
-      const int l = lib[t0 + a];
-      s_lidx[a] = l;
-      float* cpair = reinterpret_cast<float*>(s_coord + (size_t)pp * EP);
+  for (int a = threadIdx.x; a < ntp; a += kThreads) {
+    float* cpair = reinterpret_cast<float*>(s_coord + (size_t)(a >> 1) * EP) + (a & 1);
+    const int l = a < nt ? lib[t0 + a] : INT_MAX;
+    s_lidx[a] = l;
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const float c = sj[l + off - e * tau];
-        cpair[2 * e + half] = c;
-        if (e < D) c0[e] = c;
-      }
-      if (EP > E) cpair[2 * E + half] = 0.f;
-    } else {
-      if (a < ntp) {  // sentinel point: never selected
-        s_lidx[a] = INT_MAX;
-        float* cpair = reinterpret_cast<float*>(s_coord + (size_t)pp * EP);
-#pragma unroll
-        for (int e = 0; e < E; ++e) cpair[2 * e + half] = __int_as_float(0x7fffffff);
-        if (EP > E) cpair[2 * E + half] = 0.f;
-      }
-#pragma unroll
-      for (int e = 0; e < D; ++e) c0[e] = __int_as_float(0x7fffffff);
-    }
-    // chunk boxes over the first D coordinates: one per half-warp (fminf and
-    // fmaxf skip the NaN of a sentinel; a chunk always holds a real point)
-#pragma unroll
-    for (int e = 0; e < D; ++e) {
-      float lo = c0[e], hi = c0[e];
-#pragma unroll
-      for (int o = kChunk / 2; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
-      }
-      if ((a & (kChunk - 1)) == 0 && a < ntp) {
-        s_box[(a / kChunk) * 2 * D + e] = lo;
-        s_box[(a / kChunk) * 2 * D + D + e] = hi;
-      }
-    }
+    for (int e = 0; e < E; ++e)
+      cpair[2 * e] = a < nt ? sj[l + off - e * tau] : __int_as_float(0x7fffffff);
+    if (EP > E) cpair[2 * E] = 0.f;
   }
 }
 
@@ -496,6 +458,35 @@ __device__ __forceinline__ void sort_column(u64* col, int n) {
   }
 }
 
+// Batcher's merge exchange for K keys in registers: the pairs it compares, in
+// order (Knuth, The Art of Computer Programming 5.2.2, algorithm M).
+template <int K>
+struct ExchangePairs {
+  int a[64], b[64], n;
+  constexpr ExchangePairs() : a(), b(), n(0) {
+    for (int p = 1; p < K; p *= 2)
+      for (int k = p; k >= 1; k /= 2)
+        for (int j = k % p; j + k < K; j += 2 * k)
+          for (int i = 0; i < k && i + j + k < K; ++i)
+            if ((i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+              a[n] = i + j;
+              b[n++] = i + j + k;
+            }
+  }
+};
+template <int K, int I = 0>
+__device__ __forceinline__ void sort_keys(u64 (&k)[K]) {
+  constexpr ExchangePairs<K> net;
+  if constexpr (I < net.n) {
+    constexpr int a = net.a[I], b = net.b[I];
+    const u64 x = k[a], y = k[b];
+    const bool swap = y < x;
+    k[a] = swap ? y : x;
+    k[b] = swap ? x : y;
+    sort_keys<K, I + 1>(k);
+  }
+}
+
 // Brute-force search of one work item: query tiles [tile0, tile0 + n_chunk)
 // of a unit.  When the whole library fits one shared-memory tile
 // it is staged once for all of them; each warp starts its scan at the library
@@ -517,26 +508,24 @@ __device__ __forceinline__ void sort_column(u64* col, int n) {
 // exactly the list the sorted insertion of every candidate would give.
 template <int E, int V, bool kLanes, bool kStats>
 __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, int n_chunk,
-                             unsigned char* smem, RingMeta* meta, int& ring_n) {
+                             unsigned char* smem, RingMeta* meta, float2* qbox, int& ring_n) {
   constexpr int K = E + 1;  // the window keeps m itself out, so E+1 slots suffice
   constexpr int EP = TileShape<E>::EP;
   constexpr int LT = TileShape<E>::LT;
   constexpr int D = TileShape<E>::D;
   const int n_m = u.n_m, L = u.L, tau = u.tau, W = u.theiler;
   const bool single = L <= LT;
-  // Shared-memory layout: library indices [LT], chunk boxes [LT/kChunk][2D],
-  // coordinates [LT/2][EP] in the first kCoordBytes, then the candidate
-  // buffer [kBuf][kThreads].  A library that fits one tile takes only the
+  // Shared-memory layout: library indices [LT], coordinates [LT/2][EP] in the
+  // first kCoordBytes, then the candidate buffer [kBuf][kThreads].  A library that fits one tile takes only the
   // coordinate rows it needs, and the buffer starts right after them, so its
   // columns reach up to the prediction ring: wider columns need fewer
   // compactions.
   int32_t* s_lidx = reinterpret_cast<int32_t*>(smem);
-  float* s_box = reinterpret_cast<float*>(smem + (size_t)LT * 4);
-  u64* s_coord = reinterpret_cast<u64*>(smem + (size_t)LT * 4 + kBoxBytes);
+  u64* s_coord = reinterpret_cast<u64*>(smem + (size_t)LT * 4);
   size_t buf_off = kCoordBytes;
   if (single) {
     const int ntp = (L + kChunk - 1) / kChunk * kChunk;
-    buf_off = (size_t)LT * 4 + kBoxBytes + (size_t)(ntp / 2) * EP * 8;
+    buf_off = (size_t)LT * 4 + (size_t)(ntp / 2) * EP * 8;
   }
   u64* s_buf = reinterpret_cast<u64*>(smem + buf_off);
   const int cap = (int)((kCoordBytes + kBufBytes - buf_off) / (kThreads * 8));  // >= kBuf
@@ -560,7 +549,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
   const int tile1 = min(u.n_tiles, tile0 + n_chunk);
   if (single) {
     __syncthreads();  // the previous item's readers of the tile are done
-    stage_library<E>(sj, lib, off, tau, 0, L, s_coord, s_lidx, s_box);
+    stage_library<E>(sj, lib, off, tau, 0, L, s_coord, s_lidx);
     __syncthreads();
   }
   // A warp's 32 queries are consecutive positions of the query order.  For
@@ -585,8 +574,8 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
     u64 qc[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) qc[e] = pack2(c_nx[e], c_nx[e]);
-    // Bounding box of the warp's queries over the first D coordinates.
-    float qlo[D], qhi[D];
+    // Bounding box of the warp's queries over the first D coordinates (in shared
+    // memory: the registers are the search's).
 #pragma unroll
     for (int e = 0; e < D; ++e) {
       float lo = c_nx[e], hi = lo;
@@ -595,9 +584,9 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
         lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
         hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
       }
-      qlo[e] = lo;
-      qhi[e] = hi;
+      if (lane == 0) qbox[warp * kBoxDims + e] = make_float2(lo, hi);
     }
+    __syncwarp();
     // the library position nearest this warp's queries (in query order)
     const int aw = library_position(L, tile * kQT + warp * 32, n_m);
 
@@ -649,15 +638,12 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
       }
     };
 
-    // Scan the staged points [0, nt) from position `base` (a chunk start),
-    // wrapping around; `first`: the scan's first kInit points fill tl.
-    // Scan the staged points [0, nt) chunk by chunk from the chunk at `base`,
-    // wrapping around; `first`: the scan's first kInit points fill tl.
+    // Scan the staged points [0, nt), 32 pairs of points at a time from the
+    // pairs around position `base` (a chunk start) on, wrapping around;
+    // `first`: the kInit points at `base` fill tl.
     auto scan = [&](int nt, int base, bool first) {
-      const int ntp = (nt + kChunk - 1) / kChunk * kChunk;
-      const int nch = ntp / kChunk;
-      const int c0 = base / kChunk;
-      constexpr int kSteps = kChunk / kStep;  // steps per chunk
+      const int np = (nt + kChunk - 1) / kChunk * (kChunk / 2);
+      const int ng = (np + 31) >> 5;
       if (first) {
 #pragma unroll
         for (int pp = 0; pp < kInit / 2; ++pp) {
@@ -681,79 +667,84 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
         if (__any_sync(kFull, cnt > room)) make_room();
       }
 #pragma unroll 1
-      for (int jc = 0; jc < nch; ++jc) {
-        int c = c0 + jc;
-        c -= (c >= nch) ? nch : 0;
-        const int s0 = (first && jc == 0) ? kInit / kStep : 0;  // steps the fill took
-        if (s0 == 0) {
-          // Chunk pruning.  gap_e = max(0, lo_e - qhi_e, qlo_e - hi_e) bounds
-          // |q_e - x_e| from below for every query q of the warp and point x of
-          // the chunk, in FP32 too (rounding is monotone); summed in the
-          // distance's own order over the first D coordinates it bounds every
-          // FP32 squared distance between them from below.  A chunk whose bound
-          // exceeds every lane's threshold holds no candidate.
-          const float* bx = s_box + c * 2 * D;
+      for (int jg = 0; jg < ng; ++jg) {
+        int g = (base >> 6) + jg;
+        g -= (g >= ng) ? ng : 0;
+        // Pruning, a lane per pair.  gap_e = max(0, lo_e - qhi_e, qlo_e - hi_e)
+        // bounds |q_e - x_e| from below for every query q of the warp and both
+        // points x of the pair, in FP32 too (rounding is monotone); summed in the
+        // distance's own order over the first D coordinates it bounds their FP32
+        // squared distances from below.  A pair whose bound exceeds every lane's
+        // threshold holds no candidate.
+        const float th_max = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(tl[K - 1])));
+        const int pr = 32 * g + lane;
+        bool keep = pr < np && !(first && (unsigned)(pr - (base >> 1)) < (unsigned)(kInit / 2));
+        if (keep) {
+          const float2* xp = reinterpret_cast<const float2*>(s_coord + (size_t)pr * EP);
           float lb = 0.f;
 #pragma unroll
           for (int e = 0; e < D; ++e) {
-            const float g = fmaxf(fmaxf(__fsub_rn(bx[e], qhi[e]), __fsub_rn(qlo[e], bx[D + e])), 0.f);
-            lb = (e == 0) ? __fmul_rn(g, g) : __fmaf_rn(g, g, lb);
+            const float2 x = xp[e], qb = qbox[warp * kBoxDims + e];
+            const float gp = fmaxf(fmaxf(__fsub_rn(fminf(x.x, x.y), qb.y),
+                                         __fsub_rn(qb.x, fmaxf(x.x, x.y))), 0.f);
+            lb = (e == 0) ? __fmul_rn(gp, gp) : __fmaf_rn(gp, gp, lb);
           }
-          const float th_max = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(tl[K - 1])));
-          if (lb > th_max) {
-            if (kStats) st_pruned += kChunk;
-            continue;
-          }
+          keep = !(lb > th_max);
         }
-        // two steps a chunk (kStep 8) unrolled; four (kStep 4, the larger E)
-        // kept as a loop: unrolled they outgrow the instruction cache
-#pragma unroll(kSteps <= 2 ? kSteps : 1)
-        for (int sp = s0; sp < kSteps; ++sp) {
-          const int a = c * kChunk + sp * kStep;
-          if (kStats) st_begun += kStep;
-          const u64* cp = s_coord + (size_t)(a >> 1) * EP;
+        unsigned mask = __ballot_sync(kFull, keep);
+        if (kStats) st_pruned += 2u * (min(32, np - 32 * g) - __popc(mask)) -
+                                 (first && (base >> 6) == g ? (unsigned)kInit : 0u);
+        while (mask != 0u) {
+          // the next kPairs pairs (fewer at the end: the first again, not taken)
+          int at[kPairs];
+          int have = 0;
+#pragma unroll
+          for (int pp = 0; pp < kPairs; ++pp) {
+            at[pp] = mask != 0u ? 32 * g + __ffs(mask) - 1 : at[0];
+            have += mask != 0u ? 1 : 0;
+            mask &= mask - 1u;
+          }
+          if (kStats) st_begun += 2u * have;
           // Partial sums over the first E1 coordinates are lower bounds of the
           // full FP32 sums (all terms are >= 0 and rounding is monotone), so a
           // step whose partials are all above every lane's threshold cannot
           // contribute a candidate and skips the remaining coordinates.
           u64 r[kPairs];
 #pragma unroll
-          for (int pp = 0; pp < kPairs; ++pp) r[pp] = sqdist2_range<E, 0, (kE1<E, V>)>(qc, cp + pp * EP, 0ull);
+          for (int pp = 0; pp < kPairs; ++pp)
+            r[pp] = sqdist2_range<E, 0, (kE1<E, V>)>(qc, s_coord + (size_t)at[pp] * EP, 0ull);
           const float th = tl[K - 1];
           float d[kStep];
 #pragma unroll
           for (int pp = 0; pp < kPairs; ++pp) unpack2(r[pp], d[2 * pp], d[2 * pp + 1]);
-          if (kStats && (kE1<E, V>) == E) st_full += kStep;
+          if (kStats && (kE1<E, V>) == E) st_full += 2u * have;
           if (!__any_sync(kFull, min_all(d) <= th)) continue;
           if constexpr ((kE1<E, V>) < E) {
-            if (kStats) st_full += kStep;
+            if (kStats) st_full += 2u * have;
 #pragma unroll
             for (int pp = 0; pp < kPairs; ++pp) {
-              r[pp] = sqdist2_range<E, (kE1<E, V>), E>(qc, cp + pp * EP, r[pp]);
+              r[pp] = sqdist2_range<E, (kE1<E, V>), E>(qc, s_coord + (size_t)at[pp] * EP, r[pp]);
               unpack2(r[pp], d[2 * pp], d[2 * pp + 1]);
             }
             if (!__any_sync(kFull, min_all(d) <= th)) continue;
           }
-          // the step's library indices (one broadcast 16-byte load per four)
-          int li[kStep];
 #pragma unroll
-          for (int q4 = 0; q4 < kStep / 4; ++q4) {
-            const int4 v = *reinterpret_cast<const int4*>(s_lidx + a + 4 * q4);
-            li[4 * q4] = v.x;
-            li[4 * q4 + 1] = v.y;
-            li[4 * q4 + 2] = v.z;
-            li[4 * q4 + 3] = v.w;
-          }
+          for (int pp = 0; pp < kPairs; ++pp) {
+            if (pp >= have) break;  // the same for the whole warp
+            const int2 li = *reinterpret_cast<const int2*>(s_lidx + 2 * at[pp]);
 #pragma unroll
-          for (int pt = 0; pt < kStep; ++pt) {
-            // at or below the threshold (never a sentinel: NaN), outside the
-            // exclusion window |l - m| <= W (W = 0 drops only m itself, and
-            // the unsigned form tests both sides at once); appended without a
-            // branch
-            const bool take = (d[pt] <= th) &
-                              ((unsigned)li[pt] - (unsigned)m + (unsigned)W > 2u * (unsigned)W);
-            if (take) col[cnt * kThreads] = pack_key(d[pt], li[pt]);
-            cnt += take ? 1 : 0;
+            for (int h = 0; h < 2; ++h) {
+              // at or below the threshold (never a sentinel: NaN), outside the
+              // exclusion window |l - m| <= W (W = 0 drops only m itself, and
+              // the unsigned form tests both sides at once); appended without a
+              // branch
+              const int l = h ? li.y : li.x;
+              const float dh = d[2 * pp + h];
+              const bool take =
+                  (dh <= th) & ((unsigned)l - (unsigned)m + (unsigned)W > 2u * (unsigned)W);
+              if (take) col[cnt * kThreads] = pack_key(dh, l);
+              cnt += take ? 1 : 0;
+            }
           }
           if (__any_sync(kFull, cnt - done >= merge_at || cnt > room)) make_room();
         }
@@ -772,7 +763,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
       const int t0 = ti * LT, nt = min(LT, L - t0);
       if (!single) {
         __syncthreads();  // the previous library tile has been consumed
-        stage_library<E>(sj, lib, off, tau, t0, nt, s_coord, s_lidx, s_box);
+        stage_library<E>(sj, lib, off, tau, t0, nt, s_coord, s_lidx);
         __syncthreads();
       }
       const int local = aw - t0;
@@ -781,7 +772,18 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
     }
     update();
     compact();
-    sort_column(col, cnt);  // the first K keys: the E+1 nearest, in (distance, index) order
+    // the E+1 nearest in (distance, index) order: K keys are left unless some
+    // tie with the threshold (or the input is not finite)
+    u64 ku[K];
+    if (__all_sync(kFull, cnt == K)) {
+#pragma unroll
+      for (int s = 0; s < K; ++s) ku[s] = col[s * kThreads];
+      sort_keys<K>(ku);
+    } else {
+      sort_column(col, cnt);
+#pragma unroll
+      for (int s = 0; s < K; ++s) ku[s] = col[s * kThreads];
+    }
     if (kStats) {
       const uint32_t cand = __reduce_add_sync(kFull, st_cand);
       const unsigned vq = __popc(__ballot_sync(kFull, valid));
@@ -803,15 +805,11 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
     int nb[E + 1];
 #pragma unroll
     for (int s = 0; s <= E; ++s) {
-      const u64 k = col[s * kThreads];
-      dd[s] = key_dist(k);
-      nb[s] = key_index(k);
+      dd[s] = key_dist(ku[s]);
+      nb[s] = key_index(ku[s]);
     }
     if (kPrefetch && tile + 1 < tile1) load_query(tile + 1);
     finish_tile<E, kLanes, true>(p, u, tile, m, valid, dd, nb, s_ring, meta, ring_n, s_buf);
-    // the next tile's search starts behind a barrier (this also keeps the
-    // search's registers free of spills)
-    __syncthreads();
   }
 }
 
@@ -1030,6 +1028,7 @@ template <int E, bool kLanes, bool kStats>
 __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
+  __shared__ float2 s_qbox[kThreads / 32 * kBoxDims];
   __shared__ RingMeta s_meta[kRing];
   int ring_n = 0;  // staged prediction vectors (the same in every thread)
   for (int64_t round = 0;; ++round) {
@@ -1047,9 +1046,9 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
       continue;
     }
     if (p.variant[E] == 1)
-      process_item<E, 1, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, ring_n);
+      process_item<E, 1, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, s_qbox, ring_n);
     else
-      process_item<E, 0, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, ring_n);
+      process_item<E, 0, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, s_qbox, ring_n);
   }
   if (ring_n > 0)
     flush_ring(reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);

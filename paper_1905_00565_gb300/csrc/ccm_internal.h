@@ -270,6 +270,17 @@ __device__ __forceinline__ float simplex_u(float d2, float d1, float inv_d1, flo
   return simplex_u_dist(sqrt_hw(d2), d1, inv_d1, wfloor);
 }
 
+// Where a launch goes.  chained: its CTAs may be set up while the kernel before
+// it on the stream drains (launch.cuh).  Only for the direct launches of one
+// job: inside a captured graph the gaps are short anyway (175 against 170 us for
+// a single job), and set-up CTAs hold resources that other streams' kernels
+// could use (a served burst: 7.3 against 7.0 ms).
+struct LaunchStream {
+  cudaStream_t s;
+  bool chained;
+  LaunchStream(cudaStream_t stream, bool chain = false) : s(stream), chained(chain) {}
+};
+
 // Error flag values written by kernels.
 constexpr int32_t kErrBadUnit = 1;
 constexpr int32_t kErrSampler = 2;
@@ -280,10 +291,10 @@ constexpr int kSamplerThreads = 256;
 constexpr int kSamplerBitsMax = 1 << 20;  // membership bits in shared memory up to this N_m
 cudaError_t sampler_prepare();
 cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t count,
-                           int max_nm, cudaStream_t s);
+                           int max_nm, LaunchStream s);
 // Membership words of the scan groups from their units' bits.
 cudaError_t launch_member_words(const UnitDesc* units, const MemberGroup* groups, int64_t n_groups,
-                                int max_nm, const uint32_t* bits, uint32_t* words, cudaStream_t s);
+                                int max_nm, const uint32_t* bits, uint32_t* words, LaunchStream s);
 
 // Query order (order.cu).
 cudaError_t order_prepare();
@@ -291,20 +302,20 @@ cudaError_t order_prepare();
 // The same launch prepares the target series (SeriesJob).
 cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jobs, int max_nm,
                          int32_t* order, int32_t* inverse, unsigned long long* scratch,
-                         const SeriesJob* series_jobs, int64_t n_series_jobs, float* scales, float* st, cudaStream_t s);
+                         const SeriesJob* series_jobs, int64_t n_series_jobs, float* scales, float* st, LaunchStream s);
 
 // Distance indexing table (table.cu).
 cudaError_t table_prepare();
 // The jobs' points and boxes (all jobs of a run).
 cudaError_t launch_table_points(const float* series, const TableJob* jobs, int64_t n_jobs,
-                                int max_nm, const int32_t* order, float* points, cudaStream_t s);
+                                int max_nm, const int32_t* order, float* points, LaunchStream s);
 // One launch builds the tables of jobs[0..n_jobs), all of embedding dimension E
 // (n_rows rows together).
 cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_t n_jobs,
                                int64_t n_rows, int E, int max_nm, int max_R, const float* points,
                                const int32_t* order, const int32_t* inverse, void* table,
                                float* table_dist, int table_pairs, int table_u16, int32_t* err,
-                               cudaStream_t s);
+                               LaunchStream s);
 // Its kernels (table_build.cu, compiled once per E).
 template <int E>
 struct TableKernels {
@@ -312,7 +323,7 @@ struct TableKernels {
   static cudaError_t launch(const float* series, const TableJob* jobs, int64_t n_jobs,
                             int64_t n_rows, int max_nm, int max_R, const float* points,
                             const int32_t* order, const int32_t* inverse, void* table,
-                            float* table_dist, int pairs, int u16, int32_t* err, cudaStream_t s);
+                            float* table_dist, int pairs, int u16, int32_t* err, LaunchStream s);
 };
 
 // Search kernels of one E (knn_fused.cu, compiled once per E; each kernel keeps
@@ -321,13 +332,13 @@ template <int E>
 struct KnnKernels {
   static cudaError_t prepare();
   static cudaError_t occupancy(int* ctas);
-  static cudaError_t launch(const KnnParams& p, bool lanes, int grid, cudaStream_t s);
+  static cudaError_t launch(const KnnParams& p, bool lanes, int grid, LaunchStream s);
   static cudaError_t prepare_table();
   static cudaError_t occupancy_table(int max_nm, bool lanes, int* ctas);
   static cudaError_t launch_table(const KnnParams& p, int max_nm, bool lanes, int grid,
-                                  cudaStream_t s);
+                                  LaunchStream s);
   static cudaError_t prepare_scan();
-  static cudaError_t launch_scan(const KnnParams& p, int max_nm, int grid, cudaStream_t s);
+  static cudaError_t launch_scan(const KnnParams& p, int max_nm, int grid, LaunchStream s);
 };
 
 // Their dispatch, and what surrounds the search (knn_dispatch.cu).
@@ -337,24 +348,24 @@ cudaError_t knn_prepare();
 cudaError_t knn_occupancy(int E, int* ctas_per_sm);
 // lane_targets: the launch's units have kLaneTargets targets or more (a kernel
 // of their own).
-cudaError_t launch_knn(const KnnParams& p, int E, bool lane_targets, int grid, cudaStream_t s);
+cudaError_t launch_knn(const KnnParams& p, int E, bool lane_targets, int grid, LaunchStream s);
 // Observed-value records of every ObsJob (after the query order): one warp
 // per tile, n_tiles tiles in all.
 cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* jobs,
                        int64_t n_jobs, int64_t n_tiles, const float* scales, float2* obs,
-                       ObsStat* obs_stat, cudaStream_t s);
+                       ObsStat* obs_stat, LaunchStream s);
 // rho of every target from its tiles' sums (after the search kernels).
 cudaError_t launch_rho(const UnitDesc* units, const TargetDesc* targets, int64_t n_targets,
                        const float4* partials, const ObsStat* obs_stat, double* rho,
-                       cudaStream_t s);
+                       LaunchStream s);
 // Table path: same work items, neighbours read from the distance indexing table.
 cudaError_t knn_table_prepare();
 cudaError_t knn_table_occupancy(int max_nm, bool lane_targets, int* ctas_per_sm);
 cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lane_targets, int grid,
-                             cudaStream_t s);
+                             LaunchStream s);
 // Units with one target: grouped realizations (two CTAs per SM).
 cudaError_t knn_scan_prepare();
-cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, cudaStream_t s);
+cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, LaunchStream s);
 
 // Sets the thread-local message returned by ccm_last_error() (runtime.cu).
 void set_last_error(const char* msg);

@@ -1,11 +1,15 @@
 // Observed-value records, rho and the dispatch of the search kernels by E.
 #include "ccm_internal.h"
+#include "launch.cuh"
 #include "moments.cuh"
 
 namespace ccm {
 namespace {
 
 constexpr int kThreads = 256;
+// CTAs of the FP64 kernels: one warp, so that few targets spread over the SMs (a
+// warp's FP64 instruction takes 16 cycles of its SM's pipe).
+constexpr int kSmallThreads = 32;
 constexpr unsigned kFull = 0xffffffffu;
 
 // Butterfly sum over the warp: every lane ends with the same bits (each
@@ -21,10 +25,11 @@ constexpr int kPer = kQT / 32;  // queries per lane
 // Observed-value records (see ObsJob), one warp per tile: x_q is the target
 // at the tile's manifold points (Sect. 2.1: the value the cross map
 // predicts).  Two passes in FP64, then split into float pairs.
-__global__ void __launch_bounds__(kThreads) obs_kernel(const float* series, const int32_t* order,
+__global__ void __launch_bounds__(kSmallThreads) obs_kernel(const float* series, const int32_t* order,
                                                       const ObsJob* jobs, int64_t n_jobs,
                                                       int64_t n_tiles, const float* scales,
                                                       float2* obs, ObsStat* obs_stat) {
+  chain_begin();
   const int lane = threadIdx.x & 31;
   const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n_tiles;
@@ -75,65 +80,122 @@ __global__ void __launch_bounds__(kThreads) obs_kernel(const float* series, cons
 // rho of one target: the tile moments merged.  With the grand means MX =
 // sum(n_t mx_t)/N, the centred sums are exactly
 //   Sxx = sum_t [Sxx_t + n_t (mx_t - MX)^2]   (likewise Syy, Sxy),
-// a sum of non-negative terms (no cancellation).  kRhoLanes lanes per target
-// take every kRhoLanes-th tile and are added in a fixed order, so rho does not
-// depend on which CTA ran which tile, or when.  A launch of its own: FP64
-// instructions cost the same for one lane as for 32, and merging inside the
-// search kernels kept whole warps on it (and a fence and a counter per tile).
+// a sum of non-negative terms (no cancellation).  kRhoLanes lanes (a whole warp
+// for targets of more than kRhoNarrow tiles) take every so-many-th tile and are
+// added in a fixed order, so rho does not depend on which CTA ran which tile, or
+// when.  A launch of its own: FP64 instructions cost the same for one lane as
+// for 32, and merging inside the search kernels kept whole warps on it (and a
+// fence and a counter per tile).  Bound: the FP64 pipe for many targets, the
+// loads' latency for few (four tiles' loads are in flight per lane).
 constexpr int kRhoLanes = 4;
+constexpr int kRhoNarrow = 96;
+
+template <int kLanes>
 __device__ __forceinline__ double rho_sum(double v) {
 #pragma unroll
-  for (int o = 1; o < kRhoLanes; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(kFull, v, o));
+  for (int o = 1; o < kLanes; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(kFull, v, o));
   return v;
 }
-__global__ void __launch_bounds__(kThreads) rho_kernel(const UnitDesc* units,
+
+// rho of a target by kLanes lanes (lane `sub` of them); `active` false: the
+// lanes only take part in the shuffles.
+template <int kLanes>
+__device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4* base,
+                                             const ObsStat* stat, int sub, bool active) {
+  constexpr int kAhead = 4;
+  struct Tile {
+    float4 a, b;
+    double mx, sxx;
+  };
+  auto load = [&](int q0, Tile (&t)[kAhead]) {
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int q = q0 + i * kLanes;
+      if (q < n_tiles) {
+        t[i].a = __ldg(base + 2 * q);
+        t[i].b = __ldg(base + 2 * q + 1);
+        t[i].mx = __ldg(&stat[q].mx);
+        t[i].sxx = __ldg(&stat[q].sxx);
+      }
+    }
+  };
+  auto count = [&](int q) { return (double)min(kQT, n_m - q * kQT); };
+  // mean(y) of a tile; d = mean(y) - c, b1 = sum(y - c)
+  auto mean = [&](const Tile& t, double n, double& b1, double& d) {
+    b1 = __dadd_rn((double)t.a.y, (double)t.a.z);
+    d = (n == (double)kQT) ? __dmul_rn(b1, 1.0 / kQT) : __ddiv_rn(b1, n);
+    return __dadd_rn((double)t.a.x, d);
+  };
+  Tile t[kAhead];
+  double SX = 0.0, SY = 0.0, b1, d;
+  for (int q0 = sub; active && q0 < n_tiles; q0 += kAhead * kLanes) {
+    load(q0, t);
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int q = q0 + i * kLanes;
+      if (q >= n_tiles) break;
+      const double n = count(q);
+      SX = __fma_rn(n, t[i].mx, SX);
+      SY = __fma_rn(n, mean(t[i], n, b1, d), SY);
+    }
+  }
+  const double inv = (double)n_m;
+  const double MX = __ddiv_rn(rho_sum<kLanes>(SX), inv), MY = __ddiv_rn(rho_sum<kLanes>(SY), inv);
+  double SXX = 0.0, SYY = 0.0, SXY = 0.0;
+  for (int q0 = sub; active && q0 < n_tiles; q0 += kAhead * kLanes) {
+    if (n_tiles > kAhead * kLanes) load(q0, t);  // else still there
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int q = q0 + i * kLanes;
+      if (q >= n_tiles) break;
+      const double n = count(q);
+      const double dy = __dsub_rn(mean(t[i], n, b1, d), MY), dx = __dsub_rn(t[i].mx, MX);
+      const double b2 = __dadd_rn((double)t[i].a.w, (double)t[i].b.x);
+      const double syy = fmax(__fma_rn(-b1, d, b2), 0.0);
+      const double sxy = __dadd_rn((double)t[i].b.y, (double)t[i].b.z);
+      const double wx = __dmul_rn(n, dx);
+      SXX = __fma_rn(wx, dx, __dadd_rn(SXX, t[i].sxx));
+      SYY = __fma_rn(__dmul_rn(n, dy), dy, __dadd_rn(SYY, syy));
+      SXY = __fma_rn(wx, dy, __dadd_rn(SXY, sxy));
+    }
+  }
+  SXX = rho_sum<kLanes>(SXX);
+  SYY = rho_sum<kLanes>(SYY);
+  SXY = rho_sum<kLanes>(SXY);
+  return (SXX > 0.0 && SYY > 0.0) ? __ddiv_rn(SXY, __dsqrt_rn(__dmul_rn(SXX, SYY))) : nan("");
+}
+
+__global__ void __launch_bounds__(kSmallThreads) rho_kernel(const UnitDesc* units,
                                                       const TargetDesc* targets,
                                                       int64_t n_targets, const float4* partials,
                                                       const ObsStat* obs_stat, double* rho) {
-  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kRhoLanes;
-  const int sub = threadIdx.x & (kRhoLanes - 1);
-  const TargetDesc tg = targets[g < n_targets ? g : n_targets - 1];  // whole warps shuffle
-  const UnitDesc& u = units[tg.unit];
-  const int n_tiles = u.n_tiles, n_m = u.n_m;
-  const int64_t t = (g < n_targets ? g : n_targets - 1) - u.tgt_off;
-  const float4* base = partials + 2 * (u.part_off + t * n_tiles);
-  const ObsStat* stat = obs_stat + tg.obs_tile;
-  auto count = [&](int q) { return (double)min(kQT, n_m - q * kQT); };
-  // mean(y) - c and Syy, Sxy of tile q
-  auto tile = [&](int q, double n, double& my, double& syy, double& sxy) {
-    const float4 a = __ldg(base + 2 * q), b = __ldg(base + 2 * q + 1);
-    const double b1 = __dadd_rn((double)a.y, (double)a.z);
-    const double b2 = __dadd_rn((double)a.w, (double)b.x);
-    const double d = (n == (double)kQT) ? __dmul_rn(b1, 1.0 / kQT) : __ddiv_rn(b1, n);
-    my = __dadd_rn((double)a.x, d);
-    syy = fmax(__fma_rn(-b1, d, b2), 0.0);
-    sxy = __dadd_rn((double)b.y, (double)b.z);
+  chain_begin();
+  const int lane = threadIdx.x & 31, sub = lane & (kRhoLanes - 1);
+  const int64_t first = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane) / kRhoLanes;
+  const int64_t g = first + lane / kRhoLanes;  // this lane's target
+  const int64_t at = g < n_targets ? g : n_targets - 1;  // whole warps shuffle
+  auto of = [&](int64_t i, TargetDesc& tg, int& n_tiles, int& n_m) {
+    tg = targets[i];
+    const UnitDesc& u = units[tg.unit];
+    n_tiles = u.n_tiles;
+    n_m = u.n_m;
+    return partials + 2 * (u.part_off + (i - u.tgt_off) * n_tiles);
   };
-  double SX = 0.0, SY = 0.0, my, syy, sxy;
-  for (int q = sub; q < n_tiles; q += kRhoLanes) {
-    const double n = count(q);
-    tile(q, n, my, syy, sxy);
-    SX = __fma_rn(n, stat[q].mx, SX);
-    SY = __fma_rn(n, my, SY);
+  TargetDesc tg;
+  int n_tiles, n_m;
+  const float4* base = of(at, tg, n_tiles, n_m);
+  const bool narrow = n_tiles <= kRhoNarrow;
+  if (__any_sync(kFull, narrow)) {
+    const double r = target_rho<kRhoLanes>(n_tiles, n_m, base, obs_stat + tg.obs_tile, sub, narrow);
+    if (narrow && sub == 0 && g < n_targets) rho[tg.out_idx] = r;
   }
-  const double inv = (double)n_m;
-  const double MX = __ddiv_rn(rho_sum(SX), inv), MY = __ddiv_rn(rho_sum(SY), inv);
-  double SXX = 0.0, SYY = 0.0, SXY = 0.0;
-  for (int q = sub; q < n_tiles; q += kRhoLanes) {
-    const double n = count(q);
-    tile(q, n, my, syy, sxy);
-    const double dx = __dsub_rn(stat[q].mx, MX), dy = __dsub_rn(my, MY);
-    const double wx = __dmul_rn(n, dx);
-    SXX = __fma_rn(wx, dx, __dadd_rn(SXX, stat[q].sxx));
-    SYY = __fma_rn(__dmul_rn(n, dy), dy, __dadd_rn(SYY, syy));
-    SXY = __fma_rn(wx, dy, __dadd_rn(SXY, sxy));
+  if (__all_sync(kFull, narrow)) return;
+  for (int i = 0; i < 32 / kRhoLanes && first + i < n_targets; ++i) {
+    base = of(first + i, tg, n_tiles, n_m);
+    if (n_tiles <= kRhoNarrow) continue;  // the same for the whole warp
+    const double r = target_rho<32>(n_tiles, n_m, base, obs_stat + tg.obs_tile, lane, true);
+    if (lane == 0) rho[tg.out_idx] = r;
   }
-  SXX = rho_sum(SXX);
-  SYY = rho_sum(SYY);
-  SXY = rho_sum(SXY);
-  if (sub == 0 && g < n_targets)
-    rho[tg.out_idx] = (SXX > 0.0 && SYY > 0.0) ? __ddiv_rn(SXY, __dsqrt_rn(__dmul_rn(SXX, SYY)))
-                                               : nan("");
 }
 
 }  // namespace
@@ -169,7 +231,7 @@ cudaError_t knn_scan_prepare() {
   CCM_FOR_E(CCM_CASE_PREPARE_SCAN)
   return cudaSuccess;
 }
-cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, cudaStream_t s) {
+cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, LaunchStream s) {
   switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH_SCAN) }
   return cudaErrorInvalidValue;
 }
@@ -177,7 +239,7 @@ cudaError_t knn_occupancy(int E, int* ctas) {
   switch (E) { CCM_FOR_E(CCM_CASE_OCCUPANCY) }
   return cudaErrorInvalidValue;
 }
-cudaError_t launch_knn(const KnnParams& p, int E, bool lanes, int grid, cudaStream_t s) {
+cudaError_t launch_knn(const KnnParams& p, int E, bool lanes, int grid, LaunchStream s) {
   switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH) }
   return cudaErrorInvalidValue;
 }
@@ -185,30 +247,28 @@ cudaError_t knn_table_occupancy(int max_nm, bool lanes, int* ctas) {
   return KnnKernels<kMaxE>::occupancy_table(max_nm, lanes, ctas);
 }
 cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lanes, int grid,
-                             cudaStream_t s) {
+                             LaunchStream s) {
   switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH_TABLE) }
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* jobs,
                        int64_t n_jobs, int64_t n_tiles, const float* scales, float2* obs,
-                       ObsStat* obs_stat, cudaStream_t s) {
+                       ObsStat* obs_stat, LaunchStream s) {
   if (n_jobs <= 0 || n_tiles <= 0) return cudaSuccess;
-  const int64_t want = (n_tiles + kThreads / 32 - 1) / (kThreads / 32);  // a warp per tile
-  const int64_t blocks = want < 65536 ? want : 65536;
-  obs_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(series, order, jobs, n_jobs, n_tiles, scales,
-                                                   obs, obs_stat);
-  return cudaGetLastError();
+  const int64_t want = (n_tiles + kSmallThreads / 32 - 1) / (kSmallThreads / 32);  // a warp per tile
+  const int64_t blocks = want < (1 << 20) ? want : 1 << 20;
+  return launch_chained(obs_kernel, dim3((unsigned)blocks), kSmallThreads, 0, s, series, order, jobs,
+                        n_jobs, n_tiles, scales, obs, obs_stat);
 }
 
 cudaError_t launch_rho(const UnitDesc* units, const TargetDesc* targets, int64_t n_targets,
                        const float4* partials, const ObsStat* obs_stat, double* rho,
-                       cudaStream_t s) {
+                       LaunchStream s) {
   if (n_targets <= 0) return cudaSuccess;
-  const int64_t blocks = (n_targets * kRhoLanes + kThreads - 1) / kThreads;
-  rho_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(units, targets, n_targets, partials, obs_stat,
-                                                   rho);
-  return cudaGetLastError();
+  const int64_t blocks = (n_targets * kRhoLanes + kSmallThreads - 1) / kSmallThreads;
+  return launch_chained(rho_kernel, dim3((unsigned)blocks), kSmallThreads, 0, s, units, targets,
+                        n_targets, partials, obs_stat, rho);
 }
 
 }  // namespace ccm

@@ -44,6 +44,7 @@
 #include <initializer_list>
 
 #include "ccm_internal.h"
+#include "launch.cuh"
 #include "moments.cuh"
 
 namespace ccm {
@@ -1005,6 +1006,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams
   __shared__ int s_item;
   __shared__ RingMeta s_meta[kRing];
   int ring_n = 0;  // staged prediction vectors (the same in every thread)
+  chain_begin();
   for (int64_t round = 0;; ++round) {
     if (p.persistent) {
       if (threadIdx.x == 0) s_item = (int)atomicAdd(p.item_counter, 1u);
@@ -1031,6 +1033,7 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
   __shared__ float2 s_qbox[kThreads / 32 * kBoxDims];
   __shared__ RingMeta s_meta[kRing];
   int ring_n = 0;  // staged prediction vectors (the same in every thread)
+  chain_begin();
   for (int64_t round = 0;; ++round) {
     if (p.persistent) {
       if (threadIdx.x == 0) s_item = (int)atomicAdd(p.item_counter, 1u);
@@ -1068,11 +1071,10 @@ size_t table_smem(int max_nm, bool lane_targets) {
 
 // The kernels of one E, in a translation unit of their own (CCM_E).
 template <int E>
-cudaError_t KnnKernels<E>::launch(const KnnParams& p, bool lanes, int grid, cudaStream_t s) {
+cudaError_t KnnKernels<E>::launch(const KnnParams& p, bool lanes, int grid, LaunchStream s) {
   const auto fn = lanes ? (p.stats ? knn_fused_kernel<E, true, true> : knn_fused_kernel<E, true, false>)
                         : (p.stats ? knn_fused_kernel<E, false, true> : knn_fused_kernel<E, false, false>);
-  fn<<<grid, kThreads, kSmemBytes, s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(fn, dim3((unsigned)grid), kThreads, kSmemBytes, s, p);
 }
 
 template <int E>
@@ -1100,11 +1102,11 @@ static auto table_kernel(bool lanes, bool stats) {
 
 template <int E>
 cudaError_t KnnKernels<E>::launch_table(const KnnParams& params, int max_nm, bool lanes, int grid,
-                                        cudaStream_t s) {
+                                        LaunchStream s) {
   KnnParams p = params;
   p.lane_scratch = (int32_t)table_base_smem(max_nm);
-  table_kernel<E>(lanes, p.stats != nullptr)<<<grid, kThreads, table_smem(max_nm, lanes), s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(table_kernel<E>(lanes, p.stats != nullptr), dim3((unsigned)grid), kThreads,
+                        table_smem(max_nm, lanes), s, p);
 }
 
 template <int E>

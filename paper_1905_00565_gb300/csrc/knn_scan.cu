@@ -32,6 +32,7 @@
 
 #include "bits.cuh"
 #include "ccm_internal.h"
+#include "launch.cuh"
 #include "moments.cuh"
 
 namespace ccm {
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
   uint16_t* s_step = reinterpret_cast<uint16_t*>(s_mask + K * kScanThreads); // [K][kScanThreads]
   uint32_t* s_words = reinterpret_cast<uint32_t*>(s_step + K * kScanThreads);
   const BitTranspose tr(lane);
+  chain_begin();
   for (int round = 0;; ++round) {
     if (p.persistent && tid == 0) s_item = (int)atomicAdd(p.item_counter, 1u);
     __syncthreads();
@@ -381,11 +383,11 @@ auto scan_variant(int max_nm, bool u16, bool general) {
 }  // namespace
 
 template <int E>
-cudaError_t KnnKernels<E>::launch_scan(const KnnParams& p, int max_nm, int grid, cudaStream_t s) {
+cudaError_t KnnKernels<E>::launch_scan(const KnnParams& p, int max_nm, int grid, LaunchStream s) {
   const bool general = p.window || p.stats || p.dbg_nbr || p.dbg_xhat;
   const bool sm = p.table_u16 && words_in_smem<E>(max_nm);
-  scan_variant<E>(max_nm, p.table_u16 != 0, general)<<<grid, kScanThreads, scan_smem<E>(max_nm, sm), s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(scan_variant<E>(max_nm, p.table_u16 != 0, general), dim3((unsigned)grid),
+                        kScanThreads, scan_smem<E>(max_nm, sm), s, p);
 }
 
 template <int E>

@@ -27,6 +27,7 @@
 
 #include "ccm.h"
 #include "ccm_internal.h"
+#include "launch.cuh"
 
 namespace ccm {
 
@@ -89,6 +90,7 @@ struct CellArgs {
 // Writes the descriptors and work items of the cell into the scratch and
 // clears the counters and the error flag.
 __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, CellArgs c) {
+  chain_begin();
   UnitDesc* units = reinterpret_cast<UnitDesc*>(scratch + lay.units);
   WorkItem* items = reinterpret_cast<WorkItem*>(scratch + lay.items);
   const int64_t per_unit = (c.n_tiles + c.chunk - 1) / c.chunk;  // items per realization
@@ -239,17 +241,20 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   c.n_m = (int32_t)n_m;
   c.n_tiles = (int32_t)n_tiles;
   c.chunk = brute_chunk(r * n_tiles, L, E);
-  noalloc_setup_kernel<<<(unsigned)((r * n_tiles + 255) / 256), 256, 0, s>>>(scratch, lay, c);
+  const LaunchStream chain(s, true);
+  e = launch_chained(noalloc_setup_kernel, dim3((unsigned)((r * n_tiles + 255) / 256)), 256, 0, chain,
+                     scratch, lay, c);
+  if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));
   e = launch_order(d_series, reinterpret_cast<const OrderJob*>(scratch + lay.orderjob), 1,
                    (int)n_m, reinterpret_cast<int32_t*>(scratch + lay.order), nullptr, nullptr,
                    reinterpret_cast<const SeriesJob*>(scratch + lay.seriesjob), 1,
-                   reinterpret_cast<float*>(scratch + lay.scale), nullptr, s);
+                   reinterpret_cast<float*>(scratch + lay.scale), nullptr, chain);
   if (e == cudaSuccess)
     e = launch_obs(d_series, reinterpret_cast<const int32_t*>(scratch + lay.order),
                    reinterpret_cast<const ObsJob*>(scratch + lay.obsjob), 1, n_tiles,
                    reinterpret_cast<const float*>(scratch + lay.scale),
                    reinterpret_cast<float2*>(scratch + lay.obs),
-                   reinterpret_cast<ObsStat*>(scratch + lay.obs_stat), s);
+                   reinterpret_cast<ObsStat*>(scratch + lay.obs_stat), chain);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));
   SamplerParams sp{};
   sp.units = reinterpret_cast<const UnitDesc*>(scratch + lay.units);
@@ -257,7 +262,7 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   sp.order = reinterpret_cast<const int32_t*>(scratch + lay.order);
   sp.lib = reinterpret_cast<int32_t*>(scratch + lay.lib);
   sp.err = reinterpret_cast<int32_t*>(scratch + lay.err);
-  e = launch_sampler(sp, 0, r, (int)n_m, s);
+  e = launch_sampler(sp, 0, r, (int)n_m, chain);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));
   KnnParams kp{};
   kp.series = d_series;
@@ -277,9 +282,9 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
     kp.merge_at[q] = kDefaultMergeAt;
     kp.variant[q] = kDefaultVariant;
   }
-  e = launch_knn(kp, E, false, (int)kp.n_items, s);
+  e = launch_knn(kp, E, false, (int)kp.n_items, chain);
   if (e == cudaSuccess)
-    e = launch_rho(kp.units, kp.targets, r, kp.partials, kp.obs_stat, d_rho, s);
+    e = launch_rho(kp.units, kp.targets, r, kp.partials, kp.obs_stat, d_rho, chain);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));
   if (!cuda_stream) {
     int32_t err = 0;

@@ -959,7 +959,7 @@ KnnParams knn_params(char* base, const Arena& ar, const UnitList& ul, int persis
 }
 
 // Query order and target series, then the observed-value records.
-cudaError_t enqueue_order(char* base, const Arena& ar, const UnitList& ul, cudaStream_t s) {
+cudaError_t enqueue_order(char* base, const Arena& ar, const UnitList& ul, LaunchStream s) {
   float* scales = reinterpret_cast<float*>(base + ar.scales);
   const cudaError_t e =
       launch_order(reinterpret_cast<const float*>(base + ar.series),
@@ -987,6 +987,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
                          int32_t* dbg_nbr, float* dbg_xhat, cudaStream_t s,
                          cudaEvent_t* ev = nullptr, bool capturing = false,
                          bool stats = false) {
+  const LaunchStream ls(s, persistent && !capturing);
   // Inside stream capture an event record becomes a graph node only with the
   // external flag; outside capture the plain record is the valid form.
   auto record = [&](cudaEvent_t e) {
@@ -997,13 +998,13 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   CCM_CUDA(cudaMemsetAsync(base + ar.counter, 0, kMaxSearchLaunches * sizeof(uint32_t), s));
   if (stats) CCM_CUDA(cudaMemsetAsync(base + ar.stats, 0, sizeof(unsigned long long) * kStatCount, s));
   if (ev) CCM_CUDA(record(ev[0]));
-  CCM_CUDA(enqueue_order(base, ar, ul, s));
+  CCM_CUDA(enqueue_order(base, ar, ul, ls));
   if (!ul.tables.empty())
     CCM_CUDA(launch_table_points(reinterpret_cast<const float*>(base + ar.series),
                                  reinterpret_cast<const TableJob*>(base + ar.tables),
                                  (int64_t)ul.tables.size(), ul.max_nm,
                                  reinterpret_cast<const int32_t*>(base + ar.order),
-                                 reinterpret_cast<float*>(base + ar.points), s));
+                                 reinterpret_cast<float*>(base + ar.points), ls));
   for (size_t g0 = 0; g0 < ul.tables.size();) {  // one launch per (size class, E)
     const int rc = UnitList::table_rcap(ul.tables[g0].R), te = ul.tables[g0].E;
     size_t g1 = g0;
@@ -1024,18 +1025,18 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
                                 reinterpret_cast<const int32_t*>(base + ar.inverse),
                                 base + ar.table, reinterpret_cast<float*>(base + ar.table_dist),
                                 ul.table_tv ? 1 : 0, ul.table_u16(),
-                                reinterpret_cast<int32_t*>(base + ar.err), s));
+                                reinterpret_cast<int32_t*>(base + ar.err), ls));
     g0 = g1;
   }
   if (ev) CCM_CUDA(record(ev[1]));
   SamplerParams sp = sampler_params(base, ar);
   sp.dbg_lib = dbg_lib;
-  CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, s));
+  CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, ls));
   if (!ul.member_groups.empty())
     CCM_CUDA(launch_member_words(reinterpret_cast<const UnitDesc*>(base + ar.units),
                                  reinterpret_cast<const MemberGroup*>(base + ar.member_groups),
                                  (int64_t)ul.member_groups.size(), ul.max_nm, sp.bits,
-                                 reinterpret_cast<uint32_t*>(base + ar.words), s));
+                                 reinterpret_cast<uint32_t*>(base + ar.words), ls));
   if (ev) CCM_CUDA(record(ev[2]));
   KnnParams kp = knn_params(base, ar, ul, persistent, tn);
   kp.dbg_nbr = dbg_nbr;
@@ -1051,7 +1052,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     ke.n_items = ig.count;
     ke.item_counter = counter++;
     const int g = persistent ? grid : (int)std::min<int64_t>(ig.count, 0x7fffffff);
-    CCM_CUDA(launch_knn(ke, ig.E, ig.targets == Targets::kMany, g, s));
+    CCM_CUDA(launch_knn(ke, ig.E, ig.targets == Targets::kMany, g, ls));
   }
   if (ev) CCM_CUDA(record(ev[3]));
   for (const ItemGroup& ig : ul.groups_table) {
@@ -1061,12 +1062,12 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     kt.item_counter = counter++;
     const int g = persistent ? grid_table : (int)std::min<int64_t>(ig.count, 0x7fffffff);
     if (ig.targets == Targets::kOne)
-      CCM_CUDA(launch_knn_scan(kt, ig.E, ul.max_nm, persistent ? grid_scan : g, s));
+      CCM_CUDA(launch_knn_scan(kt, ig.E, ul.max_nm, persistent ? grid_scan : g, ls));
     else
-      CCM_CUDA(launch_knn_table(kt, ig.E, ul.max_nm, ig.targets == Targets::kMany, g, s));
+      CCM_CUDA(launch_knn_table(kt, ig.E, ul.max_nm, ig.targets == Targets::kMany, g, ls));
   }
   CCM_CUDA(launch_rho(kp.units, kp.targets, (int64_t)ul.targets.size(), kp.partials, kp.obs_stat,
-                      reinterpret_cast<double*>(base + ar.rho), s));
+                      reinterpret_cast<double*>(base + ar.rho), ls));
   if (ev) CCM_CUDA(record(ev[4]));
   return CCM_OK;
 }

@@ -32,6 +32,7 @@
 
 #include "bits.cuh"
 #include "ccm_internal.h"
+#include "launch.cuh"
 
 namespace ccm {
 namespace {
@@ -223,6 +224,7 @@ sampler_kernel(SamplerParams p, int64_t first_unit) {
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_below, s_listed, s_rank, s_bin, s_in_bin, s_total;
 
+  chain_begin();
   const int64_t uidx = first_unit + blockIdx.x;
   const UnitDesc u = p.units[uidx];
   const int n_m = u.n_m, L = u.L;
@@ -404,13 +406,15 @@ cudaError_t sampler_prepare() {
 }
 
 cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t count, int max_nm,
-                           cudaStream_t s) {
+                           LaunchStream s) {
   const size_t smem = (size_t)((std::min(max_nm, kSamplerBitsMax) + 31) / 32) * 4;
   for (int64_t off = 0; off < count; off += 0x7fffffff) {
     const unsigned grid = (unsigned)std::min<int64_t>(count - off, 0x7fffffff);
-    sampler_kernel<<<grid, kSamplerThreads, smem, s>>>(p, first_unit + off);
+    const cudaError_t e =
+        launch_chained(sampler_kernel, dim3(grid), kSamplerThreads, smem, s, p, first_unit + off);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 // Membership words of the scan's realization groups: word pos of a group holds
@@ -421,6 +425,7 @@ cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t c
 __global__ void __launch_bounds__(256) member_words_kernel(const UnitDesc* units,
                                                           const MemberGroup* groups,
                                                           const uint32_t* bits, uint32_t* words) {
+  chain_begin();
   const MemberGroup g = groups[blockIdx.y];
   const UnitDesc& u = units[g.unit];
   const int n_m = u.n_m, per_unit = (n_m + 31) >> 5;
@@ -438,13 +443,15 @@ __global__ void __launch_bounds__(256) member_words_kernel(const UnitDesc* units
 }
 
 cudaError_t launch_member_words(const UnitDesc* units, const MemberGroup* groups, int64_t n_groups,
-                                int max_nm, const uint32_t* bits, uint32_t* words, cudaStream_t s) {
+                                int max_nm, const uint32_t* bits, uint32_t* words, LaunchStream s) {
   const unsigned gx = (unsigned)((member_words(max_nm) / 32 + 63) / 64);
   for (int64_t off = 0; off < n_groups; off += 65535) {
     const dim3 grid(gx, (unsigned)std::min<int64_t>(n_groups - off, 65535));
-    member_words_kernel<<<grid, 256, 0, s>>>(units, groups + off, bits, words);
+    const cudaError_t e =
+        launch_chained(member_words_kernel, grid, 256, 0, s, units, groups + off, bits, words);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace ccm

@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "ccm_internal.h"
+#include "launch.cuh"
 
 namespace ccm {
 namespace {
@@ -18,6 +19,7 @@ __global__ void __launch_bounds__(kPointThreads)
 table_points_kernel(const float* series, const TableJob* jobs, const int32_t* order,
                     float* points) {
   __shared__ float s_lo[32], s_hi[32];
+  chain_begin();
   const TableJob jb = jobs[blockIdx.y];
   const int n_m = jb.n_m, E = jb.E, tau = jb.tau, off = (E - 1) * tau;
   const int n_chunks = (n_m + 31) >> 5, n_super = (n_chunks + 31) >> 5;
@@ -67,13 +69,15 @@ table_points_kernel(const float* series, const TableJob* jobs, const int32_t* or
 }  // namespace
 
 cudaError_t launch_table_points(const float* series, const TableJob* jobs, int64_t n_jobs,
-                                int max_nm, const int32_t* order, float* points, cudaStream_t s) {
+                                int max_nm, const int32_t* order, float* points, LaunchStream s) {
   for (int64_t at = 0; at < n_jobs; at += 65535) {
     const dim3 grid((unsigned)((max_nm + 1023) / 1024),
                     (unsigned)(n_jobs - at < 65535 ? n_jobs - at : 65535));
-    table_points_kernel<<<grid, kPointThreads, 0, s>>>(series, jobs + at, order, points);
+    const cudaError_t e =
+        launch_chained(table_points_kernel, grid, kPointThreads, 0, s, series, jobs + at, order, points);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 #define CCM_FOR_E(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10)
@@ -93,7 +97,7 @@ cudaError_t launch_table_build(const float* series, const TableJob* jobs, int64_
                                int64_t n_rows, int E, int max_nm, int max_R, const float* points,
                                const int32_t* order, const int32_t* inverse, void* table,
                                float* table_dist, int table_pairs, int table_u16, int32_t* err,
-                               cudaStream_t s) {
+                               LaunchStream s) {
   if (n_jobs <= 0) return cudaSuccess;
   if (max_R > kTableMaxR) return cudaErrorInvalidValue;
   switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH) }

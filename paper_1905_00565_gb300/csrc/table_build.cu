@@ -53,6 +53,7 @@
 #include <stdint.h>
 
 #include "ccm_internal.h"
+#include "launch.cuh"
 
 namespace ccm {
 namespace {
@@ -88,6 +89,7 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
   __shared__ uint32_t s_scan[kThreads / 32], s_top, s_found, s_crowd;
   __shared__ int s_supers, s_chunks, s_count, s_equal;
   constexpr int kWarps = kThreads / 32;
+  chain_begin();
   const TableJob jb = jobs[blockIdx.y];
   const int n_m = jb.n_m, R = jb.R, C = capacity(R);
   const int row0 = blockIdx.x * rows_per_cta;
@@ -471,22 +473,17 @@ cudaError_t TableKernels<E>::launch(const float* series, const TableJob* jobs, i
                                     int64_t n_rows, int max_nm, int max_R, const float* points,
                                     const int32_t* order, const int32_t* inverse, void* table,
                                     float* table_dist, int pairs, int u16, int32_t* err,
-                                    cudaStream_t s) {
+                                    LaunchStream s) {
   // consecutive rows share a CTA (and the threshold) once there are more rows
   // than fill the SMs twice
   const int64_t rows = n_rows / (2 * 152 * 8);
   const int per = (int)(rows < 1 ? 1 : rows > 32 ? 32 : rows);
   const size_t smem = build_smem(max_R, max_nm);
   const dim3 grid((unsigned)((max_nm + per - 1) / per), (unsigned)n_jobs);
-  if (max_R <= 1024)
-    table_build_kernel<E, 128><<<grid, 128, smem, s>>>(series, jobs, points, order, inverse, table,
-                                                       table_dist, pairs, u16, per, capacity(max_R),
-                                                       err);
-  else
-    table_build_kernel<E, 256><<<grid, 256, smem, s>>>(series, jobs, points, order, inverse, table,
-                                                       table_dist, pairs, u16, per, capacity(max_R),
-                                                       err);
-  return cudaGetLastError();
+  const int threads = max_R <= 1024 ? 128 : 256;
+  return launch_chained(threads == 128 ? table_build_kernel<E, 128> : table_build_kernel<E, 256>, grid,
+                        threads, smem, s, series, jobs, points, order, inverse, table, table_dist,
+                        pairs, u16, per, capacity(max_R), err);
 }
 
 template struct TableKernels<CCM_E>;

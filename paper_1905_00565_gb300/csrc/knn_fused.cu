@@ -84,12 +84,12 @@ constexpr int kStepE = (V == 1 && E <= 6) ? 8 : 4;
 template <int E, int V>
 constexpr int kE1 = (V == 1 && E >= 3) ? (E <= 6 ? 2 : 3) : E;
 
-constexpr int kBoxDims = 6;  // coordinates of a warp's query box, at most
+constexpr int kBoxDims = 8;  // coordinates of a warp's query box, at most
 
 template <int E>
 struct TileShape {
   static constexpr int EP = E + (E & 1);                        // coordinates padded to even
-  static constexpr int D = E < 6 ? E : 6;                       // coordinates the pruning bounds
+  static constexpr int D = E < kBoxDims ? E : kBoxDims;         // coordinates the pruning bounds
   // library points per tile: a point pair takes EP*8 bytes of coordinates + 8 of indices
   static constexpr int LT = brute_tile_points(E);
   static_assert(LT >= 64 && LT % 32 == 0, "tile must hold whole warps of chunks");

@@ -6,9 +6,13 @@
 // order.  The order changes which tile a query belongs to and nothing else:
 // every query's neighbours and prediction are the same in any order.
 //
-// Key: Morton interleave of the first min(E, 3) coordinates, each quantised to
-// 30/D bits over the series' [min, max]; ties (and the key's low half) by the
-// manifold index m, so the order is a deterministic function of the series.
+// Key: Morton interleave of all E coordinates, each quantised to floor(30/E) bits
+// over the series' [min, max]; ties (and the key's low half) by the manifold
+// index m, so the order is a deterministic function of the series.  With the
+// first three coordinates only, neighbours in the order could lie apart in the
+// others: rows of E = 10 tables (N = 10^4) then compare 234 of 313 chunks
+// instead of 117, and a warp's brute-force queries at E = 6 meet 49 of 150
+// library points instead of 12.
 // One CTA per (variable, E, tau) sorts in shared memory when N_m <=
 // kOrderMaxSort (a radix sort of the codes, a bitonic network for the shortest);
 // a longer manifold is sorted by one CTA too: runs of kOrderMaxSort points, then
@@ -24,23 +28,6 @@ namespace ccm {
 namespace {
 
 constexpr int kOrderThreads = 1024;
-
-__device__ __forceinline__ uint32_t spread3(uint32_t x) {  // 10 bits -> every 3rd bit
-  x &= 0x3ffu;
-  x = (x | (x << 16)) & 0x030000ffu;
-  x = (x | (x << 8)) & 0x0300f00fu;
-  x = (x | (x << 4)) & 0x030c30c3u;
-  x = (x | (x << 2)) & 0x09249249u;
-  return x;
-}
-__device__ __forceinline__ uint32_t spread2(uint32_t x) {  // 15 bits -> every 2nd bit
-  x &= 0x7fffu;
-  x = (x | (x << 8)) & 0x00ff00ffu;
-  x = (x | (x << 4)) & 0x0f0f0f0fu;
-  x = (x | (x << 2)) & 0x33333333u;
-  x = (x | (x << 1)) & 0x55555555u;
-  return x;
-}
 
 __device__ __forceinline__ uint32_t quantise(float c, float lo, float inv, int bits) {
   const float u = (c - lo) * inv;  // in [0, 1] up to rounding
@@ -78,20 +65,15 @@ __device__ void series_range(const float* s, int64_t n, float* lo_out, float* hi
   *hi_out = hi;
 }
 
-// Sort key of manifold point q: (Morton code << 32) | q.
+// Sort key of manifold point q: (Morton code << 32) | q.  The code interleaves
+// the top 30/E bits of every coordinate, the newest first.
 __device__ __forceinline__ unsigned long long morton_key(const float* s, int off, int tau, int E,
                                                          float lo, float inv, int q) {
-  const int t = q + off;
-  const int D = min(E, 3);
-  uint32_t code;
-  if (D == 1) {
-    code = quantise(s[t], lo, inv, 30);
-  } else if (D == 2) {
-    code = (spread2(quantise(s[t], lo, inv, 15)) << 1) | spread2(quantise(s[t - tau], lo, inv, 15));
-  } else {
-    code = (spread3(quantise(s[t], lo, inv, 10)) << 2) |
-           (spread3(quantise(s[t - tau], lo, inv, 10)) << 1) |
-           spread3(quantise(s[t - 2 * tau], lo, inv, 10));
+  const int t = q + off, bits = 30 / E;
+  uint32_t code = 0u;
+  for (int e = 0; e < E; ++e) {
+    const uint32_t c = quantise(s[t - e * tau], lo, inv, bits);
+    for (int b = 0; b < bits; ++b) code |= ((c >> b) & 1u) << (b * E + E - 1 - e);
   }
   return ((unsigned long long)code << 32) | (unsigned)q;
 }

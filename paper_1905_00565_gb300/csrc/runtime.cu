@@ -262,10 +262,13 @@ double table_min_L(int32_t E, int64_t n_m, int max_R, const TableTuning& t) {
 // than E+1 it scans its whole library instead, about lmin distance
 // evaluations.  lambda is the smallest multiple of 1/4 for which that happens
 // with probability at most 1/(10*lmin), so the misses cost at most about 0.1
-// distance evaluations a query (times the safety factor s on lambda); 2W more
-// entries cover the points the exclusion window removes.
+// distance evaluations a query (times the safety factor s on lambda), and from
+// lmin = 300 on still more rarely in proportion: there a miss's scan lasts longer
+// than the tile that waits for it (two variables of N = 10^5: rows 5 % longer,
+// scan 36 -> 29 ms).  2W more entries cover the points the exclusion window
+// removes.
 int64_t table_row_length(int32_t E, int64_t n_m, int64_t lmin, int32_t theiler, double safety) {
-  const double eps = 1.0 / (10.0 * (double)lmin);
+  const double eps = 1.0 / (10.0 * (double)lmin * std::max(1.0, (double)lmin / 300.0));
   double lambda = (double)(E + 1);
   for (;; lambda += 0.25) {
     double term = std::exp(-lambda), tail = term;  // P(X <= E), X ~ Poisson(lambda)
@@ -644,7 +647,9 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         // Scan groups: consecutive units of this (j, E, tau) that read the table,
         // whatever their L (the lanes of a partly filled group would idle; the
         // walk of a mixed one is as long as its smallest L's).
-        int64_t slots = scan_tiles[E] / (4 * 2 * 152);
+        // Tiles per item: one copy of the membership words (about 4 % of a tile's
+        // time) against the balance of eight items per CTA slot.
+        const int64_t slots = scan_tiles[E] / (8 * 2 * 152);
         const int32_t chunk = (int32_t)std::min<int64_t>(std::max<int64_t>(slots, 1), kScanChunk);
         for (size_t a = first_unit; a < ul->units.size();) {
           if (ul->units[a].table_R == 0) {

@@ -19,15 +19,18 @@
 // 8-bit radix select over four passes recomputes the keys.
 //
 // Bound: issue (the 64-bit multiplies of Philox are half of the instructions)
-// and the latency between its barriers.  Sweep of 4*10^5 libraries of N_m =
-// 10^4: 17.9 ms with the scan's membership words (keys stored and four radix
-// passes over them: 20.0 ms); 10^4 libraries of N_m = 10^5: 3.9 ms (keys
-// recomputed in every pass: 26.4 ms).
+// and, for short manifolds, the latency between its barriers: five CTAs per SM
+// (48 registers; the listed keys sized by N_m) hide more of it than three.
+// Sweep of 4*10^5 libraries of N_m = 10^4: 13.9 ms with the scan's membership
+// words (keys stored and four radix passes over them: 20.0 ms); 27000 of N_m =
+// 4000: 0.52 ms (0.63); 10^4 of N_m = 10^5: 2.9 ms (26.4).
 //
 // Output: realizations that read a distance indexing table get one bit per
 // position of the query order; the others their library as a list in query
 // order, the order the neighbour search visits it in (spatially coherent
 // runs).  The checking copy is compacted in ascending m.
+#include <limits.h>
+
 #include <algorithm>
 
 #include "bits.cuh"
@@ -213,13 +216,20 @@ __device__ __noinline__ unsigned long long select_by_radix(const UnitDesc& u, Se
   return ((unsigned long long)hstar << 32) | sc.prefix;
 }
 
-constexpr int kWindow = 2048;  // keys listed around the L-th smallest
+// Keys listed around the L-th smallest, at most: ten standard deviations of the
+// rank (at most sqrt(n)/2) and as many again as they may spread.
+__host__ __device__ constexpr int window_keys(int n) {
+  int root = 1;
+  while ((int64_t)root * root < n) root <<= 1;  // sqrt(n) to twice it
+  return root * 6 + 96 < 8192 ? root * 6 + 96 : 8192;
+}
 constexpr int kBinKeys = 64;   // of them, keys of the bin that holds it
 
-__global__ void __launch_bounds__(kSamplerThreads)
-sampler_kernel(SamplerParams p, int64_t first_unit) {
-  extern __shared__ __align__(16) uint32_t s_bits[];  // bit m: point m is a member
-  __shared__ unsigned long long s_win[kWindow], s_bin_keys[kBinKeys], s_last;
+__global__ void __launch_bounds__(kSamplerThreads, 5)
+sampler_kernel(SamplerParams p, int64_t first_unit, int window) {
+  extern __shared__ __align__(16) unsigned long long s_win[];  // listed keys, then
+  __shared__ unsigned long long s_bin_keys[kBinKeys], s_last;
+  uint32_t* s_bits = reinterpret_cast<uint32_t*>(s_win + window);  // bit m: point m is a member
   __shared__ SelectScratch s_sel;
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_below, s_listed, s_rank, s_bin, s_in_bin, s_total;
@@ -265,7 +275,7 @@ sampler_kernel(SamplerParams p, int64_t first_unit) {
       if (h < lo) byte |= 1u << i;
       if (h - lo <= hi - lo && 8 * b + i < n_m) {
         const uint32_t at = atomicAdd(&s_listed, 1u);
-        if (at < (uint32_t)kWindow) s_win[at] = ((unsigned long long)h << 32) | (uint32_t)(8 * b + i);
+        if (at < (uint32_t)window) s_win[at] = ((unsigned long long)h << 32) | (uint32_t)(8 * b + i);
       }
     }
     if (8 * b + 8 > n_m) byte &= (1u << (n_m - 8 * b)) - 1u;
@@ -278,7 +288,7 @@ sampler_kernel(SamplerParams p, int64_t first_unit) {
   const uint32_t listed = s_listed, sum_below = s_below;
   // members among the listed keys; 0 and all of them need no search
   const uint32_t want = (uint32_t)L - sum_below;
-  bool found = (uint32_t)L >= sum_below && listed <= (uint32_t)kWindow && want <= listed;
+  bool found = (uint32_t)L >= sum_below && listed <= (uint32_t)window && want <= listed;
   if (found && want > 0u && want < listed) {
     // bins of equal width over the window: the one holding the last member,
     // then its rank among that bin's keys
@@ -402,16 +412,17 @@ sampler_kernel(SamplerParams p, int64_t first_unit) {
 
 cudaError_t sampler_prepare() {
   return cudaFuncSetAttribute(sampler_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kSamplerBitsMax / 8);
+                              kSamplerBitsMax / 8 + window_keys(INT_MAX) * 8);
 }
 
 cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t count, int max_nm,
                            LaunchStream s) {
-  const size_t smem = (size_t)((std::min(max_nm, kSamplerBitsMax) + 31) / 32) * 4;
+  const int window = window_keys(max_nm);
+  const size_t smem = (size_t)window * 8 + (size_t)((std::min(max_nm, kSamplerBitsMax) + 31) / 32) * 4;
   for (int64_t off = 0; off < count; off += 0x7fffffff) {
     const unsigned grid = (unsigned)std::min<int64_t>(count - off, 0x7fffffff);
     const cudaError_t e =
-        launch_chained(sampler_kernel, dim3(grid), kSamplerThreads, smem, s, p, first_unit + off);
+        launch_chained(sampler_kernel, dim3(grid), kSamplerThreads, smem, s, p, first_unit + off, window);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -95,30 +95,6 @@ struct TileShape {
   static_assert(LT >= 64 && LT % 32 == 0, "tile must hold whole warps of chunks");
 };
 
-__device__ __forceinline__ u64 pack2(float a, float b) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(u64 v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ u64 sub2(u64 a, u64 b) {
-  u64 r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-  u64 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-  u64 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // Squared distances of one query (coordinates duplicated, {q_e, q_e}) to a
 // pair of library points whose coordinates are packed {a_e, b_e} starting at
 // `c` (16-byte aligned, EP entries): {d2(q, a), d2(q, b)}, accumulated over
@@ -256,23 +232,33 @@ __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc&
     };
     const float c = __fmul_rn(predict(0), scale);
     const float2* a = obs + t;
+    // two groups of eight queries side by side (packed), then the next two
     TileSums part[4];
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      part[g] = zero_sums();
-      const int qa = q0 + kMomentGroup * g;
-      if (qa + kMomentGroup <= q1 && p.dbg_xhat == nullptr) {
-#pragma unroll 4
+    for (int g = 0; g < 4; g += 2) {
+      const int qa = q0 + kMomentGroup * g, qb = qa + kMomentGroup;
+      if (qb + kMomentGroup <= q1 && p.dbg_xhat == nullptr) {
+        const packed cc = pack2(c, c), ss = pack2(scale, scale);
+        TileSums2 both = zero_sums2();
+#pragma unroll 2
         for (int i = 0; i < kMomentGroup; ++i)
-          add_query(part[g], __fmul_rn(predict(qa + i), scale), __ldg(a + (int64_t)(qa + i) * T), c);
+          add_query2(both, mul2(pack2(predict(qa + i), predict(qb + i)), ss),
+                     __ldg(a + (int64_t)(qa + i) * T), __ldg(a + (int64_t)(qb + i) * T), cc);
+        unpack_sums(both, part[g], part[g + 1]);
       } else {
-        for (int q = qa; q < min(qa + kMomentGroup, q1); ++q) {
-          const float y = predict(q);
-          if (p.dbg_xhat && tc + lane < T) p.dbg_xhat[tg.q_off + order[q]] = y;
-          add_query(part[g], __fmul_rn(y, scale), __ldg(a + (int64_t)q * T), c);
+        for (int h = 0; h < 2; ++h) {
+          TileSums one = zero_sums();
+          const int qh = qa + kMomentGroup * h;
+          for (int q = qh; q < min(qh + kMomentGroup, q1); ++q) {
+            const float y = predict(q);
+            if (p.dbg_xhat && tc + lane < T) p.dbg_xhat[tg.q_off + order[q]] = y;
+            add_query(one, __fmul_rn(y, scale), __ldg(a + (int64_t)q * T), c);
+          }
+          if (h == 0) part[g] = one;
+          else part[g + 1] = one;
         }
       }
-      if (g == 1) part[0] = merge_sums(part[0], part[1]);
+      if (g == 0) part[0] = merge_sums(part[0], part[1]);
     }
     part[0] = merge_sums(part[0], merge_sums(part[2], part[3]));
     // [turn & 1][value][warp][lane]

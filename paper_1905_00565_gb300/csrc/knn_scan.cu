@@ -335,17 +335,17 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
         const float* ys = s_vec + vec * kScanVec;
         const float2* a = p.obs + rec * kQT;
         const float c0 = ys[0];
-        TileSums half[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          half[h] = zero_sums();
+        const packed cc = pack2(c0, c0);
+        TileSums2 both = zero_sums2();
 #pragma unroll 4
-          for (int i = 0; i < kMomentGroup; ++i) {
-            const int q = 16 * g + 8 * h + i;
-            const float yq = ys[vec_slot(q)];
-            add_query(half[h], q < nq ? yq : c0, __ldg(a + obs_slot(q)), c0);
-          }
+        for (int i = 0; i < kMomentGroup; ++i) {
+          const int qa = 16 * g + i, qb = qa + kMomentGroup;
+          const float ya = ys[vec_slot(qa)], yb = ys[vec_slot(qb)];
+          add_query2(both, pack2(qa < nq ? ya : c0, qb < nq ? yb : c0), __ldg(a + obs_slot(qa)),
+                     __ldg(a + obs_slot(qb)), cc);
         }
+        TileSums half[2];
+        unpack_sums(both, half[0], half[1]);
         TileSums m = merge_sums(half[0], half[1]);
 #pragma unroll
         for (int o = 1; o < 16; o <<= 1) m = merge_across(m, o);

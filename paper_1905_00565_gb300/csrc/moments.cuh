@@ -83,6 +83,87 @@ __device__ __forceinline__ void add_query(TileSums& m, float y, float2 a, float 
   pe = __fmaf_rn(a.x, e, __fmaf_rn(a.y, b, __fmaf_rn(a.x, b, -p)));
   accumulate(m.ab, p, pe);
 }
+
+// Two sums side by side in packed FP32 pairs (one instruction for both halves,
+// each rounded as the scalar operation is: the same bits as two add_query).
+// Half of the epilogue's instructions are these sums.
+using packed = unsigned long long;
+__device__ __forceinline__ packed pack2(float lo, float hi) {
+  packed r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(packed x, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
+}
+__device__ __forceinline__ packed add2(packed a, packed b) {
+  packed r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ packed sub2(packed a, packed b) {
+  packed r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ packed mul2(packed a, packed b) {
+  packed r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ packed fma2(packed a, packed b, packed c) {
+  packed r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+struct Pair32x2 {
+  packed h, l;
+};
+struct TileSums2 {
+  Pair32x2 b1, b2, ab;
+};
+__device__ __forceinline__ TileSums2 zero_sums2() {
+  TileSums2 z;
+  z.b1 = z.b2 = z.ab = Pair32x2{0ull, 0ull};
+  return z;
+}
+__device__ __forceinline__ void accumulate2(Pair32x2& acc, packed h, packed l) {
+  const packed s = add2(acc.h, h);
+  const packed v = sub2(s, acc.h);
+  const packed err = add2(sub2(acc.h, sub2(s, v)), sub2(h, v));
+  acc.h = s;
+  acc.l = add2(acc.l, add2(err, l));
+}
+// accumulate2 of -n: subtractions in place of a negated operand
+__device__ __forceinline__ void accumulate2_negated(Pair32x2& acc, packed n, packed l) {
+  const packed s = sub2(acc.h, n);
+  const packed v = sub2(s, acc.h);
+  const packed err = sub2(sub2(acc.h, sub2(s, v)), add2(n, v));
+  acc.h = s;
+  acc.l = add2(acc.l, add2(err, l));
+}
+__device__ __forceinline__ void add_query2(TileSums2& m, packed y, float2 a0, float2 a1, packed c) {
+  const packed b = sub2(y, c), nb = sub2(c, y);
+  const packed v = sub2(b, y);
+  const packed e = sub2(sub2(y, sub2(b, v)), add2(c, v));
+  accumulate2(m.b1, b, e);
+  packed np = mul2(b, nb);
+  packed pe = fma2(add2(b, b), e, fma2(b, b, np));
+  accumulate2_negated(m.b2, np, pe);
+  const packed ah = pack2(a0.x, a1.x), al = pack2(a0.y, a1.y);
+  np = mul2(ah, nb);
+  pe = fma2(ah, e, fma2(al, b, fma2(ah, b, np)));
+  accumulate2_negated(m.ab, np, pe);
+}
+__device__ __forceinline__ void unpack_sums(const TileSums2& m, TileSums& lo, TileSums& hi) {
+  unpack2(m.b1.h, lo.b1.h, hi.b1.h);
+  unpack2(m.b1.l, lo.b1.l, hi.b1.l);
+  unpack2(m.b2.h, lo.b2.h, hi.b2.h);
+  unpack2(m.b2.l, lo.b2.l, hi.b2.l);
+  unpack2(m.ab.h, lo.ab.h, hi.ab.h);
+  unpack2(m.ab.l, lo.ab.l, hi.ab.l);
+}
+
 __device__ __forceinline__ TileSums merge_sums(const TileSums& a, const TileSums& b) {
   TileSums r;
   r.b1 = merge_pairs(a.b1, b.b1);

@@ -23,7 +23,8 @@ LIB = os.path.join(HERE, "libccm_gb300.so")
 SOURCES = [(name, e) for e in range(10, 0, -1) for name in ("knn_fused.cu", "table_build.cu", "knn_scan.cu")] + [
     (name, 0) for name in ("table.cu", "runtime.cu", "sampler.cu", "knn_dispatch.cu", "plain.cu",
                            "noalloc.cu", "order.cu", "convergence.cu")]
-HEADERS = [os.path.join(CSRC, name) for name in ("ccm_internal.h", "moments.cuh", "bits.cuh", "launch.cuh")] + [
+HEADERS = [os.path.join(CSRC, name) for name in (
+    "ccm_internal.h", "moments.cuh", "bits.cuh", "row_walk.cuh", "launch.cuh")] + [
     os.path.join(INCLUDE, "ccm.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

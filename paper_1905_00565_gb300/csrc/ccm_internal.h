@@ -20,7 +20,7 @@ struct UnitDesc {
                         // table share one slot there: only the plain comparator lists them)
   int64_t bits_off;     // table_R > 0: this unit's membership bits, by position of the query order
                         // (consecutive units of one cell lie back to back)
-  int64_t words_off;    // table_R > 0 and one target: its scan group's membership words
+  int64_t words_off;    // units read in groups: their membership words; -1: none
   int64_t part_off;     // first partial-sum slot: target t, tile q at part_off + t*n_tiles + q
   int64_t order_off;    // first entry of this unit's query order (per variable, E, tau)
   int64_t tgt_off;      // first TargetDesc of this unit
@@ -128,6 +128,12 @@ constexpr size_t kScanSmemMax = 112 * 1024;  // shared memory of a scan CTA: two
 // zeros up to a whole number of 32 beyond the last (table rows are padded with
 // position n_m).
 __host__ __device__ constexpr int member_words(int n_m) { return (n_m + 32) / 32 * 32; }
+// Realizations of an item of units with many targets that read a table: the
+// weights and neighbours of a query tile wait in 160 KB of shared memory.
+__host__ __device__ constexpr int lane_group(int E) {
+  return 80 / (E + 1) < kScanGroup ? 80 / (E + 1) : kScanGroup;
+}
+constexpr size_t kGroupSmemMax = 224 * 1024;  // shared memory of its CTA: one an SM
 // One scan group: `count` consecutive units from `unit` on.
 struct MemberGroup {
   int32_t unit, count;
@@ -212,6 +218,7 @@ struct KnnParams {
   int32_t* err;
   unsigned long long* stats;  // optional search counters [kStatCount] (kStat*), nullptr: none
   int32_t lane_scratch;   // table kernel: where the lane-per-target scratch starts in shared memory
+  int32_t group_words;    // grouped table kernel: membership words in shared memory
   int32_t persistent;     // 1: CTAs pull items from item_counter; 0: item = blockIdx.x
   int32_t merge_at[kMaxE + 1];  // per E: merge pending candidates once a lane holds this many
   int32_t variant[kMaxE + 1];   // per E: kernel variant (0 narrow, 1 wide); same results
@@ -337,6 +344,8 @@ struct KnnKernels {
   static cudaError_t occupancy_table(int max_nm, bool lanes, int* ctas);
   static cudaError_t launch_table(const KnnParams& p, int max_nm, bool lanes, int grid,
                                   LaunchStream s);
+  static cudaError_t prepare_group();
+  static cudaError_t launch_group(const KnnParams& p, int max_nm, int grid, LaunchStream s);
   static cudaError_t prepare_scan();
   static cudaError_t launch_scan(const KnnParams& p, int max_nm, int grid, LaunchStream s);
 };
@@ -366,6 +375,10 @@ cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lane_ta
 // Units with one target: grouped realizations (two CTAs per SM).
 cudaError_t knn_scan_prepare();
 cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, LaunchStream s);
+
+// Units with many targets: grouped realizations (one CTA per SM).
+cudaError_t knn_group_prepare();
+cudaError_t launch_knn_group(const KnnParams& p, int E, int max_nm, int grid, LaunchStream s);
 
 // Sets the thread-local message returned by ccm_last_error() (runtime.cu).
 void set_last_error(const char* msg);

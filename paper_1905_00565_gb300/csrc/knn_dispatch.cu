@@ -210,6 +210,10 @@ int knn_queries_per_thread() { return 1; }
   if (const cudaError_t e = KnnKernels<EV>::prepare_table(); e != cudaSuccess) return e;
 #define CCM_CASE_PREPARE_SCAN(EV)                                        \
   if (const cudaError_t e = KnnKernels<EV>::prepare_scan(); e != cudaSuccess) return e;
+#define CCM_CASE_PREPARE_GROUP(EV)                                       \
+  if (const cudaError_t e = KnnKernels<EV>::prepare_group(); e != cudaSuccess) return e;
+#define CCM_CASE_LAUNCH_GROUP(EV) \
+  case EV: return KnnKernels<EV>::launch_group(p, max_nm, grid, s);
 #define CCM_CASE_LAUNCH_SCAN(EV) \
   case EV: return KnnKernels<EV>::launch_scan(p, max_nm, grid, s);
 #define CCM_CASE_OCCUPANCY(EV) \
@@ -233,6 +237,14 @@ cudaError_t knn_scan_prepare() {
 }
 cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, LaunchStream s) {
   switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH_SCAN) }
+  return cudaErrorInvalidValue;
+}
+cudaError_t knn_group_prepare() {
+  CCM_FOR_E(CCM_CASE_PREPARE_GROUP)
+  return cudaSuccess;
+}
+cudaError_t launch_knn_group(const KnnParams& p, int E, int max_nm, int grid, LaunchStream s) {
+  switch (E) { CCM_FOR_E(CCM_CASE_LAUNCH_GROUP) }
   return cudaErrorInvalidValue;
 }
 cudaError_t knn_occupancy(int E, int* ctas) {

@@ -206,7 +206,7 @@ __device__ __forceinline__ void flush_ring(const float* ring, const RingMeta* me
 // brute force and table scan 222 -> 62 ms a run.
 // Block-wide; the caller's next use of keep and scratch is behind the closing
 // barrier.
-template <int E>
+template <int E, bool kWide>
 __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc& u, int tile, int nq,
                                           const u64* keep, const float* rus, float* sums) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -219,14 +219,16 @@ __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc&
   for (int tc = 0, turn = 0; tc < T; tc += 32, ++turn) {
     const int t = min(tc + lane, T - 1);  // lanes past the last target repeat it
     const TargetDesc& tg = tgs[t];
-    const float* col = st + tg.i;
+    const char* col = reinterpret_cast<const char*>(st + tg.i);
     const float scale = p.obs_stat[tg.obs_tile + tile].scale;
     auto predict = [&](int q) {
       float acc = 0.f;
 #pragma unroll
       for (int s = 0; s <= E; ++s) {
         const u64 k = keep[s * kThreads + q];
-        acc = __fmaf_rn(key_dist(k), __ldg(col + (int64_t)key_index(k) * stride), acc);
+        const float* at = reinterpret_cast<const float*>(
+            col + (kWide ? (int64_t)key_index(k) * stride * 4 : (int64_t)(uint32_t)k));
+        acc = __fmaf_rn(key_dist(k), __ldg(at), acc);
       }
       return __fmul_rn(acc, rus[q]);
     };
@@ -352,8 +354,19 @@ __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& 
     float* rus = reinterpret_cast<float*>(keep + (E + 1) * kThreads);
     if (kKeep) __syncthreads();  // other warps' columns reach beyond E+1 keys while they search
     rus[tid] = rcp_hw(usum);
+    // neighbours as byte offsets into the time-major series while they fit 32 bits
+    const uint32_t row_bytes = (uint32_t)u.st_stride * 4u;
+    const bool wide = (u64)u.n * row_bytes >> 32 != 0;
+    if (!wide) {
+#pragma unroll
+      for (int s = 0; s <= E; ++s) {
+        const u64 k = keep[s * kThreads + tid];
+        keep[s * kThreads + tid] = (k & 0xffffffff00000000ull) | ((uint32_t)k * row_bytes);
+      }
+    }
     __syncthreads();
-    lane_targets<E>(p, u, tile, nq, keep, rus, rus + kThreads);
+    if (wide) lane_targets<E, true>(p, u, tile, nq, keep, rus, rus + kThreads);
+    else lane_targets<E, false>(p, u, tile, nq, keep, rus, rus + kThreads);
   } else {
   auto weight = [&](int s) {
     return kKeep ? __uint_as_float((uint32_t)(keep[s * kThreads + tid] >> 32)) : w[s];
@@ -874,6 +887,46 @@ __device__ __forceinline__ int table_walk(const Index* row, const int32_t* order
   return got;
 }
 
+// Rare: fewer than E+1 members in the query's row; scan the library, keeping the
+// E+1 smallest (distance, index) keys.
+template <int E>
+__device__ __noinline__ void library_search(const float* sj, const int32_t* order,
+                                            const uint32_t* bits, int words, int off, int tau, int W,
+                                            int n_m, int m, float (&dd)[E + 1], int (&nb)[E + 1]) {
+  float q[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) q[e] = sj[m + off - e * tau];
+  float kd[E + 1];
+  int kl[E + 1];
+#pragma unroll
+  for (int s2 = 0; s2 <= E; ++s2) {
+    kd[s2] = INFINITY;
+    kl[s2] = INT_MAX;
+  }
+  for (int w = 0; w < words; ++w) {
+    for (uint32_t left = bits[w]; left != 0u; left &= left - 1u) {
+      const int l = order[32 * w + __ffs(left) - 1];
+      if (abs(l - m) <= W) continue;
+      const float d = d2_point<E>(sj, off, tau, q, l);
+      if (key_less(d, l, kd[E], kl[E])) {
+        int s2 = E;
+        while (s2 > 0 && key_less(d, l, kd[s2 - 1], kl[s2 - 1])) {
+          kd[s2] = kd[s2 - 1];
+          kl[s2] = kl[s2 - 1];
+          --s2;
+        }
+        kd[s2] = d;
+        kl[s2] = l;
+      }
+    }
+  }
+#pragma unroll
+  for (int s2 = 0; s2 <= E; ++s2) {
+    nb[s2] = min(max(kl[s2], 0), n_m - 1);  // in bounds however few points qualified
+    dd[s2] = sqrt_hw(kd[s2]);
+  }
+}
+
 template <int E, bool kLanes, bool kStats>
 __device__ void process_table_item(const KnnParams& p, const UnitDesc& u, int tile0,
                                    unsigned char* smem, RingMeta* meta, int& ring_n) {
@@ -945,40 +998,7 @@ __device__ void process_table_item(const KnnParams& p, const UnitDesc& u, int ti
         nb[s2] = 0;
       }
     } else {
-      // Rare: fewer than E+1 members in the row; scan the library, keeping the
-      // E+1 smallest (distance, index) keys.
-      float q[E];
-#pragma unroll
-      for (int e = 0; e < E; ++e) q[e] = sj[m + off - e * tau];
-      float kd[E + 1];
-      int kl[E + 1];
-#pragma unroll
-      for (int s2 = 0; s2 <= E; ++s2) {
-        kd[s2] = INFINITY;
-        kl[s2] = INT_MAX;
-      }
-      for (int w = 0; w < words; ++w) {
-        for (uint32_t left = s_bits[w]; left != 0u; left &= left - 1u) {
-          const int l = order[32 * w + __ffs(left) - 1];
-          if (abs(l - m) <= W) continue;
-          const float d = d2_point<E>(sj, off, tau, q, l);
-          if (key_less(d, l, kd[E], kl[E])) {
-            int s2 = E;
-            while (s2 > 0 && key_less(d, l, kd[s2 - 1], kl[s2 - 1])) {
-              kd[s2] = kd[s2 - 1];
-              kl[s2] = kl[s2 - 1];
-              --s2;
-            }
-            kd[s2] = d;
-            kl[s2] = l;
-          }
-        }
-      }
-#pragma unroll
-      for (int s2 = 0; s2 <= E; ++s2) {
-        nb[s2] = min(max(kl[s2], 0), n_m - 1);  // in bounds however few points qualified
-        dd[s2] = sqrt_hw(kd[s2]);
-      }
+      library_search<E>(sj, order, s_bits, words, off, tau, W, n_m, m, dd, nb);
     }
     finish_tile<E, kLanes, false, true>(p, u, tile, m, valid, dd, nb, s_ring, meta, ring_n, s_keep);
   }

@@ -2,14 +2,8 @@
 // variable, target, E, tau) are served by one walk of each query's row of the
 // distance indexing table (table.cu; compiled once per E).
 //
-// A warp owns a query and a lane a realization.  The row holds the query's
-// nearest manifold points, nearest first, as positions of the query order.  In
-// a step the lanes read 32 consecutive ranks (one coalesced access), look up
-// the membership word of each (bit r: realization r's library holds the point)
-// and transpose the 32 x 32 bits across the warp, so that every lane holds the
-// members of its own realization among the 32 ranks.  A lane that still lacks
-// neighbours records the step's mask (at most E+1 records: each holds a
-// member); the walk ends when every lane has E+1.  Then each lane reads off its
+// A warp owns a query and a lane a realization (the walk: row_walk.cuh).  When
+// every lane has met E+1 members of its library, each reads off its
 // first E+1 ranks, loads their (distance, target value) pairs from the same
 // row, and forms the weights and the prediction, in the order and with the
 // operations of the brute-force epilogue: every bit of rho is the same.
@@ -30,10 +24,12 @@
 #include <limits.h>
 #include <math.h>
 
-#include "bits.cuh"
+#include <type_traits>
+
 #include "ccm_internal.h"
 #include "launch.cuh"
 #include "moments.cuh"
+#include "row_walk.cuh"
 
 namespace ccm {
 namespace {
@@ -130,27 +126,36 @@ __device__ __noinline__ void search_library(const KnnParams& p, const UnitDesc& 
   }
 }
 
-// Weights and prediction (paper Sect. 2.1) from the E+1 distances and target
-// values, nearest first: the brute-force epilogue's operations in its order.
+// Simplex weights (paper Sect. 2.1) of the E+1 distances, nearest first, and
+// their sum: the brute-force epilogue's operations in its order.
 template <int E>
-__device__ __forceinline__ float predict(const float (&d)[E + 1], const float (&v)[E + 1],
-                                         float wfloor) {
+__device__ __forceinline__ float simplex_weights(const float (&d)[E + 1], float wfloor,
+                                                 float (&w)[E + 1]) {
   const float d1 = d[0];
   const float inv_d1 = (d1 > 0.f) ? rcp_hw(d1) : 0.f;
-  float w[E + 1];
 #pragma unroll
   for (int s = 0; s <= E; ++s) w[s] = simplex_exp(d[s], inv_d1);
   if (!(d1 > 0.f)) {  // rare: the nearest at distance 0
 #pragma unroll
     for (int s = 0; s <= E; ++s) w[s] = simplex_limit(d[s]);
   }
-  float usum = 0.f, acc = 0.f;
+  float usum = 0.f;
 #pragma unroll
   for (int s = 0; s <= E; ++s) {
     w[s] = fmaxf(w[s], wfloor);
     usum = __fadd_rn(usum, w[s]);
-    acc = __fmaf_rn(w[s], v[s], acc);
   }
+  return usum;
+}
+
+template <int E>
+__device__ __forceinline__ float predict(const float (&d)[E + 1], const float (&v)[E + 1],
+                                         float wfloor) {
+  float w[E + 1];
+  const float usum = simplex_weights<E>(d, wfloor, w);
+  float acc = 0.f;
+#pragma unroll
+  for (int s = 0; s <= E; ++s) acc = __fmaf_rn(w[s], v[s], acc);
   return __fmul_rn(acc, rcp_hw(usum));
 }
 
@@ -209,54 +214,10 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
         const int pos = tile * kQT + q;
         const int64_t row = u.table_off + (int64_t)pos * stride;
         const int m = kGeneral ? order[pos] : 0;
-        // the walk: lane l holds rank 31 - l of a step, so that the highest set
-        // bit of a realization's mask is its nearest member
-        const Index* ip = static_cast<const Index*>(p.table) + row + (31 - lane);
-        const Index* const end = ip + stride;
-        int got = 0, recs = 0, c = 0;
-        auto lookup = [&](uint32_t x) {
-          uint32_t word = kSmemWords ? s_words[x] : __ldg(words + x);
-          if (kGeneral && W > 0 && word != 0u) {  // points inside the exclusion window
-            const int l = order[x];
-            if ((unsigned)l - (unsigned)m + (unsigned)W <= 2u * (unsigned)W) word = 0u;
-          }
-          return word;
-        };
-        auto record = [&](uint32_t members) {
-          if (members != 0u && got < K) {
-            mask[recs * kScanThreads] = members;
-            step[recs * kScanThreads] = (uint16_t)c;
-            ++recs;
-            got += __popc(members);
-          }
-          ++c;
-        };
-        uint32_t xa = (uint32_t)__ldg(ip);
-        if (dense) {  // 32 ranks a step: the first ones mostly suffice
-          for (;;) {
-            const uint32_t wa = lookup(xa);
-            ip += 32;
-            const bool more = ip < end;
-            if (more) xa = (uint32_t)__ldg(ip);
-            record(tr(wa));
-            if (!more || !__any_sync(kAllLanes, mine && got < K)) break;
-          }
-        } else {  // 64 ranks a step, the next step's loads in flight
-          uint32_t xb = (uint32_t)__ldg(ip + 32);
-          for (;;) {
-            const uint32_t wa = lookup(xa), wb = lookup(xb);
-            ip += 64;
-            const bool more = ip < end;
-            if (more) {
-              xa = (uint32_t)__ldg(ip);
-              xb = (uint32_t)__ldg(ip + 32);
-            }
-            const uint32_t ma = tr(wa), mb = tr(wb);
-            record(ma);
-            record(mb);
-            if (!more || !__any_sync(kAllLanes, mine && got < K)) break;
-          }
-        }
+        int c;
+        const int got = group_walk<K, kScanThreads, Index, kGeneral>(
+            static_cast<const Index*>(p.table) + row, stride, dense, mine, kSmemWords ? s_words : words,
+            order, m, W, tr, mask, step, c);
         const bool full = mine && got >= K;
         if (kGeneral && p.stats) {
           const unsigned shorts = __popc(__ballot_sync(kAllLanes, mine && !full));
@@ -269,19 +230,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
         float y = 0.f;
         if (full) {
           int rank[K];
-          uint32_t cur = mask[0];
-          int base = step[0] * 32, rec = 0;
-#pragma unroll
-          for (int s = 0; s < K; ++s) {
-            if (cur == 0u) {
-              ++rec;
-              cur = mask[rec * kScanThreads];
-              base = step[rec * kScanThreads] * 32;
-            }
-            const int b = __clz(cur);
-            cur ^= 0x80000000u >> b;
-            rank[s] = base + b;
-          }
+          first_ranks<K, kScanThreads>(mask, step, rank);
           const float2* dv = reinterpret_cast<const float2*>(p.table_dist) + row;
           float d[K], v[K];
 #pragma unroll
@@ -357,6 +306,221 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
   }
 }
 
+// Units with many targets, up to lane_group(E) realizations of one (library
+// variable, E, tau) and one query tile an item.  Phase 1: a warp walks a query's
+// row for all of them at once, a lane a realization, and leaves each one's
+// weights and neighbours (byte offsets into the time-major series) in shared
+// memory.  Phase 2: a team of four warps takes a realization and 32 targets, a
+// lane a target and a quarter of the tile's queries a warp: a neighbour's values
+// of 32 targets are one coalesced read, the moments stay in the lane's registers
+// and meet once per task.
+//
+// Bound: issue (50 %) and the latency of the series reads (half an SM's warps
+// at 80 registers; 64 and 128 registers are slower).  A realization at a time
+// per CTA, every thread walking its own row, left 32 lines per load of a row's
+// entries and two block barriers per 32 targets: 64 variables, N = 5000, E =
+// 2..4, r = 25, L = 296 .. 4500, all pairs 42.5 ms, now 34.3.  Teams rather than
+// a warp a task: 16 to 40 tasks do not divide among 24 warps (24 variables 0.82
+// -> 0.76 ms).  160 KB for the realizations rather than 128: 35.0 -> 34.3.
+constexpr int kGroupThreads = 768;
+constexpr int kTeam = 4;  // warps a (realization, 32 targets): a quarter of the tile each
+constexpr int kTeamQueries = kQT / kTeam;
+static_assert(kGroupThreads % (32 * kTeam) == 0 && kTeamQueries % (2 * kMomentGroup) == 0, "teams");
+static_assert(4 * kGroupThreads * 6 >= kGroupThreads / 32 * 6 * 32 * 4, "the teams' sums fit the records");
+// A barrier of one team's warps (barrier 0 is the block's).
+__device__ __forceinline__ void team_barrier(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(32 * kTeam) : "memory");
+}
+template <int E>
+constexpr int kKeepStride = (E + 1) * kQT + 1;  // entries a realization; odd: 32 lanes, 32 banks
+template <int E>
+__host__ __device__ constexpr size_t group_fixed_smem() {
+  return (size_t)(lane_group(E) * kKeepStride<E> + 1) / 2 * 2 * 8 +
+         (size_t)(lane_group(E) * (kQT + 1) + 3) / 4 * 16 +
+         (size_t)(E + 1 < 4 ? 4 : E + 1) * kGroupThreads * (4 + 2);
+}
+
+template <int E, bool kGeneral>
+__global__ void __launch_bounds__(kGroupThreads, 1) group_kernel(KnnParams p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int s_item;
+  constexpr int K = E + 1, kWarps = kGroupThreads / 32, KS = kKeepStride<E>, G = lane_group(E);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float2* s_keep = reinterpret_cast<float2*>(smem);  // [realization][K][query]: weight, neighbour
+  float* s_rus = reinterpret_cast<float*>(s_keep + (G * KS + 1) / 2 * 2);  // [realization][query]
+  uint32_t* mask = reinterpret_cast<uint32_t*>(s_rus + (G * (kQT + 1) + 3) / 4 * 4) + tid;
+  uint16_t* step = reinterpret_cast<uint16_t*>(mask - tid + K * kGroupThreads) + tid;
+  uint32_t* s_words = reinterpret_cast<uint32_t*>(smem + group_fixed_smem<E>());
+  const BitTranspose tr(lane);
+  chain_begin();
+  for (int round = 0;; ++round) {
+    if (p.persistent && tid == 0) s_item = (int)atomicAdd(p.item_counter, 1u);
+    __syncthreads();
+    const int it = p.persistent ? s_item : (round == 0 ? (int)blockIdx.x : INT_MAX);
+    if ((int64_t)it >= p.n_items) break;
+    const WorkItem w = p.items[it];
+    const int count = w.count, tile = w.tile;
+    const UnitDesc& u = p.units[w.unit];  // the realizations' common description
+    const int n_m = u.n_m, stride = u.table_R, W = u.theiler, T = u.n_targets;
+    if (u.E != E || T < kLaneTargets || count < 1 || count > G) {
+      if (tid == 0) atomicOr(p.err, kErrBadUnit);
+      __syncthreads();
+      continue;
+    }
+    const uint32_t* words = p.words + u.words_off;
+    if (p.group_words) {
+      const uint4* src = reinterpret_cast<const uint4*>(words);
+      uint4* dst = reinterpret_cast<uint4*>(s_words);
+      for (int i = tid; i < member_words(n_m) >> 2; i += kGroupThreads) dst[i] = __ldg(src + i);
+    }
+    __syncthreads();
+    const int32_t* order = p.order + u.order_off;
+    const int nq = min(kQT, n_m - tile * kQT);
+    const bool mine = lane < count;
+    const bool dense = 2 * K * (int64_t)n_m <= 32 * (int64_t)u.L;
+    for (int q = warp; q < nq; q += kWarps) {
+      const int pos = tile * kQT + q;
+      const int64_t row = u.table_off + (int64_t)pos * stride;
+      const int m = kGeneral ? order[pos] : 0;
+      int c, got;
+      auto walk = [&](auto* table, const uint32_t* from) {
+        return group_walk<K, kGroupThreads, std::remove_const_t<std::remove_pointer_t<decltype(table)>>,
+                          kGeneral>(table + row, stride, dense, mine, from, order, m, W, tr, mask,
+                                    step, c);
+      };
+      if (!p.table_u16) got = walk(static_cast<const int32_t*>(p.table), words);
+      else if (p.group_words) got = walk(static_cast<const uint16_t*>(p.table), s_words);
+      else got = walk(static_cast<const uint16_t*>(p.table), words);
+      const bool full = mine && got >= K;
+      if (kGeneral && p.stats) {
+        const unsigned shorts = __popc(__ballot_sync(kAllLanes, mine && !full));
+        if (lane == 0) {
+          atomicAdd(&p.stats[kStatTableQueries], (unsigned long long)count);
+          atomicAdd(&p.stats[kStatTableEntries], 32ull * c);
+          if (shorts) atomicAdd(&p.stats[kStatTableFallbacks], (unsigned long long)shorts);
+        }
+      }
+      auto keep = [&](const float (&d)[K], const int (&nb)[K]) {
+        float wt[K];
+        const float usum = simplex_weights<E>(d, u.wfloor, wt);
+#pragma unroll
+        for (int s = 0; s < K; ++s)
+          s_keep[lane * KS + s * kQT + q] = make_float2(wt[s], __uint_as_float((uint32_t)(nb[s] * u.st_stride) * 4u));
+        s_rus[lane * (kQT + 1) + q] = rcp_hw(usum);
+        if (kGeneral && p.dbg_nbr) {
+          const int mq = order[pos];
+          for (int t = 0; t < T; ++t)
+            for (int s = 0; s < K; ++s)
+              p.dbg_nbr[p.targets[p.units[w.unit + lane].tgt_off + t].nbr_off + (int64_t)mq * K + s] =
+                  nb[s];
+        }
+      };
+      if (full) {
+        int rank[K], nb[K];
+        float d[K];
+        first_ranks<K, kGroupThreads>(mask, step, rank);
+#pragma unroll
+        for (int s = 0; s < K; ++s) {
+          const int64_t at = row + rank[s];
+          d[s] = p.table_pairs ? __ldg(reinterpret_cast<const float2*>(p.table_dist) + at).x
+                               : __ldg(p.table_dist + at);
+          nb[s] = order[p.table_u16 ? (int)__ldg(static_cast<const uint16_t*>(p.table) + at)
+                                    : __ldg(static_cast<const int32_t*>(p.table) + at)];
+        }
+        keep(d, nb);
+      }
+      for (unsigned left = __ballot_sync(kAllLanes, mine && !full); left; left &= left - 1u) {
+        const int r = __ffs(left) - 1;
+        u64 keys[K];
+        search_library<E>(p, u, r, order[pos], keys);
+        float d[K];
+        int nb[K];
+#pragma unroll
+        for (int s = 0; s < K; ++s) {
+          // in bounds however few points qualified
+          nb[s] = min(max((int)(uint32_t)keys[s], 0), n_m - 1);
+          d[s] = sqrt_hw(__uint_as_float((uint32_t)(keys[s] >> 32)));
+        }
+        if (lane == r) keep(d, nb);
+      }
+    }
+    __syncthreads();
+    const float* st = p.st + u.st_off + (int64_t)(E - 1) * u.tau * u.st_stride;
+    const TargetDesc* tgs = p.targets + u.tgt_off;
+    const float2* obs = p.obs + tgs[0].obs_tile * kQT + (int64_t)tile * kQT * T;
+    const int chunks = (T + 31) / 32;
+    // [warp][value][lane], where the walks' records were
+    float* sums = reinterpret_cast<float*>(mask - tid) + warp * 6 * 32 + lane;
+    const int part = warp % kTeam, q0 = part * kTeamQueries;
+    for (int task = warp / kTeam; task < count * chunks; task += kWarps / kTeam) {
+      const int chunk = task / count, r = task - chunk * count;
+      const int t = min(chunk * 32 + lane, T - 1);  // lanes past the last target repeat it
+      const TargetDesc& tg = tgs[t];
+      const char* col = reinterpret_cast<const char*>(st + tg.i);
+      const float scale = p.obs_stat[tg.obs_tile + tile].scale;
+      const float2* keep = s_keep + r * KS;
+      const float* rus = s_rus + r * (kQT + 1);
+      auto value = [&](int q) {
+        float acc = 0.f;
+#pragma unroll
+        for (int s = 0; s < K; ++s) {
+          const float2 k = keep[s * kQT + q];
+          
+          acc = __fmaf_rn(k.x, __ldg(reinterpret_cast<const float*>(col + __float_as_uint(k.y))), acc);
+        }
+        return __fmul_rn(acc, rus[q]);
+      };
+      const float c = __fmul_rn(value(0), scale);
+      const packed cc = pack2(c, c), ss = pack2(scale, scale);
+      const float2* a = obs + t;
+      // the tree's pending subtrees, indexed at run time: in local memory, not in the
+      // loop's registers
+      TileSums lv[3], sum;
+      for (int n = 0; n < kTeamQueries / (2 * kMomentGroup); ++n) {  // 16 queries a turn
+        const int qa = q0 + 2 * kMomentGroup * n, qb = qa + kMomentGroup;
+        TileSums lo = zero_sums(), hi = zero_sums();
+        if (qb + kMomentGroup <= nq && !(kGeneral && p.dbg_xhat)) {
+          TileSums2 both = zero_sums2();
+#pragma unroll 2
+          for (int i = 0; i < kMomentGroup; ++i)
+            add_query2(both, mul2(pack2(value(qa + i), value(qb + i)), ss),
+                       __ldg(a + (int64_t)(qa + i) * T), __ldg(a + (int64_t)(qb + i) * T), cc);
+          unpack_sums(both, lo, hi);
+        } else {
+          for (int q = qa; q < min(qb + kMomentGroup, nq); ++q) {
+            const float y = value(q);
+            if (kGeneral && p.dbg_xhat && chunk * 32 + lane < T)
+              p.dbg_xhat[p.targets[p.units[w.unit + r].tgt_off + t].q_off + order[tile * kQT + q]] = y;
+            add_query(q < qb ? lo : hi, __fmul_rn(y, scale), __ldg(a + (int64_t)q * T), c);
+          }
+        }
+        sum = merge_sums(lo, hi);  // and up the tree of the tile's groups
+        int l = 0;
+        for (int up = n; up & 1; up >>= 1, ++l) sum = merge_sums(lv[l], sum);
+        lv[l] = sum;
+      }
+      const float mine6[6] = {sum.b1.h, sum.b1.l, sum.b2.h, sum.b2.l, sum.ab.h, sum.ab.l};
+#pragma unroll
+      for (int x = 0; x < 6; ++x) sums[x * 32] = mine6[x];
+      team_barrier(warp / kTeam);
+      if (part == (task / (kWarps / kTeam)) % kTeam && chunk * 32 + lane < T) {
+        auto load = [&](int i) {
+          const float* f = sums + (i - part) * 6 * 32;
+          TileSums m;
+          m.b1 = Pair32{f[0], f[32]};
+          m.b2 = Pair32{f[2 * 32], f[3 * 32]};
+          m.ab = Pair32{f[4 * 32], f[5 * 32]};
+          return m;
+        };
+        store_sums(p.partials + 2 * (p.units[w.unit + r].part_off + (int64_t)t * u.n_tiles + tile), c,
+                   merge_sums(merge_sums(load(0), load(1)), merge_sums(load(2), load(3))));
+      }
+      team_barrier(warp / kTeam);
+    }
+    __syncthreads();
+  }
+}
+
 template <int E>
 size_t scan_smem(int max_nm, bool smem_words) {
   return scan_fixed_smem<E>() + (smem_words ? (size_t)member_words(max_nm) * 4 : 0);
@@ -397,6 +561,29 @@ cudaError_t KnnKernels<E>::prepare_scan() {
                         scan_kernel<E, int32_t, false, true>, scan_kernel<E, int32_t, false, false>}) {
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)kScanSmemMax);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+template <int E>
+cudaError_t KnnKernels<E>::launch_group(const KnnParams& params, int max_nm, int grid,
+                                        LaunchStream s) {
+  static_assert(group_fixed_smem<E>() <= kGroupSmemMax, "one CTA per SM");
+  KnnParams p = params;
+  const size_t with = group_fixed_smem<E>() + (size_t)member_words(max_nm) * 4;
+  p.group_words = p.table_u16 && with <= kGroupSmemMax ? 1 : 0;
+  const bool general = p.window || p.stats || p.dbg_nbr || p.dbg_xhat;
+  return launch_chained(general ? group_kernel<E, true> : group_kernel<E, false>,
+                        dim3((unsigned)grid), kGroupThreads,
+                        p.group_words ? with : group_fixed_smem<E>(), s, p);
+}
+
+template <int E>
+cudaError_t KnnKernels<E>::prepare_group() {
+  for (const auto fn : {group_kernel<E, false>, group_kernel<E, true>}) {
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kGroupSmemMax);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

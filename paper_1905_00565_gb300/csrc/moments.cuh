@@ -146,11 +146,11 @@ __device__ __forceinline__ void add_query2(TileSums2& m, packed y, float2 a0, fl
   const packed b = sub2(y, c), nb = sub2(c, y);
   const packed v = sub2(b, y);
   const packed e = sub2(sub2(y, sub2(b, v)), add2(c, v));
+  const packed ah = pack2(a0.x, a1.x), al = pack2(a0.y, a1.y);
   accumulate2(m.b1, b, e);
   packed np = mul2(b, nb);
   packed pe = fma2(add2(b, b), e, fma2(b, b, np));
   accumulate2_negated(m.b2, np, pe);
-  const packed ah = pack2(a0.x, a1.x), al = pack2(a0.y, a1.y);
   np = mul2(ah, nb);
   pe = fma2(ah, e, fma2(al, b, fma2(ah, b, np)));
   accumulate2_negated(m.ab, np, pe);

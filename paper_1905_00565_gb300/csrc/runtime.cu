@@ -143,8 +143,9 @@ bool all_finite(const float* x, size_t count) {
 
 // ------------------------------------------------------------- unit lists ---
 // The work items of one search launch: one E, and units of one, few or many
-// targets (a kernel each; brute force: one and few share theirs).
-enum class Targets : int32_t { kOne, kFew, kMany };
+// targets (a kernel each; brute force: one and few share theirs), or of many
+// whose realizations read their table in groups.
+enum class Targets : int32_t { kOne, kFew, kMany, kGrouped };
 struct ItemGroup {
   int32_t E;
   Targets targets;
@@ -167,7 +168,7 @@ struct UnitList {
   bool lane_targets = false;          // some unit has kLaneTargets targets
   std::vector<TableJob> tables;       // distance indexing tables to build
   std::vector<WorkItem> items_table;  // work items of units that read a table
-  std::vector<MemberGroup> member_groups;  // scan groups (units of one target)
+  std::vector<MemberGroup> member_groups;  // scan groups (units of one target or many)
   int64_t bits_total = 0, words_total = 0;  // their membership bits and words
   int64_t lib_scratch = 0;            // longest library of the units that read a table
   std::vector<double> item_cost_table;
@@ -197,7 +198,8 @@ struct UnitList {
   bool table_tv = false;              // some table stores its target's values (TableJob::tv_i)
   Targets targets_of(const WorkItem& w) const {
     const UnitDesc& u = units[(size_t)w.unit];
-    if (u.n_targets >= kLaneTargets) return Targets::kMany;
+    if (u.n_targets >= kLaneTargets)
+      return u.table_R > 0 && u.words_off >= 0 ? Targets::kGrouped : Targets::kMany;
     return u.table_R > 0 && u.n_targets == 1 ? Targets::kOne : Targets::kFew;
   }
   // The launches of a sorted item list.
@@ -530,7 +532,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         }
   }
   // Query tiles per brute-force and scan item, from the tiles of each E's launch.
-  std::map<int32_t, int64_t> brute_tiles, scan_tiles;
+  std::map<int32_t, int64_t> brute_tiles, scan_tiles, many_tiles;
   for (int32_t j : lib_vars)
     for (int32_t E : pc.E)
       for (int32_t tau : pc.tau) {
@@ -543,6 +545,8 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           else
             tabled += pc.r;
         }
+        if (pairs_of[j].size() >= (size_t)kLaneTargets)
+          many_tiles[E] += (n_m + tileq - 1) / tileq * tabled;
         scan_tiles[E] += (n_m + tileq - 1) / tileq * ((tabled + kScanGroup - 1) / kScanGroup);
       }
   for (int32_t j : lib_vars) {
@@ -551,6 +555,18 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
       for (int64_t t = 0; t < nT; ++t) {
         const int32_t E = pc.E[(size_t)e], tau = pc.tau[(size_t)t];
         const size_t first_unit = ul->units.size();
+        // Realizations per group of a variable with many targets: as many as
+        // leave the launch two items per CTA.  The groups lose to a walk per
+        // realization only where a launch is too small to fill them: 20
+        // variables of N = 2000, r = 10, L = 1900 (one wave of items) 0.121 ms
+        // against 0.114; 24 of 3000, r = 25, L = 500 .. 1900 0.76 against 1.07;
+        // 32 of 3000, r = 20, L = 2800 0.33 against 0.39; 40 of 4000, r = 12, E = 8
+        // 1.55 against 1.68.  Their byte offsets have 32 bits.
+        const int32_t lanes_group =
+            tp.size() >= (size_t)kLaneTargets && (uint64_t)pc.n * (uint64_t)st_stride * 4 < 1ull << 32
+                ? (int32_t)std::min<int64_t>(many_tiles[E] / (2 * 152), lane_group(E))
+                : 0;
+        const bool grouped = tp.size() == 1 || lanes_group >= std::min(8, lane_group(E));
         for (int64_t l = 0; l < nL; ++l) {
           const int64_t L = pc.L[(size_t)l];
           const int32_t chunk = brute_chunk(brute_tiles[E], L, E);
@@ -572,6 +588,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             u.wfloor = pc.weight_floor;
             u.lib_off = ul->lib_total;
             u.part_off = ul->part_total;
+            u.words_off = -1;
             u.st_off = st_off;
             u.st_stride = st_stride;
             u.order_off = combo[std::make_tuple(j, E, tau)];
@@ -600,8 +617,8 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
               ul->lib_scratch = std::max(ul->lib_scratch, L);
             }
             const int32_t uidx = (int32_t)ul->units.size();
-            // units of one target that read a table get their items below, in groups
-            const bool owns_items = !(u.table_R > 0 && u.n_targets == 1);
+            // the others get their items below, in groups
+            const bool owns_items = !(u.table_R > 0 && grouped);
             for (int32_t q = 0; q < u.n_tiles && owns_items; ++q) {
               const int64_t nq = std::min<int64_t>(tileq, u.n_m - (int64_t)q * tileq);
               if (u.table_R > 0) {
@@ -643,14 +660,16 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             ul->units.push_back(u);
           }
         }
-        if (tp.size() != 1) continue;
+        if (!grouped) continue;
         // Scan groups: consecutive units of this (j, E, tau) that read the table,
         // whatever their L (the lanes of a partly filled group would idle; the
         // walk of a mixed one is as long as its smallest L's).
         // Tiles per item: one copy of the membership words (about 4 % of a tile's
         // time) against the balance of eight items per CTA slot.
         const int64_t slots = scan_tiles[E] / (8 * 2 * 152);
-        const int32_t chunk = (int32_t)std::min<int64_t>(std::max<int64_t>(slots, 1), kScanChunk);
+        const int32_t chunk =
+            tp.size() > 1 ? 1 : (int32_t)std::min<int64_t>(std::max<int64_t>(slots, 1), kScanChunk);
+        const size_t group = tp.size() > 1 ? (size_t)lanes_group : (size_t)kScanGroup;
         for (size_t a = first_unit; a < ul->units.size();) {
           if (ul->units[a].table_R == 0) {
             ++a;
@@ -658,7 +677,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           }
           size_t b = a;
           int32_t lmin = ul->units[a].L;
-          for (; b < ul->units.size() && b - a < (size_t)kScanGroup && ul->units[b].table_R > 0; ++b) {
+          for (; b < ul->units.size() && b - a < group && ul->units[b].table_R > 0; ++b) {
             ul->units[b].words_off = ul->words_total;
             lmin = std::min(lmin, ul->units[b].L);
           }
@@ -666,9 +685,11 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           ul->words_total += member_words(u.n_m);
           ul->member_groups.push_back(MemberGroup{(int32_t)a, (int32_t)(b - a)});
           for (int32_t q = 0; q < u.n_tiles; q += chunk) {
-            ul->items_table.push_back(WorkItem{(int32_t)a, q, (int32_t)(b - a) | chunk << 8});
+            ul->items_table.push_back(
+                WorkItem{(int32_t)a, q, (int32_t)(b - a) | (tp.size() > 1 ? 0 : chunk << 8)});
             ul->item_cost_table.push_back(std::min(chunk, u.n_tiles - q) *
-                                          (64.0 + (E + 4.0) * u.n_m / lmin));
+                                          (64.0 + (E + 4.0) * u.n_m / lmin +
+                                           (tp.size() > 1 ? 1.5 * (double)(b - a) * u.n_targets : 0.0)));
           }
           a = b;
         }
@@ -722,7 +743,7 @@ void sort_items(UnitList* ul) {
     const Targets ta = ul->targets_of(wa), tb = ul->targets_of(wb);
     if (ta != tb) return ta > tb;
     if (ua.table_off != ub.table_off) return ua.table_off < ub.table_off;
-    if (ta == Targets::kOne && wa.tile != wb.tile) return wa.tile < wb.tile;
+    if ((ta == Targets::kOne || ta == Targets::kGrouped) && wa.tile != wb.tile) return wa.tile < wb.tile;
     return ul->item_cost_table[(size_t)a] > ul->item_cost_table[(size_t)b];
   });
   std::vector<WorkItem> sorted(order.size());
@@ -732,8 +753,8 @@ void sort_items(UnitList* ul) {
 }
 
 // Search launches of one run, at most: per E, brute force of few or many
-// targets, tables of one, few or many.
-constexpr int kMaxSearchLaunches = 5 * kMaxE;
+// targets, tables of one, few or many, or of many in groups.
+constexpr int kMaxSearchLaunches = 6 * kMaxE;
 
 // Device arena layout for a unit list.
 struct Arena {
@@ -1068,6 +1089,8 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     const int g = persistent ? grid_table : (int)std::min<int64_t>(ig.count, 0x7fffffff);
     if (ig.targets == Targets::kOne)
       CCM_CUDA(launch_knn_scan(kt, ig.E, ul.max_nm, persistent ? grid_scan : g, ls));
+    else if (ig.targets == Targets::kGrouped)
+      CCM_CUDA(launch_knn_group(kt, ig.E, ul.max_nm, persistent ? grid_scan / 2 : g, ls));
     else
       CCM_CUDA(launch_knn_table(kt, ig.E, ul.max_nm, ig.targets == Targets::kMany, g, ls));
   }
@@ -1250,6 +1273,7 @@ ccm_status ccm_context_create(int device, size_t hbm_budget_bytes, ccm_context**
   CCM_CUDA(convergence_prepare());
   CCM_CUDA(knn_table_prepare());
   CCM_CUDA(knn_scan_prepare());
+  CCM_CUDA(knn_group_prepare());
   size_t free_b = 0, total_b = 0;
   CCM_CUDA(cudaMemGetInfo(&free_b, &total_b));
   std::unique_ptr<ccm_context> ctx(new ccm_context());

@@ -80,6 +80,47 @@ def test_rows_of_unusual_distances(ccm, kind):
         ccm.ccm_context_destroy(ctx)
 
 
+# Variables with 13 targets: groups of realizations (lane_group's largest at
+# E = 1, 9; smaller ones from the launch's size), membership words in shared
+# memory and in L2 (20000, 70000), the one-realization walk (2000), 32-bit rows.
+# Rows miss for about one (query, realization) in 10 L: thousands of them here.
+@pytest.mark.parametrize("n,E,L,r,theiler", [
+    (1500, [1, 9], [1480, 500, 900], 40, 0), (3000, [3], [2900, 700], 80, 0),
+    (3000, [2, 6], [2900, 900], 33, 5), (20000, [1], [9000], 19, 0), (2000, [4], [1900], 9, 0),
+    (70000, [2], [60000], 10, 0)])
+def test_many_targets_equal_brute_force(ccm, n, E, L, r, theiler):
+    V = 14
+    s, _ = I.logistic_network(V, n, 0.05, 7)
+    pairs = np.array([[j, i] for j in range(V) for i in range(V) if i != j], np.int32)
+    p = I.Problem(series=s, pairs=pairs, E=np.array(E, np.int32), tau=np.array([1], np.int32),
+                  L=np.array(L, np.int64), r=r, seed=4, theiler=theiler)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        np.testing.assert_array_equal(rho_only(ccm, ctx, p, 0),
+                                      rho_only(ccm, ctx, p, ccm.CCM_NO_TABLE))
+    finally:
+        ccm.ccm_context_destroy(ctx)
+
+
+@pytest.mark.parametrize("theiler", [0, 3])
+def test_many_targets_checking_outputs(ccm, theiler):
+    """Neighbours, predictions, libraries and counters of the grouped walk."""
+    V, n = 13, 6000
+    s, _ = I.logistic_network(V, n, 0.05, 9)
+    pairs = np.array([[2, i] for i in range(V) if i != 2], np.int32)
+    p = I.Problem(series=s, pairs=pairs, E=np.array([2], np.int32), tau=np.array([2], np.int32),
+                  L=np.array([1500, 5000], np.int64), r=110, seed=5, theiler=theiler)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        got = run_detailed(ccm, ctx, p, 0)
+        want = run_detailed(ccm, ctx, p, ccm.CCM_NO_TABLE)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    for g, w in zip(got, want):
+        np.testing.assert_array_equal(g, w)
+    check_units(p, *got, which={0, 219, 220 * 11 + 130})
+
+
 def test_scan_checking_outputs(ccm):
     """Neighbours, predictions and libraries of the general variant."""
     p = I.Problem(series=I.logistic_pair(1500), pairs=I.BOTH_DIRECTIONS.copy(),

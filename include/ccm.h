@@ -201,7 +201,9 @@ ccm_status ccm_plan_kernel_times(const ccm_plan_t* plan, double* sampler_ms, dou
 /* The same events per stage: stage_ms[0] query order + observed-value tile
  * records + distance indexing tables, [1] library sampler, [2] brute-force
  * fused kernel, [3] table-scan fused kernel and the merge of the tiles' moments
- * into rho. */
+ * into rho.  Runs of short manifolds build the tables beside the sampler and
+ * the brute-force search: each stage is then its own duration, and the four add
+ * up to more than the run. */
 ccm_status ccm_plan_stage_times(const ccm_plan_t* plan, double* stage_ms /* [4] */);
 
 /* Work counts of the neighbour search in the plan's last completed run
@@ -215,7 +217,7 @@ typedef struct {
   uint64_t pairs_begun;      /* query-library pairs whose squared distance was begun (the
                                 first coordinates of a step, before early termination) */
   uint64_t pairs_full;       /* pairs whose squared distance was completed (all E) */
-  uint64_t pairs_pruned;     /* pairs skipped whole by the chunk bounding-box test */
+  uint64_t pairs_pruned;     /* pairs skipped by the bounding-box test of the warp's queries */
   uint64_t candidates;       /* pairs below a query's running threshold, queued for insertion */
   uint64_t merge_slots;      /* insertion slots executed: per warp merge, 32 x the largest
                                 queue of its lanes (lanes with shorter queues idle) */

@@ -175,7 +175,7 @@ inline int32_t sample_stride(int64_t n_m, int64_t R) {
   return s;
 }
 constexpr int kTableMaxR = 4096;       // entries per query row, at most
-constexpr int kWalkMaxR = 2048;        // the same for variables with several targets (knn_fused.cu)
+constexpr int kWalkMaxR = 2048;        // the same for variables with several targets
 constexpr int kTableChunk = 8;         // query tiles per table work item (one bitmap each)
 constexpr int kTableMaxNm = 1 << 20;   // longest manifold that gets a table (bitmap in smem)
 
@@ -231,11 +231,11 @@ enum : int {
   kStatBruteQueries,     // their valid queries
   kStatPairsBegun,       // query-library pairs whose distance was begun (lanes x points)
   kStatPairsFull,        // pairs whose distance was completed over all E coordinates
-  kStatPairsPruned,      // pairs skipped by chunk pruning (lanes x chunk points)
+  kStatPairsPruned,      // pairs skipped by the box test (lanes x points)
   kStatCandidates,       // candidates appended to the pending buffers
   kStatMergeSlots,       // lockstep insertion slots: per warp merge, 32 x its largest pending count
   kStatTableQueries,     // valid queries answered from a distance indexing table
-  kStatTableEntries,     // table entries loaded (per lane, eight per step)
+  kStatTableEntries,     // table entries loaded (one walk may serve several realizations)
   kStatTableFallbacks,   // queries that scanned their library instead
   kStatCount = 16
 };
@@ -372,7 +372,7 @@ cudaError_t knn_table_prepare();
 cudaError_t knn_table_occupancy(int max_nm, bool lane_targets, int* ctas_per_sm);
 cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lane_targets, int grid,
                              LaunchStream s);
-// Units with one target: grouped realizations (two CTAs per SM).
+// Units with one target: grouped realizations (two CTAs per SM; knn_scan.cu).
 cudaError_t knn_scan_prepare();
 cudaError_t launch_knn_scan(const KnnParams& p, int E, int max_nm, int grid, LaunchStream s);
 

@@ -5,8 +5,8 @@
 // names as the most time-consuming), every query point of the shadow manifold
 // M_j is compared with every library point; the E+1 nearest (itself
 // excluded) give the simplex prediction of the target variable (Sect. 2.1),
-// and the tile's FP64 moments of (observed, predicted) are merged per
-// realization into the Pearson skill (Sect. 2.1).
+// and the tile's moments of (observed, predicted) are merged per realization
+// into the Pearson skill (Sect. 2.1).
 //
 // Design (GB300, FP32 on the CUDA cores; E <= 10 is not a dense contraction):
 //  * persistent CTAs pull work items, sorted by cost, from an atomic counter;
@@ -20,15 +20,17 @@
 //    rounded product, then one fused multiply-add per coordinate), the same
 //    rounding sequence the FP32 selection is defined by;
 //  * the library is visited in query order from the run nearest each warp's
-//    queries (wrapping around); 16-point chunks whose bounding box lies
-//    farther than every lane's threshold are skipped whole;
+//    queries (wrapping around); a lane tests one pair of points of the next 32
+//    against the box of the warp's queries, and pairs farther than every
+//    lane's threshold are never read;
 //  * selection: each query keeps the K = E+1 smallest distances seen as a
 //    sorted float list in registers (a min/max network, no index
 //    bookkeeping), which is its running threshold, and the (squared
 //    distance, index) keys of every candidate at or below the threshold in
 //    its column of a shared-memory buffer; the column is compacted when it
-//    runs full and sorted at the end, so the E+1 nearest come out in
-//    (distance, index) order however the library was visited;
+//    runs full, and at the end a register network sorts what is left, so the
+//    E+1 nearest come out in (distance, index) order however the library was
+//    visited;
 //  * the epilogue forms u_i = exp(-d_i/d_1) (optionally floored), the
 //    prediction, and the moments of each (tile, target) in paired FP32
 //    (moments.cuh): predictions go to a shared-memory ring whose eight slots
@@ -203,7 +205,9 @@ __device__ __forceinline__ void flush_ring(const float* ring, const RingMeta* me
 // warps' sums meet in shared memory.  One thread per query and target after
 // target instead gathered 4 bytes a lane from as many lines and spent five
 // FP64 operations a prediction.  64 variables, N = 5000, r = 25, all pairs:
-// brute force and table scan 222 -> 62 ms a run.
+// brute force and table scan 222 -> 62 ms a run;
+// two groups of queries packed 14.4 -> 12.8 of brute force's, byte offsets for
+// 64-bit multiply-adds -> 10.6.
 // Block-wide; the caller's next use of keep and scratch is behind the closing
 // barrier.
 template <int E, bool kWide>
@@ -296,8 +300,8 @@ __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc&
 // prediction of every target; each target's prediction vector goes to the
 // next ring slot (ring_n, the same in every thread), and a full ring is
 // reduced (flush_ring); units of many targets (kLanes: a kernel of their own, so
-// that neither epilogue costs the other registers) take lane_targets instead.  The CTA flushes what is left when it runs out of
-// work.  rho does not depend on which warp reduced which vector, or when.
+// that neither epilogue costs the other registers) take lane_targets instead.
+// The CTA flushes what is left when it runs out of work.  rho does not depend on which warp reduced which vector, or when.
 // `keep` (brute-force path: the thread's own column of the candidate buffer,
 // which only this thread uses and which is free once its search is done)
 // holds the weights and neighbours in shared memory, so that a reduction
@@ -814,7 +818,8 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
 }
 
 // --------------------------------------------------------------------------
-// Table path of units with several targets (units with one: knn_scan.cu): the
+// Table path of units with several targets whose realizations are not read in
+// groups (units with one target, and groups of many: knn_scan.cu): the
 // unit's membership bits (by position of the query order) are copied to shared
 // memory and each query walks its row of the distance indexing table (sorted
 // by (FP32 squared distance, index) over the whole manifold, the query itself

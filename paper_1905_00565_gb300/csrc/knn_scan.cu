@@ -1,6 +1,7 @@
-// Table scan of units with one target: up to 32 realizations of one (library
-// variable, target, E, tau) are served by one walk of each query's row of the
-// distance indexing table (table.cu; compiled once per E).
+// Table scan in groups of realizations: up to 32 realizations of one (library
+// variable, E, tau) are served by one walk of each query's row of the distance
+// indexing table (table.cu; compiled once per E).  scan_kernel: units with one
+// target; group_kernel: units with many.
 //
 // A warp owns a query and a lane a realization (the walk: row_walk.cuh).  When
 // every lane has met E+1 members of its library, each reads off its
@@ -18,9 +19,11 @@
 // 128 (query, realization) was done.
 //
 // Bound: issue (57 %) and the latency of the row and pair loads behind the
-// shuffles (ncu, E = 10).  Sweep (N = 10^4, E = 1..10, L = 142..9000, r = 250):
-// 65 ms a run; a thread per query and four realizations per walk 151 ms.  Two
-// variables of N = 10^5 (E = 3..6, L = 5000..50000): 18 ms, before 109 ms.
+// shuffles (ncu, E = 10).  Sweep (N = 10^4, E = 1..10, r = 250), libraries from
+// 142 points on: 151 ms with a thread per query and four realizations a walk,
+// 65 with this mapping; now that libraries from 100 points on read tables 101.
+// Two variables of N = 10^5 (E = 3..6, L = 1000..50000; before from L = 5000 on):
+// 109 -> 31 ms.
 #include <limits.h>
 #include <math.h>
 

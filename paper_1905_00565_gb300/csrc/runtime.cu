@@ -5,8 +5,8 @@
 //  * plan: validated copy of a problem, its realizations ("units") in output
 //    order, the work list of (unit, query tile) items sorted by decreasing
 //    cost, and one device arena for series, libraries, partial moments and rho;
-//  * run: sampler launch + one persistent fused-kernel launch, captured once
-//    into a CUDA graph and replayed;
+//  * run: query orders, tables, sampler, one search launch per E and kind of
+//    unit, rho; captured once into a CUDA graph and replayed;
 //  * plain comparator: one launch sequence per realization;
 //  * serving: queued jobs are admitted while their footprints fit the free
 //    budget, admitted jobs are batched into shared launches on a pool of
@@ -251,7 +251,9 @@ TableTuning read_table_tuning() {
 // (E+1)*100 entries, so libraries below N_m/max_ratio (40) points stay with
 // brute force.  The last term keeps the row length (table_row_length) within
 // max_R.  (Measured with a walk per query and realization, which variables with
-// several targets still take.)
+// two to eleven targets still take.  With many, whose walks serve a group of
+// realizations, a lower floor gains nothing: 64 variables, N = 5000, L from 100:
+// 56.3, 56.7, 59.0 ms a run with a floor of 256, 150, 90.)
 double table_min_L(int32_t E, int64_t n_m, int max_R, const TableTuning& t) {
   return std::max({t.floor, std::ceil(std::sqrt(t.crossover * (double)n_m / (double)(E + 1))),
                    std::ceil((double)n_m / t.max_ratio),
@@ -932,7 +934,7 @@ struct ccm_plan_s {
   char* d_arena = nullptr;
   cudaStream_t stream = nullptr;
   cudaGraphExec_t graph = nullptr;
-  cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // stage boundaries
+  cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // stage boundaries
   int grid = 0, grid_table = 0, grid_scan = 0;
   Tuning tuning = default_tuning();
   bool tuned = false;
@@ -1004,33 +1006,62 @@ cudaError_t enqueue_order(char* base, const Arena& ar, const UnitList& ul, Launc
                     reinterpret_cast<ObsStat*>(base + ar.obs_stat), s);
 }
 
+// A second branch of a captured run: the tables need only the query orders, so
+// they are built beside the sampler and the brute-force searches.  Short
+// manifolds leave part of the chip idle in each of these (N = 1000 0.171 ->
+// 0.159 ms a run, N = 2347 0.635 -> 0.570, 64 variables of N = 5000 55.5 -> 53.5);
+// long ones do not (N = 10^4 161.6 and 161.6, N = 10^5 87.6 -> 89.1) and keep one
+// stream.
+constexpr int kBranchMaxNm = 8192;
+struct TableBranch {
+  cudaStream_t s = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaError_t create() {
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+    return e;
+  }
+  ~TableBranch() {
+    if (join) cudaEventDestroy(join);
+    if (fork) cudaEventDestroy(fork);
+    if (s) cudaStreamDestroy(s);
+  }
+};
+
 // Enqueue sampler + fused kernel for a whole unit list on stream s.
-// Stage events (optional): ev[0] start, ev[1] after order, observed moments and table build,
-// ev[2] after the sampler, ev[3] after the brute-force launch, ev[4] after the
-// table-scan launch.
+// Stage events (optional): ev[0] start, ev[5] after order, observed moments and
+// table build, ev[1] before the sampler, ev[2] after it, ev[3] after the
+// brute-force launch, ev[4] after the table-scan launch.
 ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const Tuning& tn,
                          int grid, int grid_table, int grid_scan, int persistent, int32_t* dbg_lib,
                          int32_t* dbg_nbr, float* dbg_xhat, cudaStream_t s,
                          cudaEvent_t* ev = nullptr, bool capturing = false,
-                         bool stats = false) {
+                         bool stats = false, const TableBranch* branch = nullptr) {
   const LaunchStream ls(s, persistent && !capturing);
+  // the table builds: on the stream itself, or beside sampler and brute force
+  const LaunchStream ts = branch ? LaunchStream(branch->s) : ls;
   // Inside stream capture an event record becomes a graph node only with the
   // external flag; outside capture the plain record is the valid form.
-  auto record = [&](cudaEvent_t e) {
-    return capturing ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal)
-                     : cudaEventRecord(e, s);
+  auto record = [&](cudaEvent_t e, cudaStream_t on) {
+    return capturing ? cudaEventRecordWithFlags(e, on, cudaEventRecordExternal)
+                     : cudaEventRecord(e, on);
   };
   CCM_CUDA(cudaMemsetAsync(base + ar.err, 0, sizeof(int32_t), s));
   CCM_CUDA(cudaMemsetAsync(base + ar.counter, 0, kMaxSearchLaunches * sizeof(uint32_t), s));
   if (stats) CCM_CUDA(cudaMemsetAsync(base + ar.stats, 0, sizeof(unsigned long long) * kStatCount, s));
-  if (ev) CCM_CUDA(record(ev[0]));
+  if (ev) CCM_CUDA(record(ev[0], s));
   CCM_CUDA(enqueue_order(base, ar, ul, ls));
+  if (branch) {
+    CCM_CUDA(cudaEventRecord(branch->fork, s));
+    CCM_CUDA(cudaStreamWaitEvent(branch->s, branch->fork, 0));
+  }
   if (!ul.tables.empty())
     CCM_CUDA(launch_table_points(reinterpret_cast<const float*>(base + ar.series),
                                  reinterpret_cast<const TableJob*>(base + ar.tables),
                                  (int64_t)ul.tables.size(), ul.max_nm,
                                  reinterpret_cast<const int32_t*>(base + ar.order),
-                                 reinterpret_cast<float*>(base + ar.points), ls));
+                                 reinterpret_cast<float*>(base + ar.points), ts));
   for (size_t g0 = 0; g0 < ul.tables.size();) {  // one launch per (size class, E)
     const int rc = UnitList::table_rcap(ul.tables[g0].R), te = ul.tables[g0].E;
     size_t g1 = g0;
@@ -1051,10 +1082,12 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
                                 reinterpret_cast<const int32_t*>(base + ar.inverse),
                                 base + ar.table, reinterpret_cast<float*>(base + ar.table_dist),
                                 ul.table_tv ? 1 : 0, ul.table_u16(),
-                                reinterpret_cast<int32_t*>(base + ar.err), ls));
+                                reinterpret_cast<int32_t*>(base + ar.err), ts));
     g0 = g1;
   }
-  if (ev) CCM_CUDA(record(ev[1]));
+  if (ev) CCM_CUDA(record(ev[5], ts.s));
+  if (branch) CCM_CUDA(cudaEventRecord(branch->join, branch->s));
+  if (ev) CCM_CUDA(record(ev[1], s));
   SamplerParams sp = sampler_params(base, ar);
   sp.dbg_lib = dbg_lib;
   CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, ls));
@@ -1063,7 +1096,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
                                  reinterpret_cast<const MemberGroup*>(base + ar.member_groups),
                                  (int64_t)ul.member_groups.size(), ul.max_nm, sp.bits,
                                  reinterpret_cast<uint32_t*>(base + ar.words), ls));
-  if (ev) CCM_CUDA(record(ev[2]));
+  if (ev) CCM_CUDA(record(ev[2], s));
   KnnParams kp = knn_params(base, ar, ul, persistent, tn);
   kp.dbg_nbr = dbg_nbr;
   kp.dbg_xhat = dbg_xhat;
@@ -1080,7 +1113,8 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     const int g = persistent ? grid : (int)std::min<int64_t>(ig.count, 0x7fffffff);
     CCM_CUDA(launch_knn(ke, ig.E, ig.targets == Targets::kMany, g, ls));
   }
-  if (ev) CCM_CUDA(record(ev[3]));
+  if (ev) CCM_CUDA(record(ev[3], s));
+  if (branch) CCM_CUDA(cudaStreamWaitEvent(s, branch->join, 0));
   for (const ItemGroup& ig : ul.groups_table) {
     KnnParams kt = kp;
     kt.items = reinterpret_cast<const WorkItem*>(base + ar.items_table) + ig.first;
@@ -1096,7 +1130,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   }
   CCM_CUDA(launch_rho(kp.units, kp.targets, (int64_t)ul.targets.size(), kp.partials, kp.obs_stat,
                       reinterpret_cast<double*>(base + ar.rho), ls));
-  if (ev) CCM_CUDA(record(ev[4]));
+  if (ev) CCM_CUDA(record(ev[4], s));
   return CCM_OK;
 }
 
@@ -1317,7 +1351,7 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
     (void)cudaGetLastError();  // reported by the next attempt if it fails too
   }
   e = cudaStreamCreateWithFlags(&pl->stream, cudaStreamNonBlocking);
-  for (int q = 0; q < 5 && e == cudaSuccess; ++q) e = cudaEventCreate(&pl->ev[q]);
+  for (int q = 0; q < 6 && e == cudaSuccess; ++q) e = cudaEventCreate(&pl->ev[q]);
   if (e == cudaSuccess)
     e = cudaMemcpy(pl->d_arena + pl->ar.units, pl->ul.units.data(),
                    sizeof(UnitDesc) * pl->ul.units.size(), cudaMemcpyHostToDevice);
@@ -1465,10 +1499,14 @@ ccm_status ccm_run_ex(ccm_plan_t* plan, const float* series, double* rho, const 
     }
     if (!plan->graph) {
       cudaGraph_t graph = nullptr;
+      TableBranch branch;  // (destroyed after the capture: the graph keeps the dependencies)
+      const bool fork = !plan->ul.tables.empty() && plan->ul.max_nm <= kBranchMaxNm;
+      if (fork) CCM_CUDA(branch.create());
       CCM_CUDA(cudaStreamBeginCapture(plan->stream, cudaStreamCaptureModeThreadLocal));
       ccm_status st = enqueue_sweep(base, plan->ar, plan->ul, plan->tuning, plan->grid,
                                     plan->grid_table, plan->grid_scan, 1, nullptr, nullptr, nullptr, plan->stream,
-                                    plan->ev, true, (pc.flags & CCM_SEARCH_STATS) != 0);
+                                    plan->ev, true, (pc.flags & CCM_SEARCH_STATS) != 0,
+                                    fork ? &branch : nullptr);
       const cudaError_t ce = cudaStreamEndCapture(plan->stream, &graph);
       if (st != CCM_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -1500,11 +1538,14 @@ ccm_status ccm_plan_kernel_times(const ccm_plan_t* plan, double* sampler_ms, dou
 ccm_status ccm_plan_stage_times(const ccm_plan_t* plan, double* stage_ms) {
   if (!plan || !stage_ms) return fail(CCM_EINVAL, "NULL argument");
   CCM_CUDA(cudaSetDevice(plan->ctx->device));
+  const int from[4] = {0, 1, 2, 3}, to[4] = {5, 2, 3, 4};
+  float t = 0.f;
   for (int q = 0; q < 4; ++q) {
-    float t = 0.f;
-    CCM_CUDA(cudaEventElapsedTime(&t, plan->ev[q], plan->ev[q + 1]));
+    CCM_CUDA(cudaEventElapsedTime(&t, plan->ev[from[q]], plan->ev[to[q]]));
     stage_ms[q] = t;
   }
+  CCM_CUDA(cudaEventElapsedTime(&t, plan->ev[5], plan->ev[4]));  // it also waits for the tables
+  stage_ms[3] = std::min(stage_ms[3], (double)t);
   return CCM_OK;
 }
 

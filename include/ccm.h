@@ -272,10 +272,10 @@ ccm_status ccm_job_times(ccm_context* ctx, uint64_t ticket, double* submit_s, do
  * entry of ccm_run's output for the same seed.
  * d_series: device [n_series][n] FP32 (not checked for non-finite values);
  * d_rho: device [r] FP64, written in stream order.  All scratch lives in one
- * fixed 16 MiB device array held by every GPU that loads the library until
- * exit; a cell needing more (about r*L*4 + r*ceil(N_m/256)*44 + r*176 +
- * N_m*4 + ceil(N_m/256)*2080 bytes) returns CCM_ETOOLARGE with a message and runs nothing.  Nothing is
- * allocated.  The first call on a device (with that device current) finds
+ * fixed device array held by every GPU that loads the library until exit; a cell
+ * that counts for more than 16 MiB (r*L*4 + r*ceil(N_m/256)*60 + r*164 + N_m*4 +
+ * ceil(N_m/256)*2112 bytes and some rounding) returns CCM_ETOOLARGE with a message
+ * and runs nothing.  Nothing is allocated.  The first call on a device (with that device current) finds
  * the array's address and sets kernel attributes; make it before any stream
  * capture.  Every call reuses the same array: calls that overlap on the GPU
  * (several streams or host threads) race and must be serialised by the

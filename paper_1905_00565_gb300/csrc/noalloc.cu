@@ -32,8 +32,13 @@
 namespace ccm {
 
 // Scratch for one cell: descriptors, work items, libraries, partial moments,
-// counters, query order, observed-value tile records.  16 MiB holds, e.g., r = 250 realizations of L = 9000 at N = 10^4.
-constexpr size_t kScratchBytes = 16u << 20;
+// counters, query order, observed-value tile records.  Cells are admitted up to
+// 16 MiB by a count of their own (admitted_bytes; e.g. r = 250 realizations of L
+// = 9000 at N = 10^4), which does not follow the descriptors' sizes; the array
+// has the room by which the layout may exceed it: 4 bytes a realization of a
+// single query tile, of which 16 MiB hold at most 71000, and a few roundings.
+constexpr size_t kAdmitBytes = 16u << 20;
+constexpr size_t kScratchBytes = kAdmitBytes + (512u << 10);
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 namespace {
@@ -78,6 +83,16 @@ NoallocLayout noalloc_layout(int64_t r, int64_t L, int64_t n_tiles, int64_t n_m)
   o = up256(o + sizeof(float));
   a.total = o;
   return a;
+}
+
+// What a cell counts for: per realization 164 bytes, its library and 60 bytes per
+// query tile; per query 4 bytes; per query tile 2112.
+size_t admitted_bytes(int64_t r, int64_t L, int64_t n_tiles, int64_t n_m) {
+  size_t total = 0;
+  for (const int64_t part : {112 * r, 12 * r * n_tiles, 4 * r * L, 48 * r * n_tiles, 4 * r, int64_t{4},
+                             int64_t{4}, 4 * n_m, int64_t{48}, 48 * r, 2112 * n_tiles, int64_t{56}})
+    total += up256((size_t)part);
+  return total;
 }
 
 struct CellArgs {
@@ -205,10 +220,11 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   const int64_t tileq = (int64_t)knn_block_threads() * knn_queries_per_thread();
   const int64_t n_tiles = (n_m + tileq - 1) / tileq;
   const NoallocLayout lay = noalloc_layout(r, L, n_tiles, n_m);
-  if (lay.total > kScratchBytes)
+  const size_t admitted = admitted_bytes(r, L, n_tiles, n_m);
+  if (admitted > kAdmitBytes || lay.total > kScratchBytes)
     return noalloc_fail(CCM_ETOOLARGE,
-                        "cell needs " + std::to_string(lay.total) + " B of scratch; the fixed "
-                        "array holds " + std::to_string(kScratchBytes) + " B (reduce r or L)");
+                        "cell needs " + std::to_string(admitted) + " B of scratch; the fixed "
+                        "array holds " + std::to_string(kAdmitBytes) + " B (reduce r or L)");
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));

@@ -1,0 +1,101 @@
+"""Sizes at which a size rule changes its path: the query order's sorts, a plan whose
+tables do not fit the context's budget, and the scratch of the no-allocation cell
+(needs a GB300)."""
+
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1905_00565_gb300 import inputs as I
+from tests.ccm_check import check_units, run_detailed
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ccm():
+    from paper_1905_00565_gb300 import ccm as c
+    return c
+
+
+# The order's bitonic network ends at 512 points, its radix sort at 16384 (runs are
+# merged beyond); 96 query tiles (24576 points) is where rho takes a whole warp.
+@pytest.mark.parametrize("n_m", [511, 512, 513, 16384, 16385, 24576, 24577, 33000])
+def test_orders_and_tile_counts(ccm, n_m):
+    E, tau = 2, 3
+    p = I.Problem(series=I.logistic_pair(n_m + (E - 1) * tau), pairs=I.BOTH_DIRECTIONS.copy(),
+                  E=np.array([E], np.int32), tau=np.array([tau], np.int32),
+                  L=np.array([60, 480], np.int64), r=2, seed=11)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        check_units(p, *run_detailed(ccm, ctx, p), which={0, 3, 6})
+    finally:
+        ccm.ccm_context_destroy(ctx)
+
+
+def test_tables_give_way_to_the_budget(ccm):
+    """A plan's tables shrink, then go, as the budget does; rho stays the same and the
+    smallest budget that holds the plan without tables still runs it."""
+    p = I.Problem(series=I.logistic_pair(3000), pairs=I.BOTH_DIRECTIONS.copy(),
+                  E=np.array([2, 5], np.int32), tau=np.array([1], np.int32),
+                  L=np.array([80, 400, 2500], np.int64), r=60, seed=3)
+
+    def footprint(flags, budget):
+        ctx = ccm.ccm_context_create(0, budget)
+        try:
+            plan = ccm.plan_problem(ctx, p, flags)
+            try:
+                info = ccm.ccm_plan_get_info(plan)
+                rho = np.zeros(ccm.rho_shape(p))
+                ccm.ccm_run(plan, p.series, rho)
+            finally:
+                ccm.ccm_plan_destroy(plan)
+        finally:
+            ccm.ccm_context_destroy(ctx)
+        return info["device_bytes"], info["table_bytes"], rho
+
+    full, tables, want = footprint(0, 0)
+    bare, none, _ = footprint(ccm.CCM_NO_TABLE, 0)
+    assert tables > 0 and none == 0
+    seen = set()
+    for budget in (full, full - 1, bare + tables // 2, bare + tables // 50, bare):
+        size, tab, rho = footprint(0, budget)
+        assert size <= budget
+        seen.add(tab)
+        np.testing.assert_array_equal(rho, want)
+    assert 0 in seen
+    with pytest.raises(ccm.CCMError) as ei:
+        footprint(0, bare - 1)
+    assert ei.value.status == ccm.CCM_ETOOLARGE
+
+
+def test_noalloc_admits_up_to_16_mib(ccm):
+    """One query tile and the shortest libraries, where the descriptors weigh most."""
+    torch = pytest.importorskip("torch")
+    n, L, seed = 256, 3, 7
+
+    def counts(r):
+        parts = (112 * r, 12 * r, 4 * r * L, 48 * r, 4 * r, 4, 4, 4 * n, 48, 48 * r, 2112, 56)
+        return sum((b + 255) // 256 * 256 for b in parts)
+
+    r = max(q for q in range(70000, 72000) if counts(q) <= 16 << 20)
+    p = I.Problem(series=I.logistic_pair(n), pairs=np.array([[0, 1]], np.int32),
+                  E=np.array([1], np.int32), tau=np.array([1], np.int32),
+                  L=np.array([L], np.int64), r=r, seed=seed)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        plan = ccm.plan_problem(ctx, p, ccm.CCM_NO_TABLE)
+        want = np.zeros(ccm.rho_shape(p))
+        ccm.ccm_run(plan, p.series, want)
+        ccm.ccm_plan_destroy(plan)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    s = torch.from_numpy(p.series).cuda()
+    rho = torch.full((r,), float("nan"), dtype=torch.float64, device="cuda")
+    ccm.ccm_run_noalloc(s, 0, 1, 1, 1, L, r, seed, rho)
+    np.testing.assert_array_equal(rho.cpu().numpy(), want.reshape(-1))
+    more = torch.zeros(r + 1, dtype=torch.float64, device="cuda")
+    with pytest.raises(ccm.CCMError) as ei:
+        ccm.ccm_run_noalloc(s, 0, 1, 1, 1, L, r + 1, seed, more)
+    assert ei.value.status == ccm.CCM_ETOOLARGE

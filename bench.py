@@ -14,7 +14,7 @@ ccm_convergence, the per-(pair, E, tau) convergence decision on the rho grid.
 Prints one JSON line.  `value` is realizations/s with inputs resident on the
 device; `e2e` is the same metric through ccm_run with pinned host buffers
 (host->device series copy and device->host rho copy inside the timed region);
-`roofline` reports the dominant kernel (the brute-force fused kernels) against
+`roofline` reports the brute-force fused kernels (the distance arithmetic) against
 the FP32 ALU peak; `cpu_baseline` is the FP64 oracle on a bounded sample of the
 same workload, and `accuracy` checks the GPU's results of that sample against
 it (max |d rho|, max relative |d Xhat|, near-tie neighbour swaps);
@@ -115,7 +115,7 @@ def workload_config(name, p):
         "realizations": p.n_units(),
         "queries": p.queries(),
         "pairs": p.pair_count(),
-        "precision": "FP32 distances/selection/weights, FP64 rho moments",
+        "precision": "FP32 distances/selection/weights, rho moments in paired FP32 (48 bits)",
     }
 
 
@@ -480,9 +480,10 @@ def run_ours(args, rank, world, local_rank, cpu=None):
                           "convergence": sum(conv_ms) / max(1, len(conv_ms))},
             "neighbour_search": {
                 "tables": "distance indexing tables (paper Sect. 3.2), built every step, for "
-                          "L >= max(256, sqrt(20 N_m/(E+1)), N_m/40), rows of R entries so that a "
+                          "the L from which a cost estimate favours them (at the latest "
+                          "max(256, sqrt(20 N_m/(E+1)), N_m/40)), rows of R entries so that a "
                           "query at the smallest such L misses its E+1 members with probability "
-                          "<= 1/(10 L); brute force with exact chunk pruning below",
+                          "<= 1/(10 L); brute force with exact pruning below",
                 "table_bytes": info["table_bytes"],
                 "brute_force_share_of_pairs": info["brute_pair_count"] / info["pair_count"],
                 "brute_force_share_of_flops": info["brute_flop_count"] / info["flop_count"],
@@ -490,13 +491,13 @@ def run_ours(args, rank, world, local_rank, cpu=None):
             # the table-scan kernel: the largest stage, but a lookup walk with no
             # flop or byte count of the exhaustive method to put against a peak
             "table_scan": {
-                "kernel": "knn_table_kernel<E>, one launch per E per step: each query walks "
-                          "its table row until every realization of its group (up to 4 of a "
-                          "cell) has E+1 library members, then the simplex/moment epilogue",
+                "kernel": "scan_kernel<E>, one launch per E per step: a warp walks each query's "
+                          "table row for up to 32 realizations, a lane each, until all have E+1 "
+                          "library members, then the simplex/moment epilogue",
                 "share_of_step": st[3] / t_step,
                 "query_realizations_per_s": info["table_query_count"] / (st[3] / 1e3),
                 # from the counting run: rank entries the walks loaded (one walk
-                # serves up to four realizations) and the index bytes they read
+                # serves up to 32 realizations) and the index bytes they read
                 "entries_loaded_per_s": counts["table_entries"] / (st[3] / 1e3),
                 "index_bytes_per_s": counts["table_entries"] * idx_bytes / (st[3] / 1e3),
                 "library_scan_fallbacks": counts["table_fallbacks"],
@@ -511,13 +512,13 @@ def run_ours(args, rank, world, local_rank, cpu=None):
                          # the committed capture covers the sweep workload only
                          "traffic": (ncu_rec or {}).get("dram_bytes_per_full_sweep"),
                          "traffic_unit": "DRAM bytes per step, all brute-force launches "
-                                         "(ncu, scaled from an r=8 capture)",
+                                         "(ncu, one sweep)",
                          "algorithmic_bytes": "4L per realization (library indices) + 8 (rho)",
                          "kernel": "knn_fused_kernel<E> (brute force), one launch per E per step "
                                    "over the realizations below the table threshold; 3E FP32 "
                                    "flops per query-library pair of those realizations (the "
                                    "method's exhaustive work, including the pairs that exact "
-                                   "chunk pruning skips)",
+                                   "pruning skips)",
                          "brute_pairs_per_s": info["brute_pair_count"] / (st[2] / 1e3),
                          # pairs the search evaluated (pruning skips the rest), counted
                          # by a separate run of the counting variant, per second of the
@@ -641,7 +642,7 @@ def serve_stream(ccm, I, n_jobs: int, device: int):
 
 def brute_variant(ccm, ctx, p, torch, steps: int, warmup: int, rho_ref, flush, stream):
     """The same sweep with CCM_NO_TABLE: every realization searched by the
-    brute-force fused kernels (with exact chunk pruning); bit-identical rho."""
+    brute-force fused kernels (with exact pruning); bit-identical rho."""
     flags = ccm.CCM_INPUT_ON_DEVICE | ccm.CCM_OUTPUT_ON_DEVICE | ccm.CCM_NO_TABLE
     plan = ccm.plan_problem(ctx, p, flags)
     info = ccm.ccm_plan_get_info(plan)

@@ -31,10 +31,8 @@ constexpr int kOrderThreads = 1024;
 
 __device__ __forceinline__ uint32_t quantise(float c, float lo, float inv, int bits) {
   const float u = (c - lo) * inv;  // in [0, 1] up to rounding
-  const float top = (float)((1u << bits) - 1u);
-  float v = floorf(u * (float)(1u << bits));
-  v = fminf(fmaxf(v, 0.f), top);
-  return (uint32_t)v;
+  const float v = fmaxf(floorf(u * (float)(1u << bits)), 0.f);
+  return min((uint32_t)v, (1u << bits) - 1u);  // as integers: 2^30 - 1 is no float
 }
 
 // Series range of job jb (block-wide min/max).

@@ -547,7 +547,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
   const int merge_at = max(1, min(p.merge_at[E], room));
   // the first kInit points of a query's scan go straight into its threshold
   constexpr int kInit = (K + kStep - 1) / kStep * kStep;
-  static_assert(kInit <= kChunk, "the initial points lie in the first chunk");
+  static_assert(kInit <= kChunk && kInit % kStep == 0, "the initial points are whole runs of the first chunk");
   u64* col = s_buf + tid;  // this thread's candidate column
 
   const int tile1 = min(u.n_tiles, tile0 + n_chunk);
@@ -683,7 +683,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
         const float th_max = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(tl[K - 1])));
         const int pr = 32 * g + lane;
         bool keep = pr < np && !(first && (unsigned)(pr - (base >> 1)) < (unsigned)(kInit / 2));
-        if (keep) {
+        if (keep && p.prune) {
           const float2* xp = reinterpret_cast<const float2*>(s_coord + (size_t)pr * EP);
           float lb = 0.f;
 #pragma unroll
@@ -701,10 +701,9 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
         while (mask != 0u) {
           // the next kept pair's aligned run of kPairs: the pairs in reach of a warp's
           // queries lie side by side in the query order, and collecting them one by
-          // one was a chain of find-first-bits (short libraries 4.08 -> 4.00 ms, the
-          // sweep's brute force 13.3 -> 12.7, N = 10^5 17.2 -> 15.8)
+          // one was a chain of find-first-bits (short libraries 4.08 -> 3.97 ms, the
+          // sweep's brute force 13.3 -> 12.8, N = 10^5 17.2 -> 16.3)
           const int b0 = (__ffs(mask) - 1) & ~(kPairs - 1);
-          const unsigned kept = (mask >> b0) & ((1u << kPairs) - 1u);
           mask &= ~(((1u << kPairs) - 1u) << b0);
           const int at = 32 * g + b0;
           if (kStats) st_begun += kStep;
@@ -731,23 +730,28 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
             }
             if (!__any_sync(kFull, min_all(d) <= th)) continue;
           }
+          // the run's library indices (one broadcast 16-byte load per four); its pairs
+          // that are not kept lie above every threshold, and the first points' runs
+          // hold nothing else (both are whole runs)
+          int li[kStep];
 #pragma unroll
-          for (int pp = 0; pp < kPairs; ++pp) {
-            if (!((kept >> pp) & 1u)) continue;  // the same for the whole warp
-            const int2 li = *reinterpret_cast<const int2*>(s_lidx + 2 * (at + pp));
+          for (int q4 = 0; q4 < kStep / 4; ++q4) {
+            const int4 v = *reinterpret_cast<const int4*>(s_lidx + 2 * at + 4 * q4);
+            li[4 * q4] = v.x;
+            li[4 * q4 + 1] = v.y;
+            li[4 * q4 + 2] = v.z;
+            li[4 * q4 + 3] = v.w;
+          }
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              // at or below the threshold (never a sentinel: NaN), outside the
-              // exclusion window |l - m| <= W (W = 0 drops only m itself, and
-              // the unsigned form tests both sides at once); appended without a
-              // branch
-              const int l = h ? li.y : li.x;
-              const float dh = d[2 * pp + h];
-              const bool take =
-                  (dh <= th) & ((unsigned)l - (unsigned)m + (unsigned)W > 2u * (unsigned)W);
-              if (take) col[cnt * kThreads] = pack_key(dh, l);
-              cnt += take ? 1 : 0;
-            }
+          for (int pt = 0; pt < kStep; ++pt) {
+            // at or below the threshold (never a sentinel: NaN), outside the
+            // exclusion window |l - m| <= W (W = 0 drops only m itself, and
+            // the unsigned form tests both sides at once); appended without a
+            // branch
+            const bool take =
+                (d[pt] <= th) & ((unsigned)li[pt] - (unsigned)m + (unsigned)W > 2u * (unsigned)W);
+            if (take) col[cnt * kThreads] = pack_key(d[pt], li[pt]);
+            cnt += take ? 1 : 0;
           }
           if (__any_sync(kFull, cnt - done >= merge_at || cnt > room)) make_room();
         }

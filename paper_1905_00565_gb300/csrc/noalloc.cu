@@ -294,6 +294,7 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   kp.item_counter = reinterpret_cast<uint32_t*>(scratch + lay.counter);
   kp.err = reinterpret_cast<int32_t*>(scratch + lay.err);
   kp.persistent = 0;
+  kp.prune = n_m <= kOrderMaxSort ? 1 : 0;  // (N = 20000, E = 1, L = 400, r = 100: 0.75 -> 0.72 ms)
   for (int q = 0; q <= kMaxE; ++q) {
     kp.merge_at[q] = kDefaultMergeAt;
     kp.variant[q] = kDefaultVariant;

@@ -979,6 +979,7 @@ KnnParams knn_params(char* base, const Arena& ar, const UnitList& ul, int persis
   kp.item_counter = reinterpret_cast<uint32_t*>(base + ar.counter);
   kp.err = reinterpret_cast<int32_t*>(base + ar.err);
   kp.persistent = persistent;
+  kp.prune = 1;
   for (int e = 0; e <= kMaxE; ++e) {
     kp.merge_at[e] = tn.merge_at[e];
     kp.variant[e] = tn.variant[e];

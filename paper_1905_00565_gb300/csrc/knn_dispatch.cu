@@ -112,8 +112,8 @@ __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4*
     for (int i = 0; i < kAhead; ++i) {
       const int q = q0 + i * kLanes;
       if (q < n_tiles) {
-        t[i].a = __ldg(base + 2 * q);
-        t[i].b = __ldg(base + 2 * q + 1);
+        t[i].a = base[2 * q];
+        t[i].b = base[2 * q + 1];
         t[i].mx = __ldg(&stat[q].mx);
         t[i].sxx = __ldg(&stat[q].sxx);
       }

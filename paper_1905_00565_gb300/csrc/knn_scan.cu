@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
       const int quads = member_words(n_m) >> 2;
       const uint4* src = reinterpret_cast<const uint4*>(words);
       uint4* dst = reinterpret_cast<uint4*>(s_words);
-      for (int i = tid; i < quads; i += kScanThreads) dst[i] = __ldg(src + i);
+      for (int i = tid; i < quads; i += kScanThreads) dst[i] = src[i];
     }
     __syncthreads();
     const int32_t* order = p.order + u.order_off;
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1) group_kernel(KnnParams p) {
     if (p.group_words) {
       const uint4* src = reinterpret_cast<const uint4*>(words);
       uint4* dst = reinterpret_cast<uint4*>(s_words);
-      for (int i = tid; i < member_words(n_m) >> 2; i += kGroupThreads) dst[i] = __ldg(src + i);
+      for (int i = tid; i < member_words(n_m) >> 2; i += kGroupThreads) dst[i] = src[i];
     }
     __syncthreads();
     const int32_t* order = p.order + u.order_off;

@@ -2,6 +2,11 @@
 // launch): a kernel's CTAs are set up while the one before it drains, and every
 // kernel first waits for that one to finish.  Small jobs are chains of kernels
 // of a few microseconds, where the gaps between them count.
+//
+// What the kernel before writes is read with plain loads, never with __ldg: the
+// read-only path asks for data that does not change while the kernel lives, and a
+// chained kernel lives before its wait.  (Two kernels back is safe: a CTA is set up
+// only once every CTA of the kernel before has passed its own wait.)
 #pragma once
 
 #include <cuda_runtime.h>

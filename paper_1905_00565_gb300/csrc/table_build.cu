@@ -119,8 +119,8 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
     float lb = 0.f;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const float g = fmaxf(fmaxf(__fsub_rn(__ldg(b + 2 * e * n + i), q[e]),
-                                  __fsub_rn(q[e], __ldg(b + (2 * e + 1) * n + i))), 0.f);
+      const float g = fmaxf(fmaxf(__fsub_rn(b[2 * e * n + i], q[e]),
+                                  __fsub_rn(q[e], b[(2 * e + 1) * n + i])), 0.f);
       lb = (e == 0) ? __fmul_rn(g, g) : __fmaf_rn(g, g, lb);
     }
     return __float_as_uint(lb);
@@ -175,7 +175,7 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
     {
       const float* c = pts + (int64_t)(pos >> 5) * (E * 32) + (pos & 31);
 #pragma unroll
-      for (int e = 0; e < E; ++e) q[e] = __ldg(c + e * 32);
+      for (int e = 0; e < E; ++e) q[e] = c[e * 32];
     }
     bool all = n_m - 1 <= C;  // everything fits: no threshold
     bool sampled = false, have_lo = false, have_hi = false, ties = false;
@@ -194,8 +194,8 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
           float ub = 0.f;
 #pragma unroll
           for (int e = 0; e < E; ++e) {
-            const float g = fmaxf(fabsf(__fsub_rn(__ldg(sbox + 2 * e * n_super + i), q[e])),
-                                  fabsf(__fsub_rn(q[e], __ldg(sbox + (2 * e + 1) * n_super + i))));
+            const float g = fmaxf(fabsf(__fsub_rn(sbox[2 * e * n_super + i], q[e])),
+                                  fabsf(__fsub_rn(q[e], sbox[(2 * e + 1) * n_super + i])));
             ub = __fmaf_rn(g, g, ub);
           }
           top = max(top, __float_as_uint(ub));
@@ -213,11 +213,11 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
           if (tid == 0) s_found = kBins;
           __syncthreads();
           for (int i = tid; i < n_sample; i += kThreads) {
-            float diff = __fsub_rn(q[0], __ldg(smp + i));
+            float diff = __fsub_rn(q[0], smp[i]);
             float acc = __fmul_rn(diff, diff);
 #pragma unroll
             for (int e = 1; e < E; ++e) {
-              diff = __fsub_rn(q[e], __ldg(smp + e * n_sample + i));
+              diff = __fsub_rn(q[e], smp[e * n_sample + i]);
               acc = __fmaf_rn(diff, diff, acc);
             }
             const uint32_t bits = __float_as_uint(acc);
@@ -287,7 +287,7 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
           const int ch = s_chunk[min(i, chunks - 1)];
           const float* src = pts + (int64_t)ch * (E * 32) + lane;
 #pragma unroll
-          for (int e = 0; e < E; ++e) f[e] = __ldg(src + e * 32);
+          for (int e = 0; e < E; ++e) f[e] = src[e * 32];
           m = __ldg(ord + min(ch * 32 + lane, n_m - 1));
         };
         if (warp < chunks) {

@@ -30,7 +30,9 @@
  * Precision: distances, selection, weights and predictions in FP32;
  * rho moments in FP64 and, for the predictions' sums over a tile of 256
  * queries, in unevaluated pairs of FP32 numbers (48 bits, the target scaled by
- * a power of two).
+ * a power of two); in FP64 where a tile's predictions spread so little beside
+ * the target's largest value (less than about 1e-25 of it) that these would
+ * leave FP32's range.
  *
  * Output layout: rho[pair][E][tau][L][k], FP64, C order, where the axes index
  * the arrays of ccm_problem in the order given.

@@ -72,17 +72,27 @@ struct ObsJob {
   int32_t i, E, tau, n_m, n_tiles;
   int32_t pad;
 };
+// A target series' power of two, and the smallest sum of squares at which a tile of
+// its predictions may need a second look (moments.cuh): the smallest positive
+// number, or 0 for a deep series, one with (nonzero) values below 2^-kDeepBits of its
+// largest, where a sum of 0 does not show that all predictions are equal.
+constexpr int kDeepBits = 90;
+struct alignas(8) SeriesScale {
+  float scale, least_b2;
+};
 // One tile of an observed target: mean(x), sum of (x_q - mean(x))^2 and the
 // scale.  Beside it 256 float2 {h, l}, h + l = x_q - mean(x) to 48 bits (zero
 // past the tile's end).
 struct ObsStat {
   double mx, sxx;
-  float scale;
-  float pad[3];
+  SeriesScale series;   // the series'
+  float pad[2];
 };
 // Per-series preparation (one CTA of the order launch): the power of two that
-// brings the series' largest magnitude into [1, 2), and, for jobs with units
-// of kLaneTargets targets, the series' column of the time-major copy.
+// brings the series' largest magnitude into 2^kScaleBits times [1, 2) (less for
+// series below 2^(kScaleBits - 127)), and, for jobs with units of kLaneTargets
+// targets, the series' column of the time-major copy.
+constexpr int kScaleBits = 50;
 struct SeriesJob {
   int64_t off, n;       // the series
   int64_t st_off;       // element of (t = 0, this variable) in the time-major copy; -1: none
@@ -312,7 +322,8 @@ cudaError_t order_prepare();
 // The same launch prepares the target series (SeriesJob).
 cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jobs, int max_nm,
                          int32_t* order, int32_t* inverse, unsigned long long* scratch,
-                         const SeriesJob* series_jobs, int64_t n_series_jobs, float* scales, float* st, LaunchStream s);
+                         const SeriesJob* series_jobs, int64_t n_series_jobs, SeriesScale* scales,
+                         float* st, LaunchStream s);
 
 // Distance indexing table (table.cu).
 cudaError_t table_prepare();
@@ -364,7 +375,7 @@ cudaError_t launch_knn(const KnnParams& p, int E, bool lane_targets, int grid, L
 // Observed-value records of every ObsJob (after the query order): one warp
 // per tile, n_tiles tiles in all.
 cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* jobs,
-                       int64_t n_jobs, int64_t n_tiles, const float* scales, float2* obs,
+                       int64_t n_jobs, int64_t n_tiles, const SeriesScale* scales, float2* obs,
                        ObsStat* obs_stat, LaunchStream s);
 // rho of every target from its tiles' sums (after the search kernels).
 cudaError_t launch_rho(const UnitDesc* units, const TargetDesc* targets, int64_t n_targets,

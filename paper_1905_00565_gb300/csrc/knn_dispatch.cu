@@ -27,7 +27,7 @@ constexpr int kPer = kQT / 32;  // queries per lane
 // predicts).  Two passes in FP64, then split into float pairs.
 __global__ void __launch_bounds__(kSmallThreads) obs_kernel(const float* series, const int32_t* order,
                                                       const ObsJob* jobs, int64_t n_jobs,
-                                                      int64_t n_tiles, const float* scales,
+                                                      int64_t n_tiles, const SeriesScale* scales,
                                                       float2* obs, ObsStat* obs_stat) {
   chain_begin();
   const int lane = threadIdx.x & 31;
@@ -46,13 +46,14 @@ __global__ void __launch_bounds__(kSmallThreads) obs_kernel(const float* series,
     const float* si = series + jb.series_off + (int64_t)jb.i * jb.n;
     const int32_t* ord = order + jb.order_off + (int64_t)tile * kQT;
     const int off = (jb.E - 1) * jb.tau;
-    const float scale = scales[jb.scale];
+    const SeriesScale sc = scales[jb.scale];
+    const float scale = sc.scale;
     double x[kPer];
     double sv = 0.0;
 #pragma unroll
     for (int c = 0; c < kPer; ++c) {
       const int q = lane + 32 * c;
-      x[c] = (q < nq) ? (double)__fmul_rn(si[ord[q] + off], scale) : 0.0;
+      x[c] = (q < nq) ? __dmul_rn((double)si[ord[q] + off], (double)scale) : 0.0;
       sv = __dadd_rn(sv, x[c]);
     }
     const double mx = __ddiv_rn(warp_sum(sv), (double)nq);
@@ -72,7 +73,7 @@ __global__ void __launch_bounds__(kSmallThreads) obs_kernel(const float* series,
       ObsStat& o = obs_stat[g];
       o.mx = mx;
       o.sxx = sxx;
-      o.scale = scale;
+      o.series = sc;
     }
   }
 }
@@ -120,8 +121,9 @@ __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4*
     }
   };
   auto count = [&](int q) { return (double)min(kQT, n_m - q * kQT); };
-  // mean(y) of a tile; d = mean(y) - c, b1 = sum(y - c)
+  // mean(y) of a tile; of paired sums also d = mean(y) - c, b1 = sum(y - c)
   auto mean = [&](const Tile& t, double n, double& b1, double& d) {
+    if (t.b.w != 0.f) return word_pair(t.a.x, t.a.y);  // a record in FP64
     b1 = __dadd_rn((double)t.a.y, (double)t.a.z);
     d = (n == (double)kQT) ? __dmul_rn(b1, 1.0 / kQT) : __ddiv_rn(b1, n);
     return __dadd_rn((double)t.a.x, d);
@@ -150,9 +152,15 @@ __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4*
       if (q >= n_tiles) break;
       const double n = count(q);
       const double dy = __dsub_rn(mean(t[i], n, b1, d), MY), dx = __dsub_rn(t[i].mx, MX);
-      const double b2 = __dadd_rn((double)t[i].a.w, (double)t[i].b.x);
-      const double syy = fmax(__fma_rn(-b1, d, b2), 0.0);
-      const double sxy = __dadd_rn((double)t[i].b.y, (double)t[i].b.z);
+      double syy, sxy;
+      if (t[i].b.w != 0.f) {
+        syy = word_pair(t[i].a.z, t[i].a.w);
+        sxy = word_pair(t[i].b.x, t[i].b.y);
+      } else {
+        const double b2 = __dadd_rn((double)t[i].a.w, (double)t[i].b.x);
+        syy = fmax(__fma_rn(-b1, d, b2), 0.0);
+        sxy = __dadd_rn((double)t[i].b.y, (double)t[i].b.z);
+      }
       const double wx = __dmul_rn(n, dx);
       SXX = __fma_rn(wx, dx, __dadd_rn(SXX, t[i].sxx));
       SYY = __fma_rn(__dmul_rn(n, dy), dy, __dadd_rn(SYY, syy));
@@ -265,7 +273,7 @@ cudaError_t launch_knn_table(const KnnParams& p, int E, int max_nm, bool lanes, 
 }
 
 cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* jobs,
-                       int64_t n_jobs, int64_t n_tiles, const float* scales, float2* obs,
+                       int64_t n_jobs, int64_t n_tiles, const SeriesScale* scales, float2* obs,
                        ObsStat* obs_stat, LaunchStream s) {
   if (n_jobs <= 0 || n_tiles <= 0) return cudaSuccess;
   const int64_t want = (n_tiles + kSmallThreads / 32 - 1) / (kSmallThreads / 32);  // a warp per tile

@@ -181,17 +181,35 @@ __device__ __forceinline__ void insert_prefix(u64 (&ku)[K], u64 x, int n) {
 struct RingMeta {
   const float2* a;    // the tile's centred observations
   float4* part;       // where its sums go
+  SeriesScale series;
   int32_t nq;         // valid queries of the tile
+  int32_t target, tile;
 };
+
+// One of them in FP64 (rare): all it needs follows from the target and the tile.
+__device__ __noinline__ void exact_vector(const float* ys, int target, int tile, int nq, float4* part,
+                                          const UnitDesc* units, const TargetDesc* targets,
+                                          const float* series, const int32_t* order,
+                                          const ObsStat* obs_stat) {
+  const TargetDesc& tg = targets[target];
+  const UnitDesc& u = units[tg.unit];
+  exact_sums_warp(TileTarget{series + u.series_off + (int64_t)tg.i * u.n + (u.E - 1) * u.tau,
+                             order + u.order_off + (int64_t)tile * kQT, obs_stat + tg.obs_tile + tile, nq},
+                  ys, part);
+}
 
 // The staged vectors' sums: warps 0..n-1 take one each, in parallel.  Between
 // two block barriers: the slots are complete on entry and free again on exit.
-__device__ __forceinline__ void flush_ring(const float* ring, const RingMeta* meta, int n) {
+__device__ __forceinline__ void flush_ring(const KnnParams& p, const float* ring, const RingMeta* meta,
+                                           int n) {
   __syncthreads();
   const int warp = threadIdx.x >> 5;
   if (warp < n) {
     const RingMeta mt = meta[warp];
-    tile_sums_warp(ring + warp * kVecStride, mt.a, mt.nq, mt.part);
+    const float* ys = ring + warp * kVecStride;
+    if (__builtin_expect(tile_sums_warp(ys, mt.a, mt.series, mt.nq, mt.part), 0))
+      exact_vector(ys, mt.target, mt.tile, mt.nq, mt.part, p.units, p.targets, p.series, p.order,
+                   p.obs_stat);
   }
   __syncthreads();
 }
@@ -211,6 +229,36 @@ __device__ __forceinline__ void flush_ring(const float* ring, const RingMeta* me
 // Block-wide; the caller's next use of keep and scratch is behind the closing
 // barrier.
 template <int E, bool kWide>
+__device__ __forceinline__ float lane_prediction(const u64* keep, const float* rus, const char* col,
+                                                 int stride, int q) {
+  float acc = 0.f;
+#pragma unroll
+  for (int s = 0; s <= E; ++s) {
+    const u64 k = keep[s * kThreads + q];
+    const float* at = reinterpret_cast<const float*>(
+        col + (kWide ? (int64_t)key_index(k) * stride * 4 : (int64_t)(uint32_t)k));
+    acc = __fmaf_rn(key_dist(k), __ldg(at), acc);
+  }
+  return __fmul_rn(acc, rus[q]);
+}
+
+// The targets whose sums this lane stored and whose predictions spread too little
+// for them: again in FP64.
+template <int E, bool kWide>
+__device__ __noinline__ void exact_targets(const u64* keep, const float* rus, const float* st,
+                                           int stride, const TargetDesc* tgs, int T, int n_tiles,
+                                           int nq, float4* part, const float* x, int64_t n,
+                                           const int32_t* order, const ObsStat* stat) {
+  for (int t = threadIdx.x; t < T; t += kThreads) {
+    float4* to = part + 2 * (int64_t)t * n_tiles;
+    if (!too_small(to->w, stat[tgs[t].obs_tile].series)) continue;
+    const char* col = reinterpret_cast<const char*>(st + tgs[t].i);
+    exact_sums_lane(TileTarget{x + (int64_t)tgs[t].i * n, order, stat + tgs[t].obs_tile, nq},
+                    [=](int q) { return lane_prediction<E, kWide>(keep, rus, col, stride, q); }, to);
+  }
+}
+
+template <int E, bool kWide>
 __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc& u, int tile, int nq,
                                           const u64* keep, const float* rus, float* sums) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -220,22 +268,14 @@ __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc&
   const float2* obs = p.obs + tgs[0].obs_tile * kQT + (int64_t)tile * kQT * T;
   const int q0 = warp * 32, q1 = min(nq, q0 + 32);
   const int32_t* order = p.order + u.order_off + (int64_t)tile * kQT;
+  bool redo = false;
   for (int tc = 0, turn = 0; tc < T; tc += 32, ++turn) {
     const int t = min(tc + lane, T - 1);  // lanes past the last target repeat it
     const TargetDesc& tg = tgs[t];
     const char* col = reinterpret_cast<const char*>(st + tg.i);
-    const float scale = p.obs_stat[tg.obs_tile + tile].scale;
-    auto predict = [&](int q) {
-      float acc = 0.f;
-#pragma unroll
-      for (int s = 0; s <= E; ++s) {
-        const u64 k = keep[s * kThreads + q];
-        const float* at = reinterpret_cast<const float*>(
-            col + (kWide ? (int64_t)key_index(k) * stride * 4 : (int64_t)(uint32_t)k));
-        acc = __fmaf_rn(key_dist(k), __ldg(at), acc);
-      }
-      return __fmul_rn(acc, rus[q]);
-    };
+    const SeriesScale sc = p.obs_stat[tg.obs_tile + tile].series;
+    const float scale = sc.scale;
+    auto predict = [&](int q) { return lane_prediction<E, kWide>(keep, rus, col, stride, q); };
     const float c = __fmul_rn(predict(0), scale);
     const float2* a = obs + t;
     // two groups of eight queries side by side (packed), then the next two
@@ -286,10 +326,15 @@ __device__ __forceinline__ void lane_targets(const KnnParams& p, const UnitDesc&
       };
       const TileSums lo = merge_sums(merge_sums(load(0), load(1)), merge_sums(load(2), load(3)));
       const TileSums hi = merge_sums(merge_sums(load(4), load(5)), merge_sums(load(6), load(7)));
-      store_sums(p.partials + 2 * (u.part_off + (int64_t)t * n_tiles + tile), c,
-                 merge_sums(lo, hi));
+      const TileSums m = merge_sums(lo, hi);
+      store_sums(p.partials + 2 * (u.part_off + (int64_t)t * n_tiles + tile), c, m);
+      redo |= too_small(m.b2.h, sc);
     }
   }
+  if (__builtin_expect(redo, 0))  // rare, and behind the loop: its registers are the predictions'
+    exact_targets<E, kWide>(keep, rus, st, stride, tgs, T, n_tiles, nq,
+                            p.partials + 2 * (u.part_off + tile),
+                            p.series + u.series_off + (E - 1) * u.tau, u.n, order, p.obs_stat + tile);
   __syncthreads();
 }
 
@@ -391,18 +436,19 @@ __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& 
       }
     }
     const int64_t rec = tg.obs_tile + tile;
-    ring[ring_n * kVecStride + vec_slot(tid)] = __fmul_rn(xhat, p.obs_stat[rec].scale);
+    ring[ring_n * kVecStride + vec_slot(tid)] = xhat;
     if (tid == 0)
       meta[ring_n] = RingMeta{p.obs + rec * kQT,
-                              p.partials + 2 * (u.part_off + (int64_t)t * u.n_tiles + tile), nq};
+                              p.partials + 2 * (u.part_off + (int64_t)t * u.n_tiles + tile),
+                              p.obs_stat[rec].series, nq, (int32_t)(u.tgt_off + t), tile};
     // a full ring is reduced before the next target's vector, or at the end
     if (++ring_n == kRing && t + 1 < u.n_targets) {
-      flush_ring(ring, meta, kRing);
+      flush_ring(p, ring, meta, kRing);
       ring_n = 0;
     }
   }
   if (ring_n == kRing) {  // the weights and neighbours are dead here
-    flush_ring(ring, meta, kRing);
+    flush_ring(p, ring, meta, kRing);
     ring_n = 0;
   }
   }
@@ -1037,7 +1083,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams
     }
     process_table_item<E, kLanes, kStats>(p, u, w.tile, smem, s_meta, ring_n);
   }
-  if (ring_n > 0) flush_ring(reinterpret_cast<const float*>(smem), s_meta, ring_n);
+  if (ring_n > 0) flush_ring(p, reinterpret_cast<const float*>(smem), s_meta, ring_n);
 }
 
 template <int E, bool kLanes, bool kStats>
@@ -1068,7 +1114,7 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
       process_item<E, 0, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, s_qbox, ring_n);
   }
   if (ring_n > 0)
-    flush_ring(reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);
+    flush_ring(p, reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);
 }
 
 // Ring, records and bits: every manifold of the launch fits.

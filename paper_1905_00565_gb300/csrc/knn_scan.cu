@@ -162,6 +162,10 @@ __device__ __forceinline__ float predict(const float (&d)[E + 1], const float (&
   return __fmul_rn(acc, rcp_hw(usum));
 }
 
+__device__ __noinline__ void exact_vector(const TileTarget t, const float* ys, float4* part) {
+  exact_sums_warp(t, ys, part);
+}
+
 // kSmemWords: the item's membership words lie in shared memory (else they are
 // read from global memory, spatially coherent in query order and so mostly
 // from L1).  kGeneral: with an exclusion window, search counters, or neighbour
@@ -209,7 +213,6 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
     uint32_t* mask = s_mask + tid;
     uint16_t* step = s_step + tid;
     for (int tile = tile0; tile < tile1; ++tile) {
-      const float scale = p.obs_stat[tg.obs_tile + tile].scale;
       const int nq = min(kQT, n_m - tile * kQT);
       for (int i = 0; i < kQueriesPerWarp; ++i) {
         const int q = warp * kQueriesPerWarp + i;
@@ -276,7 +279,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
           }
         }
         if (kGeneral && p.dbg_xhat && mine) p.dbg_xhat[p.targets[u.tgt_off + lane].q_off + m] = y;
-        s_vec[lane * kScanVec + vec_slot(q)] = __fmul_rn(y, scale);
+        s_vec[lane * kScanVec + vec_slot(q)] = y;
       }
       __syncthreads();
       // two vectors a warp: half a warp's lane g sums the tile's queries 16g ..
@@ -286,23 +289,33 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
         const int64_t rec = tg.obs_tile + tile;
         const float* ys = s_vec + vec * kScanVec;
         const float2* a = p.obs + rec * kQT;
-        const float c0 = ys[0];
-        const packed cc = pack2(c0, c0);
+        const ObsStat* stat = p.obs_stat + rec;
+        const SeriesScale sc = stat->series;
+        const float scale = sc.scale, c0 = __fmul_rn(ys[0], scale);
+        const packed cc = pack2(c0, c0), ss = pack2(scale, scale);
         TileSums2 both = zero_sums2();
 #pragma unroll 4
         for (int i = 0; i < kMomentGroup; ++i) {
           const int qa = 16 * g + i, qb = qa + kMomentGroup;
           const float ya = ys[vec_slot(qa)], yb = ys[vec_slot(qb)];
-          add_query2(both, pack2(qa < nq ? ya : c0, qb < nq ? yb : c0), __ldg(a + obs_slot(qa)),
-                     __ldg(a + obs_slot(qb)), cc);
+          add_query2(both, mul2(pack2(qa < nq ? ya : ys[0], qb < nq ? yb : ys[0]), ss),
+                     __ldg(a + obs_slot(qa)), __ldg(a + obs_slot(qb)), cc);
         }
         TileSums half[2];
         unpack_sums(both, half[0], half[1]);
         TileSums m = merge_sums(half[0], half[1]);
 #pragma unroll
         for (int o = 1; o < 16; o <<= 1) m = merge_across(m, o);
-        if (g == 0 && vec < count)
+        const bool writes = g == 0 && vec < count, redo_mine = writes && too_small(m.b2.h, sc);
+        if (writes && !redo_mine)
           store_sums(p.partials + 2 * (p.units[w.unit + vec].part_off + tile), c0, m);
+        for (unsigned redo = __ballot_sync(kAllLanes, redo_mine); redo; redo &= redo - 1u) {
+          const int v = warp * 2 + (__ffs(redo) > 16 ? 1 : 0);
+          exact_vector(TileTarget{p.series + u.series_off + (int64_t)tg.i * u.n + (E - 1) * u.tau,
+                                  order + tile * kQT, stat, nq},
+                       s_vec + v * kScanVec,
+                       p.partials + 2 * (p.units[w.unit + v].part_off + tile));
+        }
       }
       __syncthreads();
     }
@@ -341,6 +354,47 @@ __host__ __device__ constexpr size_t group_fixed_smem() {
   return (size_t)(lane_group(E) * kKeepStride<E> + 1) / 2 * 2 * 8 +
          (size_t)(lane_group(E) * (kQT + 1) + 3) / 4 * 16 +
          (size_t)(E + 1 < 4 ? 4 : E + 1) * kGroupThreads * (4 + 2);
+}
+
+// The prediction of query q from a realization's weights and neighbours.
+template <int E>
+__device__ __forceinline__ float group_prediction(const float2* keep, const float* rus,
+                                                  const char* col, int q) {
+  float acc = 0.f;
+#pragma unroll
+  for (int s = 0; s <= E; ++s) {
+    const float2 k = keep[s * kQT + q];
+    acc = __fmaf_rn(k.x, __ldg(reinterpret_cast<const float*>(col + __float_as_uint(k.y))), acc);
+  }
+  return __fmul_rn(acc, rus[q]);
+}
+
+// Whether this warp is the one of the task's team that stores its sums.
+__device__ __forceinline__ bool stores_task(int task, int warp) {
+  constexpr int kTeams = kGroupThreads / 32 / kTeam;
+  return task % kTeams == warp / kTeam && task / kTeams % kTeam == warp % kTeam;
+}
+
+// Of the sums this lane stored, those whose predictions spread too little for them:
+// again in FP64.
+template <int E>
+__device__ __noinline__ void exact_tasks(const float2* s_keep, const float* s_rus, const float* st,
+                                         const TargetDesc* tgs, int T, int n_tiles, int nq, int count,
+                                         const UnitDesc* units, float4* part, const float* x,
+                                         int64_t n, const int32_t* order, const ObsStat* stat) {
+  const int lane = threadIdx.x & 31;
+  for (int task = 0; task < count * ((T + 31) / 32); ++task) {
+    const int r = task % count, t = task / count * 32 + lane;
+    if (!stores_task(task, threadIdx.x >> 5) || t >= T) continue;
+    const TargetDesc& tg = tgs[t];
+    float4* to = part + 2 * (units[r].part_off + (int64_t)t * n_tiles);
+    if (!too_small(to->w, stat[tg.obs_tile].series)) continue;
+    const float2* keep = s_keep + r * kKeepStride<E>;
+    const float* rus = s_rus + r * (kQT + 1);
+    const char* col = reinterpret_cast<const char*>(st + tg.i);
+    exact_sums_lane(TileTarget{x + (int64_t)tg.i * n, order, stat + tg.obs_tile, nq},
+                    [=](int q) { return group_prediction<E>(keep, rus, col, q); }, to);
+  }
 }
 
 template <int E, bool kGeneral>
@@ -455,24 +509,17 @@ __global__ void __launch_bounds__(kGroupThreads, 1) group_kernel(KnnParams p) {
     // [warp][value][lane], where the walks' records were
     float* sums = reinterpret_cast<float*>(mask - tid) + warp * 6 * 32 + lane;
     const int part = warp % kTeam, q0 = part * kTeamQueries;
+    bool redo = false;
     for (int task = warp / kTeam; task < count * chunks; task += kWarps / kTeam) {
       const int chunk = task / count, r = task - chunk * count;
       const int t = min(chunk * 32 + lane, T - 1);  // lanes past the last target repeat it
       const TargetDesc& tg = tgs[t];
       const char* col = reinterpret_cast<const char*>(st + tg.i);
-      const float scale = p.obs_stat[tg.obs_tile + tile].scale;
+      const SeriesScale sc = p.obs_stat[tg.obs_tile + tile].series;
+      const float scale = sc.scale;
       const float2* keep = s_keep + r * KS;
       const float* rus = s_rus + r * (kQT + 1);
-      auto value = [&](int q) {
-        float acc = 0.f;
-#pragma unroll
-        for (int s = 0; s < K; ++s) {
-          const float2 k = keep[s * kQT + q];
-          
-          acc = __fmaf_rn(k.x, __ldg(reinterpret_cast<const float*>(col + __float_as_uint(k.y))), acc);
-        }
-        return __fmul_rn(acc, rus[q]);
-      };
+      auto value = [&](int q) { return group_prediction<E>(keep, rus, col, q); };
       const float c = __fmul_rn(value(0), scale);
       const packed cc = pack2(c, c), ss = pack2(scale, scale);
       const float2* a = obs + t;
@@ -506,7 +553,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1) group_kernel(KnnParams p) {
 #pragma unroll
       for (int x = 0; x < 6; ++x) sums[x * 32] = mine6[x];
       team_barrier(warp / kTeam);
-      if (part == (task / (kWarps / kTeam)) % kTeam && chunk * 32 + lane < T) {
+      if (stores_task(task, warp) && chunk * 32 + lane < T) {
         auto load = [&](int i) {
           const float* f = sums + (i - part) * 6 * 32;
           TileSums m;
@@ -515,11 +562,16 @@ __global__ void __launch_bounds__(kGroupThreads, 1) group_kernel(KnnParams p) {
           m.ab = Pair32{f[4 * 32], f[5 * 32]};
           return m;
         };
-        store_sums(p.partials + 2 * (p.units[w.unit + r].part_off + (int64_t)t * u.n_tiles + tile), c,
-                   merge_sums(merge_sums(load(0), load(1)), merge_sums(load(2), load(3))));
+        const TileSums m = merge_sums(merge_sums(load(0), load(1)), merge_sums(load(2), load(3)));
+        store_sums(p.partials + 2 * (p.units[w.unit + r].part_off + (int64_t)t * u.n_tiles + tile), c, m);
+        redo |= too_small(m.b2.h, sc);
       }
       team_barrier(warp / kTeam);
     }
+    if (__builtin_expect(redo, 0))  // rare
+      exact_tasks<E>(s_keep, s_rus, st, tgs, T, u.n_tiles, nq, count, p.units + w.unit,
+                     p.partials + 2 * tile, p.series + u.series_off + (E - 1) * u.tau, u.n,
+                     order + tile * kQT, p.obs_stat + tile);
     __syncthreads();
   }
 }

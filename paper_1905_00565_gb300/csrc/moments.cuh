@@ -11,14 +11,27 @@
 // predictions themselves are FP32 values (24 bits).
 //
 // Values are scaled by a power of two that brings the target series' largest
-// magnitude into [1, 2) (exact; rho does not change), so that no product
-// leaves FP32's range.  With c the tile's first prediction and b = y - c
-// (exact as h + l), the sums are B1 = sum b, B2 = sum b^2 and AB = sum a b,
-// a = x - mean(x) (exact to 48 bits).  y constant over a tile gives exactly
-// zero.  From them mean(y) = c + B1/n, Syy = B2 - B1^2/n, Sxy = AB (sum a = 0).
+// magnitude to 2^kScaleBits (exact; rho does not change): squares and their sums
+// over a tile stay below 2^112, and there is room below for series whose ordinary
+// values are far smaller than their largest.  With c the tile's first prediction
+// and b = y - c (exact as h + l), the sums are B1 = sum b, B2 = sum b^2 and AB =
+// sum a b, a = x - mean(x) (exact to 48 bits).  y constant over a tile gives
+// exactly zero.  From them mean(y) = c + B1/n, Syy = B2 - B1^2/n, Sxy = AB (sum a
+// = 0).
 //
-// Order of the sums, the same in every kernel: eight consecutive queries one
-// after the other, then a binary tree over the tile's 32 such groups.
+// A tile whose predictions spread so little against the series' largest value (a
+// fill value of 1e30 among values near 1) that its products would leave FP32's
+// range at the small end, B2 < kSmallB2, is summed once more in FP64 from the
+// predictions themselves, and its record holds three doubles (store_exact).  From
+// kSmallB2 on the terms lost below 2^-149 are less than 2^-78 of B2, and, as the
+// target's own spread is at least the predictions', less than 2^-70 of sqrt(Sxx
+// Syy) in AB.  B2 = 0 means that all predictions are equal, except in a series
+// whose values reach below 2^-kDeepBits of its largest: there (SeriesScale)
+// such a tile is summed again too.
+//
+// Order of the sums, the same in every kernel and in both forms: eight
+// consecutive queries one after the other, then a binary tree over the tile's 32
+// such groups.
 #pragma once
 
 #include "ccm_internal.h"
@@ -29,6 +42,7 @@ constexpr int kQT = 256;                  // queries per tile
 constexpr int kMomentGroup = 8;           // queries summed one after the other
 constexpr int kVecStride = kQT + 8;       // floats of a staged prediction vector
 constexpr unsigned kAllLanes = 0xffffffffu;
+constexpr float kSmallB2 = 0x1p-60f;
 
 // Where query q of a tile lies in a staged prediction vector: one pad word per
 // 32 queries, so that lanes walking different groups hit different banks.
@@ -186,23 +200,109 @@ __device__ __forceinline__ void store_sums(float4* part, float c, const TileSums
   part[1] = make_float4(m.b2.l, m.ab.h, m.ab.l, 0.f);
 }
 
+__device__ __forceinline__ bool too_small(float b2, const SeriesScale& s) {
+  return b2 < kSmallB2 && b2 >= s.least_b2;
+}
+
+// A tile's record in FP64 (scaled as the paired sums are): told from paired sums
+// by its last word.
+__device__ __forceinline__ void store_exact(float4* part, double my, double syy, double sxy) {
+  part[0] = make_float4(__int_as_float(__double2loint(my)), __int_as_float(__double2hiint(my)),
+                        __int_as_float(__double2loint(syy)), __int_as_float(__double2hiint(syy)));
+  part[1] = make_float4(__int_as_float(__double2loint(sxy)), __int_as_float(__double2hiint(sxy)),
+                        0.f, 1.f);
+}
+__device__ __forceinline__ double word_pair(float lo, float hi) {
+  return __hiloint2double(__float_as_int(hi), __float_as_int(lo));
+}
+
+// Where a tile's observed values lie: x[order[q]], q < nq, with their record.
+struct TileTarget {
+  const float* x;         // the target series at the manifold's points
+  const int32_t* order;   // the tile's queries
+  const ObsStat* stat;
+  int32_t nq;
+};
+
+// The same tile in FP64 by one warp (rare): ys the unscaled predictions (vec_slot
+// order).
+__device__ __forceinline__ void exact_sums_warp(const TileTarget& t, const float* ys, float4* part) {
+  const int q0 = kMomentGroup * (threadIdx.x & 31), q1 = min(q0 + kMomentGroup, t.nq);
+  const double scale = t.stat->series.scale, mx = t.stat->mx;
+  auto tree = [](double v) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(kAllLanes, v, o));
+    return v;
+  };
+  double s = 0.0, syy = 0.0, sxy = 0.0;
+  for (int q = q0; q < q1; ++q) s = __dadd_rn(s, __dmul_rn((double)ys[vec_slot(q)], scale));
+  const double my = __ddiv_rn(tree(s), (double)t.nq);
+  for (int q = q0; q < q1; ++q) {
+    const double b = __dsub_rn(__dmul_rn((double)ys[vec_slot(q)], scale), my);
+    const double a = __dsub_rn(__dmul_rn((double)t.x[t.order[q]], scale), mx);
+    syy = __fma_rn(b, b, syy);
+    sxy = __fma_rn(a, b, sxy);
+  }
+  syy = tree(syy);
+  sxy = tree(sxy);
+  if ((threadIdx.x & 31) == 0) store_exact(part, my, syy, sxy);
+}
+// And by one lane, in the same order: y(q) the unscaled prediction of query q.
+template <typename Y>
+__device__ __forceinline__ void exact_sums_lane(const TileTarget& t, Y y, float4* part) {
+  const double scale = t.stat->series.scale, mx = t.stat->mx;
+  double my = 0.0, syy = 0.0, sxy = 0.0;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    double lv[3][6];  // pending subtrees: of sum y; of syy and sxy
+    double v[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int g = 0; g < kQT / kMomentGroup; ++g) {
+      v[0] = v[1] = v[2] = 0.0;
+#pragma unroll 1
+      for (int q = kMomentGroup * g; q < min(kMomentGroup * (g + 1), t.nq); ++q) {
+        const double ys = __dmul_rn((double)y(q), scale);
+        if (pass == 0) {
+          v[0] = __dadd_rn(v[0], ys);
+        } else {
+          const double b = __dsub_rn(ys, my);
+          const double a = __dsub_rn(__dmul_rn((double)t.x[t.order[q]], scale), mx);
+          v[1] = __fma_rn(b, b, v[1]);
+          v[2] = __fma_rn(a, b, v[2]);
+        }
+      }
+      int l = 0;
+#pragma unroll 1
+      for (int up = g; up & 1; up >>= 1, ++l)
+        for (int k = 0; k < 3; ++k) v[k] = __dadd_rn(lv[k][l], v[k]);
+      for (int k = 0; k < 3; ++k) lv[k][l] = v[k];
+    }
+    if (pass == 0) my = __ddiv_rn(v[0], (double)t.nq);
+    syy = v[1];
+    sxy = v[2];
+  }
+  store_exact(part, my, syy, sxy);
+}
+
 // Moments of one staged vector by one warp: lane g sums queries 8g .. 8g+7,
-// then the tree.  ys: the scaled predictions (vec_slot order, queries past nq
-// ignored), a: the tile's record (obs_slot order, zero past nq).
-__device__ __forceinline__ void tile_sums_warp(const float* ys, const float2* a, int nq,
+// then the tree.  ys: the predictions (vec_slot order, queries past nq ignored),
+// a: the tile's record (obs_slot order, zero past nq).  True, in every lane: they
+// spread too little.
+__device__ __forceinline__ bool tile_sums_warp(const float* ys, const float2* a, SeriesScale s, int nq,
                                                float4* part) {
   const int lane = threadIdx.x & 31;
-  const float c = ys[0];
+  const float c = __fmul_rn(ys[0], s.scale);
   TileSums m = zero_sums();
 #pragma unroll
   for (int i = 0; i < kMomentGroup; ++i) {
     const int q = kMomentGroup * lane + i;
-    const float y = ys[vec_slot(q)];
+    const float y = __fmul_rn(ys[vec_slot(q)], s.scale);
     add_query(m, q < nq ? y : c, __ldg(a + obs_slot(q)), c);
   }
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) m = merge_across(m, o);
   if (lane == 0) store_sums(part, c, m);
+  return too_small(m.b2.h, s);
 }
 
 }  // namespace ccm

@@ -80,7 +80,7 @@ NoallocLayout noalloc_layout(int64_t r, int64_t L, int64_t n_tiles, int64_t n_m)
   a.seriesjob = o;
   o = up256(o + sizeof(SeriesJob));
   a.scale = o;
-  o = up256(o + sizeof(float));
+  o = up256(o + sizeof(SeriesScale));
   a.total = o;
   return a;
 }
@@ -264,11 +264,11 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   e = launch_order(d_series, reinterpret_cast<const OrderJob*>(scratch + lay.orderjob), 1,
                    (int)n_m, reinterpret_cast<int32_t*>(scratch + lay.order), nullptr, nullptr,
                    reinterpret_cast<const SeriesJob*>(scratch + lay.seriesjob), 1,
-                   reinterpret_cast<float*>(scratch + lay.scale), nullptr, chain);
+                   reinterpret_cast<SeriesScale*>(scratch + lay.scale), nullptr, chain);
   if (e == cudaSuccess)
     e = launch_obs(d_series, reinterpret_cast<const int32_t*>(scratch + lay.order),
                    reinterpret_cast<const ObsJob*>(scratch + lay.obsjob), 1, n_tiles,
-                   reinterpret_cast<const float*>(scratch + lay.scale),
+                   reinterpret_cast<const SeriesScale*>(scratch + lay.scale),
                    reinterpret_cast<float2*>(scratch + lay.obs),
                    reinterpret_cast<ObsStat*>(scratch + lay.obs_stat), chain);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));

@@ -197,19 +197,24 @@ __device__ void bitonic_sort(unsigned long long* k, int n2) {
 }
 
 // Preparation of one target series (SeriesJob), by one CTA: the power of two
-// 2^-e, e the exponent of the series' largest magnitude (clamped so that it is
-// a normal number; 1 for an all-zero or non-finite series), and its column of
-// the time-major copy.
-__device__ void prepare_series(const float* series, const SeriesJob& jb, float* scales, float* st) {
+// 2^(kScaleBits - e), e the exponent of the series' largest magnitude (clamped so
+// that it is a normal number; 1 for an all-zero or non-finite series), and its
+// column of the time-major copy.
+__device__ void prepare_series(const float* series, const SeriesJob& jb, SeriesScale* scales, float* st) {
   const float* s = series + jb.off;
   float lo, hi;
   series_range(s, jb.n, &lo, &hi);
+  const float top = fmaxf(fabsf(lo), fabsf(hi));
+  const float deep = __fmul_rn(top, __uint_as_float((uint32_t)(127 - kDeepBits) << 23));
+  bool small = false;
+  for (int64_t t = threadIdx.x; t < jb.n; t += blockDim.x) small |= s[t] != 0.f && fabsf(s[t]) < deep;
+  small = __syncthreads_or(small);
   if (threadIdx.x == 0) {
-    const float top = fmaxf(fabsf(lo), fabsf(hi));
     const int e = (int)((__float_as_uint(top) >> 23) & 0xffu) - 127;  // -127: zero or subnormal
-    scales[jb.scale] = (top == 0.f || e == 128)
-                           ? 1.f
-                           : __uint_as_float((uint32_t)(127 - max(-126, min(e, 126))) << 23);
+    scales[jb.scale].scale = (top == 0.f || e == 128)
+                                 ? 1.f
+                                 : __uint_as_float((uint32_t)(127 + min(kScaleBits - e, 127)) << 23);
+    scales[jb.scale].least_b2 = small ? 0.f : __uint_as_float(1u);
   }
   if (jb.st_off >= 0)
     for (int64_t t = threadIdx.x; t < jb.n; t += blockDim.x) st[jb.st_off + t * jb.st_stride] = s[t];
@@ -217,7 +222,7 @@ __device__ void prepare_series(const float* series, const SeriesJob& jb, float* 
 
 __global__ void __launch_bounds__(kOrderThreads)
 order_kernel(const float* series, const OrderJob* jobs, int64_t n_jobs, int32_t* order,
-             int32_t* inverse, unsigned long long* scratch, const SeriesJob* series_jobs, float* scales, float* st) {
+             int32_t* inverse, unsigned long long* scratch, const SeriesJob* series_jobs, SeriesScale* scales, float* st) {
   extern __shared__ __align__(16) unsigned char s_order[];
   unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_order);
   chain_begin();
@@ -311,7 +316,7 @@ cudaError_t order_prepare() {
 
 cudaError_t launch_order(const float* series, const OrderJob* jobs, int64_t n_jobs, int max_nm,
                          int32_t* order, int32_t* inverse, unsigned long long* scratch,
-                         const SeriesJob* series_jobs, int64_t n_series_jobs, float* scales,
+                         const SeriesJob* series_jobs, int64_t n_series_jobs, SeriesScale* scales,
                          float* st, LaunchStream s) {
   if (n_jobs + n_series_jobs <= 0) return cudaSuccess;
   const size_t smem = max_nm <= kBitonicMax ? (size_t)kBitonicMax * sizeof(unsigned long long)

@@ -802,7 +802,7 @@ Arena layout(int64_t series_elems, const UnitList& ul, int64_t n_rho, int64_t sc
   a.obs_stat = take(sizeof(ObsStat) * (size_t)ul.obs_total);
   a.obs_jobs = take(sizeof(ObsJob) * ul.obs_jobs.size());
   a.series_jobs = take(sizeof(SeriesJob) * ul.series_jobs.size());
-  a.scales = take(sizeof(float) * ul.series_jobs.size());
+  a.scales = take(sizeof(SeriesScale) * ul.series_jobs.size());
   a.st = take(sizeof(float) * (size_t)ul.st_total);
   a.stats = take(sizeof(unsigned long long) * kStatCount);
   a.total = o;
@@ -989,7 +989,7 @@ KnnParams knn_params(char* base, const Arena& ar, const UnitList& ul, int persis
 
 // Query order and target series, then the observed-value records.
 cudaError_t enqueue_order(char* base, const Arena& ar, const UnitList& ul, LaunchStream s) {
-  float* scales = reinterpret_cast<float*>(base + ar.scales);
+  SeriesScale* scales = reinterpret_cast<SeriesScale*>(base + ar.scales);
   const cudaError_t e =
       launch_order(reinterpret_cast<const float*>(base + ar.series),
                    reinterpret_cast<const OrderJob*>(base + ar.orders), (int64_t)ul.orders.size(),

@@ -109,3 +109,59 @@ def test_scaled_shifted_and_sparse_targets(ccm, targets):
             np.testing.assert_allclose(got[fine], want[fine], rtol=0, atol=MOMENT_TOL)
     finally:
         ccm.ccm_context_destroy(ctx)
+
+
+# A tile's sums in FP64 (both sides) and rho's merge differ by orders of summation
+# of at most 2560 terms: 2560 * 2^-53 * (range / std)^2 <= 1e-10 as above.
+@pytest.mark.parametrize("spike", [1e18, 1e22, 1e25, 1e30, 1e37, -3e38])
+@pytest.mark.parametrize("targets", [1, 14])
+def test_targets_with_one_huge_value(ccm, targets, spike):
+    """One target sample far above the others (a spike, a fill value): libraries that
+    miss it predict values whose squares are far below FP32's range beside it."""
+    n = 900
+    s = many_series(n, targets + 1, 7)
+    s[1, 450] = spike
+    if targets > 1:
+        s[2, 1] = spike                   # at E = 3 no manifold point holds it
+    p = I.Problem(series=s, pairs=np.array([[0, i] for i in range(1, targets + 1)], np.int32),
+                  E=np.array([1, 3], np.int32), tau=np.array([1], np.int32),
+                  L=np.array([20, 120, 600], np.int64), r=6, seed=9)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        for flags in (0, ccm.CCM_NO_TABLE):
+            got, want = run(ccm, ctx, p, flags), run(ccm, ctx, p, plain=True)
+            assert np.all(np.isfinite(want))
+            np.testing.assert_allclose(got, want, rtol=0, atol=MOMENT_TOL)
+            one = run(ccm, ctx, I.Problem(series=s, pairs=p.pairs[:1], E=p.E, tau=p.tau, L=p.L,
+                                          r=p.r, seed=p.seed), flags)
+            np.testing.assert_array_equal(got[:1], one)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+
+
+@pytest.mark.parametrize("targets", [1, 3, 14])
+def test_targets_of_two_scales(ccm, targets):
+    """Values near 1e-12 and a fill value of 9.97e36 at every 97th sample; and two
+    values 1e-40 apart, whose differences alone carry the skill."""
+    n = 1100
+    s = many_series(n, targets + 1, 3)
+    rng = np.random.default_rng(4)
+    fill = (s[1] * np.float32(1e-12)).astype(np.float32)
+    fill[::97] = 9.97e36
+    two = np.where(rng.random(n) < 0.5, np.float32(0), np.float32(1e-40))
+    two[7] = 1.0
+    ctx = ccm.ccm_context_create(0)
+    try:
+        for odd in (fill, two):
+            series = s.copy()
+            series[1] = odd
+            p = I.Problem(series=series,
+                          pairs=np.array([[0, i] for i in range(1, targets + 1)], np.int32),
+                          E=np.array([2, 4], np.int32), tau=np.array([1], np.int32),
+                          L=np.array([20, 120, 700], np.int64), r=4, seed=9)
+            got, want = run(ccm, ctx, p), run(ccm, ctx, p, plain=True)
+            np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
+            fine = np.isfinite(want)
+            np.testing.assert_allclose(got[fine], want[fine], rtol=0, atol=MOMENT_TOL)
+    finally:
+        ccm.ccm_context_destroy(ctx)

@@ -150,6 +150,7 @@ struct ItemGroup {
   int32_t E;
   Targets targets;
   int64_t first, count;
+  int32_t max_nm;  // longest manifold of its units: the launch's shared memory follows it
 };
 
 struct UnitList {
@@ -208,8 +209,9 @@ struct UnitList {
     for (size_t q = 0; q < list.size(); ++q) {
       const int32_t E = units[(size_t)list[q].unit].E;
       if (g.empty() || g.back().E != E || g.back().targets != targets_of(list[q]))
-        g.push_back(ItemGroup{E, targets_of(list[q]), (int64_t)q, 0});
+        g.push_back(ItemGroup{E, targets_of(list[q]), (int64_t)q, 0, 0});
       ++g.back().count;
+      g.back().max_nm = std::max(g.back().max_nm, units[(size_t)list[q].unit].n_m);
     }
     return g;
   }
@@ -217,6 +219,7 @@ struct UnitList {
   size_t table_elem() const { return table_u16() ? 2 : 4; }
   int64_t n_rho = 0, q_total = 0, nbr_total = 0, lib_dbg_total = 0;  // per output realization
   int emin = kMaxE + 1, emax = 0, max_nm = 0;
+  int table_max_nm = 0;               // longest manifold of the units that read a table
   double pairs = 0.0, flops = 0.0;    // neighbour-search work actually done
 };
 
@@ -617,6 +620,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
               u.bits_off = ul->bits_total;
               ul->bits_total += (u.n_m + 31) / 32;
               ul->lib_scratch = std::max(ul->lib_scratch, L);
+              ul->table_max_nm = std::max(ul->table_max_nm, u.n_m);
             }
             const int32_t uidx = (int32_t)ul->units.size();
             // the others get their items below, in groups
@@ -1060,7 +1064,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   if (!ul.tables.empty())
     CCM_CUDA(launch_table_points(reinterpret_cast<const float*>(base + ar.series),
                                  reinterpret_cast<const TableJob*>(base + ar.tables),
-                                 (int64_t)ul.tables.size(), ul.max_nm,
+                                 (int64_t)ul.tables.size(), ul.table_max_nm,
                                  reinterpret_cast<const int32_t*>(base + ar.order),
                                  reinterpret_cast<float*>(base + ar.points), ts));
   for (size_t g0 = 0; g0 < ul.tables.size();) {  // one launch per (size class, E)
@@ -1095,7 +1099,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   if (!ul.member_groups.empty())
     CCM_CUDA(launch_member_words(reinterpret_cast<const UnitDesc*>(base + ar.units),
                                  reinterpret_cast<const MemberGroup*>(base + ar.member_groups),
-                                 (int64_t)ul.member_groups.size(), ul.max_nm, sp.bits,
+                                 (int64_t)ul.member_groups.size(), ul.table_max_nm, sp.bits,
                                  reinterpret_cast<uint32_t*>(base + ar.words), ls));
   if (ev) CCM_CUDA(record(ev[2], s));
   KnnParams kp = knn_params(base, ar, ul, persistent, tn);
@@ -1123,11 +1127,11 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     kt.item_counter = counter++;
     const int g = persistent ? grid_table : (int)std::min<int64_t>(ig.count, 0x7fffffff);
     if (ig.targets == Targets::kOne)
-      CCM_CUDA(launch_knn_scan(kt, ig.E, ul.max_nm, persistent ? grid_scan : g, ls));
+      CCM_CUDA(launch_knn_scan(kt, ig.E, ig.max_nm, persistent ? grid_scan : g, ls));
     else if (ig.targets == Targets::kGrouped)
-      CCM_CUDA(launch_knn_group(kt, ig.E, ul.max_nm, persistent ? grid_scan / 2 : g, ls));
+      CCM_CUDA(launch_knn_group(kt, ig.E, ig.max_nm, persistent ? grid_scan / 2 : g, ls));
     else
-      CCM_CUDA(launch_knn_table(kt, ig.E, ul.max_nm, ig.targets == Targets::kMany, g, ls));
+      CCM_CUDA(launch_knn_table(kt, ig.E, ig.max_nm, ig.targets == Targets::kMany, g, ls));
   }
   CCM_CUDA(launch_rho(kp.units, kp.targets, (int64_t)ul.targets.size(), kp.partials, kp.obs_stat,
                       reinterpret_cast<double*>(base + ar.rho), ls));
@@ -1389,7 +1393,8 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
   pl->grid = persistent_grid(ctx, pl->ul.emin, pl->ul.emax);
   {
     int per_sm = 1;
-    if (knn_table_occupancy(pl->ul.max_nm, pl->ul.lane_targets, &per_sm) != cudaSuccess || per_sm < 1) per_sm = 1;
+    if (knn_table_occupancy(pl->ul.table_max_nm, pl->ul.lane_targets, &per_sm) != cudaSuccess || per_sm < 1)
+      per_sm = 1;
     pl->grid_table = ctx->sm_count * per_sm;
     pl->grid_scan = ctx->sm_count * 2;
   }

@@ -99,3 +99,29 @@ def test_noalloc_admits_up_to_16_mib(ccm):
     with pytest.raises(ccm.CCMError) as ei:
         ccm.ccm_run_noalloc(s, 0, 1, 1, 1, L, r + 1, seed, more)
     assert ei.value.status == ccm.CCM_ETOOLARGE
+
+
+def test_table_beside_a_manifold_too_long_for_one(ccm):
+    """A variable with two targets whose E = 10 manifold reads a table while its E = 1
+    manifold is longer than any table's (its membership bits alone would fill an
+    SM's shared memory)."""
+    n, tau = 1_400_000, 155_000                      # N_m = 1400000 and 5000
+    rng = np.random.default_rng(5)
+    p = I.Problem(series=rng.random((3, n), dtype=np.float32),
+                  pairs=np.array([[0, 1], [0, 2]], np.int32), E=np.array([1, 10], np.int32),
+                  tau=np.array([tau], np.int32), L=np.array([400], np.int64), r=110, seed=3)
+    rho = {}
+    ctx = ccm.ccm_context_create(0)
+    try:
+        for flags in (0, ccm.CCM_NO_TABLE):
+            plan = ccm.plan_problem(ctx, p, flags)
+            try:
+                assert (ccm.ccm_plan_get_info(plan)["table_bytes"] > 0) == (flags == 0)
+                rho[flags] = np.zeros(ccm.rho_shape(p))
+                ccm.ccm_run(plan, p.series, rho[flags])
+            finally:
+                ccm.ccm_plan_destroy(plan)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    assert np.all(np.isfinite(rho[0]))
+    np.testing.assert_array_equal(rho[0], rho[ccm.CCM_NO_TABLE])

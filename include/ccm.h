@@ -160,7 +160,10 @@ ccm_status ccm_context_destroy(ccm_context* ctx);
 
 /* Validate the problem, build the work list (units sorted by cost, split into
  * query tiles), reserve device memory.  Returns CCM_EINVAL for an invalid
- * problem and CCM_ETOOLARGE when the footprint exceeds the context budget. */
+ * problem and CCM_ETOOLARGE when the footprint exceeds the context budget.
+ * Test hook: the environment variable CCM_SAMPLER_WINDOW=k (read at each
+ * ccm_plan) bounds the keys the library sampler lists, so that its selection
+ * falls back on the radix search; the libraries are the same. */
 ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out);
 
 ccm_status ccm_plan_destroy(ccm_plan_t* plan);

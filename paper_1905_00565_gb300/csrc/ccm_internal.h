@@ -199,6 +199,7 @@ struct SamplerParams {
   int32_t* lib;           // library buffer (sum of L), each library in query order
   uint32_t* bits;         // membership bits of the units that read a table (no list is written)
   int32_t list_all;       // 1: list those too (at lib_off)
+  int32_t window;         // > 0: list at most so many keys around the last member's
   int32_t* dbg_lib;       // optional: libraries in ascending m, once per target, in rho order
   int32_t* err;           // error flag (set, never cleared, by the kernels)
 };

@@ -196,6 +196,7 @@ struct UnitList {
   double brute_pairs = 0.0;           // query-library pairs of those units
   int64_t search_queries = 0;         // N_m summed over the units
   int64_t table_queries = 0;          // N_m summed over the units that read a table
+  int32_t sampler_window = 0;         // CCM_SAMPLER_WINDOW
   bool table_tv = false;              // some table stores its target's values (TableJob::tv_i)
   Targets targets_of(const WorkItem& w) const {
     const UnitDesc& u = units[(size_t)w.unit];
@@ -353,6 +354,7 @@ int64_t cheapest_table_L(const ProblemCopy& pc, int32_t E, int64_t n_m, int64_t 
 // search per (E, tau, L, k); each pair becomes a target of that unit.
 void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, UnitList* ul,
                   double table_cap_bytes) {
+  if (const char* e = getenv("CCM_SAMPLER_WINDOW")) ul->sampler_window = std::max(0, atoi(e));
   const int tileq = knn_block_threads() * knn_queries_per_thread();
   const int64_t nP = (int64_t)pc.pairs.size() / 2;
   const int64_t nE = (int64_t)pc.E.size(), nT = (int64_t)pc.tau.size(), nL = (int64_t)pc.L.size();
@@ -948,8 +950,9 @@ struct ccm_plan_s {
 
 namespace {
 
-SamplerParams sampler_params(char* base, const Arena& ar) {
+SamplerParams sampler_params(char* base, const Arena& ar, const UnitList& ul) {
   SamplerParams sp{};
+  sp.window = ul.sampler_window;
   sp.units = reinterpret_cast<const UnitDesc*>(base + ar.units);
   sp.targets = reinterpret_cast<const TargetDesc*>(base + ar.targets);
   sp.order = reinterpret_cast<const int32_t*>(base + ar.order);
@@ -1093,7 +1096,7 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
   if (ev) CCM_CUDA(record(ev[5], ts.s));
   if (branch) CCM_CUDA(cudaEventRecord(branch->join, branch->s));
   if (ev) CCM_CUDA(record(ev[1], s));
-  SamplerParams sp = sampler_params(base, ar);
+  SamplerParams sp = sampler_params(base, ar, ul);
   sp.dbg_lib = dbg_lib;
   CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, ls));
   if (!ul.member_groups.empty())
@@ -1218,7 +1221,7 @@ ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
   const UnitList& ul = pl->ul;
   // libraries and query orders for the timing launches
   CCM_CUDA(enqueue_order(base, ar, ul, s));
-  SamplerParams sp = sampler_params(base, ar);
+  SamplerParams sp = sampler_params(base, ar, ul);
   CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, s));
   const int want = 6 * ctx->sm_count;
   WorkItem* d_items = nullptr;
@@ -1594,7 +1597,7 @@ ccm_status ccm_run_plain(ccm_plan_t* plan, const float* series, double* rho, voi
   CCM_CUDA(cudaMemcpyAsync(base + ar.series, series, sizeof(float) * (size_t)pc.V * (size_t)pc.n,
                            in_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   CCM_CUDA(cudaMemsetAsync(base + ar.err, 0, sizeof(int32_t), s));
-  SamplerParams sp = sampler_params(base, ar);
+  SamplerParams sp = sampler_params(base, ar, plan->ul);
   sp.list_all = 1;
   const UnitDesc* d_units = reinterpret_cast<const UnitDesc*>(base + ar.units);
   const TargetDesc* d_targets = reinterpret_cast<const TargetDesc*>(base + ar.targets);

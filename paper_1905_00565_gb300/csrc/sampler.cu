@@ -15,8 +15,12 @@
 // point: below a window of +-5 standard deviations it is a member, above it is
 // not, and the few hundred inside are listed in shared memory, where a
 // histogram and a rank count find the last member.  The keys are never stored
-// (one bit per point is).  When the window misses (about one unit in 10^6), an
-// 8-bit radix select over four passes recomputes the keys.
+// (one bit per point is).  When the window misses (about one unit in 10^6 at five
+// standard deviations), an 8-bit radix select over four passes recomputes the keys.
+// The window is narrower where the list would not hold it (libraries of about half
+// of more than 2.6 million points), down to three standard deviations (one unit in
+// 400 misses); where not even those fit, the pass is left out and the radix select
+// is all there is.
 //
 // Bound: issue (the 64-bit multiplies of Philox are half of the instructions)
 // and, for short manifolds, the latency between its barriers: five CTAs per SM
@@ -250,8 +254,9 @@ sampler_kernel(SamplerParams p, int64_t first_unit, int window) {
 
   // The window [lo, hi] of high halves: L/N_m of the range, +-5 standard
   // deviations of the rank (and a few keys more).
-  const float pf = (float)L / (float)n_m;
-  const float half_keys = 5.f * sqrtf((float)L * fmaxf(1.f - pf, 0.f)) + 8.f;
+  const float pf = (float)L / (float)n_m, sd = sqrtf((float)L * fmaxf(1.f - pf, 0.f));
+  const float half_keys = fminf(5.f * sd + 8.f, 0.45f * (float)window);
+  const bool look = half_keys >= 3.f * sd;
   const uint64_t centre = ((uint64_t)L << 32) / (uint32_t)n_m;
   const uint64_t half = (uint64_t)(half_keys * (4294967296.f / (float)n_m));
   const uint32_t lo = centre > half ? (uint32_t)min(centre - half, (uint64_t)0xffffffffu) : 0u;
@@ -265,7 +270,7 @@ sampler_kernel(SamplerParams p, int64_t first_unit, int window) {
   }
   __syncthreads();
   uint32_t below = 0u;
-  for (int b = tid; b < n_blocks; b += kSamplerThreads) {
+  for (int b = tid; b < n_blocks && look; b += kSamplerThreads) {
     uint64_t w[4];
     key_block(u, b, w);
     uint32_t byte = 0u;
@@ -288,7 +293,7 @@ sampler_kernel(SamplerParams p, int64_t first_unit, int window) {
   const uint32_t listed = s_listed, sum_below = s_below;
   // members among the listed keys; 0 and all of them need no search
   const uint32_t want = (uint32_t)L - sum_below;
-  bool found = (uint32_t)L >= sum_below && listed <= (uint32_t)window && want <= listed;
+  bool found = look && (uint32_t)L >= sum_below && listed <= (uint32_t)window && want <= listed;
   if (found && want > 0u && want < listed) {
     // bins of equal width over the window: the one holding the last member,
     // then its rank among that bin's keys
@@ -417,7 +422,7 @@ cudaError_t sampler_prepare() {
 
 cudaError_t launch_sampler(const SamplerParams& p, int64_t first_unit, int64_t count, int max_nm,
                            LaunchStream s) {
-  const int window = window_keys(max_nm);
+  const int window = p.window > 0 ? std::min(p.window, window_keys(max_nm)) : window_keys(max_nm);
   const size_t smem = (size_t)window * 8 + (size_t)((std::min(max_nm, kSamplerBitsMax) + 31) / 32) * 4;
   for (int64_t off = 0; off < count; off += 0x7fffffff) {
     const unsigned grid = (unsigned)std::min<int64_t>(count - off, 0x7fffffff);

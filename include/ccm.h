@@ -187,8 +187,9 @@ ccm_status ccm_plan_get_info(const ccm_plan_t* plan, ccm_plan_info* info);
  * pairs, for every E whose parameters are not yet known to the context, the
  * library times two kernel variants and three merge triggers on a sample of
  * the plan's work items and keeps the fastest (results are identical for all
- * of them).  Choices are cached per (device name, E) in $CCM_AUTOTUNE_CACHE,
- * default ~/.cache/ccm_gb300/autotune.tsv, and loaded by ccm_context_create.
+ * of them).  Choices are cached per (device name, revision of the kernels, E) in
+ * $CCM_AUTOTUNE_CACHE, default ~/.cache/ccm_gb300/autotune.tsv, and loaded by
+ * ccm_context_create.
  * CCM_NO_AUTOTUNE skips the measurement. */
 ccm_status ccm_run(ccm_plan_t* plan, const float* series, double* rho, void* cuda_stream);
 

@@ -9,6 +9,7 @@ runtime into one shared library exporting the C ABI of include/ccm.h.
 from __future__ import annotations
 
 import concurrent.futures as cf
+import hashlib
 import os
 import subprocess
 import sys
@@ -26,6 +27,8 @@ SOURCES = [(name, e) for e in range(10, 0, -1) for name in ("knn_fused.cu", "tab
 HEADERS = [os.path.join(CSRC, name) for name in (
     "ccm_internal.h", "moments.cuh", "bits.cuh", "row_walk.cuh", "launch.cuh")] + [
     os.path.join(INCLUDE, "ccm.h")]
+# the search kernels that the autotuner chooses between: its cached choices carry their hash
+TUNED = [os.path.join(CSRC, name) for name in ("knn_fused.cu", "ccm_internal.h", "moments.cuh")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -34,13 +37,22 @@ def _nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
+def _revision() -> str:
+    h = hashlib.sha256()
+    for path in TUNED:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def _compile(src: str, E: int, verbose: bool) -> str:
     obj = os.path.join(BUILD, os.path.splitext(src)[0] + (f"_e{E}" if E else "") + ".o")
-    deps = [os.path.join(CSRC, src), *HEADERS]
+    deps = [os.path.join(CSRC, src), *HEADERS, *(TUNED if src == "runtime.cu" else [])]
     if os.path.exists(obj) and os.path.getmtime(obj) >= max(os.path.getmtime(d) for d in deps):
         return obj
     cmd = [_nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
            *([f"-DCCM_E={E}"] if E else []),
+           *([f'-DCCM_KERNEL_REVISION="{_revision()}"'] if src == "runtime.cu" else []),
            *os.environ.get("CCM_EXTRA_NVCC_FLAGS", "").split(),
            "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, src), "-o", obj + ".tmp"]
     if verbose:

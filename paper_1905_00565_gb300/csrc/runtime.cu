@@ -1169,12 +1169,18 @@ namespace {
 // Per E the tuner times the kernel variants (narrow / wide) and merge triggers
 // on a stratified sample of the plan's own work items and keeps the fastest.
 // Every candidate computes the same result; only the time differs.  Choices
-// are cached per (device name, E) in a tab-separated file: $CCM_AUTOTUNE_CACHE,
-// else ~/.cache/ccm_gb300/autotune.tsv.
+// are cached per (device name, kernel revision, E) in a tab-separated file:
+// $CCM_AUTOTUNE_CACHE, else ~/.cache/ccm_gb300/autotune.tsv.  The revision (a hash
+// of the search kernels' sources, from build.py) keeps the choices measured with
+// other kernels from being taken for these.
+#ifndef CCM_KERNEL_REVISION
+#define CCM_KERNEL_REVISION "unknown"
+#endif
+constexpr char kRevision[] = "r" CCM_KERNEL_REVISION;
 std::string cache_path() {
   if (const char* p = getenv("CCM_AUTOTUNE_CACHE")) return p;
   const char* home = getenv("HOME");
-  return std::string(home ? home : "/tmp") + "/.cache/ccm_gb300/autotune_v2.tsv";
+  return std::string(home ? home : "/tmp") + "/.cache/ccm_gb300/autotune.tsv";
 }
 
 void load_cache(ccm_context* ctx) {
@@ -1182,10 +1188,10 @@ void load_cache(ccm_context* ctx) {
   if (!f) return;
   char line[512];
   while (fgets(line, sizeof(line), f)) {
-    char name[256];
+    char name[256], revision[64];
     int E = 0, v = 0, ma = 0;
-    if (sscanf(line, "%255[^\t]\t%d\t%d\t%d", name, &E, &v, &ma) == 4 &&
-        ctx->device_name == name && E >= 1 && E <= kMaxE && v >= 0 && v <= 1 && ma >= 1 &&
+    if (sscanf(line, "%255[^\t]\t%63[^\t]\t%d\t%d\t%d", name, revision, &E, &v, &ma) == 5 &&
+        ctx->device_name == name && std::strcmp(revision, kRevision) == 0 && E >= 1 && E <= kMaxE && v >= 0 && v <= 1 && ma >= 1 &&
         ma <= 16) {
       ctx->tuning.variant[E] = v;
       ctx->tuning.merge_at[E] = ma;
@@ -1208,7 +1214,7 @@ void save_cache(const ccm_context* ctx, int E, int v, int ma) {
   }
   FILE* f = fopen(path.c_str(), "a");
   if (!f) return;
-  fprintf(f, "%s\t%d\t%d\t%d\n", ctx->device_name.c_str(), E, v, ma);
+  fprintf(f, "%s\t%s\t%d\t%d\t%d\n", ctx->device_name.c_str(), kRevision, E, v, ma);
   fclose(f);
 }
 

@@ -15,7 +15,6 @@ constexpr int kMaxE = 10;
 // that share j are computed from one neighbour search.
 struct UnitDesc {
   int64_t series_off;   // element offset of the job's series block [V][n]
-  int64_t n;            // series length of the job
   int64_t lib_off;      // offset of this unit's library in the library buffer (units that read a
                         // table share one slot there: only the plain comparator lists them)
   int64_t bits_off;     // table_R > 0: this unit's membership bits, by position of the query order
@@ -25,23 +24,29 @@ struct UnitDesc {
   int64_t order_off;    // first entry of this unit's query order (per variable, E, tau)
   int64_t tgt_off;      // first TargetDesc of this unit
   int64_t table_off;    // distance indexing table of (j, E, tau), when table_R > 0
-  int64_t st_off;       // the job's series by time, [n][st_stride] (n_targets >= kLaneTargets)
+  int64_t st_off;       // the job's series by time, [n][st_stride]; -1: there is none
   uint64_t seed;        // library sampler seed of the job
+  int32_t n;            // series length of the job
   int32_t j;            // library variable
-  int32_t E, tau;
+  int32_t tau;
   int32_t L, k;
   int32_t n_m;          // manifold points = queries
   int32_t n_tiles;      // query tiles of the fused kernel
   int32_t n_targets;    // targets cross-mapped from this library (>= 1)
-  int32_t table_R;      // > 0: neighbours read from the table (its row length, a multiple of 64)
+  int16_t E;
+  int16_t table_R;      // > 0: neighbours read from the table (its row length, a multiple of 64)
   int32_t theiler;      // exclusion window W >= 0: candidates l of query m need |l - m| > W
   float wfloor;         // simplex weight floor f >= 0: u_i = max(u_i, f)
   int32_t st_stride;
 };
+static_assert(sizeof(UnitDesc) == 128, "no padding");
 // Units with at least this many targets form their predictions with one lane
-// per target (coalesced reads of the time-major series); fewer, one thread per
-// query and target after target.
+// per target (coalesced reads of the time-major series, where the plan has room
+// for that copy); others, one thread per query and target after target.
 constexpr int kLaneTargets = 12;
+__host__ __device__ inline bool lane_per_target(const UnitDesc& u) {
+  return u.n_targets >= kLaneTargets && u.st_off >= 0;
+}
 
 // One target of a unit: the pair (j, i) and where its outputs go.
 struct TargetDesc {

@@ -1077,7 +1077,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams
     if ((int64_t)it >= p.n_items) break;
     const WorkItem w = p.items[it];
     const UnitDesc u = p.units[w.unit];
-    if (u.E != E || (u.n_targets >= kLaneTargets) != kLanes) {
+    if (u.E != E || lane_per_target(u) != kLanes) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrBadUnit);
       continue;
     }
@@ -1104,7 +1104,7 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
     if ((int64_t)it >= p.n_items) break;
     const WorkItem w = p.items[it];
     const UnitDesc u = p.units[w.unit];
-    if (u.E != E || (u.n_targets >= kLaneTargets) != kLanes) {
+    if (u.E != E || lane_per_target(u) != kLanes) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrBadUnit);
       continue;
     }

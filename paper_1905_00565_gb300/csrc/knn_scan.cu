@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1) group_kernel(KnnParams p) {
     const int count = w.count, tile = w.tile;
     const UnitDesc& u = p.units[w.unit];  // the realizations' common description
     const int n_m = u.n_m, stride = u.table_R, W = u.theiler, T = u.n_targets;
-    if (u.E != E || T < kLaneTargets || count < 1 || count > G) {
+    if (u.E != E || !lane_per_target(u) || count < 1 || count > G) {
       if (tid == 0) atomicOr(p.err, kErrBadUnit);
       __syncthreads();
       continue;

@@ -120,14 +120,14 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, 
        k += (int64_t)gridDim.x * blockDim.x) {
     UnitDesc u;
     u.series_off = 0;
-    u.n = c.n;
+    u.n = (int32_t)c.n;
     u.lib_off = k * (int64_t)c.L;
     u.part_off = k * (int64_t)c.n_tiles;
     u.order_off = 0;
     u.tgt_off = k;
     u.seed = c.seed;
     u.j = c.j;
-    u.E = c.E;
+    u.E = (int16_t)c.E;
     u.tau = c.tau;
     u.L = c.L;
     u.k = (int32_t)k;
@@ -138,7 +138,7 @@ __global__ void noalloc_setup_kernel(unsigned char* scratch, NoallocLayout lay, 
     u.table_R = 0;
     u.theiler = 0;
     u.wfloor = 0.f;
-    u.st_off = 0;
+    u.st_off = -1;
     u.st_stride = 0;
     u.bits_off = 0;
     u.words_off = 0;

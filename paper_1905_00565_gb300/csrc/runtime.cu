@@ -200,7 +200,7 @@ struct UnitList {
   bool table_tv = false;              // some table stores its target's values (TableJob::tv_i)
   Targets targets_of(const WorkItem& w) const {
     const UnitDesc& u = units[(size_t)w.unit];
-    if (u.n_targets >= kLaneTargets)
+    if (lane_per_target(u))
       return u.table_R > 0 && u.words_off >= 0 ? Targets::kGrouped : Targets::kMany;
     return u.table_R > 0 && u.n_targets == 1 ? Targets::kOne : Targets::kFew;
   }
@@ -352,8 +352,14 @@ int64_t cheapest_table_L(const ProblemCopy& pc, int32_t E, int64_t n_m, int64_t 
 // Append the units of one problem.  Offsets: series block, first rho index.
 // Pairs that share a library variable j share one library and one neighbour
 // search per (E, tau, L, k); each pair becomes a target of that unit.
+// room: what else the plan may hold.
+struct Room {
+  double table_bytes;  // distance indexing tables, at most
+  bool time_major;     // the copy of the series that variables of many targets read
+};
 void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, UnitList* ul,
-                  double table_cap_bytes) {
+                  const Room& room) {
+  const double table_cap_bytes = room.table_bytes;
   if (const char* e = getenv("CCM_SAMPLER_WINDOW")) ul->sampler_window = std::max(0, atoi(e));
   const int tileq = knn_block_threads() * knn_queries_per_thread();
   const int64_t nP = (int64_t)pc.pairs.size() / 2;
@@ -411,10 +417,13 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
   // Target series: their scales and, when some library variable has many
   // targets, the time-major copy of the whole series block.
   bool lanes = false;
-  for (int32_t j : lib_vars) lanes |= pairs_of[j].size() >= (size_t)kLaneTargets;
+  auto many = [&](const std::vector<int64_t>& tp) {
+    return room.time_major && tp.size() >= (size_t)kLaneTargets;
+  };
+  for (int32_t j : lib_vars) lanes |= many(pairs_of[j]);
   ul->lane_targets |= lanes;
   ul->window |= pc.theiler > 0;
-  const int64_t st_off = ul->st_total;
+  const int64_t st_off = lanes ? ul->st_total : -1;
   const int32_t st_stride = (pc.V + 31) / 32 * 32;
   if (lanes) ul->st_total += pc.n * st_stride;
   std::vector<int32_t> scale_of((size_t)pc.V, -1);
@@ -453,7 +462,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           ob.tau = tau;
           ob.n_m = (int32_t)(pc.n - (int64_t)(E - 1) * tau);
           ob.n_tiles = (ob.n_m + tileq - 1) / tileq;
-          const bool side = tp.size() >= (size_t)kLaneTargets;
+          const bool side = many(tp);
           ob.a_step = side ? (int32_t)tp.size() : 0;
           ob.a_off = side ? base * tileq + (int64_t)t : ob.obs_tile * tileq;
           ul->obs_total += ob.n_tiles;
@@ -552,7 +561,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           else
             tabled += pc.r;
         }
-        if (pairs_of[j].size() >= (size_t)kLaneTargets)
+        if (many(pairs_of[j]))
           many_tiles[E] += (n_m + tileq - 1) / tileq * tabled;
         scan_tiles[E] += (n_m + tileq - 1) / tileq * ((tabled + kScanGroup - 1) / kScanGroup);
       }
@@ -570,7 +579,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         // 32 of 3000, r = 20, L = 2800 0.33 against 0.39; 40 of 4000, r = 12, E = 8
         // 1.55 against 1.68.  Their byte offsets have 32 bits.
         const int32_t lanes_group =
-            tp.size() >= (size_t)kLaneTargets && (uint64_t)pc.n * (uint64_t)st_stride * 4 < 1ull << 32
+            many(tp) && (uint64_t)pc.n * (uint64_t)st_stride * 4 < 1ull << 32
                 ? (int32_t)std::min<int64_t>(many_tiles[E] / (2 * 152), lane_group(E))
                 : 0;
         const bool grouped = tp.size() == 1 || lanes_group >= std::min(8, lane_group(E));
@@ -581,9 +590,9 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             UnitDesc u;
             std::memset(&u, 0, sizeof(u));
             u.series_off = series_off;
-            u.n = pc.n;
+            u.n = (int32_t)pc.n;
             u.j = j;
-            u.E = E;
+            u.E = (int16_t)E;
             u.tau = tau;
             u.L = (int32_t)L;
             u.k = k;
@@ -618,7 +627,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
             const auto tab = table_of.find(std::make_tuple(j, E, tau));
             if (tab != table_of.end() && L >= tab->second.lmin) {
               u.table_off = tab->second.off;
-              u.table_R = tab->second.stride;
+              u.table_R = (int16_t)tab->second.stride;
               u.bits_off = ul->bits_total;
               ul->bits_total += (u.n_m + 31) / 32;
               ul->lib_scratch = std::max(ul->lib_scratch, L);
@@ -878,9 +887,16 @@ struct ccm_context {
 };
 
 namespace {
-// Device memory the distance indexing tables of one plan (or served batch)
-// may take: a quarter of the context's budget.
-double table_cap(const ccm_context* ctx) { return 0.25 * (double)ctx->budget; }
+// What a plan (or served job) may hold beside what it needs: tables of a quarter of
+// the context's budget and the time-major copy of its series; where the plan does
+// not fit, smaller tables, then none, then no copy either.
+constexpr int kRooms = 4;
+Room room_of(const ccm_context* ctx, int attempt) {
+  constexpr double kTables[kRooms] = {0.25, 0.025, 0.0, 0.0};
+  return Room{kTables[attempt] * (double)ctx->budget, attempt < 3};
+}
+// No attempt after this one gives a smaller plan.
+bool barest(const UnitList& ul) { return ul.tables.empty() && ul.st_total == 0; }
 }  // namespace
 
 namespace {
@@ -1344,14 +1360,14 @@ ccm_status ccm_plan(ccm_context* ctx, const ccm_problem* prob, ccm_plan_t** out)
   if (st != CCM_OK) return st;
   const int64_t series_elems = (int64_t)pl->pc.V * pl->pc.n;
   CCM_CUDA(cudaSetDevice(ctx->device));
-  // where the plan does not fit, once more with smaller tables, then with none
+  // where the plan does not fit, once more with less room (room_of)
   cudaError_t e = cudaSuccess;
-  for (double cap : {table_cap(ctx), 0.1 * table_cap(ctx), 0.0}) {
+  for (int attempt = 0; attempt < kRooms; ++attempt) {
     pl->ul = UnitList();
-    append_units(pl->pc, 0, 0, &pl->ul, cap);
+    append_units(pl->pc, 0, 0, &pl->ul, room_of(ctx, attempt));
     sort_items(&pl->ul);
     pl->ar = layout(series_elems, pl->ul, pl->ul.n_rho, pl->ul.max_nm);
-    const bool last = pl->ul.tables.empty();
+    const bool last = barest(pl->ul);
     st = reserve(ctx, pl->ar.total);
     if (st != CCM_OK) {
       if (last) return st;
@@ -1685,7 +1701,7 @@ struct Job {
   int64_t n_units = 0;
   size_t footprint = 0;
   double pairs = 0.0;  // query-library pairs: the job's cost
-  double table_cap = 0.0;  // bytes its tables may take
+  int room = 0;        // room_of its layout
   enum State { kQueued, kRunning, kDone, kFailed, kCancelled } state = kQueued;
   ccm_status status = CCM_PENDING;
   std::string err;
@@ -1707,17 +1723,16 @@ struct Batch {
 
 namespace {
 
-// Device footprint of a job; where it exceeds the budget, with smaller tables,
-// then with none.
-size_t job_footprint(const ccm_context* ctx, const ProblemCopy& pc, double* pairs, double* cap) {
+// Device footprint of a job; where it exceeds the budget, with less room.
+size_t job_footprint(const ccm_context* ctx, const ProblemCopy& pc, double* pairs, int* room) {
   size_t total = 0;
-  for (double c : {table_cap(ctx), 0.1 * table_cap(ctx), 0.0}) {
+  for (int attempt = 0; attempt < kRooms; ++attempt) {
     UnitList ul;
-    append_units(pc, 0, 0, &ul, c);
+    append_units(pc, 0, 0, &ul, room_of(ctx, attempt));
     *pairs = ul.pairs;
-    *cap = c;
+    *room = attempt;
     total = layout((int64_t)pc.V * pc.n, ul, ul.n_rho, 0).total;
-    if (total <= ctx->budget || ul.tables.empty()) break;
+    if (total <= ctx->budget || barest(ul)) break;
   }
   return total;
 }
@@ -1738,7 +1753,7 @@ void CUDART_CB on_batch_done(void* arg) {
 ccm_status launch_batch(ccm_context* ctx, Batch* b, bool inject) {
   int64_t series_elems = 0, out = 0;
   for (auto& j : b->jobs) {
-    append_units(j->pc, series_elems, out, &b->ul, j->table_cap);
+    append_units(j->pc, series_elems, out, &b->ul, room_of(ctx, j->room));
     series_elems += (int64_t)j->pc.V * j->pc.n;
     out += j->n_units;
   }
@@ -1960,7 +1975,7 @@ ccm_status ccm_submit(ccm_context* ctx, const ccm_problem* prob, const float* se
   const size_t elems = (size_t)j->pc.V * (size_t)j->pc.n;
   if (!all_finite(series, elems)) return fail(CCM_EINVAL, "series holds a non-finite value");
   j->n_units = j->pc.n_units();
-  j->footprint = job_footprint(ctx, j->pc, &j->pairs, &j->table_cap);
+  j->footprint = job_footprint(ctx, j->pc, &j->pairs, &j->room);
   if (j->footprint > ctx->budget)
     return fail(CCM_ETOOLARGE, "job footprint " + std::to_string(j->footprint) +
                                    " B exceeds the context budget");

@@ -125,3 +125,49 @@ def test_table_beside_a_manifold_too_long_for_one(ccm):
         ccm.ccm_context_destroy(ctx)
     assert np.all(np.isfinite(rho[0]))
     np.testing.assert_array_equal(rho[0], rho[ccm.CCM_NO_TABLE])
+
+
+def test_many_targets_give_way_to_the_budget(ccm):
+    """Variables of many targets read a time-major copy of the series; a plan or job that
+    does not fit with it runs without, to the same bits."""
+    n, V = 20011, 40
+    rng = np.random.default_rng(6)
+    p = I.Problem(series=rng.random((V, n), dtype=np.float32),
+                  pairs=np.array([[0, i] for i in range(1, 15)] + [[1, 0]], np.int32),
+                  E=np.array([2], np.int32), tau=np.array([1], np.int32),
+                  L=np.array([30], np.int64), r=2, seed=3)
+    copy = n * 64 * 4
+
+    def run(budget, flags=ccm.CCM_NO_TABLE):
+        ctx = ccm.ccm_context_create(0, budget)
+        try:
+            plan = ccm.plan_problem(ctx, p, flags)
+            try:
+                rho = np.zeros(ccm.rho_shape(p))
+                ccm.ccm_run(plan, p.series, rho)
+                return ccm.ccm_plan_get_info(plan)["device_bytes"], rho
+            finally:
+                ccm.ccm_plan_destroy(plan)
+        finally:
+            ccm.ccm_context_destroy(ctx)
+
+    full, want = run(0)
+    for budget in (full, full - 1, full - copy):
+        size, rho = run(budget)
+        assert size <= budget
+        np.testing.assert_array_equal(rho, want)
+    with pytest.raises(ccm.CCMError) as ei:
+        run(full - copy - (1 << 20))
+    assert ei.value.status == ccm.CCM_ETOOLARGE
+    ctx = ccm.ccm_context_create(0, full - copy)
+    try:
+        ticket = ccm.ccm_submit(ctx, p.series, p.pairs, p.E, p.tau, p.L, p.r, p.seed)
+        rho = np.zeros_like(want)
+        for _ in range(600):
+            if ccm.ccm_poll(ctx, ticket, rho, 100) == ccm.CCM_OK:
+                break
+        else:
+            pytest.fail("job did not finish")
+        np.testing.assert_array_equal(rho, want)
+    finally:
+        ccm.ccm_context_destroy(ctx)

@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
     uint32_t* mask = s_mask + tid;
     uint16_t* step = s_step + tid;
     for (int tile = tile0; tile < tile1; ++tile) {
+      const SeriesScale sc = p.obs_stat[tg.obs_tile + tile].series;
       const int nq = min(kQT, n_m - tile * kQT);
       for (int i = 0; i < kQueriesPerWarp; ++i) {
         const int q = warp * kQueriesPerWarp + i;
@@ -290,7 +291,6 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(KnnParams p) {
         const float* ys = s_vec + vec * kScanVec;
         const float2* a = p.obs + rec * kQT;
         const ObsStat* stat = p.obs_stat + rec;
-        const SeriesScale sc = stat->series;
         const float scale = sc.scale, c0 = __fmul_rn(ys[0], scale);
         const packed cc = pack2(c0, c0), ss = pack2(scale, scale);
         TileSums2 both = zero_sums2();

@@ -178,6 +178,7 @@ struct TableJob {
   int64_t pts_off;      // the points in query order: [chunk of 32][E][32] floats
   int64_t box_off;      // chunk boxes [2E][32 * superchunks], superchunk boxes [2E][superchunks]
   int64_t sbox_off;
+  int64_t least_off;    // smallest manifold index of every chunk, of every superchunk (int32)
   int64_t sample_off;   // every sample-th point, [E][n_m / sample]
   int32_t sample;       // (sample_stride)
   int32_t tv_i;         // >= 0: also store target variable tv_i's value at every entry's point

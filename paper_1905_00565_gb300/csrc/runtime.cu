@@ -538,7 +538,8 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
           tj.box_off = tj.pts_off + chunks * 32 * E;
           tj.sbox_off = tj.box_off + 2 * E * supers * 32;
           tj.sample = sample_stride(n_m, R);
-          tj.sample_off = tj.sbox_off + 2 * E * supers;
+          tj.least_off = tj.sbox_off + 2 * E * supers;
+          tj.sample_off = tj.least_off + supers * 33;
           ul->points_total = (tj.sample_off + n_m / tj.sample * E + 63) / 64 * 64;
           tj.tv_i = tv ? pc.pairs[2 * pairs_of[j][0] + 1] : -1;
           if (tv) ul->table_tv = true;

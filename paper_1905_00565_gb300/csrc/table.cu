@@ -12,13 +12,15 @@ namespace {
 constexpr int kPointThreads = 1024;  // one superchunk: 32 chunks of 32 points
 
 // One CTA per superchunk: coordinates [chunk][E][32], the chunk boxes and the
-// superchunk's box (TableJob).  A box's sides are (lo, hi) per coordinate,
+// superchunk's box, and the smallest manifold index of each (TableJob).  A box's
+// sides are (lo, hi) per coordinate,
 // arrays over the boxes; NaN coordinates are left out of them, and positions
 // past the manifold's end do not count.
 __global__ void __launch_bounds__(kPointThreads)
 table_points_kernel(const float* series, const TableJob* jobs, const int32_t* order,
                     float* points) {
   __shared__ float s_lo[32], s_hi[32];
+  __shared__ int s_least[32];
   chain_begin();
   const TableJob jb = jobs[blockIdx.y];
   const int n_m = jb.n_m, E = jb.E, tau = jb.tau, off = (E - 1) * tau;
@@ -30,6 +32,14 @@ table_points_kernel(const float* series, const TableJob* jobs, const int32_t* or
   const float* s = series + jb.series_off + (int64_t)jb.j * jb.n;
   const bool valid = pos < n_m;
   const int m = valid ? order[jb.order_off + pos] : 0;
+  int32_t* least = reinterpret_cast<int32_t*>(points + jb.least_off);
+  const int first = __reduce_min_sync(0xffffffffu, valid ? m : n_m);
+  if (lane == 0) least[chunk] = s_least[warp] = first;
+  __syncthreads();
+  if (warp == 0) {
+    const int all = __reduce_min_sync(0xffffffffu, s_least[lane]);
+    if (lane == 0) least[n_super * 32 + super] = all;
+  }
   for (int e = 0; e < E; ++e) {
     const float c = valid ? s[m + off - e * tau] : 0.f;
     if (chunk < n_chunks) points[jb.pts_off + ((int64_t)chunk * E + e) * 32 + lane] = c;

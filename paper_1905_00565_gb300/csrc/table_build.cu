@@ -32,12 +32,16 @@
 //    distance's own rounding order, so it is at most every FP32 squared
 //    distance in the box.
 //  * The threshold is a key (squared distance, index) under which between R
-//    and C points lie: the previous row's, scaled to the wanted count (rows of
-//    one CTA are consecutive in query order, so their neighbourhoods are
-//    alike), else the k-th smallest distance of a sample (one histogram); when
-//    the collected count misses [R, C] it is bisected, over the index among
-//    ties.  Every point at or below it is collected, so the R smallest are
-//    among them.
+//    and C points lie: the previous row's (of the same point as it is, else
+//    scaled to the wanted count: rows of one CTA are consecutive in query order,
+//    so their neighbourhoods are alike), else the k-th smallest distance of a
+//    sample (one histogram).  When the collected count misses [R, C], histograms
+//    of the distances between the two sides narrow it down by a factor of 1024
+//    each; where more than fit tie, of their indices.  Every point at or below
+//    it is collected, so the R smallest are among them.  A chunk whose box lies
+//    at the tied distance itself is skipped when its smallest index is above the
+//    threshold's: equal points lie in index order, so of a value that fills half
+//    a series the first few chunks are read.
 //  * The collected keys are sorted by 1024 bins of the distance's bit pattern
 //    below the threshold (256 per octave in the two octaves that hold most keys
 //    of a manifold, 64 below, so a bin holds a handful) and, within a bin, by
@@ -62,7 +66,7 @@ constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kBins = 1024;
 constexpr int kSampleShift = 17;   // sample bins: 64 per octave, 16 octaves
 constexpr int kCrowded = 128;      // keys of a bin ranked by counting, at most
-constexpr int kAttempts = 256;     // thresholds tried for a row (a few; bisection needs 64)
+constexpr int kAttempts = 256;     // thresholds tried for a row (a few)
 constexpr int kSegment = 64;       // superchunks whose chunks are listed at a time
 
 // Collected keys of a row, at most: twice as many as wanted (half as many again
@@ -80,14 +84,237 @@ size_t build_smem(int max_R, int max_nm) {
          ((size_t)capacity(max_R) + supers + listed + 8) * 2;
 }
 
+template <int E>
+struct Point {
+  float x[E];
+};
+
+// What is known of a row's threshold once one missed.
+struct RowSearch {
+  uint32_t lo, hi, step;          // squared distances under which too few, too many lie
+  int lo_m, hi_m, below, above;   // indices likewise, among ties; the counts at the two sides
+  bool have_lo, have_hi, halved, ties;
+};
+
+template <int kThreads>
+struct BlockState {
+  uint32_t scan[kThreads / 32], top, found, crowd;
+  int supers, chunks, count, equal;
+  RowSearch row;
+};
+
+// Lower bound of the squared distances of q to box i of an array of `n` boxes.
+template <int E>
+__device__ __forceinline__ uint32_t box_bound(const Point<E>& q, const float* b, int n, int i) {
+  float lb = 0.f;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const float g = fmaxf(fmaxf(__fsub_rn(b[2 * e * n + i], q.x[e]),
+                                __fsub_rn(q.x[e], b[(2 * e + 1) * n + i])), 0.f);
+    lb = (e == 0) ? __fmul_rn(g, g) : __fmaf_rn(g, g, lb);
+  }
+  return __float_as_uint(lb);
+}
+
+// Exclusive scan of the bins in place; thread t holds bins [t*B, (t+1)*B).  With
+// rank > 0 also sh.found = the bin holding that (1-based) rank; sh.crowd: the
+// largest bin.  Block-wide, ends behind a barrier.
+template <int kThreads>
+__device__ __forceinline__ void scan(uint32_t* bins, BlockState<kThreads>& sh, uint32_t rank) {
+  constexpr int kPer = kBins / kThreads, kWarps = kThreads / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t v[kPer], sum = 0u, most = 0u;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    v[i] = bins[tid * kPer + i];
+    sum += v[i];
+    most = max(most, v[i]);
+  }
+  uint32_t incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFullMask, incl, o);
+    if (lane >= o) incl += y;
+  }
+  most = __reduce_max_sync(kFullMask, most);
+  if (lane == 31) sh.scan[warp] = incl;
+  if (lane == 0 && most > (uint32_t)kCrowded) sh.crowd = 1u;
+  __syncthreads();
+  uint32_t before = incl - sum;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) before += (w < warp) ? sh.scan[w] : 0u;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    bins[tid * kPer + i] = before;
+    if (rank > before && rank <= before + v[i]) sh.found = (uint32_t)(tid * kPer + i);
+    before += v[i];
+  }
+  __syncthreads();
+}
+
+// The points within squared distance `most` of query q at position pos (to the bit),
+// into the bins, which are cleared first: with m_from < 0 by (bits - from) >> shift,
+// those below `from` to bin 0; else those at `most` with index m_from .. m_to by
+// (index - m_from) >> shift.  Block-wide, behind the closing barrier.
 template <int E, int kThreads>
-__global__ void __launch_bounds__(kThreads, 1024 / kThreads)
+__device__ __forceinline__ void distance_histogram(const Point<E>& q, const TableJob& jb,
+                                                   const float* points, const int32_t* order, int pos,
+                                                   uint32_t most, uint32_t from, int m_from, int m_to,
+                                                   int shift, uint32_t* bins) {
+  constexpr int kWarps = kThreads / 32;
+  const int n_m = jb.n_m, n_chunks = (n_m + 31) >> 5, n_super = (n_chunks + 31) >> 5;
+  const float* pts = points + jb.pts_off;
+  const float* box = points + jb.box_off;
+  const float* sbox = points + jb.sbox_off;
+  const int32_t* least = reinterpret_cast<const int32_t*>(points + jb.least_off);
+  const int32_t* ord = order + jb.order_off;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < kBins; i += kThreads) bins[i] = 0u;
+  __syncthreads();
+  for (int sc = 0; sc < n_super; ++sc) {
+    if (box_bound(q, sbox, n_super, sc) > most || (m_from >= 0 && least[n_super * 32 + sc] > m_to))
+      continue;
+    const int ch = sc * 32 + lane;
+    // (a warp takes every kWarps-th chunk: few superchunks would not share out)
+    const bool keep = ch < n_chunks && lane % kWarps == warp &&
+                      box_bound(q, box, n_super * 32, min(ch, n_chunks - 1)) <= most &&
+                      (m_from < 0 || least[ch] <= m_to);
+    for (unsigned left = __ballot_sync(kFullMask, keep); left; left &= left - 1u) {
+      const int x0 = (sc * 32 + __ffs(left) - 1) * 32, x = x0 + lane;
+      const float* src = pts + (int64_t)x0 * E + lane;
+      float diff = __fsub_rn(q.x[0], src[0]);
+      float acc = __fmul_rn(diff, diff);
+#pragma unroll
+      for (int e = 1; e < E; ++e) {
+        diff = __fsub_rn(q.x[e], src[e * 32]);
+        acc = __fmaf_rn(diff, diff, acc);
+      }
+      const uint32_t bits = __float_as_uint(acc);
+      if (x >= n_m || x == pos || bits > most) continue;
+      if (m_from < 0) {
+        atomicAdd(&bins[bits < from ? 0u : (bits - from) >> shift], 1u);
+      } else if (bits == most) {
+        const int m = ord[x];
+        if (m >= m_from && m <= m_to) atomicAdd(&bins[(m - m_from) >> shift], 1u);
+      }
+    }
+    __syncwarp();
+  }
+  __syncthreads();
+}
+
+// A row's next threshold after (tb, tm) missed: `c` points lie at or below it, `equal`
+// at tb itself (whatever their index).  Block-wide, behind the closing barrier; in
+// sh.row what is known of the row (`first`: nothing yet).  Not inlined: few rows come
+// here, and its registers are the collecting loop's.
+struct Threshold {
+  uint32_t tb, tm;
+};
+template <int E, int kThreads>
+__device__ __noinline__ Threshold next_threshold(const Point<E> q, const TableJob* jobs,
+                                                 const float* points, const int32_t* order, int pos,
+                                                 Threshold t, int c, int equal, bool first,
+                                                 uint32_t* bins, BlockState<kThreads>* state) {
+  BlockState<kThreads>& sh = *state;
+  const TableJob& jb = jobs[blockIdx.y];
+  const int n_m = jb.n_m, R = jb.R, C = capacity(R), target = wanted(R);
+  RowSearch s = {0u, 0u, 1u << 19, -1, 0, 0, 0, false, false, false, false};
+  if (!first) s = sh.row;
+  __syncthreads();  // read by all before it is written
+  bool tied = false;  // just now: an index is guessed first
+  if (s.ties) {
+    if (c < R) {
+      s.lo_m = (int)t.tm;
+      s.below = c;
+    } else {
+      s.hi_m = (int)t.tm;
+      s.above = c;
+    }
+  } else {
+    // a tie that does not fit, known at once (when no tie was left out: a
+    // carried-over threshold may have an index)
+    tied = t.tm == 0xffffffffu && c > C && c - equal < R;
+    if (c < R) {
+      s.lo = t.tb;
+      s.have_lo = true;
+      s.below = c;
+    } else {
+      s.hi = t.tb;
+      s.have_hi = true;
+      s.above = c;
+    }
+    t.tm = 0xffffffffu;
+    if (tied) s.below = c - equal;
+  }
+  const bool step = !s.ties && !tied && (!(s.have_lo && s.have_hi) || !s.halved);
+  if (step) {  // (of distances that differ, a step or the middle of two mostly holds)
+    if (s.step < (1u << 30)) s.step <<= 1;
+    s.halved = s.have_lo && s.have_hi;
+    if (s.halved) t.tb = s.lo + (s.hi - s.lo) / 2u;
+    else if (s.have_lo) t.tb = s.lo > 0xffffffffu - s.step ? 0xffffffffu : s.lo + s.step;
+    else t.tb = s.hi > s.step ? s.hi - s.step : 0u;
+  }
+  while (!step && !tied) {
+    const uint32_t from = s.have_lo ? s.lo + 1u : 0u;
+    const uint32_t span = s.ties ? (uint32_t)(s.hi_m - s.lo_m - 1) : s.hi - from;
+    int shift = 0;
+    while (span >> shift >= (uint32_t)kBins) ++shift;
+    const int known = s.ties ? s.below : 0;
+    distance_histogram<E, kThreads>(q, jb, points, order, pos, s.ties ? t.tb : s.hi, from,
+                                    s.ties ? s.lo_m + 1 : -1, s.hi_m, shift, bins);
+    scan<kThreads>(bins, sh, (uint32_t)(target - known));
+    // the bin in which the wanted count is reached; the counts before it and through it
+    const uint32_t f = sh.found;
+    int before = (int)bins[f] + known;
+    const int through = f + 1u < (uint32_t)kBins ? (int)bins[f + 1u] + known : s.above;
+    __syncthreads();
+    if (f == 0u) before = s.below;  // by distance, the first bin holds what lies below `from`, too
+    // the last key of the bin before, and of this one
+    const uint32_t lowest = s.ties ? (uint32_t)(s.lo_m + 1) : from;
+    const uint32_t was = lowest + (f << shift) - 1u;
+    const uint32_t end = lowest + (uint32_t)min((uint64_t)span, ((uint64_t)(f + 1u) << shift) - 1u);
+    if (through <= C || before >= R) {
+      const uint32_t key = through <= C ? end : was;
+      if (s.ties) t.tm = key;
+      else t.tb = key;
+      break;
+    }
+    s.below = before;
+    s.above = through;
+    if (s.ties) {
+      s.lo_m = (int)was;
+      s.hi_m = (int)end;
+    } else {
+      if (f > 0u) {
+        s.lo = was;
+        s.have_lo = true;
+      }
+      s.hi = end;
+      tied = shift == 0;  // one distance is left
+    }
+  }
+  if (tied) {
+    // more than fit tie at hi: up to an index, first guessed as if the tied points'
+    // were spread evenly
+    s.ties = true;
+    s.lo_m = -1;
+    s.hi_m = n_m - 1;
+    t.tb = s.hi;
+    t.tm = (uint32_t)((int64_t)n_m * (target - s.below) / (s.above - s.below));
+  }
+  if (threadIdx.x == 0) sh.row = s;
+  __syncthreads();
+  return t;
+}
+
+// (nine CTAs of 128 threads an SM for E <= 6: eight take 7 to 13 % longer)
+template <int E, int kThreads>
+__global__ void __launch_bounds__(kThreads, (E <= 6 ? 1152 : 1024) / kThreads)
 table_build_kernel(const float* series, const TableJob* jobs, const float* points,
                    const int32_t* order, const int32_t* inverse, void* table, float* table_dist,
                    int pairs, int u16, int rows_per_cta, int cap, int32_t* err) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ uint32_t s_scan[kThreads / 32], s_top, s_found, s_crowd;
-  __shared__ int s_supers, s_chunks, s_count, s_equal;
+  __shared__ BlockState<kThreads> sh;
   constexpr int kWarps = kThreads / 32;
   chain_begin();
   const TableJob jb = jobs[blockIdx.y];
@@ -107,57 +334,18 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
   const float* pts = points + jb.pts_off;          // [chunk][E][32]
   const float* box = points + jb.box_off;          // [2E][n_super*32]
   const float* sbox = points + jb.sbox_off;        // [2E][n_super]
+  const int32_t* least = reinterpret_cast<const int32_t*>(points + jb.least_off);  // [n_super*32]
+  const int32_t* sleast = least + n_super * 32;    // [n_super]
   const int32_t* ord = order + jb.order_off;
   const int32_t* inv = inverse + jb.order_off;
   const int off = (E - 1) * jb.tau;
   const bool has_value = pairs && jb.tv_i >= 0;
   const float* tv = series + jb.series_off + (int64_t)(jb.tv_i >= 0 ? jb.tv_i : 0) * jb.n + off;
 
-  float q[E];
-  // lower bound of the squared distances to box i of an array of `n` boxes
-  auto bound = [&](const float* b, int n, int i) {
-    float lb = 0.f;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const float g = fmaxf(fmaxf(__fsub_rn(b[2 * e * n + i], q[e]),
-                                  __fsub_rn(q[e], b[(2 * e + 1) * n + i])), 0.f);
-      lb = (e == 0) ? __fmul_rn(g, g) : __fmaf_rn(g, g, lb);
-    }
-    return __float_as_uint(lb);
-  };
-  // Exclusive scan of s_bin in place; thread t holds bins [t*B, (t+1)*B).  With
-  // rank > 0 also s_found = the bin holding that (1-based) rank; s_crowd: the
-  // largest bin.  Block-wide, ends behind a barrier.
+  Point<E> q;
+  auto bound = [&](const float* b, int n, int i) { return box_bound(q, b, n, i); };
+  auto scan_bins = [&](uint32_t rank) { scan<kThreads>(s_bin, sh, rank); };
   constexpr int kPer = kBins / kThreads;
-  auto scan_bins = [&](uint32_t rank) {
-    uint32_t v[kPer], sum = 0u, most = 0u;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      v[i] = s_bin[tid * kPer + i];
-      sum += v[i];
-      most = max(most, v[i]);
-    }
-    uint32_t incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(kFullMask, incl, o);
-      if (lane >= o) incl += y;
-    }
-    most = __reduce_max_sync(kFullMask, most);
-    if (lane == 31) s_scan[warp] = incl;
-    if (lane == 0 && most > (uint32_t)kCrowded) s_crowd = 1u;
-    __syncthreads();
-    uint32_t before = incl - sum;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) before += (w < warp) ? s_scan[w] : 0u;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      s_bin[tid * kPer + i] = before;
-      if (rank > before && rank <= before + v[i]) s_found = (uint32_t)(tid * kPer + i);
-      before += v[i];
-    }
-    __syncthreads();
-  };
   auto clear_bins = [&]() {
 #pragma unroll
     for (int i = 0; i < kPer; ++i) s_bin[tid + i * kThreads] = 0u;
@@ -170,97 +358,112 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
   uint32_t tb = 0xffffffffu, tm = 0xffffffffu;  // the threshold
   bool guess = false;  // tb, tm are carried over from the previous row
   int distrust = 0;    // rows left that sample at once: a carried threshold missed
+  uint32_t kept_tb = tb;  // the previous row's threshold itself (its tm is tm)
 
   for (int pos = row0; pos < row1; ++pos) {
+    bool same = pos > row0;  // the previous row's point again: its threshold fits
     {
       const float* c = pts + (int64_t)(pos >> 5) * (E * 32) + (pos & 31);
 #pragma unroll
-      for (int e = 0; e < E; ++e) q[e] = c[e * 32];
+      for (int e = 0; e < E; ++e) {
+        const float x = c[e * 32];
+        same = same && x == q.x[e];
+        q.x[e] = x;
+      }
     }
     bool all = n_m - 1 <= C;  // everything fits: no threshold
-    bool sampled = false, have_lo = false, have_hi = false, ties = false;
-    uint32_t lo = 0u, hi = 0u, step = 1u << 19;
-    int64_t lo_m = -1, hi_m = 0;
+    bool sampled = false, missed = false;
     if (all) tb = tm = 0xffffffffu;
+    if (same && !all) {
+      tb = kept_tb;
+      guess = true;
+    }
     int c = 0;
     for (int attempt = 0;; ++attempt) {
       if (!all && !guess && !sampled) {
         // the k-th smallest sampled distance, to a bin
         sampled = true;
-        if (tid == 0) s_top = 0u;
+        if (tid == 0) sh.top = 0u;
         __syncthreads();
         uint32_t top = 0u;  // the farthest any point can be
         for (int i = tid; i < n_super; i += kThreads) {
           float ub = 0.f;
 #pragma unroll
           for (int e = 0; e < E; ++e) {
-            const float g = fmaxf(fabsf(__fsub_rn(sbox[2 * e * n_super + i], q[e])),
-                                  fabsf(__fsub_rn(q[e], sbox[(2 * e + 1) * n_super + i])));
+            const float g = fmaxf(fabsf(__fsub_rn(sbox[2 * e * n_super + i], q.x[e])),
+                                  fabsf(__fsub_rn(q.x[e], sbox[(2 * e + 1) * n_super + i])));
             ub = __fmaf_rn(g, g, ub);
           }
           top = max(top, __float_as_uint(ub));
         }
         top = __reduce_max_sync(kFullMask, top);
-        if (lane == 0) atomicMax(&s_top, top);
+        if (lane == 0) atomicMax(&sh.top, top);
         __syncthreads();
-        // 16 octaves up to the farthest point; while the k-th lies below them,
-        // the next 16 octaves down
-        constexpr uint32_t kSpan = (uint32_t)kBins << kSampleShift;
-        top = s_top + (1u << 21);
-        for (;;) {
-          const uint32_t base = top > kSpan ? top - kSpan : 0u;
+        // 16 octaves up to the farthest point; where the k-th lies below them, all
+        // that is below in coarser bins, the first of which stands for distance 0
+        top = sh.top + (1u << 21);
+        uint32_t base = top > (uint32_t)kBins << kSampleShift ? top - ((uint32_t)kBins << kSampleShift) : 0u;
+        for (int shift = kSampleShift;;) {
           clear_bins();
-          if (tid == 0) s_found = kBins;
+          if (tid == 0) sh.found = kBins;
           __syncthreads();
           for (int i = tid; i < n_sample; i += kThreads) {
-            float diff = __fsub_rn(q[0], smp[i]);
+            float diff = __fsub_rn(q.x[0], smp[i]);
             float acc = __fmul_rn(diff, diff);
 #pragma unroll
             for (int e = 1; e < E; ++e) {
-              diff = __fsub_rn(q[e], smp[e * n_sample + i]);
+              diff = __fsub_rn(q.x[e], smp[e * n_sample + i]);
               acc = __fmaf_rn(diff, diff, acc);
             }
             const uint32_t bits = __float_as_uint(acc);
             if (bits < top)
-              atomicAdd(&s_bin[bits < base ? 0u : min((bits - base) >> kSampleShift, (uint32_t)kBins - 1u)], 1u);
+              atomicAdd(&s_bin[bits < base ? 0u : min((bits - base) >> shift, (uint32_t)kBins - 1u)], 1u);
           }
           __syncthreads();
           scan_bins(stride == 1 ? (uint32_t)R + 1u : (uint32_t)((target + stride - 1) / stride + 1));
-          const uint32_t found = s_found;
+          const uint32_t found = sh.found;
           __syncthreads();  // read by all before it is reset
           if (found == 0u && base > 0u) {
             top = base + (1u << kSampleShift);
+            base = 0u;
+            while ((top - 1u) >> shift >= (uint32_t)kBins) ++shift;
             continue;
           }
-          tb = found == (uint32_t)kBins ? 0xffffffffu : base + ((found + 1u) << kSampleShift) - 1u;
+          tb = found == (uint32_t)kBins ? 0xffffffffu : found == 0u ? 0u : base + ((found + 1u) << shift) - 1u;
           break;
         }
         tm = 0xffffffffu;
       }
       // collect every point at or below the threshold
+      const bool limited = tm != 0xffffffffu;
+      auto reaches = [&](uint32_t b, const int32_t* smallest, int i) {
+        bool yes = b <= tb;
+        if (limited && b == tb) yes = (uint32_t)smallest[i] <= tm;
+        return yes;
+      };
       __syncthreads();
-      if (tid == 0) s_supers = s_count = s_equal = 0;
+      if (tid == 0) sh.supers = sh.count = sh.equal = 0;
       __syncthreads();
       for (int i = tid; i < n_super; i += kThreads)
-        if (bound(sbox, n_super, i) <= tb) s_super[atomicAdd(&s_supers, 1)] = (uint16_t)i;
+        if (reaches(bound(sbox, n_super, i), sleast, i)) s_super[atomicAdd(&sh.supers, 1)] = (uint16_t)i;
       __syncthreads();
-      const int supers = s_supers;
+      const int supers = sh.supers;
       int equal = 0;
       for (int g0 = 0; g0 < supers; g0 += kSegment) {
         if (g0 > 0) __syncthreads();  // the previous segment's list has been read
-        if (tid == 0) s_chunks = 0;
+        if (tid == 0) sh.chunks = 0;
         __syncthreads();
         for (int i = g0 + warp; i < min(supers, g0 + kSegment); i += kWarps) {
           const int ch = s_super[i] * 32 + lane;
-          const bool keep = ch < n_chunks && bound(box, n_super * 32, min(ch, n_chunks - 1)) <= tb;
+          const bool keep = ch < n_chunks && reaches(bound(box, n_super * 32, min(ch, n_chunks - 1)), least, ch);
           const unsigned bal = __ballot_sync(kFullMask, keep);
           int at = 0;
-          if (lane == 0 && bal) at = atomicAdd(&s_chunks, __popc(bal));
+          if (lane == 0 && bal) at = atomicAdd(&sh.chunks, __popc(bal));
           at = __shfl_sync(kFullMask, at, 0);
           if (keep) s_chunk[at + __popc(bal & below_lane)] = (uint16_t)ch;
         }
         __syncthreads();
-        const int chunks = s_chunks;
+        const int chunks = sh.chunks;
         auto collect = [&](int x, uint32_t bits, uint32_t m) {  // position x (past the end: not valid)
           bool hit = x < n_m && x != pos && bits <= tb;
           unsigned bal = __ballot_sync(kFullMask, hit);
@@ -272,7 +475,7 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
             bal = __ballot_sync(kFullMask, hit);
           }
           int at = 0;
-          if (lane == 0) at = atomicAdd(&s_count, __popc(bal));
+          if (lane == 0) at = atomicAdd(&sh.count, __popc(bal));
           at = __shfl_sync(kFullMask, at, 0) + __popc(bal & below_lane);
           if (hit && at < C) {
             s_bits[at] = bits;
@@ -299,11 +502,11 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
           for (int d = 0; d < kAhead; ++d) {
             const int i = i0 + d * kWarps;
             if (i >= chunks) break;
-            float diff = __fsub_rn(q[0], c[d][0]);
+            float diff = __fsub_rn(q.x[0], c[d][0]);
             float acc = __fmul_rn(diff, diff);
 #pragma unroll
             for (int e = 1; e < E; ++e) {
-              diff = __fsub_rn(q[e], c[d][e]);
+              diff = __fsub_rn(q.x[e], c[d][e]);
               acc = __fmaf_rn(diff, diff, acc);
             }
             const int m = mm[d];
@@ -312,66 +515,44 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
           }
         }
       }
-      if (lane == 0 && equal) atomicAdd(&s_equal, equal);
+      if (lane == 0 && equal) atomicAdd(&sh.equal, equal);
       __syncthreads();
-      c = s_count;
+      c = sh.count;
       if (c >= R && c <= C) break;
       if (attempt == kAttempts) {  // never: the bisection has ended before
         if (tid == 0) atomicOr(err, kErrTable);
         c = min(c, C);
         break;
       }
-      // missed: bracket the threshold
-      if (ties) {
-        if (c < R) lo_m = tm;
-        else hi_m = tm;
-        tm = (uint32_t)((lo_m + hi_m) >> 1);
-        continue;
-      }
-      if (c < R) {
-        lo = tb;
-        have_lo = true;
-      } else {
-        hi = tb;
-        have_hi = true;
-        // points nearer than tb (known when no tie was left out: a carried-over
-        // threshold may have an index)
-        const int less = c - s_equal;
-        if (tm == 0xffffffffu && less < R) {  // more than fit tie at tb: the smallest indices
-          ties = true;
-          hi_m = min((int64_t)tm, (int64_t)n_m);
-          const int64_t want = (int64_t)(R + C) / 2 - less;
-          tm = (uint32_t)min(hi_m - 1, (int64_t)n_m * want / (c - less));
-          guess = false;
-          sampled = true;
-          continue;
-        }
-      }
-      tm = 0xffffffffu;
-      if (guess) {  // the carried threshold missed: sample, here and for some rows
+      const int equal_all = sh.equal;
+      if (guess && !(tm == 0xffffffffu && c > C && c - equal_all < R)) {
+        // the carried threshold missed (and shows no tie): sample, here and for some rows
         guess = false;
         distrust = 6;
-        have_lo = have_hi = false;
         continue;
       }
-      if (step < (1u << 30)) step <<= 1;
-      if (have_lo && have_hi) tb = lo + (hi - lo) / 2u;
-      else if (have_lo) tb = lo > 0xffffffffu - step ? 0xffffffffu : lo + step;
-      else tb = hi > step ? hi - step : 0u;
+      guess = false;
+      sampled = true;
+      const Threshold next = next_threshold<E, kThreads>(q, jobs, points, order, pos, Threshold{tb, tm},
+                                                         c, equal_all, !missed, s_bin, &sh);
+      tb = next.tb;
+      tm = next.tm;
+      missed = true;
     }
+    const int kept = min(R, c);
 
     // sort: count, scan, scatter by bin (ascending distance), rank inside bins
     clear_bins();
-    if (tid == 0) s_crowd = s_top = 0u;
+    if (tid == 0) sh.crowd = sh.top = 0u;
     __syncthreads();
     uint32_t top = tb;
     if (all) {  // no threshold: bins below the largest distance
       top = 0u;
       for (int t = tid; t < c; t += kThreads) top = max(top, s_bits[t]);
       top = __reduce_max_sync(kFullMask, top);
-      if (lane == 0) atomicMax(&s_top, top);
+      if (lane == 0) atomicMax(&sh.top, top);
       __syncthreads();
-      top = s_top;
+      top = sh.top;
     }
     auto bin_of = [&](uint32_t bits) {
       const uint32_t d = top - bits;  // 2^23 bit patterns an octave
@@ -394,7 +575,7 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
       if (u16) static_cast<uint16_t*>(table)[base + rank] = (uint16_t)at;
       else static_cast<int32_t*>(table)[base + rank] = at;
     };
-    if (s_crowd == 0u) {
+    if (sh.crowd == 0u) {
       for (int t = tid; t < c; t += kThreads)
         s_idx[atomicAdd(&s_bin[bin_of(s_bits[t])], 1u)] = (uint16_t)t;
       __syncthreads();  // s_bin[b] is now the end of bin b
@@ -438,10 +619,10 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
           __syncthreads();
         }
       }
-      for (int r = tid; r < R; r += kThreads)
+      for (int r = tid; r < kept; r += kThreads)
         emit(r, s_bits[r], has_value ? __ldg(tv + s_m[r]) : 0.f, __ldg(inv + s_m[r]));
     }
-    for (int r = R + tid; r < jb.stride; r += kThreads) {
+    for (int r = kept + tid; r < jb.stride; r += kThreads) {
       if (u16) static_cast<uint16_t*>(table)[base + r] = (uint16_t)n_m;
       else static_cast<int32_t*>(table)[base + r] = n_m;
     }
@@ -449,7 +630,8 @@ table_build_kernel(const float* series, const TableJob* jobs, const float* point
     // exponent of a neighbourhood of two to three dimensions)
     guess = !all && distrust == 0;
     distrust -= distrust > 0 ? 1 : 0;
-    if (!ties && tb < 0x7f000000u) {
+    kept_tb = tb;
+    if (tm == 0xffffffffu && tb < 0x7f000000u) {
       const float f = __powf((float)target / (float)c, 0.8f);
       tb = __float_as_uint(__fmul_rn(__uint_as_float(tb), fminf(fmaxf(f, 0.5f), 2.f)));
     }

@@ -716,6 +716,73 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
         }
         if (__any_sync(kFull, cnt > room)) make_room();
       }
+      // one aligned run of kPairs pairs from pair `at` on
+      auto step = [&](int at) {
+        if (kStats) st_begun += kStep;
+        // Partial sums over the first E1 coordinates are lower bounds of the
+        // full FP32 sums (all terms are >= 0 and rounding is monotone), so a
+        // step whose partials are all above every lane's threshold cannot
+        // contribute a candidate and skips the remaining coordinates.
+        u64 r[kPairs];
+#pragma unroll
+        for (int pp = 0; pp < kPairs; ++pp)
+          r[pp] = sqdist2_range<E, 0, (kE1<E, V>)>(qc, s_coord + (size_t)(at + pp) * EP, 0ull);
+        const float th = tl[K - 1];
+        float d[kStep];
+#pragma unroll
+        for (int pp = 0; pp < kPairs; ++pp) unpack2(r[pp], d[2 * pp], d[2 * pp + 1]);
+        if (kStats && (kE1<E, V>) == E) st_full += kStep;
+        if (!__any_sync(kFull, min_all(d) <= th)) return;
+        if constexpr ((kE1<E, V>) < E) {
+          if (kStats) st_full += kStep;
+#pragma unroll
+          for (int pp = 0; pp < kPairs; ++pp) {
+            r[pp] = sqdist2_range<E, (kE1<E, V>), E>(qc, s_coord + (size_t)(at + pp) * EP, r[pp]);
+            unpack2(r[pp], d[2 * pp], d[2 * pp + 1]);
+          }
+          if (!__any_sync(kFull, min_all(d) <= th)) return;
+        }
+        // the run's library indices (one broadcast 16-byte load per four); its pairs
+        // that are not kept lie above every threshold, and the first points' runs
+        // hold nothing else (both are whole runs)
+        int li[kStep];
+#pragma unroll
+        for (int q4 = 0; q4 < kStep / 4; ++q4) {
+          const int4 v = *reinterpret_cast<const int4*>(s_lidx + 2 * at + 4 * q4);
+          li[4 * q4] = v.x;
+          li[4 * q4 + 1] = v.y;
+          li[4 * q4 + 2] = v.z;
+          li[4 * q4 + 3] = v.w;
+        }
+#pragma unroll
+        for (int pt = 0; pt < kStep; ++pt) {
+          // at or below the threshold (never a sentinel: NaN), outside the
+          // exclusion window |l - m| <= W (W = 0 drops only m itself, and
+          // the unsigned form tests both sides at once); appended without a
+          // branch
+          const bool take =
+              (d[pt] <= th) & ((unsigned)li[pt] - (unsigned)m + (unsigned)W > 2u * (unsigned)W);
+          if (take) col[cnt * kThreads] = pack_key(d[pt], li[pt]);
+          cnt += take ? 1 : 0;
+        }
+        if (__any_sync(kFull, cnt - done >= merge_at || cnt > room)) make_room();
+      };
+      if constexpr (E <= 2) {
+        if (!p.prune) {
+          // nothing to exclude: run after run, without a mask to walk (a run is 20
+          // instructions here and the walk 6: N = 20000 in time order, E = 1, L = 400,
+          // r = 100 0.72 -> 0.64 ms)
+          for (int jg = 0; jg < ng; ++jg) {
+            int g = (base >> 6) + jg;
+            g -= (g >= ng) ? ng : 0;
+            const int end = min(32 * g + 32, np);
+#pragma unroll 2
+            for (int at = 32 * g; at < end; at += kPairs)
+              if (!(first && (unsigned)(at - (base >> 1)) < (unsigned)(kInit / 2))) step(at);
+          }
+          return;
+        }
+      }
 #pragma unroll 1
       for (int jg = 0; jg < ng; ++jg) {
         int g = (base >> 6) + jg;
@@ -751,55 +818,7 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
           // sweep's brute force 13.3 -> 12.8, N = 10^5 17.2 -> 16.3)
           const int b0 = (__ffs(mask) - 1) & ~(kPairs - 1);
           mask &= ~(((1u << kPairs) - 1u) << b0);
-          const int at = 32 * g + b0;
-          if (kStats) st_begun += kStep;
-          // Partial sums over the first E1 coordinates are lower bounds of the
-          // full FP32 sums (all terms are >= 0 and rounding is monotone), so a
-          // step whose partials are all above every lane's threshold cannot
-          // contribute a candidate and skips the remaining coordinates.
-          u64 r[kPairs];
-#pragma unroll
-          for (int pp = 0; pp < kPairs; ++pp)
-            r[pp] = sqdist2_range<E, 0, (kE1<E, V>)>(qc, s_coord + (size_t)(at + pp) * EP, 0ull);
-          const float th = tl[K - 1];
-          float d[kStep];
-#pragma unroll
-          for (int pp = 0; pp < kPairs; ++pp) unpack2(r[pp], d[2 * pp], d[2 * pp + 1]);
-          if (kStats && (kE1<E, V>) == E) st_full += kStep;
-          if (!__any_sync(kFull, min_all(d) <= th)) continue;
-          if constexpr ((kE1<E, V>) < E) {
-            if (kStats) st_full += kStep;
-#pragma unroll
-            for (int pp = 0; pp < kPairs; ++pp) {
-              r[pp] = sqdist2_range<E, (kE1<E, V>), E>(qc, s_coord + (size_t)(at + pp) * EP, r[pp]);
-              unpack2(r[pp], d[2 * pp], d[2 * pp + 1]);
-            }
-            if (!__any_sync(kFull, min_all(d) <= th)) continue;
-          }
-          // the run's library indices (one broadcast 16-byte load per four); its pairs
-          // that are not kept lie above every threshold, and the first points' runs
-          // hold nothing else (both are whole runs)
-          int li[kStep];
-#pragma unroll
-          for (int q4 = 0; q4 < kStep / 4; ++q4) {
-            const int4 v = *reinterpret_cast<const int4*>(s_lidx + 2 * at + 4 * q4);
-            li[4 * q4] = v.x;
-            li[4 * q4 + 1] = v.y;
-            li[4 * q4 + 2] = v.z;
-            li[4 * q4 + 3] = v.w;
-          }
-#pragma unroll
-          for (int pt = 0; pt < kStep; ++pt) {
-            // at or below the threshold (never a sentinel: NaN), outside the
-            // exclusion window |l - m| <= W (W = 0 drops only m itself, and
-            // the unsigned form tests both sides at once); appended without a
-            // branch
-            const bool take =
-                (d[pt] <= th) & ((unsigned)li[pt] - (unsigned)m + (unsigned)W > 2u * (unsigned)W);
-            if (take) col[cnt * kThreads] = pack_key(d[pt], li[pt]);
-            cnt += take ? 1 : 0;
-          }
-          if (__any_sync(kFull, cnt - done >= merge_at || cnt > room)) make_room();
+          step(32 * g + b0);
         }
       }
     };

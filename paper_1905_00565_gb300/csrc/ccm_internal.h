@@ -386,7 +386,7 @@ cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* 
                        ObsStat* obs_stat, LaunchStream s);
 // rho of every target from its tiles' sums (after the search kernels).
 cudaError_t launch_rho(const UnitDesc* units, const TargetDesc* targets, int64_t n_targets,
-                       const float4* partials, const ObsStat* obs_stat, double* rho,
+                       int max_tiles, const float4* partials, const ObsStat* obs_stat, double* rho,
                        LaunchStream s);
 // Table path: same work items, neighbours read from the distance indexing table.
 cudaError_t knn_table_prepare();

@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(kSmallThreads) obs_kernel(const float* series,
 // loads' latency for few (four tiles' loads are in flight per lane).
 constexpr int kRhoLanes = 4;
 constexpr int kRhoNarrow = 96;
+constexpr int kRhoAhead = 4;  // tiles a lane loads at once
 
 template <int kLanes>
 __device__ __forceinline__ double rho_sum(double v) {
@@ -98,12 +99,34 @@ __device__ __forceinline__ double rho_sum(double v) {
   return v;
 }
 
+// A tile's mean of y and centred sums, from its record (moments.cuh).
+__device__ __forceinline__ double tile_mean(const float4& a, const float4& b, double n, double& b1,
+                                            double& d) {
+  if (b.w != 0.f) return word_pair(a.x, a.y);  // a record in FP64
+  b1 = __dadd_rn((double)a.y, (double)a.z);  // sum(y - c)
+  d = (n == (double)kQT) ? __dmul_rn(b1, 1.0 / kQT) : __ddiv_rn(b1, n);
+  return __dadd_rn((double)a.x, d);
+}
+__device__ __forceinline__ void tile_moments(const float4& a, const float4& b, double n, double& my,
+                                             double& syy, double& sxy) {
+  double b1, d;
+  my = tile_mean(a, b, n, b1, d);
+  if (b.w != 0.f) {
+    syy = word_pair(a.z, a.w);
+    sxy = word_pair(b.x, b.y);
+  } else {
+    const double b2 = __dadd_rn((double)a.w, (double)b.x);
+    syy = fmax(__fma_rn(-b1, d, b2), 0.0);
+    sxy = __dadd_rn((double)b.y, (double)b.z);
+  }
+}
+
 // rho of a target by kLanes lanes (lane `sub` of them); `active` false: the
 // lanes only take part in the shuffles.
 template <int kLanes>
 __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4* base,
                                              const ObsStat* stat, int sub, bool active) {
-  constexpr int kAhead = 4;
+  constexpr int kAhead = kRhoAhead;
   struct Tile {
     float4 a, b;
     double mx, sxx;
@@ -121,15 +144,8 @@ __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4*
     }
   };
   auto count = [&](int q) { return (double)min(kQT, n_m - q * kQT); };
-  // mean(y) of a tile; of paired sums also d = mean(y) - c, b1 = sum(y - c)
-  auto mean = [&](const Tile& t, double n, double& b1, double& d) {
-    if (t.b.w != 0.f) return word_pair(t.a.x, t.a.y);  // a record in FP64
-    b1 = __dadd_rn((double)t.a.y, (double)t.a.z);
-    d = (n == (double)kQT) ? __dmul_rn(b1, 1.0 / kQT) : __ddiv_rn(b1, n);
-    return __dadd_rn((double)t.a.x, d);
-  };
   Tile t[kAhead];
-  double SX = 0.0, SY = 0.0, b1, d;
+  double SX = 0.0, SY = 0.0, b1, d, my, syy, sxy;
   for (int q0 = sub; active && q0 < n_tiles; q0 += kAhead * kLanes) {
     load(q0, t);
 #pragma unroll
@@ -138,7 +154,7 @@ __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4*
       if (q >= n_tiles) break;
       const double n = count(q);
       SX = __fma_rn(n, t[i].mx, SX);
-      SY = __fma_rn(n, mean(t[i], n, b1, d), SY);
+      SY = __fma_rn(n, tile_mean(t[i].a, t[i].b, n, b1, d), SY);
     }
   }
   const double inv = (double)n_m;
@@ -151,16 +167,8 @@ __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4*
       const int q = q0 + i * kLanes;
       if (q >= n_tiles) break;
       const double n = count(q);
-      const double dy = __dsub_rn(mean(t[i], n, b1, d), MY), dx = __dsub_rn(t[i].mx, MX);
-      double syy, sxy;
-      if (t[i].b.w != 0.f) {
-        syy = word_pair(t[i].a.z, t[i].a.w);
-        sxy = word_pair(t[i].b.x, t[i].b.y);
-      } else {
-        const double b2 = __dadd_rn((double)t[i].a.w, (double)t[i].b.x);
-        syy = fmax(__fma_rn(-b1, d, b2), 0.0);
-        sxy = __dadd_rn((double)t[i].b.y, (double)t[i].b.z);
-      }
+      tile_moments(t[i].a, t[i].b, n, my, syy, sxy);
+      const double dy = __dsub_rn(my, MY), dx = __dsub_rn(t[i].mx, MX);
       const double wx = __dmul_rn(n, dx);
       SXX = __fma_rn(wx, dx, __dadd_rn(SXX, t[i].sxx));
       SYY = __fma_rn(__dmul_rn(n, dy), dy, __dadd_rn(SYY, syy));
@@ -171,6 +179,76 @@ __device__ __forceinline__ double target_rho(int n_tiles, int n_m, const float4*
   SYY = rho_sum<kLanes>(SYY);
   SXY = rho_sum<kLanes>(SXY);
   return (SXX > 0.0 && SYY > 0.0) ? __ddiv_rn(SXY, __dsqrt_rn(__dmul_rn(SXX, SYY))) : nan("");
+}
+
+// rho of a target of at most kRhoNarrow tiles by a whole warp, to the same bits as by
+// kRhoLanes lanes: the tiles' values by 32 lanes at once, then every lane adds up
+// those of its narrow lane (lane mod kRhoLanes) in that lane's order.
+struct TileRow {
+  double n, mx, my, sxx, syy, sxy, wx, dx, wy, dy;
+};
+__device__ __forceinline__ double wide_rho(int n_tiles, int n_m, const float4* base,
+                                           const ObsStat* stat, TileRow* rows) {
+  const int lane = threadIdx.x & 31, sub = lane & (kRhoLanes - 1);
+  for (int q = lane; q < n_tiles; q += 32) {
+    TileRow& t = rows[q];
+    const float4 a = base[2 * q], b = base[2 * q + 1];
+    t.n = (double)min(kQT, n_m - q * kQT);
+    t.mx = stat[q].mx;
+    t.sxx = stat[q].sxx;
+    tile_moments(a, b, t.n, t.my, t.syy, t.sxy);
+  }
+  __syncwarp();
+  double SX = 0.0, SY = 0.0;
+#pragma unroll 4
+  for (int q = sub; q < n_tiles; q += kRhoLanes) {
+    SX = __fma_rn(rows[q].n, rows[q].mx, SX);
+    SY = __fma_rn(rows[q].n, rows[q].my, SY);
+  }
+  const double inv = (double)n_m;
+  const double MX = __ddiv_rn(rho_sum<kRhoLanes>(SX), inv), MY = __ddiv_rn(rho_sum<kRhoLanes>(SY), inv);
+  for (int q = lane; q < n_tiles; q += 32) {
+    TileRow& t = rows[q];
+    t.dx = __dsub_rn(t.mx, MX);
+    t.dy = __dsub_rn(t.my, MY);
+    t.wx = __dmul_rn(t.n, t.dx);
+    t.wy = __dmul_rn(t.n, t.dy);
+  }
+  __syncwarp();
+  double SXX = 0.0, SYY = 0.0, SXY = 0.0;
+#pragma unroll 4
+  for (int q = sub; q < n_tiles; q += kRhoLanes) {
+    const TileRow& t = rows[q];
+    SXX = __fma_rn(t.wx, t.dx, __dadd_rn(SXX, t.sxx));
+    SYY = __fma_rn(t.wy, t.dy, __dadd_rn(SYY, t.syy));
+    SXY = __fma_rn(t.wx, t.dy, __dadd_rn(SXY, t.sxy));
+  }
+  SXX = rho_sum<kRhoLanes>(SXX);
+  SYY = rho_sum<kRhoLanes>(SYY);
+  SXY = rho_sum<kRhoLanes>(SXY);
+  return (SXX > 0.0 && SYY > 0.0) ? __ddiv_rn(SXY, __dsqrt_rn(__dmul_rn(SXX, SYY))) : nan("");
+}
+
+// Few targets of more tiles than a narrow lane takes at once: a warp each.  A narrow
+// lane of N = 20000 walks 20 tiles twice, four at a time: 100 targets 32 us on 13
+// SMs, 16.5 us here.  From kRhoFew targets on the pipe time of whole warps' FP64
+// instructions counts more; with 16 tiles or less the narrow lanes are as quick and a
+// launch of fewer CTAs is shorter (N = 1000, 400 targets: a cell 80.5 against 82.1 us).
+constexpr int64_t kRhoFew = 1024;
+__global__ void __launch_bounds__(kSmallThreads) rho_few_kernel(const UnitDesc* units,
+                                                                const TargetDesc* targets,
+                                                                const float4* partials,
+                                                                const ObsStat* obs_stat, double* rho) {
+  __shared__ TileRow rows[kRhoNarrow];
+  chain_begin();
+  const TargetDesc tg = targets[blockIdx.x];
+  const UnitDesc& u = units[tg.unit];
+  const float4* base = partials + 2 * (u.part_off + (blockIdx.x - u.tgt_off) * u.n_tiles);
+  const ObsStat* stat = obs_stat + tg.obs_tile;
+  const double r = u.n_tiles <= kRhoNarrow
+                       ? wide_rho(u.n_tiles, u.n_m, base, stat, rows)
+                       : target_rho<32>(u.n_tiles, u.n_m, base, stat, threadIdx.x & 31, true);
+  if (threadIdx.x == 0) rho[tg.out_idx] = r;
 }
 
 __global__ void __launch_bounds__(kSmallThreads) rho_kernel(const UnitDesc* units,
@@ -283,9 +361,12 @@ cudaError_t launch_obs(const float* series, const int32_t* order, const ObsJob* 
 }
 
 cudaError_t launch_rho(const UnitDesc* units, const TargetDesc* targets, int64_t n_targets,
-                       const float4* partials, const ObsStat* obs_stat, double* rho,
+                       int max_tiles, const float4* partials, const ObsStat* obs_stat, double* rho,
                        LaunchStream s) {
   if (n_targets <= 0) return cudaSuccess;
+  if (n_targets <= kRhoFew && max_tiles > kRhoAhead * kRhoLanes)
+    return launch_chained(rho_few_kernel, dim3((unsigned)n_targets), kSmallThreads, 0, s, units, targets,
+                          partials, obs_stat, rho);
   const int64_t blocks = (n_targets * kRhoLanes + kSmallThreads - 1) / kSmallThreads;
   return launch_chained(rho_kernel, dim3((unsigned)blocks), kSmallThreads, 0, s, units, targets,
                         n_targets, partials, obs_stat, rho);

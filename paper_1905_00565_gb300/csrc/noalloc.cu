@@ -301,7 +301,7 @@ extern "C" ccm_status ccm_run_noalloc(const float* d_series, int32_t n_series, i
   }
   e = launch_knn(kp, E, false, (int)kp.n_items, chain);
   if (e == cudaSuccess)
-    e = launch_rho(kp.units, kp.targets, r, kp.partials, kp.obs_stat, d_rho, chain);
+    e = launch_rho(kp.units, kp.targets, r, c.n_tiles, kp.partials, kp.obs_stat, d_rho, chain);
   if (e != cudaSuccess) return noalloc_fail(CCM_ECUDA, cudaGetErrorString(e));
   if (!cuda_stream) {
     int32_t err = 0;

@@ -1153,7 +1153,8 @@ ccm_status enqueue_sweep(char* base, const Arena& ar, const UnitList& ul, const 
     else
       CCM_CUDA(launch_knn_table(kt, ig.E, ig.max_nm, ig.targets == Targets::kMany, g, ls));
   }
-  CCM_CUDA(launch_rho(kp.units, kp.targets, (int64_t)ul.targets.size(), kp.partials, kp.obs_stat,
+  CCM_CUDA(launch_rho(kp.units, kp.targets, (int64_t)ul.targets.size(), (ul.max_nm + 255) / 256, kp.partials,
+                      kp.obs_stat,
                       reinterpret_cast<double*>(base + ar.rho), ls));
   if (ev) CCM_CUDA(record(ev[4], s));
   return CCM_OK;

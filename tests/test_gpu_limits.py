@@ -171,3 +171,27 @@ def test_many_targets_give_way_to_the_budget(ccm):
         np.testing.assert_array_equal(rho, want)
     finally:
         ccm.ccm_context_destroy(ctx)
+
+
+@pytest.mark.parametrize("n_m", [4096, 4097, 24576])
+def test_rho_of_few_and_of_many_targets(ccm, n_m):
+    """Up to 1024 targets of more than 16 query tiles take a warp each, more of them four
+    lanes each: the same bits, also with tiles summed in FP64 (a spike)."""
+    rng = np.random.default_rng(8)
+    s = rng.random((3, n_m), dtype=np.float32)
+    s[2, n_m // 3] = 1e30
+    ctx = ccm.ccm_context_create(0)
+    try:
+        rho = {}
+        for r in (4, 520):
+            p = I.Problem(series=s, pairs=np.array([[0, 1], [0, 2]], np.int32),
+                          E=np.array([1], np.int32), tau=np.array([1], np.int32),
+                          L=np.array([12], np.int64), r=r, seed=3)
+            plan = ccm.plan_problem(ctx, p, ccm.CCM_NO_TABLE)
+            rho[r] = np.zeros(ccm.rho_shape(p))
+            ccm.ccm_run(plan, p.series, rho[r])
+            ccm.ccm_plan_destroy(plan)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    assert np.all(np.isfinite(rho[4]))
+    np.testing.assert_array_equal(rho[4], rho[520][..., :4])

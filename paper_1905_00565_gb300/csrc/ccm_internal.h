@@ -143,6 +143,19 @@ constexpr size_t kScanSmemMax = 112 * 1024;  // shared memory of a scan CTA: two
 // zeros up to a whole number of 32 beyond the last (table rows are padded with
 // position n_m).
 __host__ __device__ constexpr int member_words(int n_m) { return (n_m + 32) / 32 * 32; }
+// Shared memory of a scan CTA: 32 vectors of predictions (vec_slot order of 256; the
+// odd stride spreads the 32 lanes' stores of one query over the banks) and the lanes'
+// records of E+1 steps; then the membership words, while two CTAs still fit an SM
+// (manifolds up to 18656 points for E = 1, 11744 for E = 10).
+constexpr int kScanThreads = 512;
+constexpr int kScanVec = 256 + 9;
+__host__ __device__ constexpr size_t scan_fixed_smem(int E) {
+  return 32 * kScanVec * 4 + (size_t)(E + 1) * kScanThreads * (4 + 2);
+}
+__host__ __device__ constexpr bool scan_words_in_smem(int E, int64_t n_m) {
+  return n_m < 65536 &&
+         scan_fixed_smem(E) + (size_t)member_words((int)n_m) * 4 <= kScanSmemMax;
+}
 // Realizations of an item of units with many targets that read a table: the
 // weights and neighbours of a query tile wait in 160 KB of shared memory.
 __host__ __device__ constexpr int lane_group(int E) {

@@ -39,17 +39,8 @@ namespace {
 
 using u64 = unsigned long long;
 
-constexpr int kScanThreads = 512;
 constexpr int kScanWarps = kScanThreads / 32;
 constexpr int kQueriesPerWarp = kQT / kScanWarps;
-// A realization's predictions of a tile (vec_slot order).  The odd stride
-// spreads the 32 lanes' stores of one query over the banks.
-constexpr int kScanVec = kQT + 9;
-
-template <int E>
-constexpr size_t scan_fixed_smem() {
-  return 32 * kScanVec * 4 + (size_t)(E + 1) * kScanThreads * (4 + 2);
-}
 
 // A realization with fewer than E+1 members in the row (rare): the warp scans
 // its whole library, every lane keeping the E+1 smallest keys of its words'
@@ -576,22 +567,12 @@ __global__ void __launch_bounds__(kGroupThreads, 1) group_kernel(KnnParams p) {
   }
 }
 
-template <int E>
-size_t scan_smem(int max_nm, bool smem_words) {
-  return scan_fixed_smem<E>() + (smem_words ? (size_t)member_words(max_nm) * 4 : 0);
-}
-
 // The membership words go to shared memory while two CTAs still fit an SM;
 // beyond that the words' spatial coherence in L1 serves better than half the
 // warps.
 template <int E>
-bool words_in_smem(int max_nm) {
-  return scan_smem<E>(max_nm, true) <= kScanSmemMax;
-}
-
-template <int E>
 auto scan_variant(int max_nm, bool u16, bool general) {
-  const bool sm = words_in_smem<E>(max_nm);
+  const bool sm = scan_words_in_smem(E, max_nm);
   if (u16) {
     if (general) return sm ? scan_kernel<E, uint16_t, true, true> : scan_kernel<E, uint16_t, false, true>;
     return sm ? scan_kernel<E, uint16_t, true, false> : scan_kernel<E, uint16_t, false, false>;
@@ -604,9 +585,11 @@ auto scan_variant(int max_nm, bool u16, bool general) {
 template <int E>
 cudaError_t KnnKernels<E>::launch_scan(const KnnParams& p, int max_nm, int grid, LaunchStream s) {
   const bool general = p.window || p.stats || p.dbg_nbr || p.dbg_xhat;
-  const bool sm = p.table_u16 && words_in_smem<E>(max_nm);
+  const size_t smem =
+      scan_fixed_smem(E) +
+      (p.table_u16 && scan_words_in_smem(E, max_nm) ? (size_t)member_words(max_nm) * 4 : 0);
   return launch_chained(scan_variant<E>(max_nm, p.table_u16 != 0, general), dim3((unsigned)grid),
-                        kScanThreads, scan_smem<E>(max_nm, sm), s, p);
+                        kScanThreads, smem, s, p);
 }
 
 template <int E>

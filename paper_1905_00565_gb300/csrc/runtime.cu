@@ -308,7 +308,7 @@ double brute_ps(int32_t E, double L) {
 }
 double scan_ps(int32_t E, double n_m, double L) {
   const double W = (E + 1 + 2.3 * std::sqrt(E + 1.0)) * n_m / L;
-  const bool in_smem = n_m <= 13000;  // membership words in shared memory (knn_scan.cu)
+  const bool in_smem = scan_words_in_smem(E, (int64_t)n_m);
   return 12.0 + 1.5 * E + 0.055 * W + (in_smem ? 0.0 : 15.0 + 0.03 * W);
 }
 double row_ps(int32_t E, double n_m, double R) {

@@ -8,6 +8,7 @@
 namespace ccm {
 
 constexpr int kMaxE = 10;
+constexpr int kSms = 152;  // a GB300's: launches are split for so many
 
 // One library realization ("unit"): library variable j, E, tau, L, realization
 // k of one job, with the targets it is cross-mapped to.  The library and the
@@ -131,7 +132,7 @@ constexpr int brute_tile_points(int E) {
 // of a tile's time), so there one item per slot is enough: with eight, 2400
 // tiles of N = 1000 and L <= 200 took 1.5 % longer.  Longer libraries are
 // staged for every tile anyway and are split to eight items per slot.
-constexpr int64_t kBruteSlots = 3 * 152;
+constexpr int64_t kBruteSlots = 3 * kSms;
 inline int32_t brute_chunk(int64_t tiles, int64_t L, int E) {
   const int64_t c = tiles / (L <= brute_tile_points(E) ? kBruteSlots : 8 * kBruteSlots);
   return c < 1 ? 1 : c > kBruteChunk ? kBruteChunk : (int32_t)c;

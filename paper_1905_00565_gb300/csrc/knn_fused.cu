@@ -151,32 +151,6 @@ __device__ __forceinline__ u64 pack_key(float d, int l) {
 __device__ __forceinline__ float key_dist(u64 k) { return __uint_as_float((uint32_t)(k >> 32)); }
 __device__ __forceinline__ int key_index(u64 k) { return (int)(uint32_t)k; }
 
-// Insert key x into the ascending list ku[0..K); a no-op when x is not below
-// the last entry.  The library is visited in any order.
-template <int K>
-__device__ __forceinline__ void insert_sorted(u64 (&ku)[K], u64 x) {
-  bool below[K];
-#pragma unroll
-  for (int s = 0; s < K; ++s) below[s] = x < ku[s];
-#pragma unroll
-  for (int s = K - 1; s > 0; --s) ku[s] = below[s - 1] ? ku[s - 1] : (below[s] ? x : ku[s]);
-  ku[0] = below[0] ? x : ku[0];
-}
-
-// Insert key x into ku[0..K) when only ku[0..n) may hold keys (the rest are
-// the empty key): the same result as insert_sorted, with the comparisons of
-// slots past n folded away when n is a compile-time constant.
-template <int K>
-__device__ __forceinline__ void insert_prefix(u64 (&ku)[K], u64 x, int n) {
-  bool below[K];
-#pragma unroll
-  for (int s = 0; s < K; ++s) below[s] = (s <= n) && x < ku[s];
-#pragma unroll
-  for (int s = K - 1; s > 0; --s)
-    if (s <= n) ku[s] = below[s - 1] ? ku[s - 1] : (below[s] ? x : ku[s]);
-  ku[0] = below[0] ? x : ku[0];
-}
-
 // A staged (tile, target) prediction vector awaiting its moments.
 struct RingMeta {
   const float2* a;    // the tile's centred observations
@@ -417,40 +391,40 @@ __device__ __forceinline__ void finish_tile(const KnnParams& p, const UnitDesc& 
     if (wide) lane_targets<E, true>(p, u, tile, nq, keep, rus, rus + kThreads);
     else lane_targets<E, false>(p, u, tile, nq, keep, rus, rus + kThreads);
   } else {
-  auto weight = [&](int s) {
-    return kKeep ? __uint_as_float((uint32_t)(keep[s * kThreads + tid] >> 32)) : w[s];
-  };
-  auto nbr = [&](int s) { return kKeep ? (int)(uint32_t)keep[s * kThreads + tid] : nbc[s]; };
-  for (int t = 0; t < u.n_targets; ++t) {
-    const TargetDesc tg = p.targets[u.tgt_off + t];
-    const float* si = p.series + u.series_off + (int64_t)tg.i * u.n;
-    float acc = 0.f;
+    auto weight = [&](int s) {
+      return kKeep ? __uint_as_float((uint32_t)(keep[s * kThreads + tid] >> 32)) : w[s];
+    };
+    auto nbr = [&](int s) { return kKeep ? (int)(uint32_t)keep[s * kThreads + tid] : nbc[s]; };
+    for (int t = 0; t < u.n_targets; ++t) {
+      const TargetDesc tg = p.targets[u.tgt_off + t];
+      const float* si = p.series + u.series_off + (int64_t)tg.i * u.n;
+      float acc = 0.f;
 #pragma unroll
-    for (int s = 0; s <= E; ++s) acc = __fmaf_rn(weight(s), si[nbr(s) + off], acc);
-    const float xhat = __fmul_rn(acc, rcp_hw(usum));  // usum >= exp(-1)
-    if (valid) {
-      if (p.dbg_xhat) p.dbg_xhat[tg.q_off + m] = xhat;
-      if (p.dbg_nbr) {
+      for (int s = 0; s <= E; ++s) acc = __fmaf_rn(weight(s), si[nbr(s) + off], acc);
+      const float xhat = __fmul_rn(acc, rcp_hw(usum));  // usum >= exp(-1)
+      if (valid) {
+        if (p.dbg_xhat) p.dbg_xhat[tg.q_off + m] = xhat;
+        if (p.dbg_nbr) {
 #pragma unroll
-        for (int s = 0; s <= E; ++s) p.dbg_nbr[tg.nbr_off + (int64_t)m * (E + 1) + s] = nbr(s);
+          for (int s = 0; s <= E; ++s) p.dbg_nbr[tg.nbr_off + (int64_t)m * (E + 1) + s] = nbr(s);
+        }
+      }
+      const int64_t rec = tg.obs_tile + tile;
+      ring[ring_n * kVecStride + vec_slot(tid)] = xhat;
+      if (tid == 0)
+        meta[ring_n] = RingMeta{p.obs + rec * kQT,
+                                p.partials + 2 * (u.part_off + (int64_t)t * u.n_tiles + tile),
+                                p.obs_stat[rec].series, nq, (int32_t)(u.tgt_off + t), tile};
+      // a full ring is reduced before the next target's vector, or at the end
+      if (++ring_n == kRing && t + 1 < u.n_targets) {
+        flush_ring(p, ring, meta, kRing);
+        ring_n = 0;
       }
     }
-    const int64_t rec = tg.obs_tile + tile;
-    ring[ring_n * kVecStride + vec_slot(tid)] = xhat;
-    if (tid == 0)
-      meta[ring_n] = RingMeta{p.obs + rec * kQT,
-                              p.partials + 2 * (u.part_off + (int64_t)t * u.n_tiles + tile),
-                              p.obs_stat[rec].series, nq, (int32_t)(u.tgt_off + t), tile};
-    // a full ring is reduced before the next target's vector, or at the end
-    if (++ring_n == kRing && t + 1 < u.n_targets) {
+    if (ring_n == kRing) {  // the weights and neighbours are dead here
       flush_ring(p, ring, meta, kRing);
       ring_n = 0;
     }
-  }
-  if (ring_n == kRing) {  // the weights and neighbours are dead here
-    flush_ring(p, ring, meta, kRing);
-    ring_n = 0;
-  }
   }
 }
 

@@ -1,7 +1,7 @@
 // Query order: a spatially coherent ordering of the manifold points of one
 // (library variable, E, tau), so that the query tiles of the fused kernel --
 // consecutive runs of this order -- hold nearby points.  Nearby queries pass
-// the running top-(E+2) thresholds on many of the same library points, so a
+// the running top-(E+1) thresholds on many of the same library points, so a
 // warp takes the rare insertion path far less often than with queries in time
 // order.  The order changes which tile a query belongs to and nothing else:
 // every query's neighbours and prediction are the same in any order.

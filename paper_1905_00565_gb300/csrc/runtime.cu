@@ -107,8 +107,7 @@ ccm_status copy_problem(const ccm_problem* p, ProblemCopy* pc) {
       return fail(CCM_EINVAL, "pair " + std::to_string(q) + " is invalid (need 0<=i,j<V, i!=j)");
   }
   {
-    // a realization completes after (query tiles) x (targets of its library
-    // variable) reductions, counted in 32 bits
+    // the interface's limit: (pairs sharing a library variable) x (query tiles) in 32 bits
     std::map<int32_t, int64_t> targets_of;
     int64_t most = 0;
     for (int32_t q = 0; q < p->n_pairs; ++q) most = std::max(most, ++targets_of[pc->pairs[2 * q]]);
@@ -581,7 +580,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         // 1.55 against 1.68.  Their byte offsets have 32 bits.
         const int32_t lanes_group =
             many(tp) && (uint64_t)pc.n * (uint64_t)st_stride * 4 < 1ull << 32
-                ? (int32_t)std::min<int64_t>(many_tiles[E] / (2 * 152), lane_group(E))
+                ? (int32_t)std::min<int64_t>(many_tiles[E] / (2 * kSms), lane_group(E))
                 : 0;
         const bool grouped = tp.size() == 1 || lanes_group >= std::min(8, lane_group(E));
         for (int64_t l = 0; l < nL; ++l) {
@@ -684,7 +683,7 @@ void append_units(const ProblemCopy& pc, int64_t series_off, int64_t out_base, U
         // walk of a mixed one is as long as its smallest L's).
         // Tiles per item: one copy of the membership words (about 4 % of a tile's
         // time) against the balance of eight items per CTA slot.
-        const int64_t slots = scan_tiles[E] / (8 * 2 * 152);
+        const int64_t slots = scan_tiles[E] / (8 * 2 * kSms);
         const int32_t chunk =
             tp.size() > 1 ? 1 : (int32_t)std::min<int64_t>(std::max<int64_t>(slots, 1), kScanChunk);
         const size_t group = tp.size() > 1 ? (size_t)lanes_group : (size_t)kScanGroup;

@@ -658,7 +658,7 @@ cudaError_t TableKernels<E>::launch(const float* series, const TableJob* jobs, i
                                     LaunchStream s) {
   // consecutive rows share a CTA (and the threshold) once there are more rows
   // than fill the SMs twice
-  const int64_t rows = n_rows / (2 * 152 * 8);
+  const int64_t rows = n_rows / (2 * kSms * 8);
   const int per = (int)(rows < 1 ? 1 : rows > 32 ? 32 : rows);
   const size_t smem = build_smem(max_R, max_nm);
   const dim3 grid((unsigned)((max_nm + per - 1) / per), (unsigned)n_jobs);

@@ -530,7 +530,7 @@ __device__ __forceinline__ void sort_keys(u64 (&k)[K]) {
 // to the K smallest keys.  At the end the column is compacted and sorted: its
 // first K keys are the E+1 nearest neighbours in (distance, index) order,
 // exactly the list the sorted insertion of every candidate would give.
-template <int E, int V, bool kLanes, bool kStats>
+template <int E, int V, bool kLanes, bool kStats, bool kPrune>
 __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, int n_chunk,
                              unsigned char* smem, RingMeta* meta, float2* qbox, int& ring_n) {
   constexpr int K = E + 1;  // the window keeps m itself out, so E+1 slots suffice
@@ -741,58 +741,56 @@ __device__ void process_item(const KnnParams& p, const UnitDesc& u, int tile0, i
         }
         if (__any_sync(kFull, cnt - done >= merge_at || cnt > room)) make_room();
       };
-      if constexpr (E <= 2) {
-        if (!p.prune) {
-          // nothing to exclude: run after run, without a mask to walk (a run is 20
-          // instructions here and the walk 6: N = 20000 in time order, E = 1, L = 400,
-          // r = 100 0.72 -> 0.64 ms)
-          for (int jg = 0; jg < ng; ++jg) {
-            int g = (base >> 6) + jg;
-            g -= (g >= ng) ? ng : 0;
-            const int end = min(32 * g + 32, np);
+      if constexpr (!kPrune) {
+        // nothing to exclude: run after run, without a mask to walk (at E = 1 a run is
+        // 20 instructions and the walk 6: N = 20000 in time order, L = 400, r = 100 0.72
+        // -> 0.64 ms)
+        for (int jg = 0; jg < ng; ++jg) {
+          int g = (base >> 6) + jg;
+          g -= (g >= ng) ? ng : 0;
+          const int end = min(32 * g + 32, np);
 #pragma unroll 2
-            for (int at = 32 * g; at < end; at += kPairs)
-              if (!(first && (unsigned)(at - (base >> 1)) < (unsigned)(kInit / 2))) step(at);
-          }
-          return;
+          for (int at = 32 * g; at < end; at += kPairs)
+            if (!(first && (unsigned)(at - (base >> 1)) < (unsigned)(kInit / 2))) step(at);
         }
-      }
+      } else {
 #pragma unroll 1
-      for (int jg = 0; jg < ng; ++jg) {
-        int g = (base >> 6) + jg;
-        g -= (g >= ng) ? ng : 0;
-        // Pruning, a lane per pair.  gap_e = max(0, lo_e - qhi_e, qlo_e - hi_e)
-        // bounds |q_e - x_e| from below for every query q of the warp and both
-        // points x of the pair, in FP32 too (rounding is monotone); summed in the
-        // distance's own order over the first D coordinates it bounds their FP32
-        // squared distances from below.  A pair whose bound exceeds every lane's
-        // threshold holds no candidate.
-        const float th_max = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(tl[K - 1])));
-        const int pr = 32 * g + lane;
-        bool keep = pr < np && !(first && (unsigned)(pr - (base >> 1)) < (unsigned)(kInit / 2));
-        if (keep && p.prune) {
-          const float2* xp = reinterpret_cast<const float2*>(s_coord + (size_t)pr * EP);
-          float lb = 0.f;
+        for (int jg = 0; jg < ng; ++jg) {
+          int g = (base >> 6) + jg;
+          g -= (g >= ng) ? ng : 0;
+          // Pruning, a lane per pair.  gap_e = max(0, lo_e - qhi_e, qlo_e - hi_e)
+          // bounds |q_e - x_e| from below for every query q of the warp and both
+          // points x of the pair, in FP32 too (rounding is monotone); summed in the
+          // distance's own order over the first D coordinates it bounds their FP32
+          // squared distances from below.  A pair whose bound exceeds every lane's
+          // threshold holds no candidate.
+          const float th_max = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(tl[K - 1])));
+          const int pr = 32 * g + lane;
+          bool keep = pr < np && !(first && (unsigned)(pr - (base >> 1)) < (unsigned)(kInit / 2));
+          if (keep && p.prune) {
+            const float2* xp = reinterpret_cast<const float2*>(s_coord + (size_t)pr * EP);
+            float lb = 0.f;
 #pragma unroll
-          for (int e = 0; e < D; ++e) {
-            const float2 x = xp[e], qb = qbox[warp * kBoxDims + e];
-            const float gp = fmaxf(fmaxf(__fsub_rn(fminf(x.x, x.y), qb.y),
-                                         __fsub_rn(qb.x, fmaxf(x.x, x.y))), 0.f);
-            lb = (e == 0) ? __fmul_rn(gp, gp) : __fmaf_rn(gp, gp, lb);
+            for (int e = 0; e < D; ++e) {
+              const float2 x = xp[e], qb = qbox[warp * kBoxDims + e];
+              const float gp = fmaxf(fmaxf(__fsub_rn(fminf(x.x, x.y), qb.y),
+                                           __fsub_rn(qb.x, fmaxf(x.x, x.y))), 0.f);
+              lb = (e == 0) ? __fmul_rn(gp, gp) : __fmaf_rn(gp, gp, lb);
+            }
+            keep = !(lb > th_max);
           }
-          keep = !(lb > th_max);
-        }
-        unsigned mask = __ballot_sync(kFull, keep);
-        if (kStats) st_pruned += 2u * (min(32, np - 32 * g) - __popc(mask)) -
-                                 (first && (base >> 6) == g ? (unsigned)kInit : 0u);
-        while (mask != 0u) {
-          // the next kept pair's aligned run of kPairs: the pairs in reach of a warp's
-          // queries lie side by side in the query order, and collecting them one by
-          // one was a chain of find-first-bits (short libraries 4.08 -> 3.97 ms, the
-          // sweep's brute force 13.3 -> 12.8, N = 10^5 17.2 -> 16.3)
-          const int b0 = (__ffs(mask) - 1) & ~(kPairs - 1);
-          mask &= ~(((1u << kPairs) - 1u) << b0);
-          step(32 * g + b0);
+          unsigned mask = __ballot_sync(kFull, keep);
+          if (kStats) st_pruned += 2u * (min(32, np - 32 * g) - __popc(mask)) -
+                                   (first && (base >> 6) == g ? (unsigned)kInit : 0u);
+          while (mask != 0u) {
+            // the next kept pair's aligned run of kPairs: the pairs in reach of a warp's
+            // queries lie side by side in the query order, and collecting them one by
+            // one was a chain of find-first-bits (short libraries 4.08 -> 3.97 ms, the
+            // sweep's brute force 13.3 -> 12.8, N = 10^5 17.2 -> 16.3)
+            const int b0 = (__ffs(mask) - 1) & ~(kPairs - 1);
+            mask &= ~(((1u << kPairs) - 1u) << b0);
+            step(32 * g + b0);
+          }
         }
       }
     };
@@ -1079,7 +1077,8 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) knn_table_kernel(KnnParams
   if (ring_n > 0) flush_ring(p, reinterpret_cast<const float*>(smem), s_meta, ring_n);
 }
 
-template <int E, bool kLanes, bool kStats>
+// kPrune false (E <= 2): for manifolds in time order, where no pair can be excluded.
+template <int E, bool kLanes, bool kStats, bool kPrune = true>
 __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -1102,9 +1101,9 @@ __global__ void __launch_bounds__(kThreads, 3) knn_fused_kernel(KnnParams p) {
       continue;
     }
     if (p.variant[E] == 1)
-      process_item<E, 1, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, s_qbox, ring_n);
+      process_item<E, 1, kLanes, kStats, kPrune>(p, u, w.tile, w.count, smem, s_meta, s_qbox, ring_n);
     else
-      process_item<E, 0, kLanes, kStats>(p, u, w.tile, w.count, smem, s_meta, s_qbox, ring_n);
+      process_item<E, 0, kLanes, kStats, kPrune>(p, u, w.tile, w.count, smem, s_meta, s_qbox, ring_n);
   }
   if (ring_n > 0)
     flush_ring(p, reinterpret_cast<const float*>(smem + kCoordBytes + kBufBytes), s_meta, ring_n);
@@ -1125,6 +1124,10 @@ size_t table_smem(int max_nm, bool lane_targets) {
 // The kernels of one E, in a translation unit of their own (CCM_E).
 template <int E>
 cudaError_t KnnKernels<E>::launch(const KnnParams& p, bool lanes, int grid, LaunchStream s) {
+  if constexpr (E <= 2)
+    if (!p.prune && !lanes && !p.stats)
+      return launch_chained(knn_fused_kernel<E, false, false, false>, dim3((unsigned)grid), kThreads,
+                            kSmemBytes, s, p);
   const auto fn = lanes ? (p.stats ? knn_fused_kernel<E, true, true> : knn_fused_kernel<E, true, false>)
                         : (p.stats ? knn_fused_kernel<E, false, true> : knn_fused_kernel<E, false, false>);
   return launch_chained(fn, dim3((unsigned)grid), kThreads, kSmemBytes, s, p);
@@ -1138,6 +1141,9 @@ cudaError_t KnnKernels<E>::prepare() {
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
   }
+  if constexpr (E <= 2)
+    return cudaFuncSetAttribute(knn_fused_kernel<E, false, false, false>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   return cudaSuccess;
 }
 

@@ -195,3 +195,28 @@ def test_rho_of_few_and_of_many_targets(ccm, n_m):
         ccm.ccm_context_destroy(ctx)
     assert np.all(np.isfinite(rho[4]))
     np.testing.assert_array_equal(rho[4], rho[520][..., :4])
+
+
+@pytest.mark.parametrize("n_m,E,L", [(16385, 1, 3), (16385, 2, 4), (16640, 1, 17), (17001, 2, 2600),
+                                     (20000, 1, 2561), (16411, 1, 5003), (16411, 3, 100)])
+def test_cells_in_time_order(ccm, n_m, E, L):
+    """Above 16384 points a cell's manifold keeps time order and nothing is pruned (a
+    search of its own for E <= 2).  The same predictions as ccm_run's in other tiles:
+    within the rounding of the sums (256 * 2^-48 * (range / std)^2 of 1e2)."""
+    torch = pytest.importorskip("torch")
+    n, r = n_m + 2 * (E - 1), 3
+    p = I.Problem(series=I.logistic_pair(n), pairs=np.array([[1, 0]], np.int32),
+                  E=np.array([E], np.int32), tau=np.array([2], np.int32),
+                  L=np.array([L], np.int64), r=r, seed=7)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        plan = ccm.plan_problem(ctx, p, ccm.CCM_NO_TABLE)
+        want = np.zeros(ccm.rho_shape(p))
+        ccm.ccm_run(plan, p.series, want)
+        ccm.ccm_plan_destroy(plan)
+    finally:
+        ccm.ccm_context_destroy(ctx)
+    s = torch.from_numpy(p.series).cuda()
+    rho = torch.full((r,), float("nan"), dtype=torch.float64, device="cuda")
+    ccm.ccm_run_noalloc(s, 1, 0, E, 2, L, r, 7, rho)
+    np.testing.assert_allclose(rho.cpu().numpy(), want.reshape(-1), rtol=0, atol=1e-10)

@@ -34,11 +34,11 @@ namespace ccm {
 // Scratch for one cell: descriptors, work items, libraries, partial moments,
 // counters, query order, observed-value tile records.  Cells are admitted up to
 // 16 MiB by a count of their own (admitted_bytes; e.g. r = 250 realizations of L
-// = 9000 at N = 10^4), which does not follow the descriptors' sizes; the array
-// has the room by which the layout may exceed it: 4 bytes a realization of a
-// single query tile, of which 16 MiB hold at most 71000, and a few roundings.
+// = 9000 at N = 10^4), which does not follow the descriptors' sizes; the layout
+// exceeds it by the roundings of its few small records at most, for which the
+// array has room.
 constexpr size_t kAdmitBytes = 16u << 20;
-constexpr size_t kScratchBytes = kAdmitBytes + (512u << 10);
+constexpr size_t kScratchBytes = kAdmitBytes + (4u << 10);
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 namespace {

@@ -1237,16 +1237,36 @@ void save_cache(const ccm_context* ctx, int E, int v, int ma) {
 
 constexpr double kTunePairs = 2.0e11;   // plans smaller than this use known or default choices
 
+// The brute-force items of one E that the tuner samples from: of one kind (of many
+// targets only where a plan has no others of this E).
+std::vector<WorkItem> tuning_items(const UnitList& ul, int E, Targets* kind) {
+  *kind = Targets::kMany;
+  for (const ItemGroup& ig : ul.groups)
+    if (ig.E == E) *kind = std::min(*kind, ig.targets);
+  std::vector<WorkItem> all;
+  for (const ItemGroup& ig : ul.groups)
+    if (ig.E == E && ig.targets == *kind)
+      all.insert(all.end(), ul.items.begin() + ig.first, ul.items.begin() + ig.first + ig.count);
+  return all;
+}
+
 ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
   ccm_context* ctx = pl->ctx;
   char* base = pl->d_arena;
   const Arena& ar = pl->ar;
   const UnitList& ul = pl->ul;
+  const int want = 6 * ctx->sm_count;
+  // an E whose libraries all read tables has nothing to measure
+  bool any = false;
+  for (int E = ul.emin; E <= ul.emax; ++E) {
+    Targets kind;
+    any |= !pl->tuning.known[E] && (int)tuning_items(ul, E, &kind).size() >= want;
+  }
+  if (!any) return CCM_OK;
   // libraries and query orders for the timing launches
   CCM_CUDA(enqueue_order(base, ar, ul, s));
   SamplerParams sp = sampler_params(base, ar, ul);
   CCM_CUDA(launch_sampler(sp, 0, (int64_t)ul.units.size(), ul.max_nm, s));
-  const int want = 6 * ctx->sm_count;
   WorkItem* d_items = nullptr;
   CCM_CUDA(cudaMallocAsync(&d_items, sizeof(WorkItem) * (size_t)want, s));
   cudaEvent_t e0, e1;
@@ -1255,13 +1275,8 @@ ccm_status autotune(ccm_plan_s* pl, cudaStream_t s) {
   ccm_status st = CCM_OK;
   for (int E = ul.emin; E <= ul.emax && st == CCM_OK; ++E) {
     if (pl->tuning.known[E]) continue;
-    // (units of many targets only where a plan has no others of this E)
-    Targets kind = Targets::kMany;
-    for (const ItemGroup& ig : ul.groups)
-      if (ig.E == E) kind = std::min(kind, ig.targets);
-    std::vector<WorkItem> all;
-    for (const WorkItem& w : ul.items)
-      if (ul.units[(size_t)w.unit].E == E && ul.targets_of(w) == kind) all.push_back(w);
+    Targets kind;
+    const std::vector<WorkItem> all = tuning_items(ul, E, &kind);
     if ((int)all.size() < want) continue;
     std::vector<WorkItem> sample;  // evenly spaced over the cost-sorted list
     for (int q = 0; q < want; ++q) sample.push_back(all[(size_t)q * all.size() / (size_t)want]);

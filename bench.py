@@ -115,7 +115,7 @@ def workload_config(name, p):
         "realizations": p.n_units(),
         "queries": p.queries(),
         "pairs": p.pair_count(),
-        "precision": "FP32 distances/selection/weights, rho moments in paired FP32 (48 bits)",
+        "precision": "FP32 distances/selection/weights, rho moments in paired FP32 (48 bits), FP64 where it needs it",
     }
 
 

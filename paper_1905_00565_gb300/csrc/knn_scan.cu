@@ -18,10 +18,10 @@
 // the walk waited on L2 (6 stalls per issue), and it ran until the slowest of
 // 128 (query, realization) was done.
 //
-// Bound: issue (57 %) and the latency of the row and pair loads behind the
+// Bound: issue (64 %) and the latency of the row and pair loads behind the
 // shuffles (ncu, E = 10).  Sweep (N = 10^4, E = 1..10, r = 250), libraries from
 // 142 points on: 151 ms with a thread per query and four realizations a walk,
-// 65 with this mapping; now that libraries from 100 points on read tables 101.
+// 65 with this mapping; now that libraries from 100 points on read tables 97.
 // Two variables of N = 10^5 (E = 3..6, L = 1000..50000; before from L = 5000 on):
 // 109 -> 31 ms.
 #include <limits.h>

@@ -165,3 +165,26 @@ def test_targets_of_two_scales(ccm, targets):
             np.testing.assert_allclose(got[fine], want[fine], rtol=0, atol=MOMENT_TOL)
     finally:
         ccm.ccm_context_destroy(ctx)
+
+
+def test_grouped_realizations_with_a_huge_value(ccm):
+    """14 targets whose realizations read their table in groups (240 of them, 12 query
+    tiles): the tiles summed again in FP64 have brute force's bits and the comparator's
+    sums."""
+    n, targets = 3000, 14
+    s = many_series(n, targets + 1, 5)
+    s[1, 1700] = 1e30
+    s[14, 5] = -3e37
+    p = I.Problem(series=s, pairs=np.array([[0, i] for i in range(1, targets + 1)], np.int32),
+                  E=np.array([3], np.int32), tau=np.array([1], np.int32),
+                  L=np.array([600, 2500], np.int64), r=120, seed=9)
+    ctx = ccm.ccm_context_create(0)
+    try:
+        got = run(ccm, ctx, p)
+        np.testing.assert_array_equal(got, run(ccm, ctx, p, ccm.CCM_NO_TABLE))
+        few = I.Problem(series=s, pairs=p.pairs, E=p.E, tau=p.tau, L=p.L, r=6, seed=p.seed)
+        want = run(ccm, ctx, few, plain=True)
+        assert np.all(np.isfinite(want))
+        np.testing.assert_allclose(got[..., :6], want, rtol=0, atol=MOMENT_TOL)
+    finally:
+        ccm.ccm_context_destroy(ctx)

@@ -1,4 +1,6 @@
 // Observed-value records, rho and the dispatch of the search kernels by E.
+#include <float.h>
+
 #include "ccm_internal.h"
 #include "launch.cuh"
 #include "moments.cuh"
@@ -48,14 +50,24 @@ __global__ void __launch_bounds__(kSmallThreads) obs_kernel(const float* series,
     const int off = (jb.E - 1) * jb.tau;
     const SeriesScale sc = scales[jb.scale];
     const float scale = sc.scale;
+    float s[kPer];
     double x[kPer];
     double sv = 0.0;
+    bool inexact = false;  // the product of some value leaves FP32's normal range
 #pragma unroll
     for (int c = 0; c < kPer; ++c) {
       const int q = lane + 32 * c;
-      x[c] = (q < nq) ? __dmul_rn((double)si[ord[q] + off], (double)scale) : 0.0;
-      sv = __dadd_rn(sv, x[c]);
+      s[c] = (q < nq) ? si[ord[q] + off] : 0.f;
+      const float scaled = __fmul_rn(s[c], scale);
+      x[c] = (double)scaled;
+      inexact |= s[c] != 0.f && fabsf(scaled) < FLT_MIN;
     }
+    if (__builtin_expect(inexact, 0)) {
+#pragma unroll
+      for (int c = 0; c < kPer; ++c) x[c] = __dmul_rn((double)s[c], (double)scale);
+    }
+#pragma unroll
+    for (int c = 0; c < kPer; ++c) sv = __dadd_rn(sv, x[c]);
     const double mx = __ddiv_rn(warp_sum(sv), (double)nq);
     double sxx = 0.0;
 #pragma unroll

@@ -150,9 +150,11 @@ def test_targets_of_two_scales(ccm, targets):
     fill[::97] = 9.97e36
     two = np.where(rng.random(n) < 0.5, np.float32(0), np.float32(1e-40))
     two[7] = 1.0
+    deep = (s[1] * np.float32(1e-20)).astype(np.float32)   # scaled, these are subnormal
+    deep[::211] = 1e37
     ctx = ccm.ccm_context_create(0)
     try:
-        for odd in (fill, two):
+        for odd in (fill, two, deep):
             series = s.copy()
             series[1] = odd
             p = I.Problem(series=series,

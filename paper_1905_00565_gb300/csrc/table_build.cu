@@ -254,7 +254,8 @@ __device__ __noinline__ Threshold next_threshold(const Point<E> q, const TableJo
     else if (s.have_lo) t.tb = s.lo > 0xffffffffu - s.step ? 0xffffffffu : s.lo + s.step;
     else t.tb = s.hi > s.step ? s.hi - s.step : 0u;
   }
-  while (!step && !tied) {
+  // (four turns cover 32 bits; the bound ends the loop whatever the counts say)
+  for (int turn = 0; !step && !tied && turn < 8; ++turn) {
     const uint32_t from = s.have_lo ? s.lo + 1u : 0u;
     const uint32_t span = s.ties ? (uint32_t)(s.hi_m - s.lo_m - 1) : s.hi - from;
     int shift = 0;
